@@ -109,12 +109,12 @@ __global__ void popularity_kernel(const IDT *tables, uint64_t n_lists, uint32_t 
     if (id < N) atomicAdd(score + id, (unsigned long long)(T - r));
 }
 
-// Library-owned copies for the input-stationary kernels (layers whose input is the (id, value) list of
-// an activator layer below them):
+// Library-owned copies for the kernels that read weights by input (a first layer with dense input, and layers
+// whose input is the (id, value) list of an activator layer below them):
 //   WT      transposed weights [D][N]; on a layer that has its own activator the node axis is stored in
 //           the order of `colpos`: nodes that sit early in many ranked lists first, so that the nodes a
 //           query selects lie close together in every row of WT
-//   colpos  [N] node id -> column of WT (activator layers only; NULL = identity)
+//   colpos  [N] node id -> column of WT (activator layers only; NULL = identity); colnode is its inverse
 //   WH      [D][32] the layer's hash rows side by side (activator layers with K*L <= 32)
 // and the plain transposed copy of a first layer fed by CSR rows.  phase 0: the CSR first layer (needed
 // by the calibration pass); phase 1: the rest (needs the finished tables).
@@ -125,9 +125,10 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
     for (uint32_t l = 0; l < m->n_layers; ++l) {
         slonn_layer &ly = m->layer[l];
         const bool csr_first = (l == 0 && m->first_sparse);
-        const bool list_input = (l > 0 && m->layer[l - 1].has_act && (uint64_t)ly.N * ly.D * esz < (1ull << 32));
-        if (phase == 0 ? !csr_first : !list_input) continue;
-        if (cudaMalloc(&ly.WT, (uint64_t)ly.N * ly.D * esz) != cudaSuccess) return SLONN_ERR_NOMEM;
+        const uint64_t wt_bytes = (uint64_t)ly.N * ly.D * esz;
+        const bool by_input = (l == 0 ? !m->first_sparse : m->layer[l - 1].has_act) && wt_bytes < (1ull << 32);
+        if (phase == 0 ? !csr_first : !by_input) continue;
+        if (cudaMalloc(&ly.WT, wt_bytes) != cudaSuccess) return SLONN_ERR_NOMEM;
         const dim3 grid((ly.D + 31) / 32, (ly.N + 31) / 32), block(32, 8);
         if (!ly.has_act || csr_first) {
             transpose_kernel<<<grid, block, 0, st>>>(ly.W, ly.WT, ly.N, ly.D, esz);
@@ -159,7 +160,9 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
         std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) { return score[a] > score[b]; });
         for (uint32_t i = 0; i < ly.N; ++i) colpos[order[i]] = i;
         if (cudaMalloc(&ly.colpos, sizeof(uint32_t) * ly.N) != cudaSuccess) return SLONN_ERR_NOMEM;
-        if (cudaMemcpyAsync(ly.colpos, colpos.data(), sizeof(uint32_t) * ly.N, cudaMemcpyHostToDevice, st) != cudaSuccess)
+        if (cudaMalloc(&ly.colnode, sizeof(uint32_t) * ly.N) != cudaSuccess) return SLONN_ERR_NOMEM;
+        if (cudaMemcpyAsync(ly.colpos, colpos.data(), sizeof(uint32_t) * ly.N, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+            cudaMemcpyAsync(ly.colnode, order.data(), sizeof(uint32_t) * ly.N, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return SLONN_ERR_CUDA;
         transpose_permuted_kernel<<<grid, block, 0, st>>>(ly.W, ly.WT, ly.N, ly.D, esz, ly.colpos);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
@@ -168,7 +171,7 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
             hash_matrix_kernel<<<(ly.D * 32 + 255) / 256, 256, 0, st>>>(ly.W, ly.WH, ly.D, esz, ly.hash_nodes, m->H);
             if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
         }
-        if (cudaStreamSynchronize(st) != cudaSuccess) return SLONN_ERR_CUDA; // colpos.data() is read by the copy above
+        if (cudaStreamSynchronize(st) != cudaSuccess) return SLONN_ERR_CUDA; // the copies above read colpos.data() and order.data()
     }
     return SLONN_OK;
 }
@@ -568,6 +571,7 @@ extern "C" void slonn_free(slonn_model *m)
         cudaFree(m->layer[l].hash_nodes);
         cudaFree(m->layer[l].WT);
         cudaFree(m->layer[l].colpos);
+        cudaFree(m->layer[l].colnode);
         cudaFree(m->layer[l].WH);
     }
     m->magic = 0;

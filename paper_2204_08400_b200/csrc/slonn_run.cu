@@ -8,6 +8,7 @@
 #include "slonn_dense_tc.cuh"
 #include "slonn_fused_kernel.cuh"
 #include "slonn_run_kernels.cuh"
+#include "slonn_tile_kernels.cuh"
 #include "slonn_cluster_kernel.cuh"
 
 namespace {
@@ -63,7 +64,14 @@ uint32_t dense_width(const slonn_model *m)
 }
 
 struct ws_layout {
-    uint64_t indptr, plan_sums, ids, vals, dense0, dense1, tc_list, tc_count, tc_a0, tc_a1, total;
+    uint64_t indptr, plan_sums, ids, vals, dense0, dense1, tc_list, tc_count, tc_a0, tc_a1;
+    uint64_t total;              // what a call needs at least
+    struct {                     // grouped products (slonn_tile_kernels.cuh), behind the rest
+        uint64_t order, key, work, items, kseg, krow, xt, ucol, ucount, bm, pre;
+        uint32_t chunk;          // queries staged at a time, 0: this batch does not take them
+        uint32_t order_stride;   // entries of `order` per chunk
+    } tile;
+    uint64_t total_tile;         // what a call needs to take them (== total when it does not)
 };
 
 // widest bf16 activation matrix row the tensor-core route needs
@@ -85,6 +93,87 @@ bool tc_route(const slonn_model *m, uint32_t max_bp, uint32_t flags)
 bool full_route_possible(const slonn_model *m, uint32_t max_bp)
 {
     return max_bp == 10000u && !m->first_sparse;
+}
+
+// ---- layers as grouped products ------------------------------------------------------
+
+// When a batch takes grouped products (measured on 4096-4096x8-1000, 1024-2048x4-500 bf16 and 1024-1536x3-300 fp32,
+// 64 to 4096 queries): from 256 queries on (50 % budget, 256 queries: 2.60 -> 1.81, 0.54 -> 0.45, 0.36 -> 0.30 ms; 128
+// queries: 1.38 -> 1.33, 0.27 -> 0.33, 0.20 -> 0.24), and from 64 queries on when the largest budget gives the batch
+// many rows (mixed budgets up to 100 %, 64 and 128 queries on the widest network: 2.66 -> 1.60, 3.03 -> 1.38 ms).
+#define SLONN_TILE_MIN_QUERIES 256u
+#define SLONN_TILE_FEW_QUERIES 64u
+#define SLONN_TILE_FEW_ROWS (148ull * 1536)
+// A layer without activator (every node): from 512 queries on (1000 outputs, 4096 queries at 10 %: 0.26 -> 0.15 ms).
+#define SLONN_TILE_DENSE_MIN_QUERIES 512u
+// Of a list-fed activator layer, the queries whose budget is at most this many nodes keep layer_cols_kernel, which needs no
+// grouping: 4096 queries, 512 nodes of 2048: 1.70 -> 1.54 ms, 307 nodes: 0.97 -> 1.03, 384 nodes of 1536: 1.04 -> 1.07;
+// 410 nodes of 4096: 3.25 -> 3.07 with 4096 queries, 0.73 -> 0.76 with 512.
+#define SLONN_TILE_NODES 512u
+#define SLONN_TILE_NODES_LARGE 400u // batches of at least SLONN_TILE_LARGE queries
+#define SLONN_TILE_LARGE 2048u
+
+// whether layer l can be evaluated as grouped products
+bool tile_layer_ok(const slonn_model *m, uint32_t l)
+{
+    const slonn_layer &ly = m->layer[l];
+    return ly.WT && !(l == 0 && m->first_sparse) && ly.N <= SLONN_TILE_MAX_N;
+}
+
+// entries a group of layer l stages at most
+uint32_t tile_kcap(const slonn_model *m, uint32_t l, uint32_t max_bp)
+{
+    const slonn_layer &ly = m->layer[l];
+    uint64_t k = ly.D;
+    if (l > 0 && m->layer[l - 1].has_act)
+        k = std::min<uint64_t>(k, (uint64_t)SLONN_TILE_G * slonn_layer_nodes(max_bp, ly.D, slonn_model_pre(m)));
+    return (uint32_t)align_up(k + 32 + SLONN_TILE_SLACK, 4);
+}
+
+// whether a batch takes them (workspace permitting)
+bool tile_wanted(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags)
+{
+    if (flags & (SLONN_FLAG_ROW_KERNELS | SLONN_FLAG_COLUMN_KERNELS | SLONN_FLAG_UNGROUPED_ROWS)) return false;
+    uint32_t rows = 0; // most rows a layer that can take them computes for a query
+    for (uint32_t l = 0; l < m->n_layers; ++l)
+        if (tile_layer_ok(m, l))
+            rows = std::max(rows, m->layer[l].has_act ? slonn_layer_nodes(max_bp, m->layer[l].N, slonn_model_pre(m)) : m->layer[l].N);
+    return rows && (n >= SLONN_TILE_MIN_QUERIES || (n >= SLONN_TILE_FEW_QUERIES && (uint64_t)n * rows >= SLONN_TILE_FEW_ROWS));
+}
+
+void carve_tile(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags, ws_layout &w)
+{
+    memset(&w.tile, 0, sizeof(w.tile));
+    w.total_tile = w.total;
+    if (!tile_wanted(m, n, max_bp, flags)) return;
+    uint32_t kcap = 0, widest = 0;
+    for (uint32_t l = 0; l < m->n_layers; ++l) {
+        if (!tile_layer_ok(m, l)) continue;
+        kcap = std::max(kcap, tile_kcap(m, l, max_bp));
+        widest = std::max(widest, m->layer[l].N);
+    }
+    const uint32_t nwords = (widest + 31u) / 32u;
+    // staged values, bitmaps and prefixes per query; at most 160 MiB of them at a time
+    const uint64_t per_query = (uint64_t)kcap * 4 + (uint64_t)nwords * 8 + ((uint64_t)kcap + 2 * widest) * 4 / SLONN_TILE_G;
+    const uint64_t fit = std::max<uint64_t>((160ull << 20) / per_query / SLONN_TILE_G, 1) * SLONN_TILE_G;
+    const uint32_t chunk = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(fit, SLONN_TILE_CHUNK), align_up(n, SLONN_TILE_G));
+    const uint64_t groups = (chunk + SLONN_TILE_G - 1) / SLONN_TILE_G, chunks = ((uint64_t)n + chunk - 1) / chunk;
+    w.tile.chunk = chunk;
+    w.tile.order_stride = (uint32_t)groups * SLONN_TILE_G;
+    uint64_t o = w.total;
+    auto take = [&](uint64_t bytes) { const uint64_t at = o; o = align_up(o + bytes, 256); return at; };
+    w.tile.order = take(chunks * w.tile.order_stride * 4);
+    w.tile.key = take((uint64_t)n * 8);
+    w.tile.work = take(256);
+    w.tile.items = take(groups * ((widest + SLONN_TILE_COLS - 1) / SLONN_TILE_COLS) * 4);
+    w.tile.kseg = take(groups * 33 * 4);
+    w.tile.krow = take(groups * kcap * 4);
+    w.tile.xt = take(groups * kcap * SLONN_TILE_G * 4);
+    w.tile.ucol = take(groups * widest * 8);
+    w.tile.ucount = take(groups * 4);
+    w.tile.bm = take(groups * nwords * SLONN_TILE_G * 4);
+    w.tile.pre = take(groups * nwords * SLONN_TILE_G * 4);
+    w.total_tile = o;
 }
 
 ws_layout carve(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags)
@@ -110,6 +199,7 @@ ws_layout carve(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
         w.tc_a1 = o; o += ab;
     }
     w.total = std::max<uint64_t>(o, 256);
+    carve_tile(m, n, max_bp, flags, w);
     return w;
 }
 
@@ -362,12 +452,43 @@ int launch_layer_cols_s(const slonn_layer_cols_params &Q, bool split, uint64_t g
                            : launch_layer_cols_t<BF16, IDT, false, false>(Q, grid, threads, smem, st);
 }
 
+template <bool BF16, typename IDT>
+int launch_select_cols_t(const slonn_layer_cols_params &Q, uint32_t n, size_t smem, cudaStream_t st)
+{
+    const int rc = set_smem(hash_select_cols_kernel<BF16, IDT>, smem);
+    if (rc) return rc;
+    hash_select_cols_kernel<BF16, IDT><<<n, SLONN_THREADS, smem, st>>>(Q);
+    return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
+}
+
+// Hash and selection of a list-fed activator layer, input-stationary.  SLONN_ERR_DIM: no side-by-side hash rows, or the
+// staging does not fit -- the caller takes hash_select_kernel.
+int launch_select_cols(const slonn_model *m, const slonn_layer &ly, uint32_t layer, slonn_gather_params G, const slonn_batch *b,
+                       uint64_t *sort_key, uint32_t n, uint32_t max_rows, cudaStream_t st)
+{
+    if (!ly.WH || G.in.kind != SLONN_IN_LIST) return SLONN_ERR_DIM;
+    const bool bf = m->dtype == SLONN_BF16, id16 = ly.id_bytes == 2;
+    G.rows_cap = max_rows;
+    size_t scratch = std::max(cols_image_bytes(G.D, bf ? 8u : 4u), (size_t)32 * 32 * 4);
+    scratch = (scratch + 15) & ~(size_t)15;
+    G.scratch_bytes = (uint32_t)scratch;
+    const size_t smem = scratch + (size_t)cols_ent_cap(G.D, G.in_cap) * 8 + (size_t)((G.N + 31u) / 32u) * 4;
+    if (smem > 200 * 1024) return SLONN_ERR_DIM;
+    slonn_layer_cols_params Q;
+    memset(&Q, 0, sizeof(Q));
+    Q.G = G; Q.WH = ly.WH; Q.hash_nodes = ly.hash_nodes; Q.tables = ly.tables; Q.cap = ly.cap;
+    Q.K = m->K; Q.L = m->L; Q.pre = slonn_model_pre(m); Q.layer = layer; Q.codes = b->codes; Q.status = b->status;
+    Q.sort_key = sort_key; Q.budget_bp = b->budget_bp;
+    if (bf) return id16 ? launch_select_cols_t<true, uint16_t>(Q, n, smem, st) : launch_select_cols_t<true, uint32_t>(Q, n, smem, st);
+    return id16 ? launch_select_cols_t<false, uint16_t>(Q, n, smem, st) : launch_select_cols_t<false, uint32_t>(Q, n, smem, st);
+}
+
 // Hash, selection and input-stationary gather of a list-fed activator layer in one launch: one block per
 // query, or, for batches of tens of queries, one block per (query, 64 nodes) with the selection repeated in
 // every block of a query.  SLONN_ERR_DIM: not applicable here (no side-by-side hash rows, or the staging
 // does not fit) -- the caller takes the separate kernels.
 int launch_layer_cols(const slonn_model *m, const slonn_layer &ly, uint32_t layer, slonn_gather_params G,
-                      const slonn_batch *b, uint32_t n, uint32_t max_rows, cudaStream_t st)
+                      const slonn_batch *b, uint32_t n, uint32_t max_rows, cudaStream_t st, uint64_t *sort_key = nullptr)
 {
     if (!ly.WH || !ly.WT || !ly.colpos || !G.use_list) return SLONN_ERR_DIM;
     const uint32_t passes = (max_rows + 63u) / 64u;
@@ -392,6 +513,7 @@ int launch_layer_cols(const slonn_model *m, const slonn_layer &ly, uint32_t laye
     memset(&Q, 0, sizeof(Q));
     Q.G = G; Q.WH = ly.WH; Q.hash_nodes = ly.hash_nodes; Q.tables = ly.tables; Q.cap = ly.cap;
     Q.K = m->K; Q.L = m->L; Q.pre = slonn_model_pre(m); Q.layer = layer; Q.codes = b->codes; Q.status = b->status;
+    Q.sort_key = sort_key; Q.budget_bp = b->budget_bp;
     const bool id16 = ly.id_bytes == 2;
     if (bf) return id16 ? launch_layer_cols_s<true, uint16_t>(Q, split, grid, warps * 32u, smem, st) : launch_layer_cols_s<true, uint32_t>(Q, split, grid, warps * 32u, smem, st);
     return id16 ? launch_layer_cols_s<false, uint16_t>(Q, split, grid, warps * 32u, smem, st) : launch_layer_cols_s<false, uint32_t>(Q, split, grid, warps * 32u, smem, st);
@@ -480,6 +602,128 @@ int launch_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, sl
     TOC();
     if (rc) return rc;
     return launch_layer_rows(m, ly, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm);
+}
+
+// ---- layers as grouped products: launches ------------------------------------------
+
+// The scratch of grouped products in a call's workspace; ws == NULL: the call does not take them.
+struct tile_ws { char *ws; const ws_layout *wl; };
+
+template <bool BF16, bool QUAD>
+int launch_tile_rows_t(const slonn_tile_params &P, cudaStream_t st)
+{
+    const int rc = set_smem(tile_rows_kernel<BF16, QUAD>, SLONN_TILE_SMEM);
+    if (rc) return rc;
+    tile_rows_kernel<BF16, QUAD><<<148u, SLONN_TILE_WARPS * 32, SLONN_TILE_SMEM, st>>>(P);
+    return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
+}
+
+template <bool BF16>
+int launch_tile_rows(const slonn_tile_params &P, cudaStream_t st)
+{
+    return !P.select && P.N % 4u == 0 ? launch_tile_rows_t<BF16, true>(P, st) : launch_tile_rows_t<BF16, false>(P, st);
+}
+
+// Sorts the batch's queries with a budget in [lo, hi] into groups by (budget, keys); the keys were written by the kernel
+// that hashed them.  *sorted: lowest budget of the groups the workspace held before (~0: none) and holds now; as long as
+// it stays, the same number of entries is overwritten.
+int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint32_t lo, uint32_t hi, uint32_t *sorted, cudaStream_t st)
+{
+    const auto &T = tw.wl->tile;
+    const uint64_t chunks = ((uint64_t)n + T.chunk - 1) / T.chunk;
+    if (*sorted != lo && cudaMemsetAsync(tw.ws + T.order, 0xff, chunks * T.order_stride * 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
+    *sorted = lo;
+    for (uint32_t c = 0, q0 = 0; q0 < n; ++c, q0 += T.chunk) {
+        slonn_order_params P;
+        P.key = (const uint64_t *)(tw.ws + T.key); P.budget_bp = b->budget_bp; P.bp_lo = lo; P.bp_hi = hi; P.q0 = q0; P.n = std::min(T.chunk, n - q0);
+        P.work = (uint32_t *)(tw.ws + T.work); P.order = (uint32_t *)(tw.ws + T.order) + (uint64_t)c * T.order_stride;
+        tile_order_kernel<<<(P.n + 31) / 32, 256, 0, st>>>(P);
+        if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
+    }
+    return SLONN_OK;
+}
+
+// One layer for the whole batch.  order_kind: 0 queries as they come (without those of skip_bp), 1 the order of
+// launch_tile_order, 2 the compacted list `list` of *count queries.  fresh_order: launch_tile_order was the launch before.
+int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, const slonn_gather_params &G, uint32_t n, uint32_t max_bp,
+                      const tile_ws &tw, int order_kind, const uint32_t *list, const uint32_t *count, bool write_ids, cudaStream_t st,
+                      bool fresh_order = false)
+{
+    const auto &T = tw.wl->tile;
+    const bool bf = m->dtype == SLONN_BF16;
+    slonn_tile_params P;
+    memset(&P, 0, sizeof(P));
+    P.in = G.in; P.D = ly.D; P.N = ly.N; P.V = bf ? 8u : 4u;
+    P.kcap = tile_kcap(m, l, max_bp); P.wps = (cols_smax(ly.D, P.V) + 31u) / 32u;
+    P.WT = ly.WT; P.ldb = ly.N * (bf ? 2u : 4u); P.colpos = ly.colpos; P.colnode = ly.colnode; P.bias = ly.bias; P.relu = G.relu;
+    P.select = G.use_list; P.n_act = G.n_act; P.a = G.a; P.indptr = G.indptr; P.ids = const_cast<uint32_t *>(G.ids); P.write_ids = write_ids ? 1u : 0u;
+    P.out_vals = G.out_vals; P.out_dense = G.out_dense; P.out_dense_ids = G.out_dense_ids; P.out_stride = G.out_stride;
+    P.nwords = (ly.N + 31u) / 32u;
+    P.work = (uint32_t *)(tw.ws + T.work); P.items = (uint32_t *)(tw.ws + T.items);
+    P.kseg = (uint32_t *)(tw.ws + T.kseg); P.krow = (uint32_t *)(tw.ws + T.krow); P.xt = (float *)(tw.ws + T.xt);
+    P.ucol = (uint2 *)(tw.ws + T.ucol); P.ucount = (uint32_t *)(tw.ws + T.ucount);
+    P.bm = (uint32_t *)(tw.ws + T.bm); P.pre = (uint32_t *)(tw.ws + T.pre);
+    const size_t smem = std::max((size_t)64 * P.wps, P.select ? (size_t)(SLONN_TILE_G + 1) * P.nwords : 0) * 4;
+    int rc = set_smem(tile_prep_kernel, smem);
+    if (rc) return rc;
+    for (uint32_t c = 0, q0 = 0; q0 < n; ++c, q0 += T.chunk) {
+        P.q0 = q0; P.s0 = q0; P.n = std::min(T.chunk, n - q0); P.skip_bp = nullptr; P.count = nullptr; P.order = nullptr;
+        if (order_kind == 0) P.skip_bp = G.skip_bp;
+        else if (order_kind == 1) P.order = (const uint32_t *)(tw.ws + T.order) + (uint64_t)c * T.order_stride;
+        else { P.order = list + q0; P.count = count; }
+        P.groups = (P.n + SLONN_TILE_G - 1) / SLONN_TILE_G;
+        // the sort cleared the count of work items; only the first chunk can rely on it
+        if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
+        tile_prep_kernel<<<dim3(P.groups, 2), 512, smem, st>>>(P);
+        if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
+        rc = bf ? launch_tile_rows<true>(P, st) : launch_tile_rows<false>(P, st);
+        if (rc) return rc;
+    }
+    return SLONN_OK;
+}
+
+// Budgets 1..limit of a list-fed activator layer keep the one-launch input-stationary kernel; the others are evaluated
+// in groups.
+uint32_t tile_budget_limit(const slonn_layer &ly, uint32_t n)
+{
+    return std::min((n >= SLONN_TILE_LARGE ? SLONN_TILE_NODES_LARGE : SLONN_TILE_NODES) * 10000u / ly.N, SLONN_COLS_MAX_BP);
+}
+
+// A list-fed activator layer of a batch that takes grouped products.  *sorted: see launch_tile_order.
+int launch_tile_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, slonn_select_params &sp, slonn_gather_params &gp,
+                          const slonn_batch *b, uint32_t n, uint32_t max_bp, uint32_t max_rows, uint32_t in_cap, const tile_ws &tw,
+                          uint32_t *sorted, cudaStream_t st, stage_timer *tm)
+{
+    uint64_t *key = (uint64_t *)(tw.ws + tw.wl->tile.key);
+    const uint16_t *skip_bp = gp.skip_bp;
+    const uint32_t limit = std::min(tile_budget_limit(ly, n), max_bp), pre = slonn_model_pre(m);
+    int rc;
+    uint32_t lo = 0;
+    if (ly.WH && limit) { // the low budgets
+        slonn_gather_params C = gp;
+        C.WT = ly.WT; C.colpos = ly.colpos;
+        if (max_bp > limit) { C.range_bp = b->budget_bp; C.bp_lo = 0; C.bp_hi = limit; }
+        C.in_cap = std::min(in_cap, slonn_layer_nodes(limit, ly.D, pre));
+        TIC(SLONN_STAGE_LAYER_COLS, C.range_bp, C.bp_lo, C.bp_hi, C.skip_bp);
+        rc = launch_layer_cols(m, ly, l, C, b, n, std::min(max_rows, slonn_layer_nodes(limit, ly.N, pre)), st, key);
+        TOC();
+        if (rc == SLONN_OK) lo = limit + 1u;
+        else if (rc != SLONN_ERR_DIM) return rc;
+    }
+    if (lo > max_bp) return SLONN_OK;
+    const uint32_t hi = skip_bp ? 9999u : 10000u;
+    if (lo) { gp.range_bp = sp.range_bp = b->budget_bp; gp.bp_lo = sp.bp_lo = lo; gp.bp_hi = sp.bp_hi = 0xffffu; }
+    sp.sort_key = key; sp.budget_bp = b->budget_bp;
+    TIC(SLONN_STAGE_HASH_SELECT, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp);
+    rc = launch_select_cols(m, ly, l, gp, b, key, n, max_rows, st);
+    if (rc == SLONN_ERR_DIM) rc = launch_select(m, sp, n, max_rows, st);
+    TOC();
+    if (rc) return rc;
+    TIC(SLONN_STAGE_GROUP_ROWS, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp);
+    rc = launch_tile_order(tw, b, n, lo, hi, sorted, st);
+    if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 1, nullptr, nullptr, false, st, true);
+    TOC();
+    return rc;
 }
 
 // ---- 100 % queries, four per block ---------------------------------------------
@@ -759,7 +1003,7 @@ extern "C" int slonn_workspace_bytes(const slonn_model *m, uint32_t n, uint32_t 
                                      uint64_t *bytes)
 {
     if (!model_ok(m) || !bytes) return SLONN_ERR_ARG;
-    *bytes = carve(m, n, eff_max_bp(max_bp), flags).total;
+    *bytes = carve(m, n, eff_max_bp(max_bp), flags).total_tile;
     return SLONN_OK;
 }
 
@@ -767,7 +1011,7 @@ extern "C" int slonn_workspace_bytes(const slonn_model *m, uint32_t n, uint32_t 
 // nothing with the other queries but the output arrays (disjoint entries), so this runs as a pass of its own.
 static int run_full_route(const slonn_model *m, const slonn_batch *b, uint32_t n, const uint32_t *list, const uint32_t *count,
                           const uint64_t *indptr, uint32_t *ids, float *vals, float *const dense[2], uint32_t stride,
-                          cudaStream_t st, stage_timer *tm)
+                          uint32_t max_bp, const tile_ws &tw, cudaStream_t st, stage_timer *tm)
 {
     slonn_input in;
     memset(&in, 0, sizeof(in));
@@ -792,7 +1036,17 @@ static int run_full_route(const slonn_model *m, const slonn_batch *b, uint32_t n
         }
         AT_LAYER(l);
         TIC(SLONN_STAGE_FULL_ROWS, b->budget_bp, 10000u, 10000u);
-        const int rc = launch_full_rows(m, fp, n, st);
+        int rc;
+        if (tw.ws && tile_layer_ok(m, l)) {
+            slonn_gather_params gp;
+            memset(&gp, 0, sizeof(gp));
+            gp.in = in; gp.n_act = m->n_act; gp.a = fp.a; gp.relu = fp.relu;
+            if (ly.has_act) { gp.indptr = indptr; gp.ids = ids; gp.out_vals = vals; }
+            gp.out_dense = fp.out_dense; gp.out_dense_ids = fp.out_dense_ids; gp.out_stride = fp.out_stride;
+            rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 2, list, count, ly.has_act != 0, st);
+        } else {
+            rc = launch_full_rows(m, fp, n, st);
+        }
         TOC();
         if (rc) return rc;
         if (ly.has_act) {
@@ -847,6 +1101,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
 
     uint32_t stride = 0;
     slonn_logit_stride(m, max_bp, &stride);
+    // grouped products: when the workspace has room for their scratch, else the kernels that need none
+    const tile_ws tw = {wl.tile.chunk && ws_bytes >= wl.total_tile ? ws : nullptr, &wl};
 
     // a handful of queries: one thread-block cluster per query, every layer in one launch (it derives the
     // list offsets itself, so no planning launch either)
@@ -963,7 +1219,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
         if (cudaMemsetAsync(full_count, 0, sizeof(uint32_t), st) != cudaSuccess) return SLONN_ERR_CUDA;
         dense_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, n, full_list, full_count);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
-        const int rc = run_full_route(m, b, n, full_list, full_count, indptr, ids, vals, dense, stride, st, tm);
+        const int rc = run_full_route(m, b, n, full_list, full_count, indptr, ids, vals, dense, stride, max_bp, tw, st, tm);
         if (rc) return rc;
         skip_bp = b->budget_bp;
     }
@@ -1002,6 +1258,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
     int dense_cur = 0;
     uint32_t in_cap = 0; // most entries the current input list holds (list inputs only)
     const group_ws gw = {(uint32_t *)(ws + wl.tc_list), (uint32_t *)(ws + wl.tc_count)};
+    uint32_t sorted = ~0u; // lowest budget of the queries the groups in the workspace hold (~0: no groups)
+    bool keyed = false;    // the workspace holds the sort keys of every query from the last activator layer
 
     for (uint32_t l = 0; l < m->n_layers; ++l) {
         const slonn_layer &ly = m->layer[l];
@@ -1041,7 +1299,15 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             max_rows = slonn_layer_nodes(max_bp, ly.N, slonn_model_pre(m));
             gp.use_list = 1; gp.a = a; gp.out_vals = vals;
             if (is_last) { gp.out_dense = b->logits; gp.out_dense_ids = b->logit_ids; gp.out_stride = stride; }
-            rc = launch_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm);
+            if (tw.ws && tile_layer_ok(m, l) && in.kind == SLONN_IN_LIST) {
+                gp.in_cap = in_cap;
+                rc = launch_tile_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, tw, &sorted, st, tm);
+                keyed = true;
+            } else {
+                keyed = tw.ws && in.kind == SLONN_IN_DENSE; // hash_select_kernel serves every query
+                if (keyed) { sp.sort_key = (uint64_t *)(ws + wl.tile.key); sp.budget_bp = b->budget_bp; }
+                rc = launch_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm);
+            }
             if (rc) return rc;
             in.kind = SLONN_IN_LIST; in.indptr = indptr; in.ids = ids; in.vals = vals;
             in.ip_mul = m->n_act; in.ip_add = a;
@@ -1054,6 +1320,17 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             // serve (budgets above the input-stationary limit) share all their weight rows, so they are
             // compacted and taken four per block.
             bool rows_done = false;
+            if (tw.ws && tile_layer_ok(m, l) && n >= SLONN_TILE_DENSE_MIN_QUERIES) {
+                TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp);
+                rc = SLONN_OK;
+                if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp ? 9999u : 10000u, &sorted, st);
+                if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, keyed);
+                TOC();
+                if (rc) return rc;
+                in.kind = SLONN_IN_DENSE; in.dense = gp.out_dense;
+                dense_cur ^= 1;
+                continue;
+            }
             const uint32_t cols_bp = cols_budget_limit(ly, gp, b, n, max_rows, max_bp);
             if (n >= 256 && (uint64_t)n * ly.N * ly.D >= (1ull << 30) && (size_t)SLONN_FULL_GROUP * ly.D * 4 <= 200 * 1024 &&
                 cols_bp < max_bp) {
@@ -1211,6 +1488,7 @@ namespace {
 struct host_layout {
     uint64_t x, indptr_in, ids_in, vals_in, bp, logits, logit_ids, pred, codes, a_indptr, a_ids, a_vals, status,
         inner, total;
+    uint64_t total_tile; // the same with room for grouped products
 };
 
 host_layout carve_host(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags, uint64_t x_nnz)
@@ -1239,8 +1517,24 @@ host_layout carve_host(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32
     h.a_vals = take(ent * 4);
     h.status = take(16);
     h.inner = o;
-    h.total = o + carve(m, n, max_bp, flags).total + 512; // + status words of a batch run in pieces
+    const ws_layout w = carve(m, n, max_bp, flags);
+    h.total = o + w.total + 512; // + status words of a batch run in pieces
+    h.total_tile = o + w.total_tile + 512;
     return h;
+}
+
+// Queries per piece of a host batch that goes through in pieces (see slonn_run_host); *pieces = 1: in one piece.
+uint32_t host_piece(const slonn_model *m, uint32_t n, uint32_t *pieces)
+{
+#ifndef SLONN_PIECE_QUERIES
+    const uint64_t row_bytes = (uint64_t)m->layer[0].D * sizeof(float);
+    const uint32_t piece_min = (uint32_t)std::min<uint64_t>(2048u, std::max<uint64_t>(1024u, (16ull << 20) / std::max<uint64_t>(row_bytes, 1)));
+#else
+    const uint32_t piece_min = SLONN_PIECE_QUERIES;
+#endif
+    *pieces = std::min(8u, std::max(1u, n / piece_min));
+    const uint32_t piece = (n + *pieces - 1) / *pieces;
+    return (piece + 255u) / 256u * 256u;
 }
 } // namespace
 
@@ -1248,7 +1542,13 @@ extern "C" int slonn_host_workspace_bytes(const slonn_model *m, uint32_t n, uint
                                           uint64_t x_nnz, uint64_t *bytes)
 {
     if (!model_ok(m) || !bytes) return SLONN_ERR_ARG;
-    *bytes = carve_host(m, n, eff_max_bp(max_bp), flags, x_nnz).total;
+    const uint32_t bp = eff_max_bp(max_bp);
+    uint64_t need = carve_host(m, n, bp, flags, x_nnz).total_tile;
+    uint32_t pieces = 1;
+    const uint32_t piece = host_piece(m, n, &pieces);
+    if (!m->first_sparse && pieces >= 2) // two piece areas at a time
+        need = std::max(need, 2 * align_up(carve_host(m, piece, bp, flags, 0).total_tile, 256) + 512);
+    *bytes = need;
     return SLONN_OK;
 }
 
@@ -1414,16 +1714,9 @@ extern "C" int slonn_run_host(const slonn_model *m, const slonn_batch *hb, void 
     // about 16 MiB of input, between 1024 and 2048 queries (4096 fp32 inputs per query: four pieces of
     // 1024 queries took 4.5 ms end to end where two of 2048 took 4.9 ms; 1024 inputs per query at
     // mixed budgets: 2048-query pieces 9.6 ms, 1024-query pieces 11.0 ms).
-#ifndef SLONN_PIECE_QUERIES
-    const uint64_t row_bytes = (uint64_t)m->layer[0].D * sizeof(float);
-    const uint32_t piece_min = (uint32_t)std::min<uint64_t>(2048u, std::max<uint64_t>(1024u, (16ull << 20) / std::max<uint64_t>(row_bytes, 1)));
-#else
-    const uint32_t piece_min = SLONN_PIECE_QUERIES;
-#endif
-    const uint32_t pieces = std::min(8u, std::max(1u, n / piece_min));
+    uint32_t pieces = 1;
+    const uint32_t piece = host_piece(m, n, &pieces);
     const bool wants_lists = hb->active_indptr || hb->active_ids || hb->active_vals;
-    uint32_t piece = (n + pieces - 1) / pieces;
-    piece = (piece + 255u) / 256u * 256u;
     const uint64_t half = ((ws_bytes - 256) / 2) & ~(uint64_t)255; // two piece areas, then the pieces' status words
     bool piecewise = !m->first_sparse && !wants_lists && pieces >= 2 && !(hb->flags & SLONN_FLAG_DENSE_TC);
     if (piecewise && carve_host(m, piece, max_bp, hb->flags, 0).total > half) piecewise = false;

@@ -153,8 +153,17 @@ struct slonn_select_params {
     const uint64_t *indptr;     // offsets of (q, a)
     uint32_t *out_ids;          // CSR payload
     uint16_t *codes;            // nullable [n][n_act][L]
+    uint64_t *sort_key;         // nullable [n]: (budget, keys of the first two tables, query) for tile_order_kernel
+    const uint16_t *budget_bp;  // read for sort_key only
     uint32_t *status;
 };
+
+// Sort key of a query: queries with equal budget whose first keys agree become neighbours.
+__device__ __forceinline__ uint64_t tile_sort_key(uint32_t bp, const uint32_t *keys, uint32_t L, uint32_t q)
+{
+    return ((uint64_t)(bp & 0x3fffu) << 48) | ((uint64_t)(keys[0] & 0xffffu) << 32) |
+           ((uint64_t)(L > 1 ? keys[1] & 0xffffu : 0u) << 16) | (q & 0xffffu);
+}
 
 template <typename IDT>
 __device__ __forceinline__ uint32_t table_entry(const void *tables, uint32_t cap, uint32_t K,
@@ -349,6 +358,7 @@ __global__ void __launch_bounds__(LAT ? 1024 : SLONN_THREADS, LAT ? 1 : SLONN_SE
         if (P.codes) P.codes[((uint64_t)q * P.n_act + P.a) * P.L + threadIdx.x] = (uint16_t)key;
     }
     __syncthreads();
+    if (P.sort_key && threadIdx.x == 0) P.sort_key[q] = tile_sort_key(P.budget_bp[q], keys, P.L, q);
 
     if (!block_select<IDT>(P.tables, P.cap, P.K, P.L, P.N, B, keys, bitmap, P.out_ids + off, scan_ws, &scan_total,
                            P.hash_nodes, P.pre) &&
@@ -1095,6 +1105,8 @@ struct slonn_layer_cols_params {
     const void *tables;
     uint32_t cap, K, L, pre, layer;
     uint16_t *codes;            // nullable
+    uint64_t *sort_key;         // nullable, see slonn_select_params
+    const uint16_t *budget_bp;  // read for sort_key only
     uint32_t *status;
 };
 
@@ -1177,6 +1189,7 @@ __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
         if (Q.codes && writer) Q.codes[((uint64_t)q * P.n_act + P.a) * Q.L + threadIdx.x] = (uint16_t)key;
     }
     __syncthreads();
+    if (Q.sort_key && writer && threadIdx.x == 0) Q.sort_key[q] = tile_sort_key(Q.budget_bp[q], keys, Q.L, q);
     // (3) + (4) bucket lists, first B distinct ids, ascending: into the layer's list, or, when several blocks
     // work on the query, into this block's own copy, which the first block then publishes
     uint32_t *global_list = const_cast<uint32_t *>(P.ids) + off;
@@ -1189,6 +1202,71 @@ __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
         for (uint32_t i = threadIdx.x; i < B; i += blockDim.x) global_list[i] = own_list[i];
     // (5) the selected nodes
     cols_order_and_gather<BF16, R, false, SPLIT>(P, S, smem4, list, zpart, q, off, B, r0, r1, scan_ws, &scan_total);
+}
+
+// Hash and selection of a list-fed activator layer, input-stationary: the first half of layer_cols_kernel for layers
+// whose nodes another kernel evaluates.  The hash functions read one 64-byte line of WH per nonzero input instead of
+// K*L whole weight rows.
+template <bool BF16, typename IDT>
+__launch_bounds__(SLONN_THREADS, 6)
+__global__ void hash_select_cols_kernel(slonn_layer_cols_params Q)
+{
+    extern __shared__ float4 smem4[];
+    constexpr int V = BF16 ? 8 : 4;
+    constexpr uint32_t ESZ = BF16 ? 2u : 4u;
+    const slonn_gather_params &P = Q.G;
+    __shared__ uint32_t segcnt[32];
+    __shared__ uint32_t segstart[33];
+    __shared__ uint32_t scan_ws[32];
+    __shared__ uint32_t scan_total;
+    __shared__ uint32_t keys[8];
+    __shared__ float zh[32];
+    const uint32_t q = blockIdx.x;
+    if (P.skip_bp && P.skip_bp[q] == 10000u) return;
+    if (!bp_in_range(P.range_bp, P.bp_lo, P.bp_hi, q)) return;
+    const uint64_t off = P.indptr[(uint64_t)q * P.n_act + P.a];
+    const uint32_t B = min((uint32_t)(P.indptr[(uint64_t)q * P.n_act + P.a + 1] - off), P.rows_cap);
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const uint32_t H = Q.K * Q.L, nwords = (P.N + 31u) >> 5;
+    // shared memory: [input image, then the hash functions' partial sums][entries][selection bitmap]
+    cols_stage S;
+    S.xs = reinterpret_cast<float *>(smem4);
+    S.ent = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(smem4) + P.scratch_bytes);
+    S.segcnt = segcnt;
+    S.segstart = segstart;
+    uint32_t *idmap = reinterpret_cast<uint32_t *>(S.ent + cols_ent_cap(P.D, P.in_cap));
+    float *zpart = reinterpret_cast<float *>(smem4);
+    const uint64_t s0 = P.in.indptr[(uint64_t)q * P.in.ip_mul + P.in.ip_add];
+    const uint32_t len = min((uint32_t)(P.in.indptr[(uint64_t)q * P.in.ip_mul + P.in.ip_add + 1] - s0), P.in_cap);
+    cols_stage_list<V>(S, P.in.ids, P.in.vals, s0, len, P.D);
+    const uint32_t cb[1] = {lane * ESZ};
+    for (uint32_t p = warp; p < 32; p += nwarps) {
+        float a[1] = {0.0f};
+        cols_segment<BF16, 1, SLONN_DEEP_WALK>(S.ent, segstart[p], segstart[p + 1], Q.WH, 32u * ESZ, cb, a);
+        zpart[p * 32u + lane] = a[0];
+    }
+    for (uint32_t i = threadIdx.x; i < nwords; i += blockDim.x) idmap[i] = 0u;
+    __syncthreads();
+    if (threadIdx.x < H) {
+        float acc[32];
+#pragma unroll
+        for (int p = 0; p < 32; ++p) acc[p] = zpart[p * 32 + threadIdx.x];
+        zh[threadIdx.x] = cols_tree(acc) + __ldg(P.bias + __ldg(Q.hash_nodes + threadIdx.x));
+    }
+    __syncthreads();
+    if (threadIdx.x < Q.L) {
+        uint32_t key = 0;
+        for (uint32_t j = 0; j < Q.K; ++j)
+            if (zh[threadIdx.x * Q.K + j] > 0.0f) key |= (1u << j);
+        keys[threadIdx.x] = key;
+        if (Q.codes) Q.codes[((uint64_t)q * P.n_act + P.a) * Q.L + threadIdx.x] = (uint16_t)key;
+    }
+    __syncthreads();
+    if (Q.sort_key && threadIdx.x == 0) Q.sort_key[q] = tile_sort_key(Q.budget_bp[q], keys, Q.L, q);
+    if (!block_select<IDT>(Q.tables, Q.cap, Q.K, Q.L, P.N, B, keys, idmap, const_cast<uint32_t *>(P.ids) + off, scan_ws, &scan_total,
+                           Q.hash_nodes, Q.pre) &&
+        threadIdx.x == 0)
+        slonn_report(Q.status, SLONN_ERR_ARG, q, Q.layer);
 }
 
 // ---------------------------------------------------------------------------

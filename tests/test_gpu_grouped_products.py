@@ -1,0 +1,77 @@
+"""Layers evaluated as grouped products (16 queries x 128 columns per work item): sizes at the edges of a tile, a group, a
+partial sum's stretch and a staged chunk, against the oracle or bit for bit against the row kernels (whose own parity the
+other tests cover; the order of every sum is fixed, so the two have to agree in every bit)."""
+import numpy as np
+import pytest
+
+from test_gpu_parity import check, custom_workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,dims,has_act,n,budgets", [
+    ("bf16", [264, 128, 136, 127], [1, 1, 1], 256, (3600, 5000, 9999)),         # one tile, one tile and 8 columns, odd width
+    ("f32", [132, 260, 124, 61], [1, 1, 0], 273, (4000, 7500, 10000)),          # ragged last group, odd output layer
+    ("bf16", [8, 32, 40, 3], [1, 1, 0], 259, (9000, 10000)),                    # partial sums without any input
+    ("f32", [64, 1032, 1024, 130], [1, 1, 1], 300, (300, 3499, 3501, 6000)),    # both sides of the split with layer_cols
+])
+def test_grouped_products_at_the_edges_of_their_tiles(dtype, dims, has_act, n, budgets):
+    wl = custom_workload(4100 + n, dims, has_act, dtype, n=n, n_cal=300, K=4, L=2, budgets=budgets)
+    check(wl)
+
+
+def _run(dm, wl, flags=0, ws_bytes=None, x=None):
+    from paper_2204_08400_b200 import binding as sl, harness
+    b = harness.DeviceBatch(dm, wl.x if x is None else x, wl.budget_bp, kernel_path=sl.PATH_STAGED, flags=flags)
+    if ws_bytes is not None:
+        b.ws_bytes = ws_bytes
+    b.run()
+    return b.results()
+
+
+KEYS = ("logits", "pred", "codes", "active_ids", "active_vals")
+
+
+def _same_bits(a, b):
+    for k in KEYS:
+        assert np.array_equal(a[k].view(np.uint8), b[k].view(np.uint8)), k
+
+
+def test_grouped_products_in_several_chunks():
+    """More queries than are sorted and staged at a time (8192), 100 % queries among them."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4201, [64, 600, 520, 20], [1, 1, 0], "bf16", n=8192 + 8192 + 17, n_cal=300, K=4, L=2,
+                         budgets=(1000, 5000, 10000))
+    dm = harness.DeviceModel(wl)
+    _same_bits(_run(dm, wl), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS))
+    dm.free()
+
+
+def test_grouped_products_need_their_scratch_and_do_without_it():
+    """A workspace of the size the other kernels need is still taken, with the same results."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4202, [128, 512, 256, 20], [1, 1, 0], "f32", n=600, n_cal=300, K=4, L=2, budgets=(2500, 6000))
+    dm = harness.DeviceModel(wl)
+    small = sl.slonn_workspace_bytes(dm.model, 600, 6000, flags=sl.FLAG_ROW_KERNELS)
+    assert small < sl.slonn_workspace_bytes(dm.model, 600, 6000)
+    _same_bits(_run(dm, wl), _run(dm, wl, ws_bytes=small))
+    dm.free()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_grouped_products_keep_queries_apart(dtype):
+    """Infinities and NaNs in some queries stay in those queries; the others, in the same groups, are untouched."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4203, [128, 256, 264, 40], [1, 1, 0], dtype, n=320, n_cal=300, K=2, L=2, budgets=(6000,))
+    dm = harness.DeviceModel(wl)
+    clean = _run(dm, wl)
+    x = wl.x.copy()
+    x[5::7, 3] = np.inf
+    x[6::7, 9] = np.nan
+    dirty = _run(dm, wl, x=x)
+    rows = _run(dm, wl, flags=sl.FLAG_ROW_KERNELS, x=x)
+    for k in KEYS:
+        assert np.array_equal(dirty[k], rows[k], equal_nan=dirty[k].dtype == np.float32), k
+    others = [q for q in range(320) if q % 7 not in (5, 6)]
+    assert np.array_equal(clean["logits"][others], dirty["logits"][others])
+    dm.free()

@@ -950,16 +950,26 @@ int launch_cluster(const slonn_model *m, const slonn_batch *b, uint32_t max_bp, 
 
 // ---- internal entry points used by the table builder --------------------------
 
-// Complete layer l (every node) for n dense input rows -> out [n][N_l].
+// Complete layer l (every node) for n dense input rows -> out [n][N_l].  Four rows per block where their staging fits
+// shared memory and there are enough of them (16,384 rows of 784 inputs, 1024 nodes: 2.42 -> 1.19 ms).
 int slonn_forward_all_rows(const slonn_model *m, uint32_t l, const float *in_dense, uint32_t n, float *out,
                            uint32_t relu, cudaStream_t st)
 {
     const slonn_layer &ly = m->layer[l];
+    const uint32_t nchunks = ly.D * (m->dtype == SLONN_BF16 ? 2u : 4u) / 16u;
+    if (n >= 256 && (size_t)SLONN_FULL_GROUP * ly.D * 4 <= 100 * 1024) {
+        slonn_full_params fp;
+        memset(&fp, 0, sizeof(fp));
+        fp.n = n; fp.in.kind = SLONN_IN_DENSE; fp.in.dense = in_dense;
+        fp.W = ly.W; fp.bias = ly.bias; fp.D = ly.D; fp.N = ly.N; fp.nchunks = nchunks;
+        fp.out_dense = out; fp.out_stride = ly.N; fp.relu = relu;
+        return launch_full_rows(m, fp, n, st);
+    }
     slonn_gather_params gp;
     memset(&gp, 0, sizeof(gp));
     gp.in.kind = SLONN_IN_DENSE; gp.in.dense = in_dense;
     gp.W = ly.W; gp.bias = ly.bias; gp.D = ly.D; gp.N = ly.N;
-    gp.nchunks = ly.D * (m->dtype == SLONN_BF16 ? 2u : 4u) / 16u;
+    gp.nchunks = nchunks;
     gp.use_list = 0; gp.out_dense = out; gp.out_stride = ly.N; gp.relu = relu;
     return launch_gather(m, gp, n, ly.N, st);
 }

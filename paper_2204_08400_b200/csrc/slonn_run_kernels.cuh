@@ -491,8 +491,9 @@ __global__ void gather_dot_kernel(slonn_gather_params P)
 // formed in the library's fixed order, so the results are those of gather_dot_kernel bit for bit.
 // `list` / `count`: the batch's 100 % queries (dense_compact_kernel); group g = entries 4g .. 4g + 3.
 struct slonn_full_params {
-    const uint32_t *list;
-    const uint32_t *count;
+    const uint32_t *list;     // nullable: queries 0 .. n - 1
+    const uint32_t *count;    // nullable with `list`
+    uint32_t n;               // queries without a list
     slonn_input in;
     const void *W;
     const float *bias;
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FULL_MIN_BLOCKS) full_row
     constexpr int G = SLONN_FULL_GROUP;
     const uint32_t g = blockIdx.x / P.ctas_per_group;
     const uint32_t chunk = blockIdx.x - g * P.ctas_per_group;
-    const uint32_t cnt = *P.count;
+    const uint32_t cnt = P.list ? *P.count : P.n;
     if (g * G >= cnt) return;
     const uint32_t r0 = chunk * P.rows_per_cta;
     if (r0 >= P.N) return;
@@ -537,7 +538,8 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FULL_MIN_BLOCKS) full_row
     uint64_t off[G];
 #pragma unroll
     for (int k = 0; k < G; ++k) {
-        q[k] = __ldg(P.list + g * G + min((uint32_t)k, nq - 1)); // a short last group repeats its last query
+        q[k] = g * G + min((uint32_t)k, nq - 1); // a short last group repeats its last query
+        if (P.list) q[k] = __ldg(P.list + q[k]);
         off[k] = P.has_act ? P.indptr[(uint64_t)q[k] * P.n_act + P.a] : 0;
         stage_input<BF16>(P.in, q[k], P.D, P.nchunks, smem4 + k * per_q);
     }

@@ -61,3 +61,23 @@ def test_round_trip_with_a_csr_first_layer():
         assert np.array_equal(got[k], want[k]), k
     sl.slonn_free(built)
     dm.free()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_nodes,K", [(1000, 6), (1024, 7), (1028, 10), (2048, 11)])   # 0.26, 0.5, 4.2 and 16.8 MB of tables
+def test_checksum_of_large_tables_is_the_plain_chain_over_the_bytes(n_nodes, K):
+    """Tables of 256 KB and more are summed on the device, in chunks of 2048 bytes and passes of 4 MiB; loading sums the
+    blob byte by byte on the host and refuses any other value."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    dims = [64, n_nodes, 8]
+    W_f32, W_store, bias = wl_mod.draw_mlp(dims, 90, "f32", bias_scale=0.2)
+    wl = Workload(name="custom", dims=dims, has_act=[1, 0], dtype="f32", W_f32=W_f32, W_store=W_store, bias=bias,
+                  first_sparse=False, calib=wl_mod.draw_dense_inputs(500, dims[0], 92, "relu_normal"),
+                  x=wl_mod.draw_dense_inputs(8, dims[0], 91, "relu_normal"), budget_bp=wl_mod.draw_mixed_budgets(8, 93),
+                  K=K, L=2, seed=94, list_cap=0)
+    dm = harness.DeviceModel(wl)
+    blob = sl.slonn_serialize(dm.model)
+    again = sl.slonn_deserialize(blob, dm.W, dm.bias)
+    assert np.array_equal(sl.slonn_serialize(again), blob)
+    sl.slonn_free(again)
+    dm.free()

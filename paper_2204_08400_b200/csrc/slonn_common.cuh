@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 #include "../../include/slonn.h"
@@ -92,19 +93,62 @@ __device__ __forceinline__ float chunk_elem(const uint4 &w)
 
 // acc[r] = fmaf(w[r][E], x[E], acc[r]) for every row, elements in ascending order; rows are
 // interleaved so that consecutive instructions belong to independent accumulation chains.
-template <bool BF16, int R, int E, int VPC>
+// PACKED: two rows per packed instruction, each half rounded on its own as fmaf does.
+template <bool BF16, int R, int E, int VPC, bool PACKED = true>
 struct chunk_fma {
     __device__ static __forceinline__ void run(const uint4 (&w)[R], const float *x, float (&acc)[R])
     {
+        if constexpr (!PACKED) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = fmaf(chunk_elem<BF16, E>(w[r]), x[E], acc[r]);
-        chunk_fma<BF16, R, E + 1, VPC>::run(w, x, acc);
+            for (int r = 0; r < R; ++r) acc[r] = fmaf(chunk_elem<BF16, E>(w[r]), x[E], acc[r]);
+        } else {
+#pragma unroll
+            for (int r = 0; r + 1 < R; r += 2) {
+                const float2 v = __ffma2_rn(make_float2(chunk_elem<BF16, E>(w[r]), chunk_elem<BF16, E>(w[r + 1])),
+                                            make_float2(x[E], x[E]), make_float2(acc[r], acc[r + 1]));
+                acc[r] = v.x;
+                acc[r + 1] = v.y;
+            }
+            if constexpr (R & 1) acc[R - 1] = fmaf(chunk_elem<BF16, E>(w[R - 1]), x[E], acc[R - 1]);
+        }
+        chunk_fma<BF16, R, E + 1, VPC, PACKED>::run(w, x, acc);
     }
 };
-template <bool BF16, int R, int VPC>
-struct chunk_fma<BF16, R, VPC, VPC> {
+template <bool BF16, int R, int VPC, bool PACKED>
+struct chunk_fma<BF16, R, VPC, VPC, PACKED> {
     __device__ static __forceinline__ void run(const uint4 (&)[R], const float *, float (&)[R]) {}
 };
+
+// One 16-byte chunk of R rows (R even) for G queries: acc[g][r / 2] takes the products of rows r and r + 1 with query g's
+// inputs, elements in ascending order.  A pair of widened weights stays put for G packed multiply-adds in a row: that order
+// issues at the full rate (128 multiply-adds per SM and cycle in registers; 102 with the queries outside).
+template <bool BF16, int R, int G>
+__device__ __forceinline__ void chunk_fma_group(const uint4 (&w)[R], const float4 *xs4, uint32_t per_q, uint32_t nchunks, uint32_t c,
+                                                float2 (&acc)[G][R / 2])
+{
+#pragma unroll
+    for (int h = 0; h < (BF16 ? 2 : 1); ++h) {
+        float x[G][4];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const float4 v = xs4[g * per_q + h * nchunks + c];
+            x[g][0] = v.x; x[g][1] = v.y; x[g][2] = v.z; x[g][3] = v.w;
+        }
+        auto element = [&](auto E) {
+#pragma unroll
+            for (int r = 0; r < R; r += 2) {
+                const float2 wp = h ? make_float2(chunk_elem<BF16, (BF16 ? 4 : 0) + E.value>(w[r]), chunk_elem<BF16, (BF16 ? 4 : 0) + E.value>(w[r + 1]))
+                                    : make_float2(chunk_elem<BF16, E.value>(w[r]), chunk_elem<BF16, E.value>(w[r + 1]));
+#pragma unroll
+                for (int g = 0; g < G; ++g) acc[g][r / 2] = __ffma2_rn(make_float2(x[g][E.value], x[g][E.value]), wp, acc[g][r / 2]);
+            }
+        };
+        element(std::integral_constant<int, 0>());
+        element(std::integral_constant<int, 1>());
+        element(std::integral_constant<int, 2>());
+        element(std::integral_constant<int, 3>());
+    }
+}
 
 // Sums of 4 rows' 32 partials with 6 shuffles instead of 20.  Same additions as the xor
 // butterfly 16, 8, 4, 2, 1 of each row (each step adds the same two operands), but after

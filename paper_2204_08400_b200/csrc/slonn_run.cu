@@ -134,6 +134,8 @@ uint32_t tile_kcap(const slonn_model *m, uint32_t l, uint32_t max_bp)
 bool tile_wanted(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags)
 {
     if (flags & (SLONN_FLAG_ROW_KERNELS | SLONN_FLAG_COLUMN_KERNELS | SLONN_FLAG_UNGROUPED_ROWS)) return false;
+    // most queries may be gone to the tensor cores, and the host does not know: sorting and staging nobody costs 0.06 ms a layer
+    if (tc_route(m, max_bp, flags)) return false;
     uint32_t rows = 0; // most rows a layer that can take them computes for a query
     for (uint32_t l = 0; l < m->n_layers; ++l)
         if (tile_layer_ok(m, l))
@@ -305,6 +307,7 @@ int launch_gather(const slonn_model *m, slonn_gather_params &P, uint32_t n, uint
 // ---- selected rows, four queries per block --------------------------------------
 
 struct group_ws { uint32_t *list, *count; }; // workspace for the compacted list of the queries a launch serves
+struct sorted_groups { const uint32_t *order; uint32_t chunk, stride, lo; }; // or the queries from budget lo on, sorted by (budget, keys): order + chunk number * stride
 
 template <bool BF16>
 int launch_group_rows_t(const slonn_group_params &Q, uint64_t grid, size_t smem, cudaStream_t st)
@@ -328,18 +331,18 @@ size_t group_rows_smem(const slonn_gather_params &P, uint32_t max_rows, uint32_t
 // once for all of them): at such budgets any four queries share most of their rows.  Below that, and for small
 // batches, layers of more than 65,535 nodes, rows of a single 512-byte round and shapes whose staging does not
 // fit two blocks per SM, every query has a block (or several) of its own.  Same values either way.
-// Measured on a 4096-wide layer with 4096 queries: 50 % budget 3.5 -> 2.8 ms per layer, 25 % 1.77 -> 1.68 ms,
-// 10 % 0.72 -> 0.79 ms (hence the limit).
-#ifndef SLONN_GROUP_MIN_BP
+// Measured on a 4096-wide layer with 4096 queries: 50 % budget 3.5 -> 2.95 ms per layer with queries as they come, 2.52 ms
+// with neighbours in (budget, keys) and packed multiply-adds; 10 % 0.72 -> 0.79 ms, sorted and packed 0.66 ms.  Small
+// batches have fewer neighbours: 777 queries of 7 to 60 % on 2328 x 1568, groups from 20 % on 0.161 ms, from 7 % on 0.174.
 #define SLONN_GROUP_MIN_BP 2000u
-#endif
+#define SLONN_GROUP_MIN_BP_SORTED 700u // batches of at least SLONN_TILE_LARGE queries, sorted
 int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch *b, uint32_t n, uint32_t max_bp,
-                uint32_t max_rows, const group_ws &gw, cudaStream_t st, stage_timer *tm)
+                uint32_t max_rows, const group_ws &gw, cudaStream_t st, stage_timer *tm, const sorted_groups *sorted = nullptr)
 {
     uint32_t shared_cap = 0;
     const size_t smem = group_rows_smem(P, max_rows, &shared_cap);
     const uint32_t lo = P.range_bp ? P.bp_lo : 0u, hi = std::min(P.range_bp ? P.bp_hi : 0xffffu, max_bp);
-    const uint32_t split = std::max(lo, SLONN_GROUP_MIN_BP + 1u); // budgets from here on are grouped
+    const uint32_t split = std::max(lo, sorted ? sorted->lo : SLONN_GROUP_MIN_BP + 1u); // budgets from here on are grouped
     const bool grouped = P.use_list && n >= 256 && P.N <= 65535u && P.nchunks > 32 && gw.list && smem <= 110 * 1024 &&
                          !(b->flags & SLONN_FLAG_UNGROUPED_ROWS) && hi >= split;
     int rc;
@@ -357,6 +360,23 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
         TOC();
         if (rc) return rc;
     }
+    slonn_group_params Q;
+    memset(&Q, 0, sizeof(Q));
+    Q.G = P; Q.rows_cap = max_rows; Q.shared_cap = shared_cap;
+    if (sorted) { // the others, neighbours in (budget, keys)
+        TIC(SLONN_STAGE_GROUP_ROWS, b->budget_bp, split, hi, P.skip_bp);
+        rc = SLONN_OK;
+        for (uint32_t c = 0, q0 = 0; q0 < n && !rc; ++c, q0 += sorted->chunk) {
+            Q.list = sorted->order + (uint64_t)c * sorted->stride;
+            Q.n = std::min(sorted->chunk, n - q0);
+            const uint32_t groups = (Q.n + SLONN_GROUP - 1) / SLONN_GROUP;
+            Q.ctas_per_group = std::max(1u, std::min(std::min(8u, (148u * 8u + groups - 1) / groups), max_rows / 32u));
+            rc = m->dtype == SLONN_BF16 ? launch_group_rows_t<true>(Q, (uint64_t)groups * Q.ctas_per_group, smem, st)
+                                        : launch_group_rows_t<false>(Q, (uint64_t)groups * Q.ctas_per_group, smem, st);
+        }
+        TOC();
+        return rc;
+    }
     // the others, compacted in two budget classes so that the queries of a group select about as many rows
     if (cudaMemsetAsync(gw.count, 0, sizeof(uint32_t), st) != cudaSuccess) return SLONN_ERR_CUDA;
     const uint32_t mid = 3750u;
@@ -365,9 +385,7 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
     if (hi > mid)
         range_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, P.skip_bp, n, std::max(split, mid + 1u), hi, gw.list, gw.count);
     if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
-    slonn_group_params Q;
-    memset(&Q, 0, sizeof(Q));
-    Q.G = P; Q.list = gw.list; Q.count = gw.count; Q.rows_cap = max_rows; Q.shared_cap = shared_cap;
+    Q.list = gw.list; Q.count = gw.count;
     const uint32_t groups = (n + SLONN_GROUP - 1) / SLONN_GROUP;
     // enough blocks for a few waves of two per SM, but no block with fewer than 32 rows of each kind
     Q.ctas_per_group = std::max(1u, std::min(std::min(8u, (148u * 8u + groups - 1) / groups), max_rows / 32u));
@@ -1316,7 +1334,17 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             } else {
                 keyed = tw.ws && in.kind == SLONN_IN_DENSE; // hash_select_kernel serves every query
                 if (keyed) { sp.sort_key = (uint64_t *)(ws + wl.tile.key); sp.budget_bp = b->budget_bp; }
-                rc = launch_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm);
+                const uint32_t from = (n >= SLONN_TILE_LARGE ? SLONN_GROUP_MIN_BP_SORTED : SLONN_GROUP_MIN_BP) + 1u;
+                if (keyed && max_bp >= from) {
+                    TIC(SLONN_STAGE_HASH_SELECT, sp.range_bp, sp.bp_lo, sp.bp_hi, sp.skip_bp);
+                    rc = launch_select(m, sp, n, max_rows, st);
+                    TOC();
+                    if (!rc) rc = launch_tile_order(tw, b, n, from, skip_bp ? 9999u : 10000u, &sorted, st);
+                    const sorted_groups sg = {(const uint32_t *)(ws + wl.tile.order), wl.tile.chunk, wl.tile.order_stride, from};
+                    if (!rc) rc = launch_rows(m, gp, b, n, max_bp, max_rows, gw, st, tm, &sg);
+                } else {
+                    rc = launch_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm);
+                }
             }
             if (rc) return rc;
             in.kind = SLONN_IN_LIST; in.indptr = indptr; in.ids = ids; in.vals = vals;

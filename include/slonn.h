@@ -221,7 +221,9 @@ typedef struct {
  * keeps of such layers.  By default the library picks per query by budget: up to SLONN_COLS_MAX_BP
  * the input list is sparse enough for the input-stationary kernels to win (batches of tens of queries
  * only when no budget exceeds 1500 bp and only for layers at least 2048 inputs wide; a handful of queries keep
- * the row kernels).  These two flags force one kind for the whole batch, for testing and
+ * the row kernels); in large batches the queries that compute more than a few hundred nodes per layer are sorted by
+ * budget and keys and evaluated 16 at a time over the union of their inputs and nodes, in the same order of sums
+ * and with the same results, when the workspace holds the scratch for it (slonn_workspace_bytes includes it).  These two flags force one kind for the whole batch, for testing and
  * tuning; setting both is an error.  They apply to the per-stage kernels and to the
  * one-warp-per-query kernel; the one-cluster-per-query kernel has row form only.
  */
@@ -413,7 +415,7 @@ int slonn_run_static(const slonn_model *m, const slonn_batch *batch, void *strea
 #define SLONN_STAGE_GATHER_COLS 8   /* selected nodes' dot products, input-stationary kernel */
 #define SLONN_STAGE_LAYER_COLS 9    /* all of 1 and 8 for a list-fed activator layer in one launch */
 #define SLONN_STAGE_FULL_ROWS 10    /* every layer of the 100 % budget queries, four queries per block */
-#define SLONN_STAGE_GROUP_ROWS 11   /* selected rows' dot products, four queries per block   */
+#define SLONN_STAGE_GROUP_ROWS 11   /* nodes' dot products, four or sixteen queries at a time */
 #define SLONN_N_STAGES 12
 int slonn_run_timed(const slonn_model *m, const slonn_batch *batch, void *workspace,
                     uint64_t workspace_bytes, void *stream, float *stage_ms,

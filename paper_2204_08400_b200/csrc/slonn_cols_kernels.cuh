@@ -20,7 +20,7 @@
 
 // Shared-memory image of one query's nonzero inputs, grouped by partial sum.
 struct cols_stage {
-    float *xs;          // [32 * smax] scratch: inputs in segment-major order (zero = absent)
+    float *xs;          // scratch while staging (cols_scratch_bytes)
     uint2 *ent;         // [cols_ent_cap] entries (j, bits of x_j), segment after segment
     uint32_t *segcnt;   // [32]
     uint32_t *segstart; // [33]
@@ -39,45 +39,50 @@ __host__ __device__ __forceinline__ uint32_t cols_ent_cap(uint32_t D, uint32_t i
     return (in_cap < D ? in_cap : D) + 96u;
 }
 
-// bytes of the input image a block scatters the list into while staging
-__host__ __device__ __forceinline__ size_t cols_image_bytes(uint32_t D, uint32_t V)
-{
-    return (size_t)32 * cols_smax(D, V) * 4;
-}
+// 32-bit words of the bitmap of one segment's inputs
+__host__ __device__ __forceinline__ uint32_t cols_words(uint32_t D, uint32_t V) { return (cols_smax(D, V) + 31u) / 32u; }
+
+// bytes of scratch a block needs while staging: the inputs' bitmap by segment, and the inputs below each word
+__host__ __device__ __forceinline__ size_t cols_scratch_bytes(uint32_t D, uint32_t V) { return (size_t)32 * cols_words(D, V) * 8; }
 
 // Builds the grouped nonzero list of query segment [s0, s0 + len) of (ids, vals).  Whole block; ends
-// with a barrier.
+// with a barrier.  An entry's place is the number of the segment's inputs below it, counted on a bitmap of the nonzero
+// inputs (one bit per input, instead of scattering the values into an image of the layer and compacting that).
 template <int V>
 __device__ __forceinline__ void cols_stage_list(const cols_stage &S, const uint32_t *ids, const float *vals, uint64_t s0,
                                                 uint32_t len, uint32_t D)
 {
-    const uint32_t smax = cols_smax(D, V);
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (uint32_t i = threadIdx.x; i < 32u * smax; i += blockDim.x) S.xs[i] = 0.0f;
+    const uint32_t words = cols_words(D, V);
+    uint32_t *bits = reinterpret_cast<uint32_t *>(S.xs), *below = bits + 32u * words;
+    for (uint32_t i = threadIdx.x; i < 32u * words; i += blockDim.x) bits[i] = 0u;
     __syncthreads();
+    // input j: chunk j / V of segment (j / V) mod 32; position in the segment
+    auto place = [&](uint32_t j, uint32_t &p, uint32_t &pos) {
+        const uint32_t c = j / V;
+        p = c & 31u;
+        pos = (c >> 5) * V + (j - c * V);
+    };
 #pragma unroll 4
     for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
         const uint32_t j = __ldg(ids + s0 + i);
         const float v = __ldg(vals + s0 + i);
-        if (j < D) {
-            const uint32_t c = j / V, p = c & 31u;
-            S.xs[p * smax + (c >> 5) * V + (j - c * V)] = v;
+        if (j < D && v != 0.0f) {
+            uint32_t p, pos;
+            place(j, p, pos);
+            atomicOr(&bits[p * words + (pos >> 5)], 1u << (pos & 31u));
         }
     }
     __syncthreads();
-    // nonzeros per segment, counted on the scattered image (so that a repeated id counts once)
-    for (uint32_t p = warp; p < 32; p += nwarps) {
-        uint32_t cnt = 0;
-        for (uint32_t pos0 = 0; pos0 < smax; pos0 += 32) {
-            const uint32_t pos = pos0 + lane;
-            const float v = pos < smax ? S.xs[p * smax + pos] : 0.0f;
-            cnt += __popc(__ballot_sync(SLONN_FULL_MASK, v != 0.0f));
+    if (threadIdx.x < 32u) { // one lane per segment; segments start at multiples of 4 entries
+        const uint32_t lane = threadIdx.x;
+        uint32_t cnt = 0, last = 0;
+        for (uint32_t w = 0; w < words; ++w) {
+            const uint32_t b = bits[lane * words + w];
+            below[lane * words + w] = cnt;
+            cnt += __popc(b);
+            if (b) last = w * 32u + 31u - (uint32_t)__clz((int)b);
         }
-        if (lane == 0) S.segcnt[p] = cnt;
-    }
-    __syncthreads();
-    if (warp == 0) { // segments start at multiples of 4 entries
-        const uint32_t c = (S.segcnt[lane] + 3u) & ~3u;
+        const uint32_t c = (cnt + 3u) & ~3u;
         uint32_t incl = c;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -86,26 +91,22 @@ __device__ __forceinline__ void cols_stage_list(const cols_stage &S, const uint3
         }
         S.segstart[lane] = incl - c;
         if (lane == 31) S.segstart[32] = incl;
+        // filled up to the next multiple of 4 with copies of the last input carrying the value 0
+        // (a multiply-add by 0 leaves the partial sum as it is)
+        const uint32_t blk = last / V, jl = (blk * 32u + lane) * V + (last - blk * V);
+        for (uint32_t k = cnt; k < c; ++k) S.ent[incl - c + k] = make_uint2(jl, 0u);
     }
     __syncthreads();
-    for (uint32_t p = warp; p < 32; p += nwarps) {
-        uint32_t base = S.segstart[p];
-        for (uint32_t pos0 = 0; pos0 < smax; pos0 += 32) {
-            const uint32_t pos = pos0 + lane;
-            const float v = pos < smax ? S.xs[p * smax + pos] : 0.0f;
-            const uint32_t m = __ballot_sync(SLONN_FULL_MASK, v != 0.0f);
-            if (v != 0.0f) {
-                const uint32_t blk = pos / V;
-                const uint32_t j = (blk * 32u + p) * V + (pos - blk * V);
-                S.ent[base + __popc(m & ((1u << lane) - 1u))] = make_uint2(j, __float_as_uint(v));
-            }
-            base += __popc(m);
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
+        const uint32_t j = __ldg(ids + s0 + i);
+        const float v = __ldg(vals + s0 + i);
+        if (j < D && v != 0.0f) {
+            uint32_t p, pos;
+            place(j, p, pos);
+            const uint32_t w = p * words + (pos >> 5);
+            S.ent[S.segstart[p] + below[w] + __popc(bits[w] & ((1u << (pos & 31u)) - 1u))] = make_uint2(j, __float_as_uint(v));
         }
-        // fill up to the next multiple of 4 with copies of the last input carrying the value 0
-        // (a multiply-add by 0 leaves the partial sum as it is)
-        __syncwarp();
-        const uint32_t pad = S.segstart[p + 1] - base;
-        if (lane < pad) S.ent[base + lane] = make_uint2(S.ent[base - 1].x, 0u);
     }
     __syncthreads();
 }

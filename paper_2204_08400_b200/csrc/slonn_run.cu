@@ -434,7 +434,7 @@ int launch_gather_cols(const slonn_model *m, slonn_gather_params &P, uint32_t n,
     P.rows_per_cta = (uint32_t)ppc * unit;
     P.ctas_per_query = (max_rows + P.rows_per_cta - 1) / P.rows_per_cta;
     P.rows_cap = max_rows;
-    size_t scratch = cols_image_bytes(P.D, bf ? 8u : 4u);
+    size_t scratch = cols_scratch_bytes(P.D, bf ? 8u : 4u);
     if (P.use_list && P.colpos) scratch = std::max(scratch, ((size_t)2 * ((P.N + 31u) / 32u) + (size_t)3 * max_rows) * 4);
     scratch = (scratch + 15) & ~(size_t)15;
     P.scratch_bytes = (uint32_t)scratch;
@@ -479,15 +479,17 @@ int launch_select_cols_t(const slonn_layer_cols_params &Q, uint32_t n, size_t sm
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
-// Hash and selection of a list-fed activator layer, input-stationary.  SLONN_ERR_DIM: no side-by-side hash rows, or the
-// staging does not fit -- the caller takes hash_select_kernel.
+// Hash and selection of a list-fed activator layer, input-stationary.  SLONN_ERR_DIM: no side-by-side hash rows, or lists too
+// long for it to pay -- the caller takes hash_select_kernel (4096 queries, 4096 x 4096: 410 entries 0.091 -> 0.07 ms, 2048
+// entries 0.165 -> 0.19).
+#define SLONN_SELECT_COLS_MAX 1536u
 int launch_select_cols(const slonn_model *m, const slonn_layer &ly, uint32_t layer, slonn_gather_params G, const slonn_batch *b,
                        uint64_t *sort_key, uint32_t n, uint32_t max_rows, cudaStream_t st)
 {
-    if (!ly.WH || G.in.kind != SLONN_IN_LIST) return SLONN_ERR_DIM;
+    if (!ly.WH || G.in.kind != SLONN_IN_LIST || G.in_cap > SLONN_SELECT_COLS_MAX) return SLONN_ERR_DIM;
     const bool bf = m->dtype == SLONN_BF16, id16 = ly.id_bytes == 2;
     G.rows_cap = max_rows;
-    size_t scratch = std::max(cols_image_bytes(G.D, bf ? 8u : 4u), (size_t)32 * 32 * 4);
+    size_t scratch = std::max(cols_scratch_bytes(G.D, bf ? 8u : 4u), (size_t)32 * 32 * 4);
     scratch = (scratch + 15) & ~(size_t)15;
     G.scratch_bytes = (uint32_t)scratch;
     const size_t smem = scratch + (size_t)cols_ent_cap(G.D, G.in_cap) * 8 + (size_t)((G.N + 31u) / 32u) * 4;
@@ -517,7 +519,7 @@ int launch_layer_cols(const slonn_model *m, const slonn_layer &ly, uint32_t laye
     G.rows_cap = max_rows;
     G.rows_per_cta = split ? 64u : passes * 64u;
     G.ctas_per_query = split ? passes : 1u;
-    size_t scratch = cols_image_bytes(G.D, bf ? 8u : 4u);
+    size_t scratch = cols_scratch_bytes(G.D, bf ? 8u : 4u);
     scratch = std::max(scratch, ((size_t)2 * ((G.N + 31u) / 32u) + (size_t)3 * max_rows) * 4);
     scratch = std::max(scratch, (size_t)32 * 32 * 4); // the hash functions' partial sums pass through it
     scratch = (scratch + 15) & ~(size_t)15;

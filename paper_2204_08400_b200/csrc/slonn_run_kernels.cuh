@@ -393,7 +393,7 @@ struct slonn_gather_params {
     const uint32_t *colpos;   // [N] node id -> column of WT; NULL = identity
     uint32_t in_cap;          // most entries an input list of this launch can hold
     uint32_t rows_cap;        // most nodes a query of this launch selects
-    uint32_t scratch_bytes;   // shared memory in front of the entries (input image, then node order)
+    uint32_t scratch_bytes;   // shared memory in front of the entries (inputs' bitmap while staging, then node order)
 };
 
 
@@ -1066,7 +1066,7 @@ __global__ void gather_cols_kernel(slonn_gather_params P)
     if (r0 >= B) return;
     const uint32_t r1 = min(B, r0 + P.rows_per_cta);
 
-    // shared memory: [scratch: input image while staging, node order afterwards][entries]
+    // shared memory: [scratch: inputs' bitmap while staging, node order afterwards][entries]
     cols_stage S;
     S.xs = reinterpret_cast<float *>(smem4);
     S.ent = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(smem4) + P.scratch_bytes);
@@ -1132,7 +1132,7 @@ __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
     const uint32_t H = Q.K * Q.L;
     const uint32_t nwords = (P.N + 31u) >> 5;
 
-    // shared memory: [scratch: input image, then the hash functions' partial sums, then node order][entries]
+    // shared memory: [scratch: inputs' bitmap, then the hash functions' partial sums, then node order][entries]
     // [selection bitmap][SPLIT: partial sums of hash functions and nodes, the query's node list]
     cols_stage S;
     S.xs = reinterpret_cast<float *>(smem4);
@@ -1215,7 +1215,7 @@ __global__ void hash_select_cols_kernel(slonn_layer_cols_params Q)
     const uint32_t B = min((uint32_t)(P.indptr[(uint64_t)q * P.n_act + P.a + 1] - off), P.rows_cap);
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const uint32_t H = Q.K * Q.L, nwords = (P.N + 31u) >> 5;
-    // shared memory: [input image, then the hash functions' partial sums][entries][selection bitmap]
+    // shared memory: [inputs' bitmap, then the hash functions' partial sums][entries][selection bitmap]
     cols_stage S;
     S.xs = reinterpret_cast<float *>(smem4);
     S.ent = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(smem4) + P.scratch_bytes);

@@ -81,6 +81,7 @@ template <bool BF16, int THREADS, int MIN_BLOCKS>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
 cluster_network_kernel(const __grid_constant__ slonn_cluster_params P)
 {
+    slonn_enter();
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ float4 smem4[];

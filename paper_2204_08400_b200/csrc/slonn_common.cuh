@@ -69,6 +69,28 @@ __host__ __device__ __forceinline__ uint32_t slonn_layer_nodes(uint32_t bp, uint
     return (B < rest ? B : rest) + pre;
 }
 
+// First statement of every kernel of a run.  The run's launches are chained with programmatic dependencies
+// (slonn_launch): a kernel may be brought onto the SMs as soon as all blocks of the one before it have started, and waits
+// here until that one has finished and its writes can be seen.  Nothing may be read or written before this; loads through
+// the read-only path stay behind it because each sits behind a branch on, or at an address from, a plain load.
+__device__ __forceinline__ void slonn_enter()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
+// Launches a kernel that begins with slonn_enter().
+template <typename... P, typename... A>
+inline cudaError_t slonn_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 __device__ __forceinline__ void slonn_report(uint32_t *status, int code, uint32_t q, uint32_t layer)
 {
     if (atomicCAS(status, 0u, (uint32_t)(-code)) == 0u) {

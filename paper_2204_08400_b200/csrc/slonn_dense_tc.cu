@@ -165,6 +165,7 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 const __grid_constant__ CUtensorMap map_out, uint32_t tma_out, const slonn_dense_epilogue E, uint32_t N,
                 uint32_t K, uint32_t bn, uint32_t probe_limit)
 {
+    slonn_enter();
     // probe_limit: 0 in normal use.  Otherwise (a test of the give-up path) the producer first waits, for at most
     // that many polls, on a barrier nobody arrives at -- before any copy or MMA has been issued.
     // map_out / tma_out: the bf16 output matrix as a tensor of 64-column x 32-row boxes (128-byte swizzle),
@@ -508,7 +509,7 @@ int slonn_dense_tc_launch(const void *A, const void *W, uint32_t N, uint32_t K, 
     }
     const uint64_t tiles = (uint64_t)((N + bn - 1) / bn) * ((E.M + BM - 1) / BM);
     const uint32_t grid = (uint32_t)std::min<uint64_t>(tiles, (uint64_t)sm_count); // one persistent block per SM
-    dense_tc_kernel<<<grid, THREADS, SMEM_BYTES, st>>>(ma, mb, mo, tma_out, E, N, K, bn, g_probe_limit.load());
+    slonn_launch(dense_tc_kernel, grid, THREADS, SMEM_BYTES, st, ma, mb, mo, tma_out, E, N, K, bn, g_probe_limit.load());
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 

@@ -213,6 +213,7 @@ template <bool BF16, int NC, int GRP, bool COLS>
 __global__ void __launch_bounds__(SLONN_FUSED_WARPS * 32, GRP == 1 ? SLONN_FUSED_MIN_BLOCKS : 1)
 fused_network_kernel(const __grid_constant__ slonn_fused_params P)
 {
+    slonn_enter();
     constexpr int VPC = fused_traits<BF16>::VPC;
     constexpr int R = SLONN_FUSED_ROWS;
     extern __shared__ float4 smem4[];

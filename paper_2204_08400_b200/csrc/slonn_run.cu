@@ -219,7 +219,7 @@ int launch_select_t(const slonn_select_params &P, uint32_t n, uint32_t threads, 
 {
     const int rc = set_smem(hash_select_kernel<BF16, IDT, LAT>, smem);
     if (rc) return rc;
-    hash_select_kernel<BF16, IDT, LAT><<<n, threads, smem, st>>>(P);
+    slonn_launch(hash_select_kernel<BF16, IDT, LAT>, n, threads, smem, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -265,7 +265,7 @@ int launch_gather_t(const slonn_gather_params &P, uint64_t grid, uint32_t thread
 {
     const int rc = set_smem(gather_dot_kernel<BF16, LAT, R>, smem);
     if (rc) return rc;
-    gather_dot_kernel<BF16, LAT, R><<<(uint32_t)grid, threads, smem, st>>>(P);
+    slonn_launch(gather_dot_kernel<BF16, LAT, R>, (uint32_t)grid, threads, smem, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -274,7 +274,7 @@ int launch_gather_short_t(const slonn_gather_params &P, uint64_t grid, size_t sm
 {
     const int rc = set_smem(gather_short_kernel<BF16>, smem);
     if (rc) return rc;
-    gather_short_kernel<BF16><<<(uint32_t)grid, SLONN_THREADS, smem, st>>>(P);
+    slonn_launch(gather_short_kernel<BF16>, (uint32_t)grid, SLONN_THREADS, smem, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -314,7 +314,7 @@ int launch_group_rows_t(const slonn_group_params &Q, uint64_t grid, size_t smem,
 {
     const int rc = set_smem(group_rows_kernel<BF16>, smem);
     if (rc) return rc;
-    group_rows_kernel<BF16><<<(uint32_t)grid, SLONN_THREADS, smem, st>>>(Q);
+    slonn_launch(group_rows_kernel<BF16>, (uint32_t)grid, SLONN_THREADS, smem, st, Q);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -381,9 +381,9 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
     if (cudaMemsetAsync(gw.count, 0, sizeof(uint32_t), st) != cudaSuccess) return SLONN_ERR_CUDA;
     const uint32_t mid = 3750u;
     if (split <= mid)
-        range_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, P.skip_bp, n, split, std::min(mid, hi), gw.list, gw.count);
+        slonn_launch(range_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, P.skip_bp, n, split, std::min(mid, hi), gw.list, gw.count);
     if (hi > mid)
-        range_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, P.skip_bp, n, std::max(split, mid + 1u), hi, gw.list, gw.count);
+        slonn_launch(range_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, P.skip_bp, n, std::max(split, mid + 1u), hi, gw.list, gw.count);
     if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     Q.list = gw.list; Q.count = gw.count;
     const uint32_t groups = (n + SLONN_GROUP - 1) / SLONN_GROUP;
@@ -410,7 +410,7 @@ int launch_gather_cols_t(const slonn_gather_params &P, uint64_t grid, uint32_t t
 {
     const int rc = set_smem(gather_cols_kernel<BF16, R, SPLIT, VEC>, smem);
     if (rc) return rc;
-    gather_cols_kernel<BF16, R, SPLIT, VEC><<<(uint32_t)grid, threads, smem, st>>>(P);
+    slonn_launch(gather_cols_kernel<BF16, R, SPLIT, VEC>, (uint32_t)grid, threads, smem, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -457,7 +457,7 @@ int launch_layer_cols_t(const slonn_layer_cols_params &Q, uint64_t grid, uint32_
 {
     const int rc = set_smem(layer_cols_kernel<BF16, IDT, SPLIT, TIGHT>, smem);
     if (rc) return rc;
-    layer_cols_kernel<BF16, IDT, SPLIT, TIGHT><<<(uint32_t)grid, threads, smem, st>>>(Q);
+    slonn_launch(layer_cols_kernel<BF16, IDT, SPLIT, TIGHT>, (uint32_t)grid, threads, smem, st, Q);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -475,7 +475,7 @@ int launch_select_cols_t(const slonn_layer_cols_params &Q, uint32_t n, size_t sm
 {
     const int rc = set_smem(hash_select_cols_kernel<BF16, IDT>, smem);
     if (rc) return rc;
-    hash_select_cols_kernel<BF16, IDT><<<n, SLONN_THREADS, smem, st>>>(Q);
+    slonn_launch(hash_select_cols_kernel<BF16, IDT>, n, SLONN_THREADS, smem, st, Q);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -634,7 +634,7 @@ int launch_tile_rows_t(const slonn_tile_params &P, cudaStream_t st)
 {
     const int rc = set_smem(tile_rows_kernel<BF16, QUAD>, SLONN_TILE_SMEM);
     if (rc) return rc;
-    tile_rows_kernel<BF16, QUAD><<<148u, SLONN_TILE_WARPS * 32, SLONN_TILE_SMEM, st>>>(P);
+    slonn_launch(tile_rows_kernel<BF16, QUAD>, 148u, SLONN_TILE_WARPS * 32, SLONN_TILE_SMEM, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -657,7 +657,7 @@ int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint3
         slonn_order_params P;
         P.key = (const uint64_t *)(tw.ws + T.key); P.budget_bp = b->budget_bp; P.bp_lo = lo; P.bp_hi = hi; P.q0 = q0; P.n = std::min(T.chunk, n - q0);
         P.work = (uint32_t *)(tw.ws + T.work); P.order = (uint32_t *)(tw.ws + T.order) + (uint64_t)c * T.order_stride;
-        tile_order_kernel<<<(P.n + 31) / 32, 256, 0, st>>>(P);
+        slonn_launch(tile_order_kernel, (P.n + 31) / 32, 256, 0, st, P);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     }
     return SLONN_OK;
@@ -694,7 +694,7 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
         P.groups = (P.n + SLONN_TILE_G - 1) / SLONN_TILE_G;
         // the sort cleared the count of work items; only the first chunk can rely on it
         if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
-        tile_prep_kernel<<<dim3(P.groups, 2), 512, smem, st>>>(P);
+        slonn_launch(tile_prep_kernel, dim3(P.groups, 2), 512, smem, st, P);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
         rc = bf ? launch_tile_rows<true>(P, st) : launch_tile_rows<false>(P, st);
         if (rc) return rc;
@@ -753,7 +753,7 @@ int launch_full_rows_t(const slonn_full_params &P, uint64_t grid, size_t smem, c
 {
     const int rc = set_smem(full_rows_kernel<BF16, SLONN_FULL_R>, smem);
     if (rc) return rc;
-    full_rows_kernel<BF16, SLONN_FULL_R><<<(uint32_t)grid, SLONN_THREADS, smem, st>>>(P);
+    slonn_launch(full_rows_kernel<BF16, SLONN_FULL_R>, (uint32_t)grid, SLONN_THREADS, smem, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -800,7 +800,7 @@ int launch_fused_g(const slonn_fused_params &P, cudaStream_t st)
     int rc = set_smem(fused_network_kernel<BF16, NC, GRP, COLS>, smem);
     if (rc) return rc;
     const uint32_t grid = (P.n + SLONN_FUSED_WARPS - 1) / SLONN_FUSED_WARPS;
-    fused_network_kernel<BF16, NC, GRP, COLS><<<grid, SLONN_FUSED_WARPS * 32, smem, st>>>(P);
+    slonn_launch(fused_network_kernel<BF16, NC, GRP, COLS>, grid, SLONN_FUSED_WARPS * 32, smem, st, P);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -1009,8 +1009,8 @@ int slonn_forward_sparse_first(const slonn_model *m, const uint64_t *indptr, con
     sp.status = status;
     const uint64_t grid = (uint64_t)n * sp.blocks_per_query;
     if (grid == 0 || grid > 0x7fffffffull) return SLONN_ERR_DIM;
-    if (m->dtype == SLONN_BF16) sparse_first_layer_kernel<true><<<(uint32_t)grid, 128, 0, st>>>(sp);
-    else sparse_first_layer_kernel<false><<<(uint32_t)grid, 128, 0, st>>>(sp);
+    if (m->dtype == SLONN_BF16) slonn_launch(sparse_first_layer_kernel<true>, (uint32_t)grid, 128, 0, st, sp);
+    else slonn_launch(sparse_first_layer_kernel<false>, (uint32_t)grid, 128, 0, st, sp);
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -1082,7 +1082,7 @@ static int run_full_route(const slonn_model *m, const slonn_batch *b, uint32_t n
         if (ly.has_act) {
             if (b->codes) { // keys from the signs of the hash nodes' values (every node was computed)
                 const uint32_t t = n * m->L;
-                dense_codes_kernel<<<(t + 127) / 128, 128, 0, st>>>(list, count, vals, indptr, m->n_act, m->act_index[l],
+                slonn_launch(dense_codes_kernel, (t + 127) / 128, 128, 0, st, list, count, vals, indptr, m->n_act, m->act_index[l],
                                                                    ly.hash_nodes, m->K, m->L, b->codes);
                 if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
             }
@@ -1180,8 +1180,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
         uint64_t *tile_sums = (uint64_t *)(ws + wl.plan_sums);
         AT_LAYER(SLONN_ALL_LAYERS);
         TIC(SLONN_STAGE_PLAN);
-        plan_partial_kernel<<<(uint32_t)tiles, SLONN_PLAN_THREADS, 0, st>>>(pp, tile_sums);
-        plan_final_kernel<<<(uint32_t)tiles, SLONN_PLAN_THREADS, 0, st>>>(pp, tile_sums);
+        slonn_launch(plan_partial_kernel, (uint32_t)tiles, SLONN_PLAN_THREADS, 0, st, pp, tile_sums);
+        slonn_launch(plan_final_kernel, (uint32_t)tiles, SLONN_PLAN_THREADS, 0, st, pp, tile_sums);
         TOC();
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     }
@@ -1206,8 +1206,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
         int rc = SLONN_OK;
         if (cudaMemsetAsync(tc_count, 0, sizeof(uint32_t), st) != cudaSuccess) rc = SLONN_ERR_CUDA;
         if (!rc) {
-            dense_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, n, tc_list, tc_count);
-            dense_gather_x_kernel<<<n, 128, 0, st>>>(b->x_dense, m->layer[0].D, tc_list, tc_count, A[0]);
+            slonn_launch(dense_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, n, tc_list, tc_count);
+            slonn_launch(dense_gather_x_kernel, n, 128, 0, st, b->x_dense, m->layer[0].D, tc_list, tc_count, A[0]);
             if (cudaGetLastError() != cudaSuccess) rc = SLONN_ERR_CUDA;
         }
         for (uint32_t l = 0; l < m->n_layers && !rc; ++l) {
@@ -1230,7 +1230,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             rc = slonn_dense_tc_launch(A[l & 1], ly.W, ly.N, ly.D, E, st);
             if (!rc && ly.has_act && b->codes) {
                 const uint32_t t = n * m->L;
-                dense_codes_kernel<<<(t + 127) / 128, 128, 0, st>>>(tc_list, tc_count, vals, indptr, m->n_act,
+                slonn_launch(dense_codes_kernel, (t + 127) / 128, 128, 0, st, tc_list, tc_count, vals, indptr, m->n_act,
                                                                    m->act_index[l], ly.hash_nodes, m->K, m->L, b->codes);
                 if (cudaGetLastError() != cudaSuccess) rc = SLONN_ERR_CUDA;
             }
@@ -1247,7 +1247,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
     if (full_route) {
         uint32_t *full_list = (uint32_t *)(ws + wl.tc_list), *full_count = (uint32_t *)(ws + wl.tc_count);
         if (cudaMemsetAsync(full_count, 0, sizeof(uint32_t), st) != cudaSuccess) return SLONN_ERR_CUDA;
-        dense_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, n, full_list, full_count);
+        slonn_launch(dense_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, n, full_list, full_count);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
         const int rc = run_full_route(m, b, n, full_list, full_count, indptr, ids, vals, dense, stride, max_bp, tw, st, tm);
         if (rc) return rc;
@@ -1274,8 +1274,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             ap.fixed_len = last.N;
         }
         TIC(SLONN_STAGE_ARGMAX, b->budget_bp, 10000u, 10000u);
-        if (stride >= 2048) argmax_block_kernel<<<n, 256, 0, st>>>(ap);
-        else argmax_kernel<<<(n + 7) / 8, 256, 0, st>>>(ap);
+        if (stride >= 2048) slonn_launch(argmax_block_kernel, n, 256, 0, st, ap);
+        else slonn_launch(argmax_kernel, (n + 7) / 8, 256, 0, st, ap);
         TOC();
         return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
     }
@@ -1376,7 +1376,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                 cols_bp < max_bp) {
                 uint32_t *glist = (uint32_t *)(ws + wl.tc_list), *gcount = (uint32_t *)(ws + wl.tc_count);
                 if (cudaMemsetAsync(gcount, 0, sizeof(uint32_t), st) != cudaSuccess) return SLONN_ERR_CUDA;
-                range_compact_kernel<<<(n + 255) / 256, 256, 0, st>>>(b->budget_bp, skip_bp, n, cols_bp ? cols_bp + 1 : 0u, 0xffffu,
+                slonn_launch(range_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, skip_bp, n, cols_bp ? cols_bp + 1 : 0u, 0xffffu,
                                                                      glist, gcount);
                 if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
                 slonn_full_params fp;
@@ -1409,8 +1409,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
         }
         AT_LAYER(SLONN_ALL_LAYERS);
         TIC(SLONN_STAGE_ARGMAX);
-        if (stride >= 2048) argmax_block_kernel<<<n, 256, 0, st>>>(ap);
-        else argmax_kernel<<<(n + 7) / 8, 256, 0, st>>>(ap);
+        if (stride >= 2048) slonn_launch(argmax_block_kernel, n, 256, 0, st, ap);
+        else slonn_launch(argmax_kernel, (n + 7) / 8, 256, 0, st, ap);
         TOC();
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     }

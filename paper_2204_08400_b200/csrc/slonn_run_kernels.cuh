@@ -95,6 +95,7 @@ __device__ __forceinline__ uint32_t plan_count(const slonn_plan_params &P, uint6
 
 __global__ void __launch_bounds__(SLONN_PLAN_THREADS) plan_partial_kernel(slonn_plan_params P, uint64_t *tile_sums)
 {
+    slonn_enter();
     __shared__ uint64_t warp_sums[32];
     __shared__ uint64_t total;
     const uint64_t M = (uint64_t)P.n * P.n_act;
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(SLONN_PLAN_THREADS) plan_partial_kernel(slonn_
 
 __global__ void __launch_bounds__(SLONN_PLAN_THREADS) plan_final_kernel(slonn_plan_params P, const uint64_t *tile_sums)
 {
+    slonn_enter();
     __shared__ uint64_t warp_sums[32];
     __shared__ uint64_t total;
     __shared__ uint64_t base_total;
@@ -305,6 +307,7 @@ __device__ __forceinline__ bool block_select(const void *tables, uint32_t cap, u
 template <bool BF16, typename IDT, bool LAT>
 __global__ void __launch_bounds__(LAT ? 1024 : SLONN_THREADS, LAT ? 1 : SLONN_SELECT_MIN_BLOCKS) hash_select_kernel(slonn_select_params P)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     float4 *xs4 = smem4;
     uint32_t *bitmap = reinterpret_cast<uint32_t *>(smem4 + (P.D >> 2));
@@ -407,6 +410,7 @@ __launch_bounds__(SLONN_THREADS)
 #endif
 __global__ void gather_dot_kernel(slonn_gather_params P)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     const uint32_t q = blockIdx.x / P.ctas_per_query;
     const uint32_t chunk = blockIdx.x - q * P.ctas_per_query;
@@ -521,6 +525,7 @@ struct slonn_full_params {
 template <bool BF16, int R>
 __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FULL_MIN_BLOCKS) full_rows_kernel(slonn_full_params P)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int VPC = BF16 ? 8 : 4;
     constexpr int G = SLONN_FULL_GROUP;
@@ -539,7 +544,7 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FULL_MIN_BLOCKS) full_row
 #pragma unroll
     for (int k = 0; k < G; ++k) {
         q[k] = g * G + min((uint32_t)k, nq - 1); // a short last group repeats its last query
-        if (P.list) q[k] = __ldg(P.list + q[k]);
+        if (P.list) q[k] = P.list[q[k]];
         off[k] = P.has_act ? P.indptr[(uint64_t)q[k] * P.n_act + P.a] : 0;
         stage_input<BF16>(P.in, q[k], P.D, P.nchunks, smem4 + k * per_q);
     }
@@ -620,6 +625,7 @@ struct slonn_group_params {
 template <bool BF16>
 __global__ void __launch_bounds__(SLONN_THREADS, SLONN_GROUP_MIN_BLOCKS) group_rows_kernel(slonn_group_params Q)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int VPC = BF16 ? 8 : 4;
     constexpr int G = SLONN_GROUP, R = 4;
@@ -629,9 +635,9 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_GROUP_MIN_BLOCKS) group_r
     const uint32_t g = blockIdx.x / Q.ctas_per_group;
     const uint32_t chunk = blockIdx.x - g * Q.ctas_per_group;
     const uint32_t cnt = Q.count ? *Q.count : Q.n;
-    if (g * G >= cnt || __ldg(Q.list + g * G) == 0xffffffffu) return; // queries come first in a list
+    if (g * G >= cnt || Q.list[g * G] == 0xffffffffu) return; // queries come first in a list
     uint32_t nq = min((uint32_t)G, cnt - g * G);
-    while (__ldg(Q.list + g * G + nq - 1u) == 0xffffffffu) --nq;
+    while (Q.list[g * G + nq - 1u] == 0xffffffffu) --nq;
     const uint32_t per_q = (BF16 ? 2u : 1u) * P.nchunks; // float4 per staged input
     const uint32_t nwords = (P.N + 31u) >> 5;
 
@@ -648,7 +654,7 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_GROUP_MIN_BLOCKS) group_r
     uint64_t off[G];
 #pragma unroll
     for (int k = 0; k < G; ++k) {
-        q[k] = __ldg(Q.list + g * G + min((uint32_t)k, nq - 1)); // a short last group repeats its last query
+        q[k] = Q.list[g * G + min((uint32_t)k, nq - 1)]; // a short last group repeats its last query
         off[k] = P.indptr[(uint64_t)q[k] * P.n_act + P.a];
         B[k] = min((uint32_t)(P.indptr[(uint64_t)q[k] * P.n_act + P.a + 1] - off[k]), Q.rows_cap);
         stage_input<BF16>(P.in, q[k], P.D, P.nchunks, smem4 + k * per_q);
@@ -784,6 +790,7 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_GROUP_MIN_BLOCKS) group_r
 template <bool BF16>
 __global__ void __launch_bounds__(SLONN_THREADS, 2) gather_short_kernel(slonn_gather_params P)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int VPC = BF16 ? 8 : 4;
     constexpr int R = 8;
@@ -1046,6 +1053,7 @@ __launch_bounds__(SLONN_THREADS)
 #endif
 __global__ void gather_cols_kernel(slonn_gather_params P)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int V = BF16 ? 8 : 4;
     __shared__ uint32_t segcnt[32];
@@ -1108,6 +1116,7 @@ template <bool BF16, typename IDT, bool SPLIT, bool TIGHT>
 __launch_bounds__(SLONN_THREADS, (SPLIT || TIGHT) ? 6 : 5) // 40 or 48 registers
 __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int V = BF16 ? 8 : 4;
     constexpr int R = 2;
@@ -1198,6 +1207,7 @@ template <bool BF16, typename IDT>
 __launch_bounds__(SLONN_THREADS, 6)
 __global__ void hash_select_cols_kernel(slonn_layer_cols_params Q)
 {
+    slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int V = BF16 ? 8 : 4;
     constexpr uint32_t ESZ = BF16 ? 2u : 4u;
@@ -1278,6 +1288,7 @@ struct slonn_sparse_params {
 template <bool BF16>
 __global__ void __launch_bounds__(128) sparse_first_layer_kernel(slonn_sparse_params P)
 {
+    slonn_enter();
     __shared__ uint32_t s_ids[128];
     __shared__ float s_vals[128];
     const uint32_t q = blockIdx.x / P.blocks_per_query;
@@ -1341,6 +1352,7 @@ struct slonn_argmax_params {
 
 __global__ void __launch_bounds__(256) argmax_kernel(slonn_argmax_params P)
 {
+    slonn_enter();
     const uint32_t q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const uint32_t lane = threadIdx.x & 31u;
     if (q >= P.n) return;
@@ -1372,6 +1384,7 @@ __global__ void __launch_bounds__(256) argmax_kernel(slonn_argmax_params P)
 // The same with one block per query, for logit rows of thousands of entries.
 __global__ void __launch_bounds__(256) argmax_block_kernel(slonn_argmax_params P)
 {
+    slonn_enter();
     __shared__ float wbest[8];
     __shared__ uint32_t wbi[8];
     const uint32_t q = blockIdx.x;
@@ -1420,6 +1433,7 @@ __global__ void __launch_bounds__(256) argmax_block_kernel(slonn_argmax_params P
 __global__ void range_compact_kernel(const uint16_t *bp, const uint16_t *skip_bp, uint32_t n, uint32_t lo, uint32_t hi,
                                      uint32_t *list, uint32_t *count)
 {
+    slonn_enter();
     const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31u;
     bool take = false;
@@ -1437,6 +1451,7 @@ __global__ void range_compact_kernel(const uint16_t *bp, const uint16_t *skip_bp
 
 __global__ void dense_compact_kernel(const uint16_t *bp, uint32_t n, uint32_t *list, uint32_t *count)
 {
+    slonn_enter();
     const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31u;
     const bool full = q < n && bp[q] == 10000u;
@@ -1460,6 +1475,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2_rne(float a, float b)
 __global__ void dense_gather_x_kernel(const float *x, uint32_t D, const uint32_t *list, const uint32_t *count,
                                       uint16_t *A)
 {
+    slonn_enter();
     const uint32_t m = blockIdx.x;
     if (m >= *count) return;
     const float4 *src = reinterpret_cast<const float4 *>(x + (uint64_t)list[m] * D);
@@ -1476,6 +1492,7 @@ __global__ void dense_codes_kernel(const uint32_t *list, const uint32_t *count, 
                                    const uint64_t *indptr, uint32_t n_act, uint32_t a, const uint32_t *hash_nodes,
                                    uint32_t K, uint32_t L, uint16_t *codes)
 {
+    slonn_enter();
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t m = t / L, b = t - m * L;
     if (m >= *count) return;

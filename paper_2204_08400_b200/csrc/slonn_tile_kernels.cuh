@@ -44,6 +44,7 @@ struct slonn_order_params {
 // queries) spread over the GPU take 3 us, less than the launches of a radix sort.  A warp ranks four queries.
 __global__ void __launch_bounds__(256) tile_order_kernel(slonn_order_params P)
 {
+    slonn_enter();
     __shared__ uint64_t s[2048];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t e0 = (blockIdx.x * 8u + warp) * 4u;
@@ -131,6 +132,7 @@ __device__ __forceinline__ uint32_t tile_query(const slonn_tile_params &P, uint3
 // nodes and adds the group's work items.  One warp per query; a warp's list reads are issued eight at a time.
 __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
 {
+    slonn_enter();
     extern __shared__ uint32_t smem_u[];
     constexpr int G = SLONN_TILE_G;
     __shared__ uint32_t slotcnt[32];
@@ -427,6 +429,7 @@ template <bool BF16, bool QUAD> struct tile_weights {
 template <bool BF16, bool QUAD>
 __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slonn_tile_params P)
 {
+    slonn_enter();
     constexpr int G = SLONN_TILE_G, NN = SLONN_TILE_NN, W = SLONN_TILE_WARPS;
     constexpr uint32_t ESZ = BF16 ? 2u : 4u;
     constexpr uint32_t BLOCK_STEPS = SLONN_TILE_BLOCK / 2;

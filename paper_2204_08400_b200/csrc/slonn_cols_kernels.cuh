@@ -64,8 +64,8 @@ __device__ __forceinline__ void cols_stage_list(const cols_stage &S, const uint3
     };
 #pragma unroll 4
     for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
-        const uint32_t j = __ldg(ids + s0 + i);
-        const float v = __ldg(vals + s0 + i);
+        const uint32_t j = ids[s0 + i];
+        const float v = vals[s0 + i];
         if (j < D && v != 0.0f) {
             uint32_t p, pos;
             place(j, p, pos);
@@ -99,8 +99,8 @@ __device__ __forceinline__ void cols_stage_list(const cols_stage &S, const uint3
     __syncthreads();
 #pragma unroll 4
     for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
-        const uint32_t j = __ldg(ids + s0 + i);
-        const float v = __ldg(vals + s0 + i);
+        const uint32_t j = ids[s0 + i];
+        const float v = vals[s0 + i];
         if (j < D && v != 0.0f) {
             uint32_t p, pos;
             place(j, p, pos);

@@ -71,8 +71,12 @@ __host__ __device__ __forceinline__ uint32_t slonn_layer_nodes(uint32_t bp, uint
 
 // First statement of every kernel of a run.  The run's launches are chained with programmatic dependencies
 // (slonn_launch): a kernel may be brought onto the SMs as soon as all blocks of the one before it have started, and waits
-// here until that one has finished and its writes can be seen.  Nothing may be read or written before this; loads through
-// the read-only path stay behind it because each sits behind a branch on, or at an address from, a plain load.
+// here until that one has finished and its writes can be seen.  Nothing may be read or written before this.
+// Read-only loads (__ldg) are for memory that nobody writes while the kernel is resident, and the compiler may move them
+// across the wait: weights and their copies, biases, tables, hash nodes and the caller's own inputs, which are complete
+// before a run's first kernel becomes resident because the run begins with a memset, a full dependency.  Whatever a kernel
+// of the same chain writes -- lists, offsets, sort order, staged values, the dense activations of a layer below -- is read
+// with plain loads, which the wait orders.
 __device__ __forceinline__ void slonn_enter()
 {
     asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
@@ -323,7 +327,7 @@ __device__ __forceinline__ void stage_input(const slonn_input &in, uint32_t q, u
         const float4 *src = reinterpret_cast<const float4 *>(in.dense + (uint64_t)q * D);
 #pragma unroll 4
         for (uint32_t i = threadIdx.x; i < nvec; i += blockDim.x) {
-            const float4 v = __ldg(src + i);
+            const float4 v = src[i]; // a kernel of the same chain may have written it: no read-only load
             if (BF16) xs4[(i & 1u) * nchunks + (i >> 1)] = v;
             else xs4[i] = v;
         }

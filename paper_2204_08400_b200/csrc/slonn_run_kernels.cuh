@@ -431,7 +431,7 @@ __global__ void gather_dot_kernel(slonn_gather_params P)
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     if (LAT) { // one row per warp, deep load prefetch
         for (uint32_t r = r0 + warp; r < r1; r += nwarps) {
-            const uint32_t nd = P.use_list ? __ldg(P.ids + off + r) : r;
+            const uint32_t nd = P.use_list ? P.ids[off + r] : r;
             const float sum = warp_dot_row1<BF16>(reinterpret_cast<const uint4 *>(P.W) + (uint64_t)nd * P.nchunks, smem4,
                                                   P.nchunks, lane);
             if (lane == 0) {
@@ -454,7 +454,7 @@ __global__ void gather_dot_kernel(slonn_gather_params P)
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const uint32_t rr = min(r + k, r1 - 1);
-            const uint32_t nd = P.use_list ? __ldg(P.ids + off + rr) : rr;
+            const uint32_t nd = P.use_list ? P.ids[off + rr] : rr;
             rows[k] = reinterpret_cast<const uint4 *>(P.W) + (uint64_t)nd * P.nchunks;
         }
         float acc[R];
@@ -472,7 +472,7 @@ __global__ void gather_dot_kernel(slonn_gather_params P)
             writer = (lane & 7u) == 0u;
         }
         if (writer && mr < r1) {
-            const uint32_t nd = P.use_list ? __ldg(P.ids + off + mr) : mr;
+            const uint32_t nd = P.use_list ? P.ids[off + mr] : mr;
             float z = sum + __ldg(P.bias + nd);
             if (P.relu) z = z > 0.0f ? z : 0.0f;
             if (P.use_list) {
@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(SLONN_THREADS, SLONN_GROUP_MIN_BLOCKS) group_r
     for (int k = 0; k < G; ++k)
         if ((uint32_t)k < nq)
             for (uint32_t i = threadIdx.x; i < B[k]; i += blockDim.x) {
-                const uint32_t id = min(__ldg(P.ids + off[k] + i), P.N - 1u);
+                const uint32_t id = min(P.ids[off[k] + i], P.N - 1u);
                 atomicOr(&bm[k * nwords + (id >> 5)], 1u << (id & 31u));
             }
     __syncthreads();
@@ -827,7 +827,7 @@ __global__ void __launch_bounds__(SLONN_THREADS, 2) gather_short_kernel(slonn_ga
     const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
     for (uint32_t base = r0 + warp * 32u; base < r1; base += nwarps * 32u) {
         const uint32_t mine = min(base + lane, r1 - 1);
-        const uint32_t myid = P.use_list ? __ldg(P.ids + off + mine) : mine;
+        const uint32_t myid = P.use_list ? P.ids[off + mine] : mine;
 #pragma unroll
         for (uint32_t sub = 0; sub < 4; ++sub) {
             const uint32_t r = base + sub * R;
@@ -865,21 +865,17 @@ __global__ void __launch_bounds__(SLONN_THREADS, 2) gather_short_kernel(slonn_ga
 
 // Second half of the input-stationary layer, shared by gather_cols_kernel and layer_cols_kernel: puts the
 // query's selected nodes in column order and evaluates nodes [r0, r1) of that order against the staged
-// input list S.  `order_mem` is block scratch of P.scratch_bytes (the staging image, dead by now).  NC: the
-// id list was written by an earlier launch and may be read through the read-only path.
+// input list S.  `order_mem` is block scratch of P.scratch_bytes (the inputs' bitmap, dead by now).
 // VEC: compiled with the path for a layer that computes every node and whose width is a multiple of the
 // 16 / element size nodes one load holds: a lane takes that many neighbouring columns.
-template <bool BF16, int R, bool NC, bool SPLIT = false, bool VEC = false>
+template <bool BF16, int R, bool SPLIT = false, bool VEC = false>
 __device__ __forceinline__ void cols_order_and_gather(const slonn_gather_params &P, const cols_stage &S, void *order_mem,
                                                       const uint32_t *idlist, float *zpart, uint32_t q, uint64_t off,
                                                       uint32_t B, uint32_t r0, uint32_t r1, uint32_t *scan_ws,
                                                       uint32_t *scan_total_p)
 {
     // idlist: the query's id-ascending node list (global or shared memory; unused when every node is computed)
-    auto list_id = [&](uint32_t e) -> uint32_t {
-        const uint32_t v = NC ? __ldg(idlist + e) : idlist[e];
-        return min(v, P.N - 1u);
-    };
+    auto list_id = [&](uint32_t e) -> uint32_t { return min(idlist[e], P.N - 1u); };
     // the query's nodes in column order: spos[slot] = column, sidx[slot] = place in the id-ascending list
     const bool ordered = P.use_list && P.colpos;
     uint32_t *bitmap = reinterpret_cast<uint32_t *>(order_mem);
@@ -1084,8 +1080,8 @@ __global__ void gather_cols_kernel(slonn_gather_params P)
     const uint32_t len = min((uint32_t)(P.in.indptr[(uint64_t)q * P.in.ip_mul + P.in.ip_add + 1] - s0), P.in_cap);
     cols_stage_list<V>(S, P.in.ids, P.in.vals, s0, len, P.D);
 
-    cols_order_and_gather<BF16, R, true, SPLIT, VEC>(P, S, smem4, P.ids + off, reinterpret_cast<float *>(S.ent + cols_ent_cap(P.D, P.in_cap)),
-                                                 q, off, B, r0, r1, scan_ws, &scan_total);
+    cols_order_and_gather<BF16, R, SPLIT, VEC>(P, S, smem4, P.ids + off, reinterpret_cast<float *>(S.ent + cols_ent_cap(P.D, P.in_cap)),
+                                           q, off, B, r0, r1, scan_ws, &scan_total);
 }
 
 // A whole list-fed activator layer for one query per block, input-stationary: the input list is grouped
@@ -1197,7 +1193,7 @@ __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
     if (SPLIT && writer)
         for (uint32_t i = threadIdx.x; i < B; i += blockDim.x) global_list[i] = own_list[i];
     // (5) the selected nodes
-    cols_order_and_gather<BF16, R, false, SPLIT>(P, S, smem4, list, zpart, q, off, B, r0, r1, scan_ws, &scan_total);
+    cols_order_and_gather<BF16, R, SPLIT>(P, S, smem4, list, zpart, q, off, B, r0, r1, scan_ws, &scan_total);
 }
 
 // Hash and selection of a list-fed activator layer, input-stationary: the first half of layer_cols_kernel for layers

@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const bool in = i0 + u * 32u + lane < len;
-                j[u] = in ? __ldg(ids + i0 + u * 32u + lane) : 0xffffffffu;
-                v[u] = in ? __ldg(vals + i0 + u * 32u + lane) : 0.0f;
+                j[u] = in ? ids[i0 + u * 32u + lane] : 0xffffffffu;
+                v[u] = in ? vals[i0 + u * 32u + lane] : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u)
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
             krow[at] = j * P.ldb;
             float v[G];
 #pragma unroll
-            for (int i = 0; i < G; ++i) v[i] = s_q[i] != 0xffffffffu ? __ldg(P.in.dense + (uint64_t)s_q[i] * P.D + j) : 0.0f;
+            for (int i = 0; i < G; ++i) v[i] = s_q[i] != 0xffffffffu ? P.in.dense[(uint64_t)s_q[i] * P.D + j] : 0.0f;
 #pragma unroll
             for (int i = 0; i < G; i += 4) xt4[((uint64_t)at * G + i) / 4] = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         }

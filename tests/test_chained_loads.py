@@ -47,3 +47,11 @@ def test_the_check_sees_direct_and_renamed_loads():
         assert names & (WRITTEN | aliases), body
     arg, names, aliases = next(iter(read_only_loads("__global__ void k(P p) { b = __ldg(P.bias + P.ids[r]); }")))
     assert not names & (WRITTEN | aliases)
+
+
+def test_no_kernel_lets_the_next_one_in_early():
+    """Blocks of the next kernel would wait in slots that another stream's blocks could use."""
+    for name in FILES:
+        with open(os.path.join(CSRC, name)) as f:
+            code = re.sub(r"//[^\n]*", "", f.read())
+        assert "launch_dependents" not in code and "TriggerProgrammaticLaunch" not in code, name

@@ -56,3 +56,43 @@ def test_csr_fed_first_layer_on_changing_inputs():
         for k in ("logits", "pred", "codes", "active_ids", "active_vals"):
             assert np.array_equal(got[k], want[turn % 3][k]), (turn, k)
     dm.free()
+
+
+def test_two_threads_with_a_stream_each():
+    """One model, two host threads, two streams, batches of different sizes and budgets that take the grouped products, each
+    with a workspace of its own: every run's results are those of the batch alone."""
+    import threading
+    import torch
+    from paper_2204_08400_b200 import harness
+    wl = custom_workload(4350, [512, 1536, 1536, 130], [1, 1, 0], "bf16", n=700, n_cal=300, K=4, L=2,
+                         budgets=(1000, 5000, 9000, 10000))
+    dm = harness.DeviceModel(wl)
+    parts = [(wl.x, wl.budget_bp), (wl.x[:300], np.full(300, 6000, np.uint16))]
+    batches = [harness.DeviceBatch(dm, x, bp, kernel_path=1) for x, bp in parts]
+    want = []
+    for b in batches:
+        b.run()
+        want.append(b.results())
+    streams = [torch.cuda.Stream() for _ in parts]
+    torch.cuda.synchronize()
+    keys = ("logits", "pred", "codes", "active_ids", "active_vals")
+    wrong = []
+
+    def work(i):
+        for _ in range(15):
+            for t in (batches[i].logits, batches[i].vals, batches[i].ids):
+                with torch.cuda.stream(streams[i]):
+                    t.zero_()
+            batches[i].run(streams[i])
+            batches[i].run(streams[i])
+            streams[i].synchronize()
+            got = batches[i].results()
+            wrong.extend((i, k) for k in keys if not np.array_equal(got[k], want[i][k]))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, wrong[:4]
+    dm.free()

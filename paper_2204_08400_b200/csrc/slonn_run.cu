@@ -341,10 +341,11 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
 {
     uint32_t shared_cap = 0;
     const size_t smem = group_rows_smem(P, max_rows, &shared_cap);
-    const uint32_t lo = P.range_bp ? P.bp_lo : 0u, hi = std::min(P.range_bp ? P.bp_hi : 0xffffu, max_bp);
+    const uint32_t lo = P.range_bp ? P.bp_lo : 0u, hi = P.range_bp ? P.bp_hi : 0xffffu;
+    const uint32_t top = std::min(hi, max_bp); // largest budget that is no error; the clamped lists above it are served with it
     const uint32_t split = std::max(lo, sorted ? sorted->lo : SLONN_GROUP_MIN_BP + 1u); // budgets from here on are grouped
     const bool grouped = P.use_list && n >= 256 && P.N <= 65535u && P.nchunks > 32 && gw.list && smem <= 110 * 1024 &&
-                         !(b->flags & SLONN_FLAG_UNGROUPED_ROWS) && hi >= split;
+                         !(b->flags & SLONN_FLAG_UNGROUPED_ROWS) && top >= split;
     int rc;
     if (!grouped) {
         TIC(SLONN_STAGE_GATHER_DOT, P.range_bp, P.bp_lo, P.bp_hi, P.skip_bp);
@@ -381,8 +382,8 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
     if (cudaMemsetAsync(gw.count, 0, sizeof(uint32_t), st) != cudaSuccess) return SLONN_ERR_CUDA;
     const uint32_t mid = 3750u;
     if (split <= mid)
-        slonn_launch(range_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, P.skip_bp, n, split, std::min(mid, hi), gw.list, gw.count);
-    if (hi > mid)
+        slonn_launch(range_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, P.skip_bp, n, split, top > mid ? mid : hi, gw.list, gw.count);
+    if (top > mid)
         slonn_launch(range_compact_kernel, (n + 255) / 256, 256, 0, st, b->budget_bp, P.skip_bp, n, std::max(split, mid + 1u), hi, gw.list, gw.count);
     if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     Q.list = gw.list; Q.count = gw.count;
@@ -644,10 +645,11 @@ int launch_tile_rows(const slonn_tile_params &P, cudaStream_t st)
     return !P.select && P.N % 4u == 0 ? launch_tile_rows_t<BF16, true>(P, st) : launch_tile_rows_t<BF16, false>(P, st);
 }
 
-// Sorts the batch's queries with a budget in [lo, hi] into groups by (budget, keys); the keys were written by the kernel
-// that hashed them.  *sorted: lowest budget of the groups the workspace held before (~0: none) and holds now; as long as
+// Sorts the batch's queries with a budget of at least lo (skip_full: but those at 10000 bp) into groups by (budget, keys); the
+// keys were written by the kernel that hashed them.  Budgets above the batch's maximum are errors, but such queries
+// have their clamped lists and are served like the others.  *sorted: lowest budget of the groups the workspace held before (~0: none) and holds now; as long as
 // it stays, the same number of entries is overwritten.
-int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint32_t lo, uint32_t hi, uint32_t *sorted, cudaStream_t st)
+int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint32_t lo, bool skip_full, uint32_t *sorted, cudaStream_t st)
 {
     const auto &T = tw.wl->tile;
     const uint64_t chunks = ((uint64_t)n + T.chunk - 1) / T.chunk;
@@ -655,7 +657,7 @@ int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint3
     *sorted = lo;
     for (uint32_t c = 0, q0 = 0; q0 < n; ++c, q0 += T.chunk) {
         slonn_order_params P;
-        P.key = (const uint64_t *)(tw.ws + T.key); P.budget_bp = b->budget_bp; P.bp_lo = lo; P.bp_hi = hi; P.q0 = q0; P.n = std::min(T.chunk, n - q0);
+        P.key = (const uint64_t *)(tw.ws + T.key); P.budget_bp = b->budget_bp; P.bp_lo = lo; P.skip_full = skip_full ? 1u : 0u; P.q0 = q0; P.n = std::min(T.chunk, n - q0);
         P.work = (uint32_t *)(tw.ws + T.work); P.order = (uint32_t *)(tw.ws + T.order) + (uint64_t)c * T.order_stride;
         slonn_launch(tile_order_kernel, (P.n + 31) / 32, 256, 0, st, P);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
@@ -731,7 +733,6 @@ int launch_tile_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t 
         else if (rc != SLONN_ERR_DIM) return rc;
     }
     if (lo > max_bp) return SLONN_OK;
-    const uint32_t hi = skip_bp ? 9999u : 10000u;
     if (lo) { gp.range_bp = sp.range_bp = b->budget_bp; gp.bp_lo = sp.bp_lo = lo; gp.bp_hi = sp.bp_hi = 0xffffu; }
     sp.sort_key = key; sp.budget_bp = b->budget_bp;
     TIC(SLONN_STAGE_HASH_SELECT, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp);
@@ -740,7 +741,7 @@ int launch_tile_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t 
     TOC();
     if (rc) return rc;
     TIC(SLONN_STAGE_GROUP_ROWS, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp);
-    rc = launch_tile_order(tw, b, n, lo, hi, sorted, st);
+    rc = launch_tile_order(tw, b, n, lo, skip_bp != nullptr, sorted, st);
     if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 1, nullptr, nullptr, false, st, true);
     TOC();
     return rc;
@@ -1341,7 +1342,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                     TIC(SLONN_STAGE_HASH_SELECT, sp.range_bp, sp.bp_lo, sp.bp_hi, sp.skip_bp);
                     rc = launch_select(m, sp, n, max_rows, st);
                     TOC();
-                    if (!rc) rc = launch_tile_order(tw, b, n, from, skip_bp ? 9999u : 10000u, &sorted, st);
+                    if (!rc) rc = launch_tile_order(tw, b, n, from, skip_bp != nullptr, &sorted, st);
                     const sorted_groups sg = {(const uint32_t *)(ws + wl.tile.order), wl.tile.chunk, wl.tile.order_stride, from};
                     if (!rc) rc = launch_rows(m, gp, b, n, max_bp, max_rows, gw, st, tm, &sg);
                 } else {
@@ -1363,7 +1364,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             if (tw.ws && tile_layer_ok(m, l) && n >= SLONN_TILE_DENSE_MIN_QUERIES) {
                 TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp);
                 rc = SLONN_OK;
-                if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp ? 9999u : 10000u, &sorted, st);
+                if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp != nullptr, &sorted, st);
                 if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, keyed);
                 TOC();
                 if (rc) return rc;

@@ -34,7 +34,8 @@ __host__ __device__ __forceinline__ uint32_t tile_slot(uint32_t p) { return (p &
 struct slonn_order_params {
     const uint64_t *key;     // [n] sort key of each query (all different)
     const uint16_t *budget_bp;
-    uint32_t bp_lo, bp_hi;   // queries whose budget lies outside are left out
+    uint32_t bp_lo;          // queries with a smaller budget are left out
+    uint32_t skip_full;      // 1: and those at exactly 10000 bp
     uint32_t q0, n;          // queries [q0, q0 + n), n <= SLONN_TILE_CHUNK
     uint32_t *order;         // out: the first entries; the rest keep the 0xffffffff (no query) they were set to
     uint32_t *work;          // cleared for the tile_prep_kernel that follows
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(256) tile_order_kernel(slonn_order_params P)
     auto key_of = [&](uint32_t e) -> uint64_t { // ~0: left out
         if (e >= P.n) return ~0ull;
         const uint32_t bp = P.budget_bp[P.q0 + e];
-        return bp < P.bp_lo || bp > P.bp_hi ? ~0ull : P.key[P.q0 + e];
+        return bp < P.bp_lo || (P.skip_full && bp == 10000u) ? ~0ull : P.key[P.q0 + e];
     };
     bool any = false;
 #pragma unroll

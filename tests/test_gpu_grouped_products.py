@@ -75,3 +75,39 @@ def test_grouped_products_keep_queries_apart(dtype):
     others = [q for q in range(320) if q % 7 not in (5, 6)]
     assert np.array_equal(clean["logits"][others], dirty["logits"][others])
     dm.free()
+
+
+@pytest.mark.parametrize("dims,has_act,n,budgets,max_bp", [
+    ([512, 640, 520, 24], [1, 1, 0], 600, (1500, 2500, 6000), 6000),    # grouped rows, grouped products, plain last layer
+    ([512, 640, 520, 300], [1, 1, 1], 600, (2500, 6000), 6000),         # budgeted last layer
+    ([512, 640, 520, 24], [1, 1, 0], 600, (1500, 3000), 3000),          # both budget classes of the compacted row groups in one
+    ([512, 640, 520, 24], [1, 1, 0], 600, (2500, 6000, 10000), 10000),  # beside 100 % queries on their own route
+    ([512, 640, 520, 24], [1, 1, 0], 2100, (600, 800, 2500), 2500),     # groups sorted from a low budget on
+])
+def test_budgets_above_the_maximum_get_the_clamped_results(dims, has_act, n, budgets, max_bp):
+    """A query whose budget is too large is reported and evaluated at the batch's maximum, whatever kernels the batch takes; the
+    output buffers hold something else before the run."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4500 + n, dims, has_act, "bf16", n=n, n_cal=300, K=4, L=2, budgets=budgets)
+    dm = harness.DeviceModel(wl)
+    bad = {7: 20000, 8: 65535, 70: 10001, 71: 0, n - 1: max_bp + 1}
+    bp, clamped = wl.budget_bp.copy(), wl.budget_bp.copy()
+    for q, v in bad.items():
+        bp[q], clamped[q] = v, 1 if v == 0 else max_bp
+    want = harness.run_once(dm, wl.x, clamped, max_budget_bp=max_bp, kernel_path=1, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS)
+    for flags in (0, sl.FLAG_ROW_KERNELS, sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS):
+        b = harness.DeviceBatch(dm, wl.x, bp, max_budget_bp=max_bp, kernel_path=1, flags=flags)
+        b.logits.fill_(777.0)
+        b.vals.fill_(777.0)
+        b.pred.fill_(7777)
+        b.run()
+        got = b.results()
+        assert got["status"][0] == 5 and got["status"][1] in bad
+        ip = want["active_indptr"].astype(np.int64)
+        assert np.array_equal(got["active_indptr"], want["active_indptr"])
+        for k in ("pred", "codes", "active_ids", "active_vals"):
+            assert np.array_equal(got[k], want[k]), (flags, k)
+        for q in range(n):
+            B = int(ip[(q + 1) * sum(has_act)] - ip[(q + 1) * sum(has_act) - 1]) if has_act[-1] else dims[-1]
+            assert np.array_equal(got["logits"][q, :B], want["logits"][q, :B]), (flags, q)
+    dm.free()

@@ -124,8 +124,11 @@ __device__ __forceinline__ float chunk_elem(const uint4 &w)
 
 // acc[r] = fmaf(w[r][E], x[E], acc[r]) for every row, elements in ascending order; rows are
 // interleaved so that consecutive instructions belong to independent accumulation chains.
-// PACKED: two rows per packed instruction, each half rounded on its own as fmaf does.
-template <bool BF16, int R, int E, int VPC, bool PACKED = true>
+// PACKED: two rows per packed instruction, each half rounded on its own as fmaf does.  That pays where the two weights are
+// formed next to one another anyway, by widening; fp32 weights of two rows come out of two 16-byte loads and would
+// first have to be moved together (2100 queries on 1536-1536-1536-1536-300 fp32, plain layers: 1430 us one by one, 1590
+// packed; 200,000 outputs, 256 queries at 5 %: 111 against 119).
+template <bool BF16, int R, int E, int VPC, bool PACKED = BF16>
 struct chunk_fma {
     __device__ static __forceinline__ void run(const uint4 (&w)[R], const float *x, float (&acc)[R])
     {
@@ -151,14 +154,33 @@ struct chunk_fma<BF16, R, VPC, VPC, PACKED> {
 };
 
 // One 16-byte chunk of R rows (R even) for G queries: acc[g][r / 2] takes the products of rows r and r + 1 with query g's
-// inputs, elements in ascending order.  A pair of widened weights stays put for G packed multiply-adds in a row: that order
-// issues at the full rate (128 multiply-adds per SM and cycle in registers; 102 with the queries outside).
+// inputs, elements in ascending order.  bf16: a pair of widened weights stays put for G packed multiply-adds in a row; that
+// order issues at the full rate (128 multiply-adds per SM and cycle in registers; 102 with the queries outside).  fp32: one
+// multiply-add at a time, query by query (see chunk_fma; 300 queries, plain 2048-wide layers: 555 us, packed 786).
 template <bool BF16, int R, int G>
 __device__ __forceinline__ void chunk_fma_group(const uint4 (&w)[R], const float4 *xs4, uint32_t per_q, uint32_t nchunks, uint32_t c,
                                                 float2 (&acc)[G][R / 2])
 {
+    if constexpr (!BF16) {
 #pragma unroll
-    for (int h = 0; h < (BF16 ? 2 : 1); ++h) {
+        for (int g = 0; g < G; ++g) {
+            const float4 v = xs4[g * per_q + c];
+            const float x[4] = {v.x, v.y, v.z, v.w};
+            auto element = [&](auto E) {
+#pragma unroll
+                for (int r = 0; r < R; r += 2) {
+                    acc[g][r / 2].x = fmaf(chunk_elem<false, E.value>(w[r]), x[E.value], acc[g][r / 2].x);
+                    acc[g][r / 2].y = fmaf(chunk_elem<false, E.value>(w[r + 1]), x[E.value], acc[g][r / 2].y);
+                }
+            };
+            element(std::integral_constant<int, 0>());
+            element(std::integral_constant<int, 1>());
+            element(std::integral_constant<int, 2>());
+            element(std::integral_constant<int, 3>());
+        }
+    } else
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
         float x[G][4];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -168,8 +190,8 @@ __device__ __forceinline__ void chunk_fma_group(const uint4 (&w)[R], const float
         auto element = [&](auto E) {
 #pragma unroll
             for (int r = 0; r < R; r += 2) {
-                const float2 wp = h ? make_float2(chunk_elem<BF16, (BF16 ? 4 : 0) + E.value>(w[r]), chunk_elem<BF16, (BF16 ? 4 : 0) + E.value>(w[r + 1]))
-                                    : make_float2(chunk_elem<BF16, E.value>(w[r]), chunk_elem<BF16, E.value>(w[r + 1]));
+                const float2 wp = h ? make_float2(chunk_elem<true, 4 + E.value>(w[r]), chunk_elem<true, 4 + E.value>(w[r + 1]))
+                                    : make_float2(chunk_elem<true, E.value>(w[r]), chunk_elem<true, E.value>(w[r + 1]));
 #pragma unroll
                 for (int g = 0; g < G; ++g) acc[g][r / 2] = __ffma2_rn(make_float2(x[g][E.value], x[g][E.value]), wp, acc[g][r / 2]);
             }

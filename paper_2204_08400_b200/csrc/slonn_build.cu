@@ -895,12 +895,16 @@ __global__ void __launch_bounds__(64) fnv_sum_kernel(const unsigned char *p, uin
 
 __global__ void fnv_next_kernel(uint64_t *h) { h[0] = h[1]; }
 
-// *h := the checksum continued over n bytes on the device (synchronous, default stream).
+// *h := the checksum continued over n bytes on the device (synchronous, default stream).  false: no memory for the scratch, or
+// an error; *h is as it was.
 bool fnv1a_device(const void *dev, uint64_t n, uint64_t *h)
 {
     const unsigned char *p = (const unsigned char *)dev;
     unsigned char *scratch = nullptr; // h, next h; maps; first low bytes
-    if (cudaMalloc(&scratch, 256 + (uint64_t)FNV_CHUNKS * 257) != cudaSuccess) return false;
+    if (cudaMalloc(&scratch, 256 + (uint64_t)FNV_CHUNKS * 257) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
     uint64_t *d_h = (uint64_t *)scratch;
     unsigned char *map = scratch + 256, *first = map + (uint64_t)FNV_CHUNKS * 256;
     bool ok = cudaMemcpyAsync(d_h, h, 8, cudaMemcpyHostToDevice, 0) == cudaSuccess;
@@ -957,8 +961,8 @@ extern "C" int slonn_serialize(const slonn_model *m, void *dst_host, uint64_t ds
         memcpy(p + o, &ly.id_bytes, 4); o += 4;
         if (ly.table_bytes >= FNV_ON_DEVICE) {
             sum = fnv1a(p + summed, o - summed, sum);
-            if (!fnv1a_device(ly.tables, ly.table_bytes, &sum)) return SLONN_ERR_CUDA;
-            summed = o + ly.table_bytes;
+            summed = o;
+            if (fnv1a_device(ly.tables, ly.table_bytes, &sum)) summed = o + ly.table_bytes; // else on the host with the rest
         }
         if (cudaMemcpy(p + o, ly.tables, ly.table_bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return SLONN_ERR_CUDA;
         o += ly.table_bytes;

@@ -20,9 +20,10 @@
  *   - Ownership: the caller owns every buffer it passes in.  Weights and biases
  *     given to slonn_build are referenced, not copied: they must stay valid and
  *     unchanged until slonn_free.  The library owns what it allocates inside
- *     slonn_model (tables, hash-node ids, transposed copies of a CSR-fed first
- *     layer and of every layer that follows an activator layer -- a snapshot of
- *     those weights taken at build time).
+ *     slonn_model (tables, hash-node ids, transposed copies of the first layer and
+ *     of every layer that follows an activator layer -- a snapshot of those
+ *     weights taken at build time; the copy of a first layer with dense input
+ *     is left out when there is no memory for it).
  *   - A model is read-only after slonn_build; slonn_run may be called
  *     concurrently on different streams with different workspaces.
  *   - Arithmetic: every dot product is summed in fp32 in one fixed order (32
@@ -218,7 +219,7 @@ typedef struct {
  * A layer whose input is the sparse output of an activator layer (Sec. 3.3) can be evaluated in two
  * ways with identical results: row kernels read each selected weight row whole; input-stationary
  * kernels walk the query's nonzero inputs and read single weights from a transposed copy the model
- * keeps of such layers.  By default the library picks per query by budget: up to SLONN_COLS_MAX_BP
+ * keeps.  By default the library picks per query by budget: up to SLONN_COLS_MAX_BP
  * the input list is sparse enough for the input-stationary kernels to win (batches of tens of queries
  * only when no budget exceeds 1500 bp and only for layers at least 2048 inputs wide; a handful of queries keep
  * the row kernels); in large batches the queries that compute more than a few hundred nodes per layer are sorted by

@@ -111,11 +111,13 @@ __global__ void popularity_kernel(const IDT *tables, uint64_t n_lists, uint32_t 
 
 // Library-owned copies for the kernels that read weights by input (a first layer with dense input, and layers
 // whose input is the (id, value) list of an activator layer below them):
-//   WT      transposed weights [D][N]; on a layer that has its own activator the node axis is stored in
+//   WT      transposed weights [D][N]; on a list-fed layer that has its own activator the node axis is stored in
 //           the order of `colpos`: nodes that sit early in many ranked lists first, so that the nodes a
 //           query selects lie close together in every row of WT
-//   colpos  [N] node id -> column of WT (activator layers only; NULL = identity); colnode is its inverse
-//   WH      [D][32] the layer's hash rows side by side (activator layers with K*L <= 32)
+//   colpos  [N] node id -> column of WT (list-fed activator layers only; NULL = identity); colnode is its inverse
+//   WH      [D][32] the layer's hash rows side by side (list-fed activator layers with K*L <= 32)
+// A first layer with dense input is read by input only where every node is computed (100 % queries, no activator), so its
+// copy keeps the nodes' order and has no WH; it is an option, and a model for which it does not fit goes without it.
 // and the plain transposed copy of a first layer fed by CSR rows.  phase 0: the CSR first layer (needed
 // by the calibration pass); phase 1: the rest (needs the finished tables).
 // Copies of 4 GiB or more are left out: the kernels address them with 32-bit byte offsets (such layers keep the row kernels).
@@ -128,9 +130,14 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
         const uint64_t wt_bytes = (uint64_t)ly.N * ly.D * esz;
         const bool by_input = (l == 0 ? !m->first_sparse : m->layer[l - 1].has_act) && wt_bytes < (1ull << 32);
         if (phase == 0 ? !csr_first : !by_input) continue;
-        if (cudaMalloc(&ly.WT, wt_bytes) != cudaSuccess) return SLONN_ERR_NOMEM;
+        if (cudaMalloc(&ly.WT, wt_bytes) != cudaSuccess) {
+            ly.WT = nullptr;
+            if (l > 0 || csr_first) return SLONN_ERR_NOMEM;
+            (void)cudaGetLastError(); // the dense first layer keeps the row kernels
+            continue;
+        }
         const dim3 grid((ly.D + 31) / 32, (ly.N + 31) / 32), block(32, 8);
-        if (!ly.has_act || csr_first) {
+        if (!ly.has_act || l == 0) {
             transpose_kernel<<<grid, block, 0, st>>>(ly.W, ly.WT, ly.N, ly.D, esz);
             if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
             continue;

@@ -25,7 +25,8 @@ struct slonn_layer {
     uint64_t table_bytes;
     uint32_t *hash_nodes; // library-owned device copy, [L*K]
     void *WT;             // library-owned transposed copy [D][N]: layer 0, and layers whose input is an
-                          // activator layer's list (node axis in colpos order when colpos != NULL)
+                          // activator layer's list (node axis in colpos order when colpos != NULL);
+                          // NULL when a dense first layer's copy did not fit
     uint32_t *colpos;     // library-owned [N]: node id -> column of WT; NULL = identity
     uint32_t *colnode;    // library-owned [N]: column of WT -> node id; NULL = identity
     void *WH;             // library-owned [D][32]: the hash rows side by side (list-input activator layers)

@@ -472,7 +472,7 @@ extern "C" int slonn_test_tc_wait_limit(uint32_t polls)
 }
 
 int slonn_dense_tc_launch(const void *A, const void *W, uint32_t N, uint32_t K, const slonn_dense_epilogue &E,
-                          cudaStream_t st)
+                          cudaStream_t st, bool chained)
 {
     if (!A || !W || E.M == 0 || N == 0 || K == 0) return SLONN_ERR_ARG;
     CUtensorMap ma, mb;
@@ -509,7 +509,8 @@ int slonn_dense_tc_launch(const void *A, const void *W, uint32_t N, uint32_t K, 
     }
     const uint64_t tiles = (uint64_t)((N + bn - 1) / bn) * ((E.M + BM - 1) / BM);
     const uint32_t grid = (uint32_t)std::min<uint64_t>(tiles, (uint64_t)sm_count); // one persistent block per SM
-    slonn_launch(dense_tc_kernel, grid, THREADS, SMEM_BYTES, st, ma, mb, mo, tma_out, E, N, K, bn, g_probe_limit.load());
+    if (chained) slonn_launch(dense_tc_kernel, grid, THREADS, SMEM_BYTES, st, ma, mb, mo, tma_out, E, N, K, bn, g_probe_limit.load());
+    else dense_tc_kernel<<<grid, THREADS, SMEM_BYTES, st>>>(ma, mb, mo, tma_out, E, N, K, bn, g_probe_limit.load());
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
@@ -526,5 +527,6 @@ extern "C" int slonn_dense_layer(const void *x_bf16, const void *w_bf16, const f
     E.out_bf16 = (uint16_t *)out_bf16; E.ld_bf16 = N;
     E.status = status;
     if (status && cudaMemsetAsync(status, 0, 4 * sizeof(uint32_t), (cudaStream_t)stream) != cudaSuccess) return SLONN_ERR_CUDA;
-    return slonn_dense_tc_launch(x_bf16, w_bf16, N, D, E, (cudaStream_t)stream);
+    // not chained: nothing of this call's own stands between the kernel and one of the caller's that may still be writing bias
+    return slonn_dense_tc_launch(x_bf16, w_bf16, N, D, E, (cudaStream_t)stream, false);
 }

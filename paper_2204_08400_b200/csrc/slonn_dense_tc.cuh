@@ -23,4 +23,4 @@ struct slonn_dense_epilogue {
 
 // A: bf16 [M][K] row-major, W: bf16 [N][K] row-major; K * 2 bytes a multiple of 16.
 int slonn_dense_tc_launch(const void *A, const void *W, uint32_t N, uint32_t K, const slonn_dense_epilogue &E,
-                          cudaStream_t st);
+                          cudaStream_t st, bool chained);

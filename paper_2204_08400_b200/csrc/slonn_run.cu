@@ -1228,7 +1228,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                     E.indptr = indptr; E.ip_mul = m->n_act; E.ip_add = m->act_index[l];
                 }
             }
-            rc = slonn_dense_tc_launch(A[l & 1], ly.W, ly.N, ly.D, E, st);
+            rc = slonn_dense_tc_launch(A[l & 1], ly.W, ly.N, ly.D, E, st, true);
             if (!rc && ly.has_act && b->codes) {
                 const uint32_t t = n * m->L;
                 slonn_launch(dense_codes_kernel, (t + 127) / 128, 128, 0, st, tc_list, tc_count, vals, indptr, m->n_act,

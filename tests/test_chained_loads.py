@@ -49,6 +49,20 @@ def test_the_check_sees_direct_and_renamed_loads():
     assert not names & (WRITTEN | aliases)
 
 
+def test_a_chain_starts_behind_a_full_dependency():
+    """What a caller's own kernel may just be writing is read through the read-only path only behind a memset of the call's own; an
+    entry point without one does not chain its kernel."""
+    with open(os.path.join(CSRC, "slonn_run.cu")) as f:
+        run = f.read()
+    body = run[run.index("static int run_impl("):]
+    assert body.index("cudaMemsetAsync(b->status") < body.index("slonn_launch(")
+    assert body.index("cudaMemsetAsync(b->status") < body.index("launch_cluster(")
+    with open(os.path.join(CSRC, "slonn_dense_tc.cu")) as f:
+        tc = f.read()
+    entry = tc[tc.index('extern "C" int slonn_dense_layer('):]
+    assert "(cudaStream_t)stream, false);" in entry, "slonn_dense_layer works without a status buffer, hence without a memset"
+
+
 def test_no_kernel_lets_the_next_one_in_early():
     """Blocks of the next kernel would wait in slots that another stream's blocks could use."""
     for name in FILES:

@@ -268,7 +268,8 @@ def roofline_of(table, workload, n, budget_bp, dense_tc):
                 frac_row_granular=k["row_granular"] / sec / 1e9 / hbm if sec > 0 else 0.0,
                 dram_frac=(traffic * k["launches"] / sec / 1e9 / hbm) if traffic else None,
                 note="bytes_per_step: hash rows, bucket lists and selected nodes x input entries (the least any form must "
-                     "load); bytes_as_run: whole rows where a layer ran row-wise.  A fraction above 1, or a traffic far "
+                     "load); bytes_as_run: whole rows where a layer ran row-wise, a sixteenth of bytes_per_step (a lower "
+                     "bound) where 16 queries were evaluated at a time.  A fraction above 1, or a traffic far "
                      "below bytes_per_step, means the rows were served from L2/L1, not HBM")
 
 
@@ -437,7 +438,9 @@ def main():
     roofline["step"] = {"bytes_algorithmic": int(sb["algorithmic"]), "bytes_row_granular": int(sb["row_granular"]),
                         "GBps_algorithmic": sb["algorithmic"] / (ms_step / 1e3) / 1e9,
                         "frac": sb["algorithmic"] / (ms_step / 1e3) / 1e9 / hbm_peak}
-    launches_per_step = len(recs) + sum(1 for r in recs if r["stage"] == "plan")   # the plan record covers two launches
+    # a plan record covers two launches, one of grouped products at least two (preparation, product) or three (the sort before)
+    launches_per_step = len(recs) + sum({"plan": 1, "full_rows": 1, "group_rows": 2}.get(r["stage"], 0) for r in recs
+                                        if r["stage"] == "plan" or accounting.grouped_products(r))
 
     latency = latency_block(rig, wl.budget_bp, max(args.steps, 1000), flags) if n <= 64 else None
 

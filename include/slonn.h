@@ -438,7 +438,9 @@ typedef struct {
     uint32_t bp_lo, bp_hi; /* it serves the queries whose budget lies in [bp_lo, bp_hi] ...           */
     uint32_t skips_full; /* ... 1: except those at 10000 bp, which another launch serves              */
     uint32_t cols_bp;    /* whole-network launches: queries with budgets up to this evaluated their   */
-                         /* list-fed activator layers input-stationary (0 = every layer row-wise)     */
+                         /* list-fed activator layers input-stationary (0 = every layer row-wise);    */
+                         /* HASH_SELECT, FULL_ROWS, GROUP_ROWS: 10000 when single weights of the        */
+                         /* transposed copy were read (the two latter: 16 queries at a time), else 0     */
     float ms;            /* device time between the event pair around the launch                      */
 } slonn_launch_record;
 int slonn_run_traced(const slonn_model *m, const slonn_batch *batch, void *workspace,

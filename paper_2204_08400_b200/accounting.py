@@ -10,12 +10,15 @@ node ids of 2 bytes up to 65,536 nodes, else 4):
     bucket lists    L * B_out * idbytes
     selected nodes  B_out * D * s      row form: every selected weight row whole
                     B_out * B_in * s   input-stationary form: selected nodes x input list entries
+                    a 16th of that     grouped products: a weight is loaded once for a group of 16 queries.  Counted as
+                                       if the 16 selected the same nodes of the same inputs; what is loaded is the
+                                       union of both (1.1 to 1.7 times as much), which the host does not know
     CSR first layer nnz * N * s        one row of the transposed weights per nonzero
 
 with B_out the node count of the query's budget in this layer (N without activator) and B_in the length of
 the list the layer below hands over (D when the input is dense).  Three totals are kept per launch:
 
-    as_run         the form each layer actually took (what the kernel had to load)
+    as_run         the form each layer actually took (what the kernel had to load; grouped products: at least)
     algorithmic    the sparse count everywhere (B_out * B_in, H * B_in): the least any form could load
     row_granular   whole rows everywhere
 """
@@ -30,6 +33,8 @@ KERNEL_OF_STAGE = {
     "dense_tc": "dense_tc_kernel", "cluster": "cluster_network_kernel", "gather_cols": "gather_cols_kernel",
     "layer_cols": "layer_cols_kernel", "full_rows": "full_rows_kernel", "group_rows": "group_rows_kernel",
 }
+
+TILE_G = 16                       # queries per group of the grouped products
 
 
 @dataclass
@@ -82,6 +87,11 @@ def served(rec: dict, bps: np.ndarray) -> np.ndarray:
     return m
 
 
+def grouped_products(rec: dict) -> bool:
+    """Whether the launch evaluated 16 queries at a time from the transposed copy."""
+    return rec["stage"] in ("full_rows", "group_rows") and bool(rec["cols_bp"])
+
+
 def launch_bytes(sh: NetShape, rec: dict, bps: Sequence[int], x_nnz: Optional[np.ndarray] = None) -> dict:
     """Totals over the queries the launch serves: as_run / algorithmic / row_granular bytes, flops (tensor-core
     launches) and the number of queries."""
@@ -112,7 +122,8 @@ def launch_bytes(sh: NetShape, rec: dict, bps: Sequence[int], x_nnz: Optional[np
         hashes = stage in ("hash_select", "layer_cols", "fused", "cluster")
         nodes = stage in ("gather_dot", "gather_cols", "layer_cols", "full_rows", "group_rows", "fused", "cluster")
         cols = np.zeros(bp.size, bool)
-        if stage in ("gather_cols", "layer_cols"):
+        tile = grouped_products(rec)
+        if stage in ("gather_cols", "layer_cols") or (stage == "hash_select" and rec["cols_bp"]):
             cols[:] = True
         elif stage == "fused" and rec["cols_bp"] and t["act"] and t["list_in"]:
             cols = bp <= rec["cols_bp"]
@@ -123,13 +134,18 @@ def launch_bytes(sh: NetShape, rec: dict, bps: Sequence[int], x_nnz: Optional[np
         if nodes:
             alg += int(t["rows_alg"].sum())
             row += int(t["rows_row"].sum())
-            run += int(np.where(cols, t["rows_alg"], t["rows_row"]).sum())
+            run += int(t["rows_alg"].sum()) // TILE_G if tile else int(np.where(cols, t["rows_alg"], t["rows_row"]).sum())
         out["as_run"] += run; out["algorithmic"] += alg; out["row_granular"] += row
     return out
 
 
 def kernel_name(sh: NetShape, rec: dict) -> str:
-    """The kernel behind a record (rows of at most one 512-byte round take the short-row gather)."""
+    """The kernel behind a record (rows of at most one 512-byte round take the short-row gather).  Grouped products are
+    three launches under one record: the sort into groups, their preparation, and the product, which takes the time."""
+    if grouped_products(rec):
+        return "tile_rows_kernel"
+    if rec["stage"] == "hash_select" and rec["cols_bp"]:
+        return "hash_select_cols_kernel"
     if rec["stage"] == "gather_dot" and rec["layer"] is not None and sh.dims[rec["layer"]] * sh.esz <= 512:
         return "gather_short_kernel"
     return KERNEL_OF_STAGE[rec["stage"]]

@@ -33,9 +33,11 @@ struct stage_timer {
         cudaEventRecord(s.a, st);
         ++n;
     }
+    void by_input() { if (n > 0 && !failed) spans[n - 1].cols_bp = 10000u; } // the last launch read single weights of a transposed copy
     void toc() { if (n > 0 && !failed) cudaEventRecord(spans[n - 1].b, st); }
 };
 #define TIC(...) do { if (tm) tm->tic(__VA_ARGS__); } while (0)
+#define TIC_BY_INPUT() do { if (tm) tm->by_input(); } while (0)
 #define TOC() do { if (tm) tm->toc(); } while (0)
 #define AT_LAYER(l) do { if (tm) tm->layer = (l); } while (0)
 
@@ -737,10 +739,11 @@ int launch_tile_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t 
     sp.sort_key = key; sp.budget_bp = b->budget_bp;
     TIC(SLONN_STAGE_HASH_SELECT, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp);
     rc = launch_select_cols(m, ly, l, gp, b, key, n, max_rows, st);
+    if (rc == SLONN_OK) TIC_BY_INPUT();
     if (rc == SLONN_ERR_DIM) rc = launch_select(m, sp, n, max_rows, st);
     TOC();
     if (rc) return rc;
-    TIC(SLONN_STAGE_GROUP_ROWS, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp);
+    TIC(SLONN_STAGE_GROUP_ROWS, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp, 10000u);
     rc = launch_tile_order(tw, b, n, lo, skip_bp != nullptr, sorted, st);
     if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 1, nullptr, nullptr, false, st, true);
     TOC();
@@ -1069,6 +1072,7 @@ static int run_full_route(const slonn_model *m, const slonn_batch *b, uint32_t n
         TIC(SLONN_STAGE_FULL_ROWS, b->budget_bp, 10000u, 10000u);
         int rc;
         if (tw.ws && tile_layer_ok(m, l)) {
+            TIC_BY_INPUT();
             slonn_gather_params gp;
             memset(&gp, 0, sizeof(gp));
             gp.in = in; gp.n_act = m->n_act; gp.a = fp.a; gp.relu = fp.relu;
@@ -1341,8 +1345,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                 if (keyed && max_bp >= from) {
                     TIC(SLONN_STAGE_HASH_SELECT, sp.range_bp, sp.bp_lo, sp.bp_hi, sp.skip_bp);
                     rc = launch_select(m, sp, n, max_rows, st);
-                    TOC();
                     if (!rc) rc = launch_tile_order(tw, b, n, from, skip_bp != nullptr, &sorted, st);
+                    TOC();
                     const sorted_groups sg = {(const uint32_t *)(ws + wl.tile.order), wl.tile.chunk, wl.tile.order_stride, from};
                     if (!rc) rc = launch_rows(m, gp, b, n, max_bp, max_rows, gw, st, tm, &sg);
                 } else {
@@ -1362,7 +1366,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             // compacted and taken four per block.
             bool rows_done = false;
             if (tw.ws && tile_layer_ok(m, l) && n >= SLONN_TILE_DENSE_MIN_QUERIES) {
-                TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp);
+                TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp, 10000u);
                 rc = SLONN_OK;
                 if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp != nullptr, &sorted, st);
                 if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, keyed);

@@ -105,3 +105,20 @@ def test_records_group_by_kernel_and_short_rows_name_their_kernel():
 
 def test_empty_batch_has_no_bytes():
     assert acc.launch_bytes(toy(), rec("fused", None), np.zeros(0, np.int64))["as_run"] == 0
+
+
+def test_grouped_products_are_named_and_counted_as_what_ran():
+    """Records that say 16 queries were evaluated at a time from the transposed copy (cols_bp) are not the four-per-block
+    row kernels: their weights are loaded once per group."""
+    sh, bp = toy(), np.full(32, 5000)                             # 100 of 200 nodes
+    g = acc.launch_bytes(sh, rec("group_rows", 1, 3501, cols_bp=10000), bp)
+    assert g["algorithmic"] == 32 * 100 * 100 * 2 and g["as_run"] == 2 * 100 * 100 * 2
+    f = acc.launch_bytes(sh, rec("full_rows", 0, 10000, 10000, cols_bp=10000), np.full(32, 10000))
+    assert f["as_run"] == 2 * 64 * 200 * 2
+    s = acc.launch_bytes(sh, rec("hash_select", 1, cols_bp=10000), bp)
+    assert s["as_run"] == s["algorithmic"] == 32 * (20 * 100 * 2 + 2 * 100 * 2)
+    assert acc.kernel_name(sh, rec("group_rows", 1, cols_bp=10000)) == "tile_rows_kernel"
+    assert acc.kernel_name(sh, rec("full_rows", 1, cols_bp=10000)) == "tile_rows_kernel"
+    assert acc.kernel_name(sh, rec("hash_select", 1, cols_bp=10000)) == "hash_select_cols_kernel"
+    assert acc.kernel_name(sh, rec("group_rows", 0)) == "group_rows_kernel"
+    assert acc.kernel_name(sh, rec("full_rows", 0)) == "full_rows_kernel"

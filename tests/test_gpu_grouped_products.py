@@ -111,3 +111,24 @@ def test_budgets_above_the_maximum_get_the_clamped_results(dims, has_act, n, bud
             B = int(ip[(q + 1) * sum(has_act)] - ip[(q + 1) * sum(has_act) - 1]) if has_act[-1] else dims[-1]
             assert np.array_equal(got["logits"][q, :B], want["logits"][q, :B]), (flags, q)
     dm.free()
+
+
+def test_launch_records_say_which_launches_took_grouped_products():
+    """What the benchmark names and counts kernels by: launches that read single weights of a transposed copy carry
+    cols_bp = 10000, the row kernels 0."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(4204, [512, 1240, 520, 120], [1, 1, 0], "bf16", n=3500, n_cal=300, K=4, L=2, budgets=(700, 5000, 10000))
+    dm = harness.DeviceModel(wl)
+    sh = acc.NetShape.of(wl)
+
+    def kernels(flags):
+        b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED, flags=flags)
+        recs = sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes)
+        assert b.results()["status"][0] == 0
+        return {(r["layer"], acc.kernel_name(sh, r), r["bp_lo"] == 10000) for r in recs if r["layer"] is not None}
+
+    tiled, rows = kernels(0), kernels(sl.FLAG_ROW_KERNELS)
+    assert {(0, "tile_rows_kernel", True), (1, "tile_rows_kernel", True), (2, "tile_rows_kernel", True),
+            (1, "hash_select_cols_kernel", False), (1, "tile_rows_kernel", False), (2, "tile_rows_kernel", False)} <= tiled
+    assert not [k for k in rows if k[1] in ("tile_rows_kernel", "hash_select_cols_kernel")]
+    dm.free()

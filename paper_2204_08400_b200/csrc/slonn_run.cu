@@ -106,8 +106,20 @@ bool full_route_possible(const slonn_model *m, uint32_t max_bp)
 #define SLONN_TILE_MIN_QUERIES 256u
 #define SLONN_TILE_FEW_QUERIES 64u
 #define SLONN_TILE_FEW_ROWS (148ull * 1536)
-// A layer without activator (every node): from 512 queries on (1000 outputs, 4096 queries at 10 %: 0.26 -> 0.15 ms).
+// A layer without activator (every node): from 512 queries on, when it has nodes for most of a tile's 128 columns (10 outputs:
+// 600 queries 13 -> 26 us, 8192 queries 60 -> 120; 32 outputs: 15 -> 30; 100 to 130 outputs: 0.9 to 1.2 times the speed) and
+// there are items for most of the SMs (600 queries, 130 outputs, 76 items: 29 -> 36 us; 300 outputs, 114 items: 66 -> 50).  A
+// list that comes from the first layers is as short as its budget, but the union of 16 such lists is not: at low budgets the
+// input-stationary kernel wins there (1000 outputs behind one layer of 2048, speed at 600 / 2100 / 4096 / 8192 queries: 5 %
+// 0.93 0.80 0.88 0.87, 10 % 0.98 0.84 0.90 0.93, 25 % 1.10 1.01 1.02 1.10; behind two of 1536: 10 % 1.02 0.91 0.98 1.00, 25 %
+// 1.27 1.13 1.17 1.26; behind eight of 4096, 4096 queries, 10 %: 260 -> 150 us), except on wide fp32 layers, where its
+// 16-byte load brings four weights instead of eight (1000 outputs behind one layer of 2048: 5 % 0.97 0.91 1.01 1.00, 10 % 1.02
+// 1.01 1.13 1.12; behind two of 4096: 5 % 1.06 1.14 1.25 1.28; but 130 outputs behind two of 1536: 10 % 0.89 0.84 0.89).
 #define SLONN_TILE_DENSE_MIN_QUERIES 512u
+#define SLONN_TILE_DENSE_MIN_NODES 96u
+#define SLONN_TILE_DENSE_MIN_ITEMS 100u
+#define SLONN_TILE_DENSE_MIN_BP 2000u  // behind the first layers, largest budget of the batch
+#define SLONN_TILE_DENSE_F32_WIDTH 2048u // fp32: any budget from this many inputs on
 // Of a list-fed activator layer, the queries whose budget is at most this many nodes keep layer_cols_kernel, which needs no
 // grouping: 4096 queries, 512 nodes of 2048: 1.70 -> 1.54 ms, 307 nodes: 0.97 -> 1.03, 384 nodes of 1536: 1.04 -> 1.07;
 // 410 nodes of 4096: 3.25 -> 3.07 with 4096 queries, 0.73 -> 0.76 with 512.
@@ -120,6 +132,23 @@ bool tile_layer_ok(const slonn_model *m, uint32_t l)
 {
     const slonn_layer &ly = m->layer[l];
     return ly.WT && !(l == 0 && m->first_sparse) && ly.N <= SLONN_TILE_MAX_N;
+}
+
+// whether layer l's input has come through two list-fed layers (three activator layers) at least
+bool tile_deep(const slonn_model *m, uint32_t l)
+{
+    return l >= 3 && m->layer[l - 1].has_act && m->layer[l - 2].has_act && m->layer[l - 3].has_act;
+}
+
+// whether a batch evaluates layer l, which has no activator, as grouped products
+bool tile_plain_wanted(const slonn_model *m, uint32_t l, uint32_t n, uint32_t max_bp)
+{
+    const slonn_layer &ly = m->layer[l];
+    const uint64_t items = (uint64_t)((n + SLONN_TILE_G - 1) / SLONN_TILE_G) * ((ly.N + SLONN_TILE_COLS - 1) / SLONN_TILE_COLS);
+    if (!tile_layer_ok(m, l) || n < SLONN_TILE_DENSE_MIN_QUERIES || ly.N < SLONN_TILE_DENSE_MIN_NODES || items < SLONN_TILE_DENSE_MIN_ITEMS)
+        return false;
+    const bool list_in = l > 0 && m->layer[l - 1].has_act;
+    return !list_in || max_bp >= SLONN_TILE_DENSE_MIN_BP || tile_deep(m, l) || (m->dtype == SLONN_F32 && ly.D >= SLONN_TILE_DENSE_F32_WIDTH);
 }
 
 // entries a group of layer l stages at most
@@ -1365,7 +1394,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             // serve (budgets above the input-stationary limit) share all their weight rows, so they are
             // compacted and taken four per block.
             bool rows_done = false;
-            if (tw.ws && tile_layer_ok(m, l) && n >= SLONN_TILE_DENSE_MIN_QUERIES) {
+            if (tw.ws && tile_plain_wanted(m, l, n, max_bp)) {
                 TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp, 10000u);
                 rc = SLONN_OK;
                 if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp != nullptr, &sorted, st);

@@ -132,3 +132,30 @@ def test_launch_records_say_which_launches_took_grouped_products():
             (1, "hash_select_cols_kernel", False), (1, "tile_rows_kernel", False), (2, "tile_rows_kernel", False)} <= tiled
     assert not [k for k in rows if k[1] in ("tile_rows_kernel", "hash_select_cols_kernel")]
     dm.free()
+
+
+@pytest.mark.parametrize("dtype,dims,has_act,n,budgets,layer,kernel", [
+    ("bf16", [512, 640, 640, 10], [1, 1, 0], 2100, (1000, 5000), 2, None),              # a tile of 128 columns for 10 nodes
+    ("bf16", [512, 640, 640, 95], [1, 1, 0], 2100, (1000, 5000), 2, None),
+    ("bf16", [512, 640, 640, 96], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_kernel"),
+    ("bf16", [512, 640, 640, 96], [1, 1, 0], 1500, (1000, 5000), 2, None),              # 94 items
+    ("bf16", [512, 640, 640, 256], [1, 1, 0], 2100, (500, 1999), 2, None),              # low budgets behind the second layer ...
+    ("bf16", [512, 640, 640, 256], [1, 1, 0], 2100, (500, 2000), 2, "tile_rows_kernel"),
+    ("bf16", [512, 640, 640, 640, 256], [1, 1, 1, 0], 2100, (500, 1999), 3, "tile_rows_kernel"),   # ... and behind the third
+    ("f32", [128, 2048, 256], [1, 0], 1000, (500, 1000), 1, "tile_rows_kernel"),        # wide and fp32
+    ("f32", [128, 2040, 256], [1, 0], 1000, (500, 1000), 1, None),
+])
+def test_grouped_products_are_taken_where_they_pay(dtype, dims, has_act, n, budgets, layer, kernel):
+    """Both sides of each line of the dispatch (None: anything but grouped products); same bits as the row kernels."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(4800 + n, dims, has_act, dtype, n=n, n_cal=300, K=4, L=2, budgets=budgets)
+    dm = harness.DeviceModel(wl)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
+    names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes)
+             if r["layer"] == layer and r["bp_lo"] <= budgets[0 if len(budgets) > 1 and budgets[0] == 2900 else -1] <= r["bp_hi"]]
+    if kernel:
+        assert names[-1] == kernel, names
+    else:
+        assert "tile_rows_kernel" not in names, names
+    _same_bits(b.results(), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()

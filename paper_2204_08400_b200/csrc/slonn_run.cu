@@ -365,8 +365,21 @@ size_t group_rows_smem(const slonn_gather_params &P, uint32_t max_rows, uint32_t
 // Measured on a 4096-wide layer with 4096 queries: 50 % budget 3.5 -> 2.95 ms per layer with queries as they come, 2.52 ms
 // with neighbours in (budget, keys) and packed multiply-adds; 10 % 0.72 -> 0.79 ms, sorted and packed 0.66 ms.  Small
 // batches have fewer neighbours: 777 queries of 7 to 60 % on 2328 x 1568, groups from 20 % on 0.161 ms, from 7 % on 0.174.
+// In batches of at least SLONN_TILE_LARGE queries sorted groups pay below 20 % too, once a query's selected rows take 3 MiB
+// (speed over the one-query kernel at 2100 / 4096 / 8192 queries; 3.2 MB: 389 of 2048 x 4096 bf16 0.99 1.06 1.16, 778 of
+// 4096 x 2048 0.97 1.03 1.05, 778 of 4096 x 1024 fp32 1.01 1.05 1.14; 1.6 MB: 195 of 1024 x 4096 0.86 0.92 1.06, 778 of
+// 4096 x 1024 0.86 0.92 0.96; 0.3 MB: 0.61 0.70 0.82).
 #define SLONN_GROUP_MIN_BP 2000u
-#define SLONN_GROUP_MIN_BP_SORTED 700u // batches of at least SLONN_TILE_LARGE queries, sorted
+#define SLONN_GROUP_MIN_BP_SORTED 700u // the least measured
+#define SLONN_GROUP_SORTED_BYTES (3ull << 20)
+// groups take the budgets above this
+uint32_t group_min_bp(const slonn_model *m, const slonn_layer &ly, uint32_t n)
+{
+    if (n < SLONN_TILE_LARGE) return SLONN_GROUP_MIN_BP;
+    const uint64_t layer_bytes = (uint64_t)ly.N * ly.D * (m->dtype == SLONN_BF16 ? 2u : 4u);
+    const uint64_t bp = (SLONN_GROUP_SORTED_BYTES * 10000u + layer_bytes - 1) / layer_bytes;
+    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(bp, SLONN_GROUP_MIN_BP_SORTED), SLONN_GROUP_MIN_BP);
+}
 int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch *b, uint32_t n, uint32_t max_bp,
                 uint32_t max_rows, const group_ws &gw, cudaStream_t st, stage_timer *tm, const sorted_groups *sorted = nullptr)
 {
@@ -1370,7 +1383,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             } else {
                 keyed = tw.ws && in.kind == SLONN_IN_DENSE; // hash_select_kernel serves every query
                 if (keyed) { sp.sort_key = (uint64_t *)(ws + wl.tile.key); sp.budget_bp = b->budget_bp; }
-                const uint32_t from = (n >= SLONN_TILE_LARGE ? SLONN_GROUP_MIN_BP_SORTED : SLONN_GROUP_MIN_BP) + 1u;
+                const uint32_t from = group_min_bp(m, ly, n) + 1u;
                 if (keyed && max_bp >= from) {
                     TIC(SLONN_STAGE_HASH_SELECT, sp.range_bp, sp.bp_lo, sp.bp_hi, sp.skip_bp);
                     rc = launch_select(m, sp, n, max_rows, st);

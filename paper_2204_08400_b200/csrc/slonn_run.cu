@@ -121,10 +121,16 @@ bool full_route_possible(const slonn_model *m, uint32_t max_bp)
 #define SLONN_TILE_DENSE_MIN_BP 2000u  // behind the first layers, largest budget of the batch
 #define SLONN_TILE_DENSE_F32_WIDTH 2048u // fp32: any budget from this many inputs on
 // Of a list-fed activator layer, the queries whose budget is at most this many nodes keep layer_cols_kernel, which needs no
-// grouping: 4096 queries, 512 nodes of 2048: 1.70 -> 1.54 ms, 307 nodes: 0.97 -> 1.03, 384 nodes of 1536: 1.04 -> 1.07;
-// 410 nodes of 4096: 3.25 -> 3.07 with 4096 queries, 0.73 -> 0.76 with 512.
+// grouping: speed of the products over that kernel's, bf16, five layers of the same width, 2100 / 4096 / 8192 queries, in the first,
+// second and third list-fed layer:
+//   404 nodes of 2048: 0.86 0.89 0.98, 1.00 1.06 1.18, 1.24 1.26 1.40;  559 nodes: 0.98 1.06 1.16, 1.24 1.32 1.42, 1.60 1.56 1.77
+//   409 nodes of 4096: 0.78 0.82 0.84, 0.91 0.99 1.00, 1.08 1.15 1.19;  559 nodes: 1.15 1.14 1.12, 1.26 1.29 1.28, 1.55 1.53 1.50
+// What sets them apart is the union of a group's input lists, which narrows from layer to layer; the host knows the place of a
+// layer, not the union.  512 queries, 410 nodes of 4096: 0.73 -> 0.76 ms.
 #define SLONN_TILE_NODES 512u
-#define SLONN_TILE_NODES_LARGE 400u // batches of at least SLONN_TILE_LARGE queries
+// A batch that holds budgets above the line anyway pays little for the others: budgets of 5 to 100 %, 512 nodes of 2048 beside the
+// higher ones, 2100 / 4096 / 8192 queries: 354 562 988 -> 327 531 963 us.
+#define SLONN_TILE_NODES_LARGE 400u // from the third list-fed layer on or beside higher budgets, at least SLONN_TILE_LARGE queries
 #define SLONN_TILE_LARGE 2048u
 
 // whether layer l can be evaluated as grouped products
@@ -750,9 +756,11 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
 
 // Budgets 1..limit of a list-fed activator layer keep the one-launch input-stationary kernel; the others are evaluated
 // in groups.
-uint32_t tile_budget_limit(const slonn_layer &ly, uint32_t n)
+uint32_t tile_budget_limit(const slonn_model *m, uint32_t l, uint32_t n, uint32_t max_bp)
 {
-    return std::min((n >= SLONN_TILE_LARGE ? SLONN_TILE_NODES_LARGE : SLONN_TILE_NODES) * 10000u / ly.N, SLONN_COLS_MAX_BP);
+    const uint32_t N = m->layer[l].N, limit = std::min(SLONN_TILE_NODES * 10000u / N, SLONN_COLS_MAX_BP);
+    if (n < SLONN_TILE_LARGE || (!tile_deep(m, l) && max_bp <= limit)) return limit;
+    return std::min(SLONN_TILE_NODES_LARGE * 10000u / N, SLONN_COLS_MAX_BP);
 }
 
 // A list-fed activator layer of a batch that takes grouped products.  *sorted: see launch_tile_order.
@@ -762,7 +770,7 @@ int launch_tile_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t 
 {
     uint64_t *key = (uint64_t *)(tw.ws + tw.wl->tile.key);
     const uint16_t *skip_bp = gp.skip_bp;
-    const uint32_t limit = std::min(tile_budget_limit(ly, n), max_bp), pre = slonn_model_pre(m);
+    const uint32_t limit = std::min(tile_budget_limit(m, l, n, max_bp), max_bp), pre = slonn_model_pre(m);
     int rc;
     uint32_t lo = 0;
     if (ly.WH && limit) { // the low budgets

@@ -146,6 +146,9 @@ def test_launch_records_say_which_launches_took_grouped_products():
     ("f32", [128, 2040, 256], [1, 0], 1000, (500, 1000), 1, None),
     ("bf16", [512, 1536, 24], [1, 0], 2100, (1900,), 0, "gather_dot_kernel"),           # 0.3 MB of selected rows a query
     ("bf16", [4096, 2048, 24], [1, 0], 2100, (1875, 1876), 0, "group_rows_kernel"),     # 3 MiB from 18.75 % on
+    ("bf16", [512, 1536, 1536, 24], [1, 1, 0], 2100, (2900,), 1, "layer_cols_kernel"),  # 445 nodes in the first list-fed layer,
+    ("bf16", [512, 1536, 1536, 1536, 1536, 24], [1, 1, 1, 1, 0], 2100, (2900,), 3, "tile_rows_kernel"),  # in the third,
+    ("bf16", [512, 1536, 1536, 24], [1, 1, 0], 2100, (2900, 5000), 1, "tile_rows_kernel"),  # and beside higher budgets
 ])
 def test_grouped_products_are_taken_where_they_pay(dtype, dims, has_act, n, budgets, layer, kernel):
     """Both sides of each line of the dispatch (None: anything but grouped products); same bits as the row kernels."""

@@ -22,7 +22,7 @@
 struct cols_stage {
     float *xs;          // scratch while staging (cols_scratch_bytes)
     uint2 *ent;         // [cols_ent_cap] entries (j, bits of x_j), segment after segment
-    uint32_t *segcnt;   // [32]
+    uint32_t *segcnt;   // [32], cols_stage_warp only
     uint32_t *segstart; // [33]
 };
 

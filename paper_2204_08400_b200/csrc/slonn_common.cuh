@@ -375,10 +375,10 @@ __device__ __forceinline__ void stage_input(const slonn_input &in, uint32_t q, u
     __syncthreads();
 }
 
-// hash nodes that are active whatever the budget (0 unless the model was built that way)
 // Lets `kernel` be launched with `bytes` of dynamic shared memory on the current device.  The 48 KB a launch gets
 // without opting in and the 227 KB a block can have both count the kernel's static shared memory (at most 1120
-// bytes in this library): the opt-in starts at 46 KB and ends at 225 KB (SLONN_ERR_DIM above).  The limit of a
+// bytes where the dynamic size varies; tile_rows_kernel has more and checks its own sum): the opt-in starts at 46 KB
+// and ends at 225 KB (SLONN_ERR_DIM above).  The limit of a
 // kernel is only ever raised, so that two host threads launching the same kernel with different sizes cannot
 // take each other's allowance away between the opt-in and the launch.
 inline int slonn_allow_smem(const void *kernel, size_t bytes)
@@ -399,6 +399,7 @@ inline int slonn_allow_smem(const void *kernel, size_t bytes)
     return SLONN_OK;
 }
 
+// hash nodes that are active whatever the budget (0 unless the model was built that way)
 inline uint32_t slonn_model_pre(const slonn_model *m) { return m->free_hash ? m->H : 0u; }
 
 // ---- internal host entry points shared between translation units ---------------

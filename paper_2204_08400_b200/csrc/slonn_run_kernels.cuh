@@ -1049,7 +1049,6 @@ __global__ void gather_cols_kernel(slonn_gather_params P)
     slonn_enter();
     extern __shared__ float4 smem4[];
     constexpr int V = BF16 ? 8 : 4;
-    __shared__ uint32_t segcnt[32];
     __shared__ uint32_t segstart[33];
     __shared__ uint32_t scan_ws[32];
     __shared__ uint32_t scan_total;
@@ -1071,7 +1070,7 @@ __global__ void gather_cols_kernel(slonn_gather_params P)
     cols_stage S;
     S.xs = reinterpret_cast<float *>(smem4);
     S.ent = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(smem4) + P.scratch_bytes);
-    S.segcnt = segcnt;
+    S.segcnt = nullptr;
     S.segstart = segstart;
     const uint64_t s0 = P.in.indptr[(uint64_t)q * P.in.ip_mul + P.in.ip_add];
     const uint32_t len = min((uint32_t)(P.in.indptr[(uint64_t)q * P.in.ip_mul + P.in.ip_add + 1] - s0), P.in_cap);
@@ -1114,7 +1113,6 @@ __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
     constexpr int V = BF16 ? 8 : 4;
     constexpr int R = 2;
     const slonn_gather_params &P = Q.G;
-    __shared__ uint32_t segcnt[32];
     __shared__ uint32_t segstart[33];
     __shared__ uint32_t scan_ws[32];
     __shared__ uint32_t scan_total;
@@ -1139,7 +1137,7 @@ __global__ void layer_cols_kernel(slonn_layer_cols_params Q)
     cols_stage S;
     S.xs = reinterpret_cast<float *>(smem4);
     S.ent = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(smem4) + P.scratch_bytes);
-    S.segcnt = segcnt;
+    S.segcnt = nullptr;
     S.segstart = segstart;
     uint32_t *idmap = reinterpret_cast<uint32_t *>(S.ent + cols_ent_cap(P.D, P.in_cap));
     // [32][R][32] of its own when the node loop needs it too (SPLIT); else [32][32] at the start of the scratch,
@@ -1205,7 +1203,6 @@ __global__ void hash_select_cols_kernel(slonn_layer_cols_params Q)
     constexpr int V = BF16 ? 8 : 4;
     constexpr uint32_t ESZ = BF16 ? 2u : 4u;
     const slonn_gather_params &P = Q.G;
-    __shared__ uint32_t segcnt[32];
     __shared__ uint32_t segstart[33];
     __shared__ uint32_t scan_ws[32];
     __shared__ uint32_t scan_total;
@@ -1222,7 +1219,7 @@ __global__ void hash_select_cols_kernel(slonn_layer_cols_params Q)
     cols_stage S;
     S.xs = reinterpret_cast<float *>(smem4);
     S.ent = reinterpret_cast<uint2 *>(reinterpret_cast<char *>(smem4) + P.scratch_bytes);
-    S.segcnt = segcnt;
+    S.segcnt = nullptr;
     S.segstart = segstart;
     uint32_t *idmap = reinterpret_cast<uint32_t *>(S.ent + cols_ent_cap(P.D, P.in_cap));
     float *zpart = reinterpret_cast<float *>(smem4);

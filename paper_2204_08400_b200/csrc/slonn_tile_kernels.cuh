@@ -390,6 +390,9 @@ __device__ __forceinline__ void tile_cp_async(uint32_t dst, const void *src)
 #define SLONN_TILE_RING_BYTES (SLONN_TILE_ROWS_AT + SLONN_TILE_RING * 4 + 16) // the first row offsets again behind the last
 #define SLONN_TILE_PART (SLONN_TILE_COLS * SLONN_TILE_G) // floats of a warp's sums
 #define SLONN_TILE_SMEM ((size_t)SLONN_TILE_WARPS * (SLONN_TILE_RING_BYTES + SLONN_TILE_PART * 4))
+#define SLONN_TILE_STATIC (2 * SLONN_TILE_COLS * 8 + 2 * SLONN_TILE_WARPS * 32 + 2 * SLONN_TILE_G * 12) // s_col, s_item, s_q and s_off
+static_assert(SLONN_TILE_SMEM > 46 * 1024 && SLONN_TILE_SMEM + SLONN_TILE_STATIC <= 227 * 1024,
+              "tile_rows_kernel must opt in to its shared memory and fit a block's 227 KB with its static part");
 
 // The four weights of a lane for one entry, as loaded from p[j] + row.  QUAD: four neighbouring columns, one load; else
 // one load each.

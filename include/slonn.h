@@ -321,7 +321,9 @@ int slonn_active_capacity(const slonn_model *m, uint32_t n_queries, uint32_t max
 /* logit_stride for this model at max_budget_bp (see slonn_batch.logits). */
 int slonn_logit_stride(const slonn_model *m, uint32_t max_budget_bp, uint32_t *stride);
 /* Bytes of device workspace slonn_run needs (256-byte aligned buffer) for a batch with these
- * n_queries, max_budget_bp and flags. */
+ * n_queries, max_budget_bp and flags.  For large batches up to about 170 MiB of it are scratch for evaluating 16 queries
+ * at a time; slonn_run also takes a workspace without that part (the size with SLONN_FLAG_ROW_KERNELS) and then
+ * uses the kernels that need none, with the same results. */
 int slonn_workspace_bytes(const slonn_model *m, uint32_t n_queries, uint32_t max_budget_bp,
                           uint32_t flags, uint64_t *bytes);
 
@@ -379,9 +381,10 @@ int slonn_test_tc_wait_limit(uint32_t polls);
  * ends).  The call performs no cudaMalloc / cudaFree and uses no allocating
  * library routine.
  *
- *   - The batch must fit: if slonn_workspace_bytes(m, n_queries, max_budget_bp, flags)
- *     exceeds SLONN_STATIC_WORKSPACE_BYTES the call returns SLONN_ERR_WORKSPACE
- *     and launches nothing.  Use smaller batches or slonn_run.
+ *   - The batch must fit: if its workspace without the scratch for 16 queries at a
+ *     time (what slonn_workspace_bytes returns with SLONN_FLAG_ROW_KERNELS) exceeds
+ *     SLONN_STATIC_WORKSPACE_BYTES the call returns SLONN_ERR_WORKSPACE and
+ *     launches nothing.  Use smaller batches or slonn_run.
  *   - The model's device must be the current device (else SLONN_ERR_ARG).
  *   - The first call on each device looks up the scratch area's device address
  *     (a one-time set-up step under a lock).  Make that first call during

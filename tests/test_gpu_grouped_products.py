@@ -134,6 +134,22 @@ def test_launch_records_say_which_launches_took_grouped_products():
     dm.free()
 
 
+@pytest.mark.parametrize("dtype,dims,has_act,n,budgets,K,L", [
+    ("bf16", [4096, 2048, 24], [1, 0], 8192 + 40, (1500, 1876, 1900), 4, 2),        # groups of four sorted below 20 %, two chunks
+    ("bf16", [512, 640, 520, 24], [1, 1, 0], 8192 + 309, (600, 2001, 2500), 4, 2),  # from 20 % on
+    ("f32", [264, 512, 512, 20], [1, 1, 1], 8192 + 33, (700, 2500, 10000), 4, 2),   # 100 % queries beside them
+    ("bf16", [128, 640, 520, 20], [1, 1, 0], 300, (2500, 6000), 9, 4),              # 36 hash functions: no side-by-side hash rows
+    ("f32", [128, 640, 520, 44], [1, 1, 1], 2100, (700, 6000), 9, 4),
+])
+def test_sorted_groups_and_many_hash_functions(dtype, dims, has_act, n, budgets, K, L):
+    """Against the row kernels, which neither sort nor read by input."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4700 + n, dims, has_act, dtype, n=n, n_cal=600, K=K, L=L, budgets=budgets)
+    dm = harness.DeviceModel(wl)
+    _same_bits(_run(dm, wl), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()
+
+
 @pytest.mark.parametrize("dtype,dims,has_act,n,budgets,layer,kernel", [
     ("bf16", [512, 640, 640, 10], [1, 1, 0], 2100, (1000, 5000), 2, None),              # a tile of 128 columns for 10 nodes
     ("bf16", [512, 640, 640, 95], [1, 1, 0], 2100, (1000, 5000), 2, None),

@@ -689,9 +689,20 @@ int launch_tile_rows_t(const slonn_tile_params &P, cudaStream_t st)
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
+template <bool BF16, bool VEC>
+int launch_tile_rows_wide_t(const slonn_tile_params &P, cudaStream_t st)
+{
+    const int rc = set_smem(tile_rows_wide_kernel<BF16, VEC>, SLONN_WIDE_SMEM);
+    if (rc) return rc;
+    slonn_launch(tile_rows_wide_kernel<BF16, VEC>, 148u, SLONN_WIDE_WARPS * 32, SLONN_WIDE_SMEM, st, P);
+    return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
+}
+
 template <bool BF16>
 int launch_tile_rows(const slonn_tile_params &P, cudaStream_t st)
 {
+    if (P.cols == SLONN_WIDE_COLS)
+        return !P.select && P.N % SLONN_WIDE_NN == 0 ? launch_tile_rows_wide_t<BF16, true>(P, st) : launch_tile_rows_wide_t<BF16, false>(P, st);
     return !P.select && P.N % 4u == 0 ? launch_tile_rows_t<BF16, true>(P, st) : launch_tile_rows_t<BF16, false>(P, st);
 }
 
@@ -713,6 +724,20 @@ int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint3
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     }
     return SLONN_OK;
+}
+
+// Columns of a work item.  Every node computed: the items are known, 148 are worked on at a time, and 256 columns take 1.8 times as
+// long as 128 (us with 128 and 256 columns, bf16: 4096 x 4096, 4096 queries, 3157 and 2763; 2048 x 2048, 777 queries, 392 items of
+// 256, 239 and 223; 300 queries, 152 items, 149 and 158; 4096 x 1000, 777 queries, 196 items, 213 and 247; fp32 1536 x 304, 2100
+// queries, 104 and 121, padding).  Selected nodes: a group's union holds at least `nodes` columns; from 1024 items of 256 on
+// (4096 x 4096, 4096 queries, 50 %: 2133 and 2060, 25 %: 993 and 980; 2100 queries, 50 %: 1151 and 1093, 25 %, 528 items: 475 and
+// 494; 2048 x 2048, 2100 queries, 50 %: 335 and 359; 777 queries, 50 % of 4096: 469 and 527).
+uint32_t tile_item_cols(uint32_t groups, bool select, uint32_t nodes)
+{
+    const uint64_t wide = (uint64_t)groups * ((nodes + SLONN_WIDE_COLS - 1) / SLONN_WIDE_COLS);
+    const uint64_t narrow = (uint64_t)groups * ((nodes + SLONN_TILE_COLS - 1) / SLONN_TILE_COLS);
+    const bool wider = select ? wide >= 1024u : (wide + 147) / 148 * 9 <= (narrow + 147) / 148 * 5;
+    return wider ? SLONN_WIDE_COLS : SLONN_TILE_COLS;
 }
 
 // One layer for the whole batch.  order_kind: 0 queries as they come (without those of skip_bp), 1 the order of
@@ -744,6 +769,7 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
         else if (order_kind == 1) P.order = (const uint32_t *)(tw.ws + T.order) + (uint64_t)c * T.order_stride;
         else { P.order = list + q0; P.count = count; }
         P.groups = (P.n + SLONN_TILE_G - 1) / SLONN_TILE_G;
+        P.cols = tile_item_cols(P.groups, P.select != 0, P.select ? slonn_layer_nodes(max_bp, ly.N, slonn_model_pre(m)) : ly.N);
         // the sort cleared the count of work items; only the first chunk can rely on it
         if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
         slonn_launch(tile_prep_kernel, dim3(P.groups, 2), 512, smem, st, P);

@@ -13,20 +13,26 @@
 //
 //   tile_order_kernel   queries -> groups (sorted by budget, then keys)
 //   tile_prep_kernel    per group: union of inputs, staged values [entry][query], union of nodes, work items
-//   tile_rows_kernel    per work item (group, 128 columns): the product, bias, ReLU, scatter to the lists
+//   tile_rows_kernel, tile_rows_wide_kernel
+//                       per work item (group, 128 or 256 columns): the product, bias, ReLU, scatter to the lists
 #pragma once
 #include "slonn_common.cuh"
 
 #define SLONN_TILE_G 16         // queries per group
-#define SLONN_TILE_WARPS 16     // warps of tile_rows_kernel: warp w owns the partial sums w and w + 16
+#define SLONN_TILE_WARPS 16     // warps of tile_rows_kernel: two partial sums each
 #define SLONN_TILE_NN 4         // columns per lane
 #define SLONN_TILE_COLS (32 * SLONN_TILE_NN)
+#define SLONN_WIDE_WARPS 8      // the same of tile_rows_wide_kernel: four partial sums each
+#define SLONN_WIDE_NN 8
+#define SLONN_WIDE_COLS (32 * SLONN_WIDE_NN)
 #define SLONN_TILE_CHUNK 8192u  // most queries sorted and staged at a time
 #define SLONN_TILE_MAX_N 32768u // widest layer: the group's G node bitmaps are built in shared memory
 #define SLONN_TILE_SLACK 64u    // entries past a group's list that a pipelined load may touch
 
-// position of partial sum p in the entry order: warp after warp, each warp's two partial sums
-__host__ __device__ __forceinline__ uint32_t tile_slot(uint32_t p) { return (p & 15u) * 2u + (p >> 4); }
+// Position of partial sum p in the entry order, and back.  Four in a row are those of a warp of eight, in bit-reversed order
+// (w, w + 16, w + 8, w + 24), so that the operands of an addition of the tree follow each other; a warp of sixteen has two of them.
+__host__ __device__ __forceinline__ uint32_t tile_slot(uint32_t p) { return (p & 7u) * 4u + ((p >> 4) | ((p >> 2) & 2u)); }
+__host__ __device__ __forceinline__ uint32_t tile_partial(uint32_t slot) { return (slot >> 2) + ((slot & 1u) << 4) + ((slot & 2u) << 2); }
 
 // ---------------------------------------------------------------------------
 // groups: queries in the order of (budget, keys)
@@ -110,6 +116,7 @@ struct slonn_tile_params {
     // scratch
     uint32_t groups;
     uint32_t nwords;          // (N + 31) / 32
+    uint32_t cols;            // columns of a work item: SLONN_TILE_COLS or SLONN_WIDE_COLS
     uint32_t *work;           // number of work items
     uint32_t *items;          // group << 16 | tile (groups <= 1024 * 8, tiles <= N / 128)
     uint32_t *kseg;           // [groups][33] first entry of each partial sum's stretch, total
@@ -239,7 +246,7 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
             ncols = all;
         }
         if (tid < 32u) {
-            const uint32_t tiles = (ncols + SLONN_TILE_COLS - 1) / SLONN_TILE_COLS;
+            const uint32_t tiles = (ncols + P.cols - 1) / P.cols;
             uint32_t base = 0;
             if (tid == 0) {
                 P.ucount[g] = ncols;
@@ -341,7 +348,7 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
         for (uint32_t i = tid; i < total * (G / 4); i += blockDim.x) xt4[i] = z;
         for (uint32_t i = tid; i < 32u * P.wps; i += blockDim.x) { // the listed inputs' rows, word by word
             const uint32_t slot = i / P.wps, w = i - slot * P.wps;
-            const uint32_t p = (slot >> 1) + 16u * (slot & 1u);
+            const uint32_t p = tile_partial(slot);
             uint32_t bits = kbits[i], at = slotstart[slot] + kpre[i];
             while (bits) {
                 const uint32_t t = __ffs(bits) - 1;
@@ -423,8 +430,8 @@ template <bool BF16, bool QUAD> struct tile_weights {
     }
 };
 
-// One block of 16 warps per SM takes work items (group, 128 columns) until none is left.  Warp w walks the entries of
-// the partial sums w and w + 16; a lane holds the 16 queries' sums of four columns (64 accumulators).  Per entry: 16
+// One block of 16 warps per SM takes work items (group, 128 columns) until none is left.  A warp walks the entries of
+// two partial sums (p and p + 16); a lane holds the 16 queries' sums of four columns (64 accumulators).  Per entry: 16
 // values broadcast from the warp's ring in shared memory, four weights loaded two entries ahead into registers, 32
 // packed multiply-adds (one value times two columns' weights; each half rounded on its own, as fmaf does).  What the
 // next item needs first (its entry stretches, its columns, the first values and weights) is fetched while the block
@@ -486,7 +493,7 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         if (lane == 4u) s_item[buf][warp][4] = item;
         if (lane < 4u)
             tile_cp_async<4>((uint32_t)__cvta_generic_to_shared(&s_item[buf][warp][lane]),
-                             lane < 3u ? P.kseg + (item >> 16) * 33u + warp * 2u + lane : P.ucount + (item >> 16));
+                             lane < 3u ? P.kseg + (item >> 16) * 33u + (warp & 7u) * 4u + (warp >> 3) * 2u + lane : P.ucount + (item >> 16));
     };
     // makes the item looked up in s_item[buf] the item at hand and starts the copies of its first blocks
     auto start_copies = [&](uint32_t buf) {
@@ -667,5 +674,340 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         }
         if (!more) return;
         __syncthreads(); // the sums have been read
+    }
+}
+
+// ---------------------------------------------------------------------------
+// the product, 256 columns at a time
+// ---------------------------------------------------------------------------
+// shared memory of tile_rows_wide_kernel
+#define SLONN_WIDE_STEP (2 * SLONN_TILE_G * 4 + 16) // bytes of a step in a warp's ring: two entries' values, their row offsets, padding
+#define SLONN_WIDE_BLOCK 8                          // steps a warp copies ahead at a time
+#define SLONN_WIDE_RING (3 * SLONN_WIDE_BLOCK)      // steps in a warp's ring
+#define SLONN_WIDE_ROWS_AT (2 * SLONN_TILE_G * 4)   // row offsets within a step
+#define SLONN_WIDE_RING_BYTES ((SLONN_WIDE_RING + 1) * SLONN_WIDE_STEP) // the first step's row offsets again behind the last step
+#define SLONN_WIDE_SMEM ((size_t)SLONN_WIDE_WARPS * (SLONN_WIDE_RING_BYTES + SLONN_WIDE_COLS * SLONN_TILE_G * 4))
+#define SLONN_WIDE_STATIC (2 * SLONN_WIDE_COLS * 8 + 2 * SLONN_TILE_G * 12 + 2 * SLONN_WIDE_WARPS * 32 + 16) // s_col, s_q, s_off, s_item, s_tmem
+#define SLONN_WIDE_TMEM 256 // columns of tensor memory: 128 sums per lane, two warps on the same lanes
+static_assert(SLONN_WIDE_SMEM > 46 * 1024 && SLONN_WIDE_SMEM + SLONN_WIDE_STATIC <= 227 * 1024,
+              "tile_rows_wide_kernel must opt in to its shared memory and fit a block's 227 KB with its static part");
+
+// 16 registers of a warp to and from 16 columns of its own 32 lanes of tensor memory
+__device__ __forceinline__ void tile_tmem_store16(uint32_t at, const uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(at), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                 : "memory");
+}
+__device__ __forceinline__ void tile_tmem_load16(uint32_t at, uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(at)
+                 : "memory");
+}
+
+// The eight weights of a lane for one entry, as loaded from p[j] + row.  VEC: neighbouring columns, 16 bytes per load; else one
+// load each.
+template <bool BF16, bool VEC> struct wide_weights {
+    uint32_t r[(BF16 && VEC) ? 4 : 8];
+    __device__ __forceinline__ void load(const unsigned char *const (&p)[VEC ? 1 : SLONN_WIDE_NN], uint32_t row)
+    {
+        if constexpr (VEC) {
+#pragma unroll
+            for (int i = 0; i < (BF16 ? 1 : 2); ++i) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p[0] + row) + i);
+                r[4 * i] = v.x; r[4 * i + 1] = v.y; r[4 * i + 2] = v.z; r[4 * i + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < SLONN_WIDE_NN; ++j)
+                r[j] = BF16 ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(p[j] + row))
+                            : __ldg(reinterpret_cast<const uint32_t *>(p[j] + row));
+        }
+    }
+    __device__ __forceinline__ float2 pair(int i) const // columns 2 i and 2 i + 1, widened (see tile_weights)
+    {
+        if constexpr (!BF16) return make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+        else if constexpr (VEC) return make_float2(__uint_as_float(__byte_perm(r[i], 0u, 0x1044)), __uint_as_float(__byte_perm(r[i], 0u, 0x3244)));
+        else return make_float2(__uint_as_float(__byte_perm(r[2 * i], 0u, 0x1044)), __uint_as_float(__byte_perm(r[2 * i + 1], 0u, 0x1044)));
+    }
+};
+
+// tile_rows_kernel with twice the columns per lane (128 accumulators) and half the warps, one block of 8 warps per SM.  What is not
+// a multiply-add takes issue slots and register writes from them (every value and weight loaded costs a cycle of the
+// scheduler): per multiply-add the 16 broadcast values, the loop and the waits are halved here.  A warp walks the entries of four
+// partial sums, w, w + 16, w + 8, w + 24; a finished one meets its partner of the tree as soon as both exist: the first of two
+// waits in tensor memory (128 registers per lane), the sum of the first two in shared memory, where the warps' sums meet in the
+// end.  VEC: a lane's columns are neighbours (every node computed, N a multiple of 8).
+template <bool BF16, bool VEC>
+__global__ void __launch_bounds__(SLONN_WIDE_WARPS * 32, 1) tile_rows_wide_kernel(slonn_tile_params P)
+{
+    slonn_enter();
+    constexpr int G = SLONN_TILE_G, NN = SLONN_WIDE_NN, W = SLONN_WIDE_WARPS, SEGS = 32 / W;
+    constexpr uint32_t ESZ = BF16 ? 2u : 4u, STEP = SLONN_WIDE_STEP, COLS = SLONN_WIDE_COLS, PART = COLS * G;
+    extern __shared__ __align__(16) unsigned char smem_b[];
+    __shared__ __align__(8) uint2 s_col[2][COLS]; // column and node of each slot (select)
+    __shared__ __align__(16) uint32_t s_item[2][W][8]; // per warp: its SEGS + 1 kseg values; column count at 5, item at 6
+    __shared__ uint64_t s_off[2][G];
+    __shared__ uint32_t s_q[2][G];
+    __shared__ uint32_t s_tmem;
+    const uint32_t n_items = P.work[0];
+    uint32_t it = blockIdx.x;
+    if (it >= n_items) return;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t ring = warp * SLONN_WIDE_RING_BYTES; // offset in smem_b
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(smem_b) + ring;
+    float *part = reinterpret_cast<float *>(smem_b + W * SLONN_WIDE_RING_BYTES); // [warp][query][column slot]
+    // this lane's column slots: 64 i + 2 lane + {0, 1}
+    float *mypart = part + warp * PART + 2u * lane;
+    // union index of column slot s of a tile
+    auto slot_index = [&](uint32_t tile, uint32_t s) -> uint32_t {
+        return tile * COLS + (VEC ? ((s & 63u) >> 1) * NN + (s >> 6) * 2u + (s & 1u) : s);
+    };
+
+    // the item at hand: the lane's columns in row 0
+    const unsigned char *p[VEC ? 1 : NN];
+    wide_weights<BF16, VEC> wn[2];
+    uint32_t at_copy = 0;              // ring block (0, 1, 2) the next copies go to
+    uint32_t src = 0, src_end = 0;     // the entry they start with, and the warp's last, of all groups' entries
+    auto copy_block = [&]() {
+        if (src < src_end) {
+            const uint32_t *krow = P.krow + src;
+            const unsigned char *xsrc = reinterpret_cast<const unsigned char *>(P.xt + (uint64_t)src * G);
+            const uint32_t dst = ring_s + at_copy * (SLONN_WIDE_BLOCK * STEP);
+            const uint32_t to = dst + (lane >> 3) * STEP + (lane & 7u) * 16u; // eight lanes copy a step's values
+            tile_cp_async<16>(to, xsrc + lane * 16u);
+            tile_cp_async<16>(to + 4u * STEP, xsrc + 512u + lane * 16u);
+            if (lane < 8u) tile_cp_async<8>(dst + lane * STEP + SLONN_WIDE_ROWS_AT, krow + lane * 2u);
+            if (lane == 8u && at_copy == 0u) tile_cp_async<8>(ring_s + SLONN_WIDE_RING * STEP + SLONN_WIDE_ROWS_AT, krow);
+            src += SLONN_WIDE_BLOCK * 2;
+            at_copy = at_copy == 2u ? 0u : at_copy + 1u;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // fetches what a warp needs to know of an item into s_item[buf][warp]
+    // (and, between the block's threads, the item's columns into s_col[buf])
+    auto look_up = [&](uint32_t index, uint32_t buf) {
+        const uint32_t item = P.items[index];
+        if (P.select) // entries behind the group's last are not used, but stay inside the scratch
+            tile_cp_async<8>((uint32_t)__cvta_generic_to_shared(&s_col[buf][tid]),
+                             P.ucol + (uint64_t)(item >> 16) * P.N + min((item & 0xffffu) * COLS + tid, P.N - 1u));
+        if (lane == 6u) s_item[buf][warp][6] = item;
+        if (lane <= (uint32_t)SEGS || lane == 5u)
+            tile_cp_async<4>((uint32_t)__cvta_generic_to_shared(&s_item[buf][warp][lane]),
+                             lane <= (uint32_t)SEGS ? P.kseg + (item >> 16) * 33u + warp * SEGS + lane : P.ucount + (item >> 16));
+    };
+    // makes the item looked up in s_item[buf] the item at hand and starts the copies of its first blocks
+    auto start_copies = [&](uint32_t buf) {
+        const uint32_t g = s_item[buf][warp][6] >> 16;
+        src = g * P.kcap + s_item[buf][warp][0];
+        src_end = g * P.kcap + s_item[buf][warp][SEGS];
+        at_copy = 0;
+        copy_block(); copy_block();
+        if (tid < (uint32_t)G) {
+            const uint32_t slot = g * G + tid;
+            const uint32_t q = slot < P.n ? tile_query(P, slot) : 0xffffffffu;
+            s_q[buf][tid] = q;
+            s_off[buf][tid] = (q != 0xffffffffu && P.indptr) ? P.indptr[(uint64_t)q * P.n_act + P.a] : 0;
+        }
+    };
+    // and, behind a barrier of the block, its first weights
+    auto start_weights = [&](uint32_t buf) {
+        const uint32_t tile = s_item[buf][warp][6] & 0xffffu, last = s_item[buf][warp][5] - tile * COLS - 1u;
+        const unsigned char *WT = reinterpret_cast<const unsigned char *>(P.WT);
+        if constexpr (VEC) {
+            p[0] = WT + (uint64_t)min(tile * COLS + lane * NN, P.N - NN) * ESZ;
+        } else {
+#pragma unroll
+            for (int j = 0; j < NN; ++j) {
+                const uint32_t s = min((j >> 1) * 64u + lane * 2u + (j & 1), last); // slots behind the last column repeat it
+                p[j] = WT + (uint64_t)(P.select ? s_col[buf][s].x : tile * COLS + s) * ESZ;
+            }
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        if (s_item[buf][warp][SEGS] != s_item[buf][warp][0]) {
+            const uint2 r = *reinterpret_cast<const uint2 *>(smem_b + ring + SLONN_WIDE_ROWS_AT);
+            wn[0].load(p, r.x);
+            wn[1].load(p, r.y);
+        }
+    };
+
+    // items are dealt out in turn: neighbours in the list are of neighbouring groups and cost about the same
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_tmem)), "r"(SLONN_WIDE_TMEM) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (uint32_t i = lane; i < SLONN_WIDE_RING_BYTES / 4; i += 32) reinterpret_cast<uint32_t *>(smem_b + ring)[i] = 0u; // row offsets that exist
+    look_up(it, 0u);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem + (((warp & 3u) * 32u) << 16) + (warp >> 2) * 128u; // this warp's 32 lanes, 128 columns
+    start_copies(0u);
+    start_weights(0u);
+
+    for (uint32_t buf = 0;; buf ^= 1u) {
+        float2 acc[G][NN / 2];
+        uint32_t left = 0; // steps of the ring block ahead
+        uint32_t at = ring; // the step at hand, in smem_b
+#pragma unroll 1
+        for (uint32_t seg = 0; seg < (uint32_t)SEGS; ++seg) { // the warp's partial sums
+#pragma unroll
+            for (int i = 0; i < G; ++i)
+#pragma unroll
+                for (int j = 0; j < NN / 2; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+            uint32_t todo = (s_item[buf][warp][seg + 1u] - s_item[buf][warp][seg]) >> 1; // steps of two entries
+#pragma unroll 1
+            while (todo) {
+                if (left == 0) { // a new ring block: the one after it must have landed too, the one before is free
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    __syncwarp();
+                    copy_block();
+                    left = SLONN_WIDE_BLOCK;
+                    if (at == ring + SLONN_WIDE_RING * STEP) at = ring;
+                }
+                const uint32_t now = min(todo, left), at_stop = at + now * STEP;
+                todo -= now;
+                left -= now;
+#pragma unroll 1
+                do {
+                    float2 w[2][NN / 2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+#pragma unroll
+                        for (int j = 0; j < NN / 2; ++j) w[e][j] = wn[e].pair(j);
+                    const uint2 r = *reinterpret_cast<const uint2 *>(smem_b + at + STEP + SLONN_WIDE_ROWS_AT); // the next step's rows (behind the last step: rows that exist, not used)
+                    wn[0].load(p, r.x);
+                    wn[1].load(p, r.y);
+                    constexpr int RUN = 8; // neighbouring multiply-adds that share the weight pair
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+#pragma unroll
+                        for (int i0 = 0; i0 < G; i0 += RUN) {
+                            float x[RUN];
+#pragma unroll
+                            for (int i = 0; i < RUN; i += 4) {
+                                const float4 v = *reinterpret_cast<const float4 *>(smem_b + at + (e * G + i0 + i) * 4);
+                                x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+                            }
+#pragma unroll
+                            for (int j = 0; j < NN / 2; ++j)
+#pragma unroll
+                                for (int i = 0; i < RUN; ++i) acc[i0 + i][j] = __ffma2_rn(make_float2(x[i], x[i]), w[e][j], acc[i0 + i][j]);
+                        }
+                    at += STEP;
+                } while (at != at_stop);
+            }
+            // the partial sum is complete: it waits for its partner, or meets it
+            auto sums = [&](int k) -> float & { float2 &v = acc[k / NN][(k % NN) >> 1]; return (k & 1) ? v.y : v.x; };
+            if (!(seg & 1u)) {
+#pragma unroll
+                for (int h = 0; h < G * NN / 16; ++h) {
+                    uint32_t t[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) t[k] = __float_as_uint(sums(16 * h + k));
+                    tile_tmem_store16(tmem + 16u * h, t);
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                continue;
+            }
+#pragma unroll
+            for (int h = 0; h < G * NN / 16; ++h) {
+                uint32_t t[16];
+                tile_tmem_load16(tmem + 16u * h, t);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) sums(16 * h + k) = __uint_as_float(t[k]) + sums(16 * h + k);
+            }
+            const bool later = seg >= (uint32_t)SEGS / 2u;
+            if (!later) {
+                __syncthreads(); // the block has read the sums of the item before
+                if (it + gridDim.x < n_items) look_up(it + gridDim.x, buf ^ 1u);
+            }
+#pragma unroll
+            for (int i = 0; i < G; ++i)
+#pragma unroll
+                for (int j = 0; j < NN / 2; ++j) {
+                    float2 *s = reinterpret_cast<float2 *>(mypart + i * COLS + j * 64);
+                    *s = later ? __fadd2_rn(*s, acc[i][j]) : acc[i][j];
+                }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+
+        it += gridDim.x;
+        const bool more = it < n_items;
+        // the item's own end, one column per thread
+        const uint32_t g = s_item[buf][warp][6] >> 16, tile = s_item[buf][warp][6] & 0xffffu, cnt = s_item[buf][warp][5];
+        const uint32_t u = slot_index(tile, tid);
+        const bool mine = u < cnt;
+        uint32_t nd = 0;
+        float b = 0.0f;
+        uint4 word[G / 4], below[G / 4];
+        if (mine) {
+            nd = P.select ? s_col[buf][tid].y : P.colnode ? __ldg(P.colnode + u) : u;
+            b = __ldg(P.bias + nd);
+            if (P.select) {
+                const uint64_t from = (((uint64_t)g * P.nwords + (nd >> 5)) * G) / 4u;
+#pragma unroll
+                for (int i = 0; i < G / 4; ++i) {
+                    word[i] = reinterpret_cast<const uint4 *>(P.bm)[from + i];
+                    below[i] = reinterpret_cast<const uint4 *>(P.pre)[from + i];
+                }
+            }
+        }
+        if (more) start_copies(buf ^ 1u);
+        __syncthreads();
+        if (more) start_weights(buf ^ 1u);
+        if (mine) {
+            // the warps' sums, strides W / 2 .. 1 of the tree; then bias, ReLU and the query's list
+            auto emit = [&](uint32_t k, uint32_t wd, uint32_t bl) {
+                float v[W];
+#pragma unroll
+                for (int w = 0; w < W; ++w) v[w] = part[w * PART + k * COLS + tid];
+#pragma unroll
+                for (int off = W / 2; off >= 1; off >>= 1)
+#pragma unroll
+                    for (int w = 0; w < off; ++w) v[w] = v[w] + v[w + off];
+                const uint32_t q = s_q[buf][k];
+                if (q == 0xffffffffu) return;
+                float z = v[0] + b;
+                if (P.relu) z = z > 0.0f ? z : 0.0f;
+                uint32_t pos = nd;
+                if (P.select) {
+                    const uint32_t bit = 1u << (nd & 31u);
+                    if (!(wd & bit)) return;
+                    pos = bl + __popc(wd & (bit - 1u));
+                }
+                const uint64_t off = s_off[buf][k];
+                if (P.out_vals) P.out_vals[off + pos] = z;
+                if (P.write_ids) P.ids[off + pos] = nd;
+                if (P.out_dense) {
+                    P.out_dense[(uint64_t)q * P.out_stride + pos] = z;
+                    if (P.out_dense_ids) P.out_dense_ids[(uint64_t)q * P.out_stride + pos] = nd;
+                }
+            };
+#pragma unroll
+            for (int i = 0; i < G / 4; ++i) {
+                emit(4 * i, word[i].x, below[i].x);
+                emit(4 * i + 1, word[i].y, below[i].y);
+                emit(4 * i + 2, word[i].z, below[i].z);
+                emit(4 * i + 3, word[i].w, below[i].w);
+            }
+        }
+        if (!more) break;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(SLONN_WIDE_TMEM) : "memory");
     }
 }

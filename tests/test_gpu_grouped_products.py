@@ -47,6 +47,22 @@ def test_grouped_products_in_several_chunks():
     dm.free()
 
 
+@pytest.mark.parametrize("dtype,dims,has_act,n,budgets", [
+    ("bf16", [40, 264, 256, 250], [1, 0, 0], 1209, (5000,)),              # every node: one item of exactly 256 columns, one short of it
+    ("f32", [36, 264, 252, 253], [1, 0, 0], 1209, (5000,)),
+    ("bf16", [8, 248, 256, 505], [1, 1, 0], 2500, (10000,)),              # 100 % queries, two items, the second not full
+    ("bf16", [1032, 520, 528, 24], [1, 1, 0], 8209, (4850, 4880, 9999)),  # selected nodes, up to one more than an item holds
+    ("f32", [132, 516, 260, 24], [1, 1, 0], 8192, (9000, 9900)),
+])
+def test_items_of_256_columns(dtype, dims, has_act, n, budgets):
+    """Enough work items for the kernel with eight columns per lane; partial sums without an input and odd widths among them."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4300 + n, dims, has_act, dtype, n=n, n_cal=300, K=4, L=2, budgets=budgets)
+    dm = harness.DeviceModel(wl)
+    _same_bits(_run(dm, wl), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()
+
+
 def test_grouped_products_need_their_scratch_and_do_without_it():
     """A workspace of the size the other kernels need is still taken, with the same results."""
     from paper_2204_08400_b200 import binding as sl, harness

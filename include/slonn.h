@@ -221,8 +221,8 @@ typedef struct {
  * kernels walk the query's nonzero inputs and read single weights from a transposed copy the model
  * keeps.  By default the library picks per query by budget: up to SLONN_COLS_MAX_BP
  * the input list is sparse enough for the input-stationary kernels to win (batches of tens of queries
- * only when no budget exceeds 1500 bp and only for layers at least 2048 inputs wide; a handful of queries keep
- * the row kernels); in large batches the queries that compute more than a few hundred nodes per layer are sorted by
+ * only for layers at least 2048 inputs wide, and, where the layer has an activator, only when no budget exceeds 1500 bp; a handful of
+ * queries keep the row kernels); in large batches the queries that compute more than a few hundred nodes per layer are sorted by
  * budget and keys and evaluated 16 at a time over the union of their inputs and nodes, in the same order of sums
  * and with the same results, when the workspace holds the scratch for it (slonn_workspace_bytes includes it).  These two flags force one kind for the whole batch, for testing and
  * tuning; setting both is an error.  They apply to the per-stage kernels and to the

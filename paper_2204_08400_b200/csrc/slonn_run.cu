@@ -471,7 +471,11 @@ int launch_gather_cols(const slonn_model *m, slonn_gather_params &P, uint32_t n,
     const uint32_t R = SLONN_COLS_R;
     const uint64_t want_ctas = 148ull * 8;
     // too few warp passes to fill the GPU: one block per pass, its warps sharing the walk over the input list
-    const bool split = (uint64_t)n * ((max_rows + 32u * R - 1u) / (32u * R)) < want_ctas;
+    // (layers without activator, whose blocks need no order of their nodes: up to 18 blocks per SM; us of whole queries per block and of
+    // this form, 20 % budgets: 4096 x 1000, 2880 blocks 78 and 56, 4000 blocks 78 and 72, but at 10 % 45 and 50; 2048 x 512, 2000
+    // blocks 44 and 29, 2800 blocks 35 and 35; fp32 2048 x 2000, 3200 blocks 43 and 39, 5760 blocks 45 and 62)
+    const uint64_t split_ctas = (uint64_t)n * ((max_rows + 32u * R - 1u) / (32u * R));
+    const bool split = split_ctas < (P.use_list ? want_ctas : 148ull * 18);
     // a layer that computes every node, its width a multiple of the nodes one 16-byte load holds: a lane takes that
     // many neighbouring columns (1000-node output layer of a 4096-wide network: 0.36 -> 0.26 ms per 4096 queries)
     const uint32_t nv = bf ? 8u : 4u;
@@ -479,7 +483,7 @@ int launch_gather_cols(const slonn_model *m, slonn_gather_params &P, uint32_t n,
     const uint32_t unit = vec ? 32u * nv : 32u * R; // nodes per warp pass
     const uint32_t passes = (max_rows + unit - 1u) / unit;
     uint64_t ppc = ((uint64_t)n * passes + want_ctas - 1) / want_ctas; // passes per block
-    ppc = std::min<uint64_t>(std::max<uint64_t>(ppc, 1), passes);
+    ppc = split ? 1 : std::min<uint64_t>(std::max<uint64_t>(ppc, 1), passes);
     const uint32_t rounds = (uint32_t)((ppc + 7) / 8);
     const uint32_t warps = split ? SLONN_SPLIT_WARPS : std::max(vec ? 1u : 4u, (uint32_t)((ppc + rounds - 1) / rounds));
     P.rows_per_cta = (uint32_t)ppc * unit;
@@ -590,6 +594,13 @@ int launch_layer_cols(const slonn_model *m, const slonn_layer &ly, uint32_t laye
     return id16 ? launch_layer_cols_s<false, uint16_t>(Q, split, grid, warps * 32u, smem, st) : launch_layer_cols_s<false, uint32_t>(Q, split, grid, warps * 32u, smem, st);
 }
 
+// Layers without activator in batches too small to fill the GPU (us with whole rows and input-stationary, budgets of 20, 25 and 35 %):
+// 4096 x 1000 bf16, 32 queries 27 27 29 and 19 21 25, 64 queries 47 48 50 and 27 31 37, 100 queries 60 60 62 and 37 41 52; fp32 2048 x
+// 2000, 32 queries 39 39 41 and 19 21 23; 3072 x 304, 64 queries 21 21 21 and 17 17 21; 4096 x 200, 64 queries 17 17 17 and 17 19
+// 23; 4096 x 1000, 16 queries 17 17 19 and 19 23 33.  A layer with activator orders its nodes and stages its list in every block:
+// 64 queries, 4096 x 4096, 25 %, 70 and 99.
+#define SLONN_COLS_PLAIN_QUERIES 32u
+#define SLONN_COLS_PLAIN_ROWS (148ull * 128)
 // Budgets 1..limit take the input-stationary kernels in this layer (0: none do).
 uint32_t cols_budget_limit(const slonn_layer &ly, const slonn_gather_params &P, const slonn_batch *b, uint32_t n, uint32_t max_rows,
                            uint32_t max_bp)
@@ -600,7 +611,11 @@ uint32_t cols_budget_limit(const slonn_layer &ly, const slonn_gather_params &P, 
     // tens of queries: the one-block-per-64-nodes variant pays only for long weight rows and very sparse lists
     // (4096-wide nine-layer network, 64 queries: 0.36 -> 0.30 ms per step at 10 %, but 0.57 -> 0.92 ms at 25 %)
     // and only when no query of the batch needs the row kernels (a second launch of idle blocks costs such a batch 6 %)
-    return ((uint64_t)n * max_rows > 148ull * 64 && ly.D >= 2048u && max_bp <= 1500u) ? 1500u : 0u;
+    if ((uint64_t)n * max_rows > 148ull * 64 && ly.D >= 2048u && max_bp <= 1500u) return 1500u;
+    // a layer without activator shares no selection between its blocks: from 64 queries on, any sparse list
+    if (!P.use_list && n >= SLONN_COLS_PLAIN_QUERIES && (uint64_t)n * max_rows >= SLONN_COLS_PLAIN_ROWS && ly.D >= 2048u && max_bp <= SLONN_COLS_MAX_BP)
+        return SLONN_COLS_MAX_BP;
+    return 0;
 }
 
 // Rows of one layer for a batch whose layer input is `P.in`: the input-stationary kernel for the queries

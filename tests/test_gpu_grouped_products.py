@@ -63,6 +63,17 @@ def test_items_of_256_columns(dtype, dims, has_act, n, budgets):
     dm.free()
 
 
+@pytest.mark.parametrize("dtype,n,last", [("bf16", 40, 505), ("f32", 33, 576), ("bf16", 200, 500), ("f32", 255, 641), ("bf16", 64, 296)])
+def test_plain_layers_of_few_queries_by_input(dtype, n, last):
+    """A layer without activator behind a list of 2048 inputs, one block per (query, 64 nodes): odd widths, a last block that is
+    not full, more blocks than one per query and pass of its warps."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(4700 + n, [64, 2048, last], [1, 0], dtype, n=n, n_cal=200, K=4, L=2, budgets=(20, 2000, 3500))
+    dm = harness.DeviceModel(wl)
+    _same_bits(_run(dm, wl), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()
+
+
 def test_grouped_products_need_their_scratch_and_do_without_it():
     """A workspace of the size the other kernels need is still taken, with the same results."""
     from paper_2204_08400_b200 import binding as sl, harness

@@ -701,24 +701,42 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
 static_assert(SLONN_WIDE_SMEM > 46 * 1024 && SLONN_WIDE_SMEM + SLONN_WIDE_STATIC <= 227 * 1024,
               "tile_rows_wide_kernel must opt in to its shared memory and fit a block's 227 KB with its static part");
 
-// 16 registers of a warp to and from 16 columns of its own 32 lanes of tensor memory
-__device__ __forceinline__ void tile_tmem_store16(uint32_t at, const uint32_t (&r)[16])
+// N values of every lane of a warp, value(0) to value(N - 1), to its own 32 lanes of tensor memory, 16 columns at a time, and back: take(k,
+// v).  All lanes have to execute these instructions together, and the code in front of them branches by lane: the warp meets first.
+template <int N, typename F>
+__device__ __forceinline__ void tile_tmem_store(uint32_t at, F value)
 {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-                 ::"r"(at), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-                 : "memory");
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < N; h += 16) {
+        uint32_t r[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(value(h + k));
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+                     "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                     ::"r"(at + h), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                     "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                     : "memory");
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tile_tmem_load16(uint32_t at, uint32_t (&r)[16])
+template <int N, typename F>
+__device__ __forceinline__ void tile_tmem_load(uint32_t at, F take)
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-                 "tcgen05.wait::ld.sync.aligned;"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(at)
-                 : "memory");
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < N; h += 16) {
+        uint32_t r[16];
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                     "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+                     "tcgen05.wait::ld.sync.aligned;"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                       "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                     : "r"(at + h)
+                     : "memory");
+#pragma unroll
+        for (int k = 0; k < 16; ++k) take(h + k, __uint_as_float(r[k]));
+    }
 }
 
 // The eight weights of a lane for one entry, as loaded from p[j] + row.  VEC: neighbouring columns, 16 bytes per load; else one
@@ -850,6 +868,7 @@ __global__ void __launch_bounds__(SLONN_WIDE_WARPS * 32, 1) tile_rows_wide_kerne
 
     // items are dealt out in turn: neighbours in the list are of neighbouring groups and cost about the same
     if (warp == 0) {
+        __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_tmem)), "r"(SLONN_WIDE_TMEM) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -918,23 +937,10 @@ __global__ void __launch_bounds__(SLONN_WIDE_WARPS * 32, 1) tile_rows_wide_kerne
             // the partial sum is complete: it waits for its partner, or meets it
             auto sums = [&](int k) -> float & { float2 &v = acc[k / NN][(k % NN) >> 1]; return (k & 1) ? v.y : v.x; };
             if (!(seg & 1u)) {
-#pragma unroll
-                for (int h = 0; h < G * NN / 16; ++h) {
-                    uint32_t t[16];
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) t[k] = __float_as_uint(sums(16 * h + k));
-                    tile_tmem_store16(tmem + 16u * h, t);
-                }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tile_tmem_store<G * NN>(tmem, sums);
                 continue;
             }
-#pragma unroll
-            for (int h = 0; h < G * NN / 16; ++h) {
-                uint32_t t[16];
-                tile_tmem_load16(tmem + 16u * h, t);
-#pragma unroll
-                for (int k = 0; k < 16; ++k) sums(16 * h + k) = __uint_as_float(t[k]) + sums(16 * h + k);
-            }
+            tile_tmem_load<G * NN>(tmem, [&](int k, float first) { sums(k) = first + sums(k); });
             const bool later = seg >= (uint32_t)SEGS / 2u;
             if (!later) {
                 __syncthreads(); // the block has read the sums of the item before
@@ -1017,6 +1023,7 @@ __global__ void __launch_bounds__(SLONN_WIDE_WARPS * 32, 1) tile_rows_wide_kerne
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(SLONN_WIDE_TMEM) : "memory");
     }
 }

@@ -131,8 +131,10 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// All lanes of the warp together; the code in front branches by lane (a wait's polls, rows that are not there), so the warp meets first.
 __device__ __forceinline__ void tmem_load32(uint32_t taddr, uint32_t (&r)[32])
 {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -198,6 +200,7 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) { // one warp allocates the accumulator columns and gives the permit back
+        __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot_addr), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -414,6 +417,7 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
+        __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     }
 }

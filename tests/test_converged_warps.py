@@ -24,7 +24,7 @@ def unsynchronised(text):
     return bad
 
 
-@pytest.mark.parametrize("name", ["slonn_tile_kernels.cuh"])
+@pytest.mark.parametrize("name", ["slonn_tile_kernels.cuh", "slonn_dense_tc.cu"])
 def test_aligned_instructions_stand_behind_a_meeting_of_the_warp(name):
     with open(os.path.join(CSRC, name)) as f:
         text = f.read()

@@ -485,20 +485,39 @@ int launch_gather_cols_t(const slonn_gather_params &P, uint64_t grid, uint32_t t
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
+// Layers without activator in batches too small to fill the GPU (us with whole rows and input-stationary, budgets of 20, 25 and 35 %):
+// 4096 x 1000 bf16, 32 queries 27 27 29 and 19 21 25, 64 queries 47 48 50 and 27 31 37, 100 queries 60 60 62 and 37 41 52; fp32 2048 x
+// 2000, 32 queries 39 39 41 and 19 21 23; 3072 x 304, 64 queries 21 21 21 and 17 17 21; 4096 x 200, 64 queries 17 17 17 and 17 19
+// 23; 4096 x 1000, 16 queries 17 17 19 and 19 23 33; 4096 x 512, 37 queries 17 17 19 and 19 21 23.  A block evaluates 64 nodes whether
+// the layer has them or not: 4096 x 10, 2000 queries 31 31 35 and 41 45 58; 2048 x 130, 733 queries, 35 %, 39 and 41.  Beyond 16
+// blocks per SM a query has a block: 4096 x 200, 750 queries, 25 %, 84 and 93.  Of 2669 points that these lines and launch_gather_cols' change
+// (1024 to 4096 inputs, 10 to 2000 nodes, 150 to 3000 blocks, both types, budgets of 1 to 35 % and two mixes with 1 %), two were slower, by
+// 1 and 3 % of the pass: one query in 32 at 15 %, the others at 1 %.  A layer with activator orders its nodes and stages its list in every
+// block: 64 queries, 4096 x 4096, 25 %, 70 and 99.
+#define SLONN_COLS_PLAIN_QUERIES 32u
+#define SLONN_COLS_PLAIN_ROWS (148ull * 160)
+#define SLONN_COLS_PLAIN_CTAS (148ull * 16)
+
 int launch_gather_cols(const slonn_model *m, slonn_gather_params &P, uint32_t n, uint32_t max_rows, cudaStream_t st)
 {
     const bool bf = m->dtype == SLONN_BF16;
     const uint32_t R = SLONN_COLS_R;
     const uint64_t want_ctas = 148ull * 8;
-    // too few warp passes to fill the GPU: one block per pass, its warps sharing the walk over the input list
-    // (layers without activator, whose blocks need no order of their nodes: up to 18 blocks per SM; us of whole queries per block and of
-    // this form, 20 % budgets: 4096 x 1000, 2880 blocks 78 and 56, 4000 blocks 78 and 72, but at 10 % 45 and 50; 2048 x 512, 2000
-    // blocks 44 and 29, 2800 blocks 35 and 35; fp32 2048 x 2000, 3200 blocks 43 and 39, 5760 blocks 45 and 62)
+    const uint32_t nv = bf ? 8u : 4u; // nodes one 16-byte load holds
+    // Too few warp passes to fill the GPU: one block per pass, its warps sharing the walk over the input list.  In layers without
+    // activator, whose blocks need no order of their nodes, at up to 16 blocks per SM (SLONN_COLS_PLAIN_CTAS) where the lists are longer
+    // than the 15 % that bring any smaller batch here; with such lists, the more blocks the longer they are, as a block's fixed part
+    // (setting up the list, adding the warps' sums) is repeated every 64 nodes, and none where a whole block's loads take one node each.
+    // Us of whole queries per block and of this form, bf16: 2048 x 304, lists of 205, 1200 blocks 25 and 19, 2000 blocks 25 and 23, 2600
+    // blocks 25 and 27; lists of 307, 1600 blocks 31 and 23; lists of 102, 1200 blocks 19 and 17, 2600 blocks 19 and 23; lists of 20, 1600
+    // blocks 13 and 15; 2048 x 50, lists of 153, 1600 blocks 17 and 19.
     const uint64_t split_ctas = (uint64_t)n * ((max_rows + 32u * R - 1u) / (32u * R));
-    const bool split = split_ctas < (P.use_list ? want_ctas : 148ull * 18);
+    uint64_t split_limit = want_ctas;
+    if (!P.use_list && P.in_cap * 20ull > P.D * 3ull) split_limit = SLONN_COLS_PLAIN_CTAS;
+    else if (!P.use_list && P.N % nv == 0u) split_limit = 148ull * (8u + std::min(8u, P.in_cap / 80u));
+    const bool split = split_ctas < split_limit;
     // a layer that computes every node, its width a multiple of the nodes one 16-byte load holds: a lane takes that
     // many neighbouring columns (1000-node output layer of a 4096-wide network: 0.36 -> 0.26 ms per 4096 queries)
-    const uint32_t nv = bf ? 8u : 4u;
     const bool vec = !split && !P.use_list && P.N % nv == 0u;
     const uint32_t unit = vec ? 32u * nv : 32u * R; // nodes per warp pass
     const uint32_t passes = (max_rows + unit - 1u) / unit;
@@ -614,13 +633,6 @@ int launch_layer_cols(const slonn_model *m, const slonn_layer &ly, uint32_t laye
     return id16 ? launch_layer_cols_s<false, uint16_t>(Q, split, grid, warps * 32u, smem, st) : launch_layer_cols_s<false, uint32_t>(Q, split, grid, warps * 32u, smem, st);
 }
 
-// Layers without activator in batches too small to fill the GPU (us with whole rows and input-stationary, budgets of 20, 25 and 35 %):
-// 4096 x 1000 bf16, 32 queries 27 27 29 and 19 21 25, 64 queries 47 48 50 and 27 31 37, 100 queries 60 60 62 and 37 41 52; fp32 2048 x
-// 2000, 32 queries 39 39 41 and 19 21 23; 3072 x 304, 64 queries 21 21 21 and 17 17 21; 4096 x 200, 64 queries 17 17 17 and 17 19
-// 23; 4096 x 1000, 16 queries 17 17 19 and 19 23 33.  A layer with activator orders its nodes and stages its list in every block:
-// 64 queries, 4096 x 4096, 25 %, 70 and 99.
-#define SLONN_COLS_PLAIN_QUERIES 32u
-#define SLONN_COLS_PLAIN_ROWS (148ull * 128)
 // Budgets 1..limit take the input-stationary kernels in this layer (0: none do).
 uint32_t cols_budget_limit(const slonn_layer &ly, const slonn_gather_params &P, const slonn_batch *b, uint32_t n, uint32_t max_rows,
                            uint32_t max_bp)
@@ -632,8 +644,10 @@ uint32_t cols_budget_limit(const slonn_layer &ly, const slonn_gather_params &P, 
     // (4096-wide nine-layer network, 64 queries: 0.36 -> 0.30 ms per step at 10 %, but 0.57 -> 0.92 ms at 25 %)
     // and only when no query of the batch needs the row kernels (a second launch of idle blocks costs such a batch 6 %)
     if ((uint64_t)n * max_rows > 148ull * 64 && ly.D >= 2048u && max_bp <= 1500u) return 1500u;
-    // a layer without activator shares no selection between its blocks: from 64 queries on, any sparse list
-    if (!P.use_list && n >= SLONN_COLS_PLAIN_QUERIES && (uint64_t)n * max_rows >= SLONN_COLS_PLAIN_ROWS && ly.D >= 2048u && max_bp <= SLONN_COLS_MAX_BP)
+    // a layer without activator shares no selection between its blocks: any sparse list, where the blocks' 64 nodes are three quarters full
+    const uint64_t blocks = (uint64_t)n * ((ly.N + 63u) / 64u);
+    if (!P.use_list && n >= SLONN_COLS_PLAIN_QUERIES && (uint64_t)n * ly.N >= SLONN_COLS_PLAIN_ROWS && blocks < SLONN_COLS_PLAIN_CTAS &&
+        (uint64_t)n * ly.N * 4u >= blocks * 192u && ly.D >= 2048u && max_bp <= SLONN_COLS_MAX_BP)
         return SLONN_COLS_MAX_BP;
     return 0;
 }

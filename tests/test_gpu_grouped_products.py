@@ -74,6 +74,30 @@ def test_plain_layers_of_few_queries_by_input(dtype, n, last):
     dm.free()
 
 
+@pytest.mark.parametrize("dtype,n,last,kernel", [
+    ("bf16", 2000, 10, "gather_dot_kernel"),    # a block's 64 nodes are mostly padding
+    ("bf16", 37, 512, "gather_dot_kernel"),     # 18,944 rows; from 23,680 on
+    ("f32", 47, 504, "gather_cols_kernel"),
+    ("bf16", 493, 48, "gather_dot_kernel"),     # 23,664
+    ("bf16", 494, 48, "gather_cols_kernel"),
+    ("bf16", 750, 200, "gather_dot_kernel"),    # 3000 blocks; below 2368
+    ("f32", 592, 200, "gather_dot_kernel"),
+    ("f32", 591, 200, "gather_cols_kernel"),
+    ("bf16", 215, 641, "gather_cols_kernel"),   # an odd width, 2365 blocks
+    ("bf16", 255, 641, "gather_cols_kernel"),   # as many rows as fill the GPU: whole queries per block
+])
+def test_plain_layers_of_few_queries_take_columns_where_they_pay(dtype, n, last, kernel):
+    """Both sides of each line of the dispatch, at budgets that smaller batches leave to the row kernels; same bits as these."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(4900 + n, [64, 2048, last], [1, 0], dtype, n=n, n_cal=200, K=4, L=2, budgets=(300, 2000, 3500))
+    dm = harness.DeviceModel(wl)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
+    names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == 1]
+    assert names == [kernel], names
+    _same_bits(b.results(), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()
+
+
 @pytest.mark.parametrize("dtype,dims,n,budgets", [
     ("f32", [64, 30000, 24], 100, (1000, 3001, 5000)),   # a last group of four queries
     ("bf16", [72, 52000, 24], 64, (1, 7, 2000)),         # lists of a few entries: ranges of ids without any

@@ -435,6 +435,8 @@ int slonn_run_timed(const slonn_model *m, const slonn_batch *batch, void *worksp
  */
 #define SLONN_ALL_LAYERS 0xffffffffu
 #define SLONN_MAX_RECORDS (10 * SLONN_MAX_LAYERS)
+#define SLONN_COLS_EVERY 10000u
+#define SLONN_COLS_EVERY_WIDE 10001u
 typedef struct {
     uint32_t stage;      /* SLONN_STAGE_*                                                             */
     uint32_t layer;      /* the layer the launch works on, or SLONN_ALL_LAYERS                        */
@@ -442,8 +444,9 @@ typedef struct {
     uint32_t skips_full; /* ... 1: except those at 10000 bp, which another launch serves              */
     uint32_t cols_bp;    /* whole-network launches: queries with budgets up to this evaluated their   */
                          /* list-fed activator layers input-stationary (0 = every layer row-wise);    */
-                         /* HASH_SELECT, FULL_ROWS, GROUP_ROWS: 10000 when single weights of the        */
-                         /* transposed copy were read (the two latter: 16 queries at a time), else 0     */
+                         /* HASH_SELECT, FULL_ROWS, GROUP_ROWS: SLONN_COLS_EVERY when single weights of  */
+                         /* the transposed copy were read (the two latter: 16 queries at a time, 128     */
+                         /* columns or, SLONN_COLS_EVERY_WIDE, 256), else 0                              */
     float ms;            /* device time between the event pair around the launch                      */
 } slonn_launch_record;
 int slonn_run_traced(const slonn_model *m, const slonn_batch *batch, void *workspace,

@@ -35,6 +35,7 @@ KERNEL_OF_STAGE = {
 }
 
 TILE_G = 16                       # queries per group of the grouped products
+COLS_EVERY_WIDE = 10001           # SLONN_COLS_EVERY_WIDE: of them, those that took 256 columns at a time
 
 
 @dataclass
@@ -141,7 +142,8 @@ def launch_bytes(sh: NetShape, rec: dict, bps: Sequence[int], x_nnz: Optional[np
 
 def kernel_name(sh: NetShape, rec: dict) -> str:
     """The kernel behind a record (rows of at most one 512-byte round take the short-row gather).  Grouped products are
-    three launches under one record: the sort into groups, their preparation, and the product, which takes the time."""
+    three launches under one record: the sort into groups, their preparation, and the product, which takes the time; both
+    of its kernels go by the one name here (see timed_kernel)."""
     if grouped_products(rec):
         return "tile_rows_kernel"
     if rec["stage"] == "hash_select" and rec["cols_bp"]:
@@ -151,11 +153,18 @@ def kernel_name(sh: NetShape, rec: dict) -> str:
     return KERNEL_OF_STAGE[rec["stage"]]
 
 
+def timed_kernel(sh: NetShape, rec: dict) -> str:
+    """kernel_name, with the two kernels of grouped products told apart: work items of 128 and of 256 columns."""
+    if grouped_products(rec) and rec["cols_bp"] == COLS_EVERY_WIDE:
+        return "tile_rows_wide_kernel"
+    return kernel_name(sh, rec)
+
+
 def per_kernel(sh: NetShape, records: List[dict], bps, x_nnz=None) -> dict:
     """Launch records of ONE step grouped by kernel: launches, ms and the three byte totals."""
     acc = {}
     for r in records:
-        k = kernel_name(sh, r)
+        k = timed_kernel(sh, r)
         b = launch_bytes(sh, r, bps, x_nnz)
         a = acc.setdefault(k, dict(launches=0, ms=0.0, as_run=0, algorithmic=0, row_granular=0, flops=0.0))
         a["launches"] += 1

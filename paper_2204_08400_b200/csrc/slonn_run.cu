@@ -33,11 +33,13 @@ struct stage_timer {
         cudaEventRecord(s.a, st);
         ++n;
     }
-    void by_input() { if (n > 0 && !failed) spans[n - 1].cols_bp = 10000u; } // the last launch read single weights of a transposed copy
+    void by_input() { if (n > 0 && !failed) spans[n - 1].cols_bp = SLONN_COLS_EVERY; } // the last launch read single weights of a transposed copy
+    void by_input_wide() { if (n > 0 && !failed) spans[n - 1].cols_bp = SLONN_COLS_EVERY_WIDE; } // and 256 columns of it at a time
     void toc() { if (n > 0 && !failed) cudaEventRecord(spans[n - 1].b, st); }
 };
 #define TIC(...) do { if (tm) tm->tic(__VA_ARGS__); } while (0)
 #define TIC_BY_INPUT() do { if (tm) tm->by_input(); } while (0)
+#define TIC_BY_INPUT_WIDE() do { if (tm) tm->by_input_wide(); } while (0)
 #define TOC() do { if (tm) tm->toc(); } while (0)
 #define AT_LAYER(l) do { if (tm) tm->layer = (l); } while (0)
 
@@ -793,7 +795,7 @@ uint32_t tile_item_cols(uint32_t groups, bool select, uint32_t nodes)
 // launch_tile_order, 2 the compacted list `list` of *count queries.  fresh_order: launch_tile_order was the launch before.
 int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, const slonn_gather_params &G, uint32_t n, uint32_t max_bp,
                       const tile_ws &tw, int order_kind, const uint32_t *list, const uint32_t *count, bool write_ids, cudaStream_t st,
-                      bool fresh_order = false)
+                      stage_timer *tm, bool fresh_order = false)
 {
     const auto &T = tw.wl->tile;
     const bool bf = m->dtype == SLONN_BF16;
@@ -823,6 +825,7 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
         if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
         slonn_launch(tile_prep_kernel, dim3(P.groups, 2), 512, smem, st, P);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
+        if (P.cols == SLONN_WIDE_COLS) TIC_BY_INPUT_WIDE();
         rc = bf ? launch_tile_rows<true>(P, st) : launch_tile_rows<false>(P, st);
         if (rc) return rc;
     }
@@ -868,9 +871,9 @@ int launch_tile_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t 
     if (rc == SLONN_ERR_DIM) rc = launch_select(m, sp, n, max_rows, st);
     TOC();
     if (rc) return rc;
-    TIC(SLONN_STAGE_GROUP_ROWS, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp, 10000u);
+    TIC(SLONN_STAGE_GROUP_ROWS, gp.range_bp, gp.bp_lo, gp.bp_hi, skip_bp, SLONN_COLS_EVERY);
     rc = launch_tile_order(tw, b, n, lo, skip_bp != nullptr, sorted, st);
-    if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 1, nullptr, nullptr, false, st, true);
+    if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 1, nullptr, nullptr, false, st, tm, true);
     TOC();
     return rc;
 }
@@ -1203,7 +1206,7 @@ static int run_full_route(const slonn_model *m, const slonn_batch *b, uint32_t n
             gp.in = in; gp.n_act = m->n_act; gp.a = fp.a; gp.relu = fp.relu;
             if (ly.has_act) { gp.indptr = indptr; gp.ids = ids; gp.out_vals = vals; }
             gp.out_dense = fp.out_dense; gp.out_dense_ids = fp.out_dense_ids; gp.out_stride = fp.out_stride;
-            rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 2, list, count, ly.has_act != 0, st);
+            rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, 2, list, count, ly.has_act != 0, st, tm);
         } else {
             rc = launch_full_rows(m, fp, n, st);
         }
@@ -1491,10 +1494,10 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
             // compacted and taken four per block.
             bool rows_done = false;
             if (tw.ws && tile_plain_wanted(m, l, n, max_bp)) {
-                TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp, 10000u);
+                TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp, SLONN_COLS_EVERY);
                 rc = SLONN_OK;
                 if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp != nullptr, &sorted, st);
-                if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, keyed);
+                if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, tm, keyed);
                 TOC();
                 if (rc) return rc;
                 in.kind = SLONN_IN_DENSE; in.dense = gp.out_dense;

@@ -122,3 +122,13 @@ def test_grouped_products_are_named_and_counted_as_what_ran():
     assert acc.kernel_name(sh, rec("hash_select", 1, cols_bp=10000)) == "hash_select_cols_kernel"
     assert acc.kernel_name(sh, rec("group_rows", 0)) == "group_rows_kernel"
     assert acc.kernel_name(sh, rec("full_rows", 0)) == "full_rows_kernel"
+
+
+def test_the_product_kernels_are_timed_apart():
+    """One name as a kind of launch, two kernels in the per-kernel table."""
+    sh, bp = toy(), np.full(32, 5000)
+    narrow, wide = rec("group_rows", 1, cols_bp=10000, ms=1.0), rec("group_rows", 1, cols_bp=10001, ms=2.0)
+    assert acc.kernel_name(sh, wide) == acc.kernel_name(sh, narrow) == "tile_rows_kernel"
+    assert acc.launch_bytes(sh, wide, bp) == acc.launch_bytes(sh, narrow, bp)
+    k = acc.per_kernel(sh, [narrow, wide, rec("full_rows", 0, 10000, 10000, cols_bp=10001, ms=4.0)], bp)
+    assert k["tile_rows_kernel"]["ms"] == 1.0 and k["tile_rows_wide_kernel"]["ms"] == 6.0

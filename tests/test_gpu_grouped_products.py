@@ -246,3 +246,22 @@ def test_grouped_products_are_taken_where_they_pay(dtype, dims, has_act, n, budg
         assert "tile_rows_kernel" not in names, names
     _same_bits(b.results(), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
     dm.free()
+
+
+@pytest.mark.parametrize("dtype,dims,has_act,n,budgets,layer,kernel", [
+    ("bf16", [512, 640, 640, 96], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_kernel"),
+    ("bf16", [512, 640, 640, 256], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_wide_kernel"),        # every node, 8 columns per load
+    ("f32", [512, 640, 640, 256], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_wide_kernel"),
+    ("f32", [512, 640, 640, 1000], [1, 1, 0], 3000, (1000, 5000), 2, "tile_rows_wide_kernel"),        # four items a group, the last not full
+    ("bf16", [512, 640, 640, 505], [1, 1, 0], 3000, (1000, 5000), 2, "tile_rows_wide_kernel"),        # one column per load
+])
+def test_which_product_kernel_is_taken(dtype, dims, has_act, n, budgets, layer, kernel):
+    """The launch records tell the kernels with 128 and 256 columns per work item apart; same bits as the row kernels."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(4900 + n, dims, has_act, dtype, n=n, n_cal=300, K=4, L=2, budgets=budgets)
+    dm = harness.DeviceModel(wl)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
+    names = [acc.timed_kernel(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == layer]
+    assert names[-1] == kernel, names
+    _same_bits(b.results(), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()

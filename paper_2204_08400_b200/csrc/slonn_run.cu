@@ -15,7 +15,7 @@ namespace {
 
 // Optional per-launch timing: an event pair around every launch, with what the launch covers.
 struct stage_timer {
-    struct span { int stage; uint32_t layer, bp_lo, bp_hi, skips_full, cols_bp; cudaEvent_t a, b; };
+    struct span { int stage; uint32_t layer, bp_lo, bp_hi, skips_full, cols_bp; const uint32_t *work; uint32_t items[2]; cudaEvent_t a, b; };
     span spans[10 * SLONN_MAX_LAYERS];
     int n = 0;
     bool failed = false;
@@ -29,17 +29,24 @@ struct stage_timer {
         s.stage = stage; s.layer = layer;
         s.bp_lo = range_bp ? lo : 0u; s.bp_hi = range_bp ? std::min(hi, 10000u) : 10000u;
         s.skips_full = skip_bp ? 1u : 0u; s.cols_bp = cols_bp;
+        s.work = nullptr; s.items[0] = s.items[1] = 0;
         if (cudaEventCreate(&s.a) != cudaSuccess || cudaEventCreate(&s.b) != cudaSuccess) { failed = true; return; }
         cudaEventRecord(s.a, st);
         ++n;
     }
     void by_input() { if (n > 0 && !failed) spans[n - 1].cols_bp = SLONN_COLS_EVERY; } // the last launch read single weights of a transposed copy
-    void by_input_wide() { if (n > 0 && !failed) spans[n - 1].cols_bp = SLONN_COLS_EVERY_WIDE; } // and 256 columns of it at a time
-    void toc() { if (n > 0 && !failed) cudaEventRecord(spans[n - 1].b, st); }
+    void items_at(const uint32_t *work) { if (n > 0 && !failed) spans[n - 1].work = work; } // where the device counts its work items of 128 and 256 columns
+    void toc()
+    {
+        if (n <= 0 || failed) return;
+        span &s = spans[n - 1];
+        cudaEventRecord(s.b, st);
+        if (s.work && cudaMemcpyAsync(s.items, s.work, sizeof(s.items), cudaMemcpyDeviceToHost, st) != cudaSuccess) failed = true;
+    }
 };
 #define TIC(...) do { if (tm) tm->tic(__VA_ARGS__); } while (0)
 #define TIC_BY_INPUT() do { if (tm) tm->by_input(); } while (0)
-#define TIC_BY_INPUT_WIDE() do { if (tm) tm->by_input_wide(); } while (0)
+#define TIC_ITEMS(work) do { if (tm) tm->items_at(work); } while (0)
 #define TOC() do { if (tm) tm->toc(); } while (0)
 #define AT_LAYER(l) do { if (tm) tm->layer = (l); } while (0)
 
@@ -749,12 +756,16 @@ int launch_tile_rows_wide_t(const slonn_tile_params &P, cudaStream_t st)
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
+// The product kernel for the items' width, or, where tile_prep_kernel decides, both: one finds no items.
 template <bool BF16>
 int launch_tile_rows(const slonn_tile_params &P, cudaStream_t st)
 {
-    if (P.cols == SLONN_WIDE_COLS)
-        return !P.select && P.N % SLONN_WIDE_NN == 0 ? launch_tile_rows_wide_t<BF16, true>(P, st) : launch_tile_rows_wide_t<BF16, false>(P, st);
-    return !P.select && P.N % 4u == 0 ? launch_tile_rows_t<BF16, true>(P, st) : launch_tile_rows_t<BF16, false>(P, st);
+    int rc = SLONN_OK;
+    if (P.cols != SLONN_TILE_COLS)
+        rc = !P.select && P.N % SLONN_WIDE_NN == 0 ? launch_tile_rows_wide_t<BF16, true>(P, st) : launch_tile_rows_wide_t<BF16, false>(P, st);
+    if (!rc && P.cols != SLONN_WIDE_COLS)
+        rc = !P.select && P.N % 4u == 0 ? launch_tile_rows_t<BF16, true>(P, st) : launch_tile_rows_t<BF16, false>(P, st);
+    return rc;
 }
 
 // Sorts the batch's queries with a budget of at least lo (skip_full: but those at 10000 bp) into groups by (budget, keys); the
@@ -777,25 +788,24 @@ int launch_tile_order(const tile_ws &tw, const slonn_batch *b, uint32_t n, uint3
     return SLONN_OK;
 }
 
-// Columns of a work item.  Every node computed: the items are known, 148 are worked on at a time, and 256 columns take 1.8 times as
-// long as 128 (us with 128 and 256 columns, bf16: 4096 x 4096, 4096 queries, 3157 and 2763; 2048 x 2048, 777 queries, 392 items of
-// 256, 239 and 223; 300 queries, 152 items, 149 and 158; 4096 x 1000, 777 queries, 196 items, 213 and 247; fp32 1536 x 304, 2100
-// queries, 104 and 121, padding).  Selected nodes: a group's union holds at least `nodes` columns; from 1024 items of 256 on
-// (4096 x 4096, 4096 queries, 50 %: 2133 and 2060, 25 %: 993 and 980; 2100 queries, 50 %: 1151 and 1093, 25 %, 528 items: 475 and
-// 494; 2048 x 2048, 2100 queries, 50 %: 335 and 359; 777 queries, 50 % of 4096: 469 and 527).
-uint32_t tile_item_cols(uint32_t groups, bool select, uint32_t nodes)
+// Columns of a work item of P's layer for P's groups, all of which (exact) or some of which are served; 0: what is served decides.
+// nodes: most that a query of a group computes.
+uint32_t tile_item_cols(const slonn_tile_params &P, uint32_t nodes, bool exact)
 {
-    const uint64_t wide = (uint64_t)groups * ((nodes + SLONN_WIDE_COLS - 1) / SLONN_WIDE_COLS);
-    const uint64_t narrow = (uint64_t)groups * ((nodes + SLONN_TILE_COLS - 1) / SLONN_TILE_COLS);
-    const bool wider = select ? wide >= 1024u : (wide + 147) / 148 * 9 <= (narrow + 147) / 148 * 5;
-    return wider ? SLONN_WIDE_COLS : SLONN_TILE_COLS;
+    const uint32_t most = P.groups * ((nodes + SLONN_WIDE_COLS - 1) / SLONN_WIDE_COLS);
+    const bool even = P.in.kind != SLONN_IN_LIST || P.count;
+    if (exact && !P.select) return tile_wide(P.groups, P.D, P.N, P.V, false, 0, even) ? SLONN_WIDE_COLS : SLONN_TILE_COLS;
+    // no part of the groups takes 256 columns: too few nodes, or, every node computed, one round of 128 columns
+    const bool none = !tile_wide_layer(P.D, P.N, P.V, P.select) || (P.select ? !tile_wide(P.groups, P.D, P.N, P.V, true, most, even) : most <= 74u);
+    return none ? SLONN_TILE_COLS : 0u;
 }
 
 // One layer for the whole batch.  order_kind: 0 queries as they come (without those of skip_bp), 1 the order of
-// launch_tile_order, 2 the compacted list `list` of *count queries.  fresh_order: launch_tile_order was the launch before.
+// launch_tile_order, 2 the compacted list `list` of *count queries.  fresh_order: launch_tile_order was the launch before.  all_queries:
+// every query of the batch is served.
 int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, const slonn_gather_params &G, uint32_t n, uint32_t max_bp,
                       const tile_ws &tw, int order_kind, const uint32_t *list, const uint32_t *count, bool write_ids, cudaStream_t st,
-                      stage_timer *tm, bool fresh_order = false)
+                      stage_timer *tm, bool fresh_order = false, bool all_queries = false)
 {
     const auto &T = tw.wl->tile;
     const bool bf = m->dtype == SLONN_BF16;
@@ -807,7 +817,7 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
     P.select = G.use_list; P.n_act = G.n_act; P.a = G.a; P.indptr = G.indptr; P.ids = const_cast<uint32_t *>(G.ids); P.write_ids = write_ids ? 1u : 0u;
     P.out_vals = G.out_vals; P.out_dense = G.out_dense; P.out_dense_ids = G.out_dense_ids; P.out_stride = G.out_stride;
     P.nwords = (ly.N + 31u) / 32u;
-    P.work = (uint32_t *)(tw.ws + T.work); P.items = (uint32_t *)(tw.ws + T.items);
+    P.items = (uint32_t *)(tw.ws + T.items);
     P.kseg = (uint32_t *)(tw.ws + T.kseg); P.krow = (uint32_t *)(tw.ws + T.krow); P.xt = (float *)(tw.ws + T.xt);
     P.ucol = (uint2 *)(tw.ws + T.ucol); P.ucount = (uint32_t *)(tw.ws + T.ucount);
     P.bm = (uint32_t *)(tw.ws + T.bm); P.pre = (uint32_t *)(tw.ws + T.pre);
@@ -820,12 +830,13 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
         else if (order_kind == 1) P.order = (const uint32_t *)(tw.ws + T.order) + (uint64_t)c * T.order_stride;
         else { P.order = list + q0; P.count = count; }
         P.groups = (P.n + SLONN_TILE_G - 1) / SLONN_TILE_G;
-        P.cols = tile_item_cols(P.groups, P.select != 0, P.select ? slonn_layer_nodes(max_bp, ly.N, slonn_model_pre(m)) : ly.N);
-        // the sort cleared the count of work items; only the first chunk can rely on it
-        if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
+        P.cols = tile_item_cols(P, P.select ? slonn_layer_nodes(max_bp, ly.N, slonn_model_pre(m)) : ly.N, all_queries);
+        P.work = (uint32_t *)(tw.ws + T.work) + (c ? 2 : 0); // the first chunk's counts stay until the layer is done (items_at)
+        // the sort cleared the counts of work items; only the first chunk can rely on it
+        if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 8, st) != cudaSuccess) return SLONN_ERR_CUDA;
         slonn_launch(tile_prep_kernel, dim3(P.groups, 2), 512, smem, st, P);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
-        if (P.cols == SLONN_WIDE_COLS) TIC_BY_INPUT_WIDE();
+        if (c == 0) TIC_ITEMS(P.work);
         rc = bf ? launch_tile_rows<true>(P, st) : launch_tile_rows<false>(P, st);
         if (rc) return rc;
     }
@@ -1497,7 +1508,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                 TIC(SLONN_STAGE_GROUP_ROWS, nullptr, 0u, 0xffffu, skip_bp, SLONN_COLS_EVERY);
                 rc = SLONN_OK;
                 if (keyed) rc = launch_tile_order(tw, b, n, 0u, skip_bp != nullptr, &sorted, st);
-                if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, tm, keyed);
+                if (!rc) rc = launch_tile_layer(m, ly, l, gp, n, max_bp, tw, keyed ? 1 : 0, nullptr, nullptr, false, st, tm, keyed, !skip_bp);
                 TOC();
                 if (rc) return rc;
                 in.kind = SLONN_IN_DENSE; in.dense = gp.out_dense;
@@ -1566,6 +1577,7 @@ static int run_with_timer(const slonn_model *m, const slonn_batch *b, void *work
         float ms = 0.0f;
         if (rc == SLONN_OK && !tm.failed && cudaEventElapsedTime(&ms, tm.spans[i].a, tm.spans[i].b) != cudaSuccess) rc = SLONN_ERR_CUDA;
         span_ms[i] = ms;
+        if (rc == SLONN_OK && tm.spans[i].items[1]) tm.spans[i].cols_bp = SLONN_COLS_EVERY_WIDE;
         cudaEventDestroy(tm.spans[i].a);
         cudaEventDestroy(tm.spans[i].b);
     }

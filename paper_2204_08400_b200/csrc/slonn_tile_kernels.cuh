@@ -44,7 +44,7 @@ struct slonn_order_params {
     uint32_t skip_full;      // 1: and those at exactly 10000 bp
     uint32_t q0, n;          // queries [q0, q0 + n), n <= SLONN_TILE_CHUNK
     uint32_t *order;         // out: the first entries; the rest keep the 0xffffffff (no query) they were set to
-    uint32_t *work;          // cleared for the tile_prep_kernel that follows
+    uint32_t *work;          // [2] cleared for the tile_prep_kernel that follows
 };
 
 // Rank by counting: a query's place is the number of smaller keys of its chunk.  n^2 compares (17 M for 4096
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256) tile_order_kernel(slonn_order_params P)
     const uint32_t e0 = (blockIdx.x * 8u + warp) * 4u;
     uint64_t mine[4];
     uint32_t rank[4] = {0u, 0u, 0u, 0u};
-    if (blockIdx.x == 0 && threadIdx.x == 0) *P.work = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 2u) P.work[threadIdx.x] = 0u;
     // ~0: left out.  The key of a query that is left out may never have been written; it is loaded beside the budget all the
     // same, so that neither load waits for the other.
     auto key_of = [&](uint32_t e) -> uint64_t {
@@ -125,8 +125,8 @@ struct slonn_tile_params {
     // scratch
     uint32_t groups;
     uint32_t nwords;          // (N + 31) / 32
-    uint32_t cols;            // columns of a work item: SLONN_TILE_COLS or SLONN_WIDE_COLS
-    uint32_t *work;           // number of work items
+    uint32_t cols;            // columns of a work item: SLONN_TILE_COLS or SLONN_WIDE_COLS, or 0: tile_prep_kernel decides
+    uint32_t *work;           // [2] number of work items of SLONN_TILE_COLS and of SLONN_WIDE_COLS columns; one of them stays 0
     uint32_t *items;          // group << 16 | tile (groups <= 1024 * 8, tiles <= N / 128)
     uint32_t *kseg;           // [groups][33] first entry of each partial sum's stretch, total
     uint32_t *krow;           // [groups][kcap] byte offset of the entry's row of WT
@@ -145,6 +145,34 @@ __device__ __forceinline__ uint32_t tile_query(const slonn_tile_params &P, uint3
     return P.skip_bp && P.skip_bp[q] == 10000u ? 0xffffffffu : q;
 }
 
+// Whether work items of a layer take 256 columns, for `groups` groups that have queries; `listed`: items of 256 columns that the first
+// queries of these groups alone fill (selected nodes; a group's union holds at least those).  Nowhere if the layer has more than
+// 40 MiB of weights (fp32 4096 x 4096, 128 and 256 columns, every node, 1300 queries 1213 and 1280 us, 656 queries 744 and 861; 90 %
+// of the nodes, 4000 queries, 3570 and 3813).
+// Every node computed (only where one load brings a lane's eight columns; 2048 x 500, 1000 queries, 91 and 101): 148 items are worked on
+// at a time, and 256 columns take 1.8 times as long as 128.  bf16 1536 x 1536, 13 groups 60 and 54, 49 groups 110 and 95, 82
+// groups (4 and 7 rounds) 177 and 171; 4096 x 4096, 256 groups, 3157 and 2763.  With more than 10 MiB the first of them start later:
+// 4096 x 4096, 7 groups (1 and 2 rounds) 142 and 155, 16 groups 249 and 245, 41 groups (5 and 9) 515 either way; fp32 4096 x 2048, 29
+// groups (2 and 4) 261 and 269, 49 groups 370 and 366.  even: the groups' inputs are about equally many.  Behind lists of mixed budgets
+// the last items are the longest, and all but a few SMs wait for them: 4096 x 1000, one query in 100 at 35 %, the others at 5 %, 1024
+// queries 90 and 106, 2100 queries (4 and 8 rounds) 118 and 140, 4096 queries (7 and 14) 180 and 181 (all at 5 %: 145 and 129).
+// Selected nodes: from 2048 items on.  bf16 4096 x 2048, 40 %, 1000 items 946 and 1009, 1628 items 1446 and 1440, 50 %, 1252 items
+// 1420 and 1460, 90 %, 2504 items 2210 and 2134; 4096 x 4096, 75 %, 1200 items 1281 and 1349, 3000 items 2910 and 2783; fp32 3072 x 3072,
+// 40 %, 2035 items 1496 and 1400.
+__host__ __device__ __forceinline__ bool tile_wide_layer(uint32_t D, uint32_t N, uint32_t V, bool select)
+{
+    return (uint64_t)D * N * (16u / V) <= (40ull << 20) && (select || N % SLONN_WIDE_NN == 0u);
+}
+__host__ __device__ __forceinline__ bool tile_wide(uint32_t groups, uint32_t D, uint32_t N, uint32_t V, bool select, uint32_t listed, bool even)
+{
+    if (!tile_wide_layer(D, N, V, select)) return false;
+    if (select) return listed >= 2048u;
+    const uint32_t wide = (groups * ((N + SLONN_WIDE_COLS - 1) / SLONN_WIDE_COLS) + 147u) / 148u; // rounds
+    const uint32_t narrow = (groups * ((N + SLONN_TILE_COLS - 1) / SLONN_TILE_COLS) + 147u) / 148u;
+    const uint32_t start = (uint64_t)D * N * (16u / V) <= (10ull << 20) ? 0u : V == 8u ? 2u : 3u;
+    return wide * 9u + start <= narrow * 5u && (even || wide >= 7u);
+}
+
 // Two blocks per group that share nothing: block (g, 0) lists the inputs and stages their values, block (g, 1) lists the
 // nodes and adds the group's work items.  One warp per query; a warp's list reads are issued eight at a time.
 __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
@@ -158,6 +186,7 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
     __shared__ uint64_t s_begin[G];
     __shared__ uint32_t s_len[G];
     __shared__ uint32_t wsum[16];
+    __shared__ uint2 wcount[16]; // per warp: groups that have queries, items their first queries fill
     const uint32_t g = blockIdx.x;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5; // warp: the query this warp reads the list of
     const bool nodes = blockIdx.y != 0u;
@@ -186,6 +215,22 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
         uint32_t ncols = P.N;
         if (P.select) for (uint32_t i = tid; i < (G + 1u) * P.nwords; i += blockDim.x) nbits[i] = 0u;
         if (!__syncthreads_or(any)) return;
+        // Which queries a launch serves only the device knows (those of a budget range, of a list): the width of the work items is
+        // decided here, by every group alike, from one query of each group (a thread's; at most 512 groups).
+        if (P.cols == 0u) {
+            uint32_t q = 0xffffffffu;
+            if (tid < P.groups) // with an order a group's queries come first
+                for (uint32_t k = 0; k < (P.order ? 1u : (uint32_t)G) && q == 0xffffffffu; ++k) q = tid * G + k < P.n ? tile_query(P, tid * G + k) : 0xffffffffu;
+            uint32_t items = 0;
+            if (P.select && q != 0xffffffffu) {
+                const uint64_t *ip = P.indptr + (uint64_t)q * P.n_act + P.a;
+                items = ((uint32_t)(ip[1] - ip[0]) + SLONN_WIDE_COLS - 1) / SLONN_WIDE_COLS;
+            }
+            const uint32_t have = __popc(__ballot_sync(SLONN_FULL_MASK, q != 0xffffffffu));
+            items = __reduce_add_sync(SLONN_FULL_MASK, items);
+            if (lane == 0) wcount[warp] = make_uint2(have, items); // read behind the next barrier
+            if (!P.select) __syncthreads();
+        }
         if (P.select) {
             const uint32_t *ids = P.ids + s_begin[warp];
             const uint32_t len = s_len[warp];
@@ -255,11 +300,18 @@ __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)
             ncols = all;
         }
         if (tid < 32u) {
-            const uint32_t tiles = (ncols + P.cols - 1) / P.cols;
+            bool wide = P.cols == SLONN_WIDE_COLS;
+            if (P.cols == 0u) {
+                const uint2 c = tid < 16u ? wcount[tid] : make_uint2(0u, 0u);
+                const uint32_t have = __reduce_add_sync(SLONN_FULL_MASK, c.x), items = __reduce_add_sync(SLONN_FULL_MASK, c.y);
+                wide = tile_wide(have, P.D, P.N, P.V, P.select != 0u, items, P.in.kind != SLONN_IN_LIST || P.count);
+            }
+            const uint32_t cols = wide ? SLONN_WIDE_COLS : SLONN_TILE_COLS;
+            const uint32_t tiles = (ncols + cols - 1) / cols;
             uint32_t base = 0;
             if (tid == 0) {
                 P.ucount[g] = ncols;
-                base = atomicAdd(P.work, tiles);
+                base = atomicAdd(P.work + (wide ? 1 : 0), tiles);
             }
             base = __shfl_sync(SLONN_FULL_MASK, base, 0);
             for (uint32_t t = tid; t < tiles; t += 32u) P.items[base + t] = (g << 16) | t;
@@ -784,7 +836,7 @@ __global__ void __launch_bounds__(SLONN_WIDE_WARPS * 32, 1) tile_rows_wide_kerne
     __shared__ uint64_t s_off[2][G];
     __shared__ uint32_t s_q[2][G];
     __shared__ uint32_t s_tmem;
-    const uint32_t n_items = P.work[0];
+    const uint32_t n_items = P.work[1];
     uint32_t it = blockIdx.x;
     if (it >= n_items) return;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;

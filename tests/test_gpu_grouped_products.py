@@ -249,11 +249,19 @@ def test_grouped_products_are_taken_where_they_pay(dtype, dims, has_act, n, budg
 
 
 @pytest.mark.parametrize("dtype,dims,has_act,n,budgets,layer,kernel", [
-    ("bf16", [512, 640, 640, 96], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_kernel"),
-    ("bf16", [512, 640, 640, 256], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_wide_kernel"),        # every node, 8 columns per load
-    ("f32", [512, 640, 640, 256], [1, 1, 0], 2100, (1000, 5000), 2, "tile_rows_wide_kernel"),
-    ("f32", [512, 640, 640, 1000], [1, 1, 0], 3000, (1000, 5000), 2, "tile_rows_wide_kernel"),        # four items a group, the last not full
-    ("bf16", [512, 640, 640, 505], [1, 1, 0], 3000, (1000, 5000), 2, "tile_rows_wide_kernel"),        # one column per load
+    ("bf16", [640, 96, 24], [0, 1], 2100, (1000, 5000), 0, "tile_rows_kernel"),
+    ("bf16", [640, 256, 24], [0, 1], 2100, (1000, 5000), 0, "tile_rows_wide_kernel"),      # every node, eight columns per load
+    ("f32", [640, 256, 24], [0, 1], 2100, (1000, 5000), 0, "tile_rows_wide_kernel"),
+    ("f32", [640, 252, 24], [0, 1], 2100, (1000, 5000), 0, "tile_rows_kernel"),            # a load of four columns, but not of eight
+    ("f32", [40, 1000, 24], [0, 1], 3000, (1000, 5000), 0, "tile_rows_wide_kernel"),       # four items a group, the last not full; stretches without inputs
+    ("bf16", [2512, 2080, 24], [0, 1], 1150, (5000,), 0, "tile_rows_wide_kernel"),         # 5 and 9 rounds of items, 9.97 MiB
+    ("bf16", [2560, 2080, 24], [0, 1], 1150, (5000,), 0, "tile_rows_kernel"),              # 10.2 MiB
+    ("f32", [2512, 1040, 24], [0, 1], 880, (5000,), 0, "tile_rows_wide_kernel"),           # 2 and 4
+    ("f32", [2560, 1040, 24], [0, 1], 880, (5000,), 0, "tile_rows_kernel"),
+    ("f32", [2560, 1040, 24], [0, 1], 1408, (5000,), 0, "tile_rows_wide_kernel"),          # 3 and 6
+    ("f32", [2560, 4104, 24], [0, 1], 1408, (5000,), 0, "tile_rows_kernel"),               # 40.1 MiB
+    ("bf16", [64, 512, 504], [1, 0], 8192, (1000, 5000), 1, "tile_rows_wide_kernel"),      # behind lists: 7 rounds,
+    ("bf16", [64, 512, 504], [1, 0], 7000, (1000, 5000), 1, "tile_rows_kernel"),           # 6
 ])
 def test_which_product_kernel_is_taken(dtype, dims, has_act, n, budgets, layer, kernel):
     """The launch records tell the kernels with 128 and 256 columns per work item apart; same bits as the row kernels."""
@@ -263,5 +271,32 @@ def test_which_product_kernel_is_taken(dtype, dims, has_act, n, budgets, layer, 
     b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
     names = [acc.timed_kernel(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == layer]
     assert names[-1] == kernel, names
+    _same_bits(b.results(), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()
+
+
+@pytest.mark.parametrize("dtype,dims,has_act,n,budgets,layer,lo,kernel", [
+    ("bf16", [512, 1240, 520, 120], [1, 1, 0], 3500, (10000,), 0, 10000, "tile_rows_wide_kernel"),  # ids written, a last load clamped
+    ("f32", [512, 1240, 520, 120], [1, 1, 0], 3500, (10000,), 0, 10000, "tile_rows_wide_kernel"),
+    ("bf16", [512, 1240, 512, 120], [1, 1, 0], 3500, (10000,), 1, 10000, "tile_rows_wide_kernel"),           # complete lists
+    ("bf16", [512, 1240, 505], [1, 0], 3500, (10000,), 1, 10000, "tile_rows_kernel"),                        # one column per load
+    ("bf16", [512, 1240, 520, 120], [1, 1, 0], 3500, (700,) * 19 + (10000,), 0, 10000, "tile_rows_kernel"),  # a dozen groups of 219
+    # selected nodes: 2304 items and (a second chunk, of few groups) 1950; one column more than four items hold
+    ("bf16", [64, 520, 1032, 24], [1, 1, 0], 8192, (9000, 9999), 1, 3501, "tile_rows_wide_kernel"),
+    ("f32", [64, 516, 1032, 24], [1, 1, 0], 8192 + 800, (9000, 9999), 1, 3501, "tile_rows_wide_kernel"),
+    ("bf16", [64, 72, 1028], [1, 1], 8192, (9000, 9999), 1, 3501, "tile_rows_wide_kernel"),   # partial sums without an input
+    ("bf16", [64, 520, 1032, 24], [1, 1, 0], 8192, (500,) * 15 + (9999,), 1, 3501, "tile_rows_kernel"),
+    ("bf16", [64, 520, 1032, 24], [1, 1, 0], 7000, (9000,), 1, 3501, "tile_rows_kernel"),            # 1752
+])
+def test_item_width_follows_the_queries_that_are_served(dtype, dims, has_act, n, budgets, layer, lo, kernel):
+    """A few queries of a large batch leave few work items: the kernel whose items are shorter; same bits as the row kernels."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(5000 + n, dims, has_act, dtype, n=n, n_cal=300, K=4, L=2, budgets=budgets)
+    dm = harness.DeviceModel(wl)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
+    sh = acc.NetShape.of(wl)
+    names = [acc.timed_kernel(sh, r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes)
+             if r["layer"] == layer and r["bp_lo"] == lo and acc.grouped_products(r)]
+    assert names == [kernel], names
     _same_bits(b.results(), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
     dm.free()

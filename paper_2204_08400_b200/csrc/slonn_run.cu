@@ -324,34 +324,14 @@ int launch_gather_short_t(const slonn_gather_params &P, uint64_t grid, size_t sm
     return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
-template <bool BF16>
-int launch_gather_short_group_t(const slonn_gather_params &P, uint32_t n, uint32_t ranges, cudaStream_t st)
-{
-    slonn_launch(gather_short_group_kernel<BF16>, (n + SLONN_SHORT_GROUP - 1) / SLONN_SHORT_GROUP * ranges, SLONN_SHORT_GROUP * 32, 0, st, P, n, ranges);
-    return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
-}
-
-// Rows of one 512-byte round: 32 queries of a block walk the same ranges of ids when the layer does not fit L1 and the batch
-// selects many rows (us with a query per block and so, 256 queries: fp32 200,000 x 128, 5 % 109 and 97, 10 % 203 and 183; bf16 100,000 x
-// 256, 10 % 138 and 121; fp32 30,000 x 64 (8 MB), 10 % 29 and 27; 64 queries, 200,000 x 128, 5 % 35 and 31, 1 % 13 and 15).
-#define SLONN_SHORT_GROUP_MIN 64u
-#define SLONN_SHORT_GROUP_BYTES (7ull << 20)
-#define SLONN_SHORT_GROUP_ROWS (148ull * 2048)
-
 #ifndef SLONN_GATHER_R
 #define SLONN_GATHER_R 4 // rows per warp pass of the row kernel for rows longer than one 512-byte round (4 or 8)
 #endif
-int launch_gather(const slonn_model *m, slonn_gather_params &P, const slonn_batch *b, uint32_t n, uint32_t max_rows, cudaStream_t st)
+int launch_gather(const slonn_model *m, slonn_gather_params &P, uint32_t n, uint32_t max_rows, cudaStream_t st)
 {
     // so few rows that the GPU cannot be filled: latency variant, 4 warps per block, one row per warp
     const bool lat = (uint64_t)n * max_rows <= 148ull * 64;
     const bool short_rows = P.nchunks <= 32; // a row is one 512-byte round: 8 rows per warp pass
-    const uint32_t groups = (n + SLONN_SHORT_GROUP - 1) / SLONN_SHORT_GROUP;
-    if (short_rows && P.use_list && P.in.kind == SLONN_IN_DENSE && n >= SLONN_SHORT_GROUP_MIN && groups <= 148u &&
-        (uint64_t)n * max_rows >= SLONN_SHORT_GROUP_ROWS && (uint64_t)P.N * P.nchunks * 16u >= SLONN_SHORT_GROUP_BYTES && !(b->flags & SLONN_FLAG_UNGROUPED_ROWS)) {
-        const uint32_t ranges = std::max(1u, 148u / groups);
-        return m->dtype == SLONN_BF16 ? launch_gather_short_group_t<true>(P, n, ranges, st) : launch_gather_short_group_t<false>(P, n, ranges, st);
-    }
     uint32_t threads = SLONN_THREADS;
     if (lat) {
         threads = 128;
@@ -428,7 +408,7 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
     int rc;
     if (!grouped) {
         TIC(SLONN_STAGE_GATHER_DOT, P.range_bp, P.bp_lo, P.bp_hi, P.skip_bp);
-        rc = launch_gather(m, P, b, n, max_rows, st);
+        rc = launch_gather(m, P, n, max_rows, st);
         TOC();
         return rc;
     }
@@ -436,7 +416,7 @@ int launch_rows(const slonn_model *m, slonn_gather_params &P, const slonn_batch 
         slonn_gather_params A = P;
         A.range_bp = b->budget_bp; A.bp_lo = lo; A.bp_hi = split - 1u;
         TIC(SLONN_STAGE_GATHER_DOT, A.range_bp, A.bp_lo, A.bp_hi, A.skip_bp);
-        rc = launch_gather(m, A, b, n, std::min(max_rows, slonn_layer_nodes(split - 1u, P.N, slonn_model_pre(m))), st);
+        rc = launch_gather(m, A, n, std::min(max_rows, slonn_layer_nodes(split - 1u, P.N, slonn_model_pre(m))), st);
         TOC();
         if (rc) return rc;
     }
@@ -1134,7 +1114,7 @@ int slonn_forward_all_rows(const slonn_model *m, uint32_t l, const float *in_den
     gp.W = ly.W; gp.bias = ly.bias; gp.D = ly.D; gp.N = ly.N;
     gp.nchunks = nchunks;
     gp.use_list = 0; gp.out_dense = out; gp.out_stride = ly.N; gp.relu = relu;
-    return launch_gather(m, gp, nullptr, n, ly.N, st); // every row: no list, no flags read
+    return launch_gather(m, gp, n, ly.N, st);
 }
 
 // Complete layer 0 for n CSR rows -> out [n][N_0].

@@ -874,82 +874,6 @@ __global__ void __launch_bounds__(SLONN_THREADS, 2) gather_short_kernel(slonn_ga
     }
 }
 
-// First position of the ascending list ids[0, B) that holds `key` or more, by one warp: 32 probes at a time.
-__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t *ids, uint32_t B, uint32_t key, uint32_t lane)
-{
-    uint32_t lo = 0, hi = B; // the answer lies in [lo, hi]
-    while (lo < hi) {
-        const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
-        const uint32_t c = __popc(__ballot_sync(SLONN_FULL_MASK, at < hi && ids[at] < key));
-        hi = min(hi, lo + c * step);
-        if (c) lo += (c - 1u) * step + 1u;
-    }
-    return lo;
-}
-
-// gather_short_kernel for batches whose queries select largely the same rows of a layer too large for L1: a warp per query, 32
-// queries per block, and every warp of the block walks its query's rows of the same range of ids, so that a row several of them
-// selected comes from L2 once.  What bounds gather_short_kernel at such sizes is L2 (200,000 fp32 rows of 512 bytes, 256
-// queries at 5 %: 1.31 GB); here it is L1's 128 bytes a cycle and the issue of about a dozen instructions a row.
-#define SLONN_SHORT_GROUP 32
-template <bool BF16>
-__global__ void __launch_bounds__(SLONN_SHORT_GROUP * 32, 1) gather_short_group_kernel(slonn_gather_params P, uint32_t n, uint32_t ranges)
-{
-    slonn_enter();
-    constexpr int VPC = BF16 ? 8 : 4;
-    constexpr int R = 8;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t g = blockIdx.x / ranges, range = blockIdx.x - g * ranges;
-    const uint32_t q = g * SLONN_SHORT_GROUP + warp;
-    if (q >= n) return;
-    if (P.skip_bp && P.skip_bp[q] == 10000u) return;
-    if (!bp_in_range(P.range_bp, P.bp_lo, P.bp_hi, q)) return;
-    const uint64_t off = P.indptr[(uint64_t)q * P.n_act + P.a];
-    const uint32_t B = (uint32_t)(P.indptr[(uint64_t)q * P.n_act + P.a + 1] - off);
-    const bool has_chunk = lane < P.nchunks;
-    float x[VPC];
-#pragma unroll
-    for (int e = 0; e < VPC; e += 4) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (has_chunk) v = reinterpret_cast<const float4 *>(P.in.dense + (uint64_t)q * P.D)[(lane * VPC + e) / 4];
-        x[e] = v.x; x[e + 1] = v.y; x[e + 2] = v.z; x[e + 3] = v.w;
-    }
-    const uint32_t r0 = range == 0u ? 0u : warp_lower_bound(P.ids + off, B, (uint32_t)((uint64_t)P.N * range / ranges), lane);
-    const uint32_t r1 = range + 1u == ranges ? B : warp_lower_bound(P.ids + off, B, (uint32_t)((uint64_t)P.N * (range + 1u) / ranges), lane);
-    const uint4 *Wl = reinterpret_cast<const uint4 *>(P.W) + lane;
-    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t base = r0; base < r1; base += 32u) {
-        const uint32_t myid = P.ids[off + min(base + lane, r1 - 1u)];
-#pragma unroll
-        for (uint32_t sub = 0; sub < 4; ++sub) {
-            const uint32_t r = base + sub * R;
-            if (r >= r1) break; // uniform
-            uint4 w[R];
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const uint32_t nd = __shfl_sync(SLONN_FULL_MASK, myid, sub * R + k); // rows past r1 repeat the last id
-                w[k] = has_chunk ? __ldg(Wl + (uint64_t)nd * P.nchunks) : zero4;
-            }
-            float acc[R];
-#pragma unroll
-            for (int k = 0; k < R; ++k) acc[k] = 0.0f;
-            chunk_fma<BF16, R, 0, VPC>::run(w, x, acc);
-            const float sum = reduce_rows8(acc, lane); // row r + (lane >> 2)
-            const uint32_t mr = r + (lane >> 2);
-            const uint32_t nd = __shfl_sync(SLONN_FULL_MASK, myid, sub * R + (lane >> 2));
-            if ((lane & 3u) == 0u && mr < r1) {
-                float z = sum + __ldg(P.bias + nd);
-                if (P.relu) z = z > 0.0f ? z : 0.0f;
-                if (P.out_vals) P.out_vals[off + mr] = z;
-                if (P.out_dense) {
-                    P.out_dense[(uint64_t)q * P.out_stride + mr] = z;
-                    if (P.out_dense_ids) P.out_dense_ids[(uint64_t)q * P.out_stride + mr] = nd;
-                }
-            }
-        }
-    }
-}
-
 // Second half of the input-stationary layer, shared by gather_cols_kernel and layer_cols_kernel: puts the
 // query's selected nodes in column order and evaluates nodes [r0, r1) of that order against the staged
 // input list S.  `order_mem` is block scratch of P.scratch_bytes (the inputs' bitmap, dead by now).

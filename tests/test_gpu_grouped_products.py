@@ -98,21 +98,6 @@ def test_plain_layers_of_few_queries_take_columns_where_they_pay(dtype, n, last,
     dm.free()
 
 
-@pytest.mark.parametrize("dtype,dims,n,budgets", [
-    ("f32", [64, 30000, 24], 100, (1000, 3001, 5000)),   # a last group of four queries
-    ("bf16", [72, 52000, 24], 64, (1, 7, 2000)),         # lists of a few entries: ranges of ids without any
-    ("bf16", [128, 70000, 24], 97, (300, 5000)),         # 32-bit list entries
-    ("f32", [128, 15000, 24], 1000, (500, 9999, 10000)),
-])
-def test_short_rows_of_32_queries_by_id_range(dtype, dims, n, budgets):
-    """Rows of one 512-byte round of a layer that does not fit L1, 32 queries per block."""
-    from paper_2204_08400_b200 import binding as sl, harness
-    wl = custom_workload(4800 + n, dims, [1, 0], dtype, n=n, n_cal=64, K=3, L=2, budgets=budgets)
-    dm = harness.DeviceModel(wl)
-    _same_bits(_run(dm, wl), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
-    dm.free()
-
-
 def test_grouped_products_need_their_scratch_and_do_without_it():
     """A workspace of the size the other kernels need is still taken, with the same results."""
     from paper_2204_08400_b200 import binding as sl, harness

@@ -1,4 +1,4 @@
-"""Layers evaluated as grouped products (16 queries x 128 columns per work item): sizes at the edges of a tile, a group, a
+"""Layers evaluated as grouped products (16 queries x 128 or 256 columns per work item): sizes at the edges of a tile, a group, a
 partial sum's stretch and a staged chunk, against the oracle or bit for bit against the row kernels (whose own parity the
 other tests cover; the order of every sum is fixed, so the two have to agree in every bit)."""
 import numpy as np
@@ -54,8 +54,9 @@ def test_grouped_products_in_several_chunks():
     ("bf16", [1032, 520, 528, 24], [1, 1, 0], 8209, (4850, 4880, 9999)),  # selected nodes, up to one more than an item holds
     ("f32", [132, 516, 260, 24], [1, 1, 0], 8192, (9000, 9900)),
 ])
-def test_items_of_256_columns(dtype, dims, has_act, n, budgets):
-    """Enough work items for the kernel with eight columns per lane; partial sums without an input and odd widths among them."""
+def test_layers_of_up_to_256_columns_and_more(dtype, dims, has_act, n, budgets):
+    """Around the 256 columns of the longer work items, whichever kernel takes them; partial sums without an input and odd widths among
+    them.  (test_which_product_kernel_is_taken and test_item_width_follows_the_queries_that_are_served ask for the kernel too.)"""
     from paper_2204_08400_b200 import binding as sl, harness
     wl = custom_workload(4300 + n, dims, has_act, dtype, n=n, n_cal=300, K=4, L=2, budgets=budgets)
     dm = harness.DeviceModel(wl)
@@ -65,8 +66,8 @@ def test_items_of_256_columns(dtype, dims, has_act, n, budgets):
 
 @pytest.mark.parametrize("dtype,n,last", [("bf16", 40, 505), ("f32", 33, 576), ("bf16", 200, 500), ("f32", 255, 641), ("bf16", 64, 296)])
 def test_plain_layers_of_few_queries_by_input(dtype, n, last):
-    """A layer without activator behind a list of 2048 inputs, one block per (query, 64 nodes): odd widths, a last block that is
-    not full, more blocks than one per query and pass of its warps."""
+    """A layer without activator behind a list of 2048 inputs: odd widths, a last block that is not full.  (The form is asked for in
+    test_plain_layers_of_few_queries_take_columns_where_they_pay.)"""
     from paper_2204_08400_b200 import binding as sl, harness
     wl = custom_workload(4700 + n, [64, 2048, last], [1, 0], dtype, n=n, n_cal=200, K=4, L=2, budgets=(20, 2000, 3500))
     dm = harness.DeviceModel(wl)
@@ -265,6 +266,7 @@ def test_which_product_kernel_is_taken(dtype, dims, has_act, n, budgets, layer, 
     ("f32", [512, 1240, 520, 120], [1, 1, 0], 3500, (10000,), 0, 10000, "tile_rows_wide_kernel"),
     ("bf16", [512, 1240, 512, 120], [1, 1, 0], 3500, (10000,), 1, 10000, "tile_rows_wide_kernel"),           # complete lists
     ("bf16", [512, 1240, 505], [1, 0], 3500, (10000,), 1, 10000, "tile_rows_kernel"),                        # one column per load
+    ("bf16", [512, 1240, 520, 120], [1, 1, 0], 3500, (700, 10000), 0, 10000, "tile_rows_wide_kernel"),       # about half of the groups
     ("bf16", [512, 1240, 520, 120], [1, 1, 0], 3500, (700,) * 19 + (10000,), 0, 10000, "tile_rows_kernel"),  # a dozen groups of 219
     # selected nodes: 2304 items and (a second chunk, of few groups) 1950; one column more than four items hold
     ("bf16", [64, 520, 1032, 24], [1, 1, 0], 8192, (9000, 9999), 1, 3501, "tile_rows_wide_kernel"),

@@ -377,7 +377,7 @@ __device__ __forceinline__ void stage_input(const slonn_input &in, uint32_t q, u
 
 // Lets `kernel` be launched with `bytes` of dynamic shared memory on the current device.  The 48 KB a launch gets
 // without opting in and the 227 KB a block can have both count the kernel's static shared memory (at most 1120
-// bytes where the dynamic size varies; tile_rows_kernel has more and checks its own sum): the opt-in starts at 46 KB
+// bytes where the dynamic size varies; the two product kernels have more and check their own sums): the opt-in starts at 46 KB
 // and ends at 225 KB (SLONN_ERR_DIM above).  The limit of a
 // kernel is only ever raised, so that two host threads launching the same kernel with different sizes cannot
 // take each other's allowance away between the opt-in and the launch.

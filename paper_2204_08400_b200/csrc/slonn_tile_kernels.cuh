@@ -173,6 +173,7 @@ __host__ __device__ __forceinline__ bool tile_wide(uint32_t groups, uint32_t D, 
     return wide * 9u + start <= narrow * 5u && (even || wide >= 7u);
 }
 
+static_assert(SLONN_TILE_CHUNK / SLONN_TILE_G <= 512, "a thread of tile_prep_kernel per group");
 // Two blocks per group that share nothing: block (g, 0) lists the inputs and stages their values, block (g, 1) lists the
 // nodes and adds the group's work items.  One warp per query; a warp's list reads are issued eight at a time.
 __global__ void __launch_bounds__(512) tile_prep_kernel(slonn_tile_params P)

@@ -99,6 +99,20 @@ def test_plain_layers_of_few_queries_take_columns_where_they_pay(dtype, n, last,
     dm.free()
 
 
+@pytest.mark.parametrize("dtype,n,last", [
+    ("bf16", 203, 512), ("bf16", 204, 512),   # lists of 307 entries: 1624 and 1632 blocks of 64 nodes, shared below 1628
+    ("f32", 203, 508), ("f32", 204, 508),
+    ("bf16", 148, 505), ("bf16", 147, 505),   # a load of one node: shared below 1184 blocks
+])
+def test_plain_layers_share_a_walk_by_the_length_of_their_lists(dtype, n, last):
+    """One block per (query, 64 nodes) or per query, at budgets that always go by input."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(5100 + n, [64, 2048, last], [1, 0], dtype, n=n, n_cal=200, K=4, L=2, budgets=(20, 700, 1500))
+    dm = harness.DeviceModel(wl)
+    _same_bits(_run(dm, wl), _run(dm, wl, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS))
+    dm.free()
+
+
 def test_grouped_products_need_their_scratch_and_do_without_it():
     """A workspace of the size the other kernels need is still taken, with the same results."""
     from paper_2204_08400_b200 import binding as sl, harness

@@ -226,7 +226,8 @@ typedef struct {
  * budget and keys and evaluated 16 at a time over the union of their inputs and nodes, in the same order of sums
  * and with the same results, when the workspace holds the scratch for it (slonn_workspace_bytes includes it).  These two flags force one kind for the whole batch, for testing and
  * tuning; setting both is an error.  They apply to the per-stage kernels and to the
- * one-warp-per-query kernel; the one-cluster-per-query kernel has row form only.
+ * one-warp-per-query kernel; the one-cluster-per-query path takes the input-stationary form by itself (no budget above 2000 bp, a
+ * list-fed layer of at least 1024 inputs) and whole rows otherwise or with SLONN_FLAG_ROW_KERNELS.
  */
 #define SLONN_COLS_MAX_BP 3500u /* default split: budgets up to this take the input-stationary kernels */
 #define SLONN_FLAG_ROW_KERNELS 2u
@@ -443,7 +444,8 @@ typedef struct {
     uint32_t bp_lo, bp_hi; /* it serves the queries whose budget lies in [bp_lo, bp_hi] ...           */
     uint32_t skips_full; /* ... 1: except those at 10000 bp, which another launch serves              */
     uint32_t cols_bp;    /* whole-network launches: queries with budgets up to this evaluated their   */
-                         /* list-fed activator layers input-stationary (0 = every layer row-wise);    */
+                         /* list-fed activator layers (CLUSTER: all list-fed layers) input-stationary */
+                         /* (0 = every layer row-wise);                                               */
                          /* HASH_SELECT, FULL_ROWS, GROUP_ROWS: SLONN_COLS_EVERY when single weights of  */
                          /* the transposed copy were read (the two latter: 16 queries at a time, 128     */
                          /* columns or, SLONN_COLS_EVERY_WIDE, 256), else 0                              */

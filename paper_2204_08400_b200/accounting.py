@@ -127,7 +127,7 @@ def launch_bytes(sh: NetShape, rec: dict, bps: Sequence[int], x_nnz: Optional[np
         tile = grouped_products(rec)
         if stage in ("gather_cols", "layer_cols") or (stage == "hash_select" and rec["cols_bp"]):
             cols[:] = True
-        elif stage == "fused" and rec["cols_bp"] and t["act"] and t["list_in"]:
+        elif rec["cols_bp"] and t["list_in"] and ((stage == "fused" and t["act"]) or stage == "cluster"):
             cols = bp <= rec["cols_bp"]
         if hashes and t["act"]:
             alg += int((t["hash_alg"] + t["lists"]).sum())
@@ -149,6 +149,8 @@ def kernel_name(sh: NetShape, rec: dict) -> str:
         return "tile_rows_kernel"
     if rec["stage"] == "hash_select" and rec["cols_bp"]:
         return "hash_select_cols_kernel"
+    if rec["stage"] == "cluster" and rec["cols_bp"]:
+        return "cluster_lists_kernel"
     if rec["stage"] == "gather_dot" and rec["layer"] is not None and sh.dims[rec["layer"]] * sh.esz <= 512:
         return "gather_short_kernel"
     return KERNEL_OF_STAGE[rec["stage"]]

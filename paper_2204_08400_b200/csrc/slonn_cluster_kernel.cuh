@@ -17,6 +17,9 @@
 // Two hardware cluster barriers per layer replace two kernel launches per layer.  Every block
 // executes the same number of barriers whatever the data (no early exit).  Arithmetic is the
 // library's fixed-order dot product (warp_dot_row1), so results are identical to the other paths.
+//
+// cluster_lists_kernel is the same for clusters of 16 blocks on networks that have list-fed layers with transposed copies:
+// those layers run input-stationary.  See there.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -41,6 +44,10 @@ struct slonn_cluster_layer {
     const void *tables;
     uint32_t D, N, nchunks, cap;
     uint32_t has_act, a, relu, id_bytes;
+    // cluster_lists_kernel only
+    const void *WT, *WH;     // transposed weights and side-by-side hash rows of a layer that runs input-stationary
+    const uint32_t *colpos;  // node id -> column of WT; NULL = identity
+    uint32_t by_input, pad;  // 1: input-stationary
 };
 
 struct slonn_cluster_params {
@@ -63,6 +70,7 @@ struct slonn_cluster_params {
     uint32_t xbuf_floats;    // floats per input buffer (two buffers)
     uint32_t ids_cap;        // entries of the id list
     uint32_t bitmap_words;
+    uint32_t scratch_bytes;  // cluster_lists_kernel: grouped inputs, or the selection's marks of a layer that runs by rows
 };
 
 // Node count of activator layer l for query q (same rule and the same clamping as the plan kernels).
@@ -75,6 +83,67 @@ __device__ __forceinline__ uint32_t cluster_count(const slonn_cluster_params &P,
     const uint32_t B = slonn_layer_nodes(bp, P.layer[l].N, P.pre);
     if (B - P.pre > P.layer[l].cap && B != P.layer[l].N) *bad = true;
     return B;
+}
+
+// List offsets and node counts of query q, by one thread: with a handful of queries every block simply adds up the counts of the
+// (query, layer) entries before its own instead of waiting for a separate planning launch.
+__device__ __forceinline__ void cluster_plan(const slonn_cluster_params &P, uint32_t q, uint32_t rank, uint64_t *s_off, uint32_t *s_cnt)
+{
+    bool bad;
+    if (P.indptr_in || !(P.out_ids || P.out_vals || P.indptr_out)) {
+        // offsets planned by an earlier launch, or not needed at all (no list is written)
+        for (uint32_t l = 0; l < P.n_layers; ++l) {
+            if (!P.layer[l].has_act) continue;
+            s_cnt[l] = cluster_count(P, q, l, &bad);
+            s_off[l] = P.indptr_in ? P.indptr_in[(uint64_t)q * P.n_act + P.layer[l].a] : 0;
+            if (bad && rank == 0) slonn_report(P.status, SLONN_ERR_BUDGET, q, l);
+        }
+        return;
+    }
+    uint64_t run = 0;
+    for (uint32_t qq = 0; qq <= q; ++qq)
+        for (uint32_t l = 0; l < P.n_layers; ++l) {
+            if (!P.layer[l].has_act) continue;
+            const uint32_t B = cluster_count(P, qq, l, &bad);
+            if (qq == q) {
+                s_off[l] = run; s_cnt[l] = B;
+                if (bad && rank == 0) slonn_report(P.status, SLONN_ERR_BUDGET, q, l);
+            }
+            if (rank == 0 && q + 1 == P.n && P.indptr_out) P.indptr_out[(uint64_t)qq * P.n_act + P.layer[l].a] = run;
+            run += B;
+        }
+    if (rank == 0 && q + 1 == P.n && P.indptr_out) P.indptr_out[(uint64_t)P.n * P.n_act] = run;
+}
+
+// Position of the largest of lg[0 .. B), the lowest of equal ones, to thread 0.  The whole block.
+__device__ __forceinline__ uint32_t cluster_argmax(const float *lg, uint32_t B)
+{
+    __shared__ float wbest[32];
+    __shared__ uint32_t wbi[32];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    float best = 0.0f;
+    uint32_t bi = 0xffffffffu;
+    for (uint32_t i = threadIdx.x; i < B; i += blockDim.x) {
+        const float v = lg[i];
+        if (bi == 0xffffffffu || v > best) { best = v; bi = i; }
+    }
+    auto meet = [&]() {
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            const float ob = __shfl_xor_sync(SLONN_FULL_MASK, best, o);
+            const uint32_t oi = __shfl_xor_sync(SLONN_FULL_MASK, bi, o);
+            if (oi != 0xffffffffu && (bi == 0xffffffffu || ob > best || (ob == best && oi < bi))) { best = ob; bi = oi; }
+        }
+    };
+    meet();
+    if (lane == 0) { wbest[warp] = best; wbi[warp] = bi; }
+    __syncthreads();
+    if (warp == 0) {
+        best = lane < nwarps ? wbest[lane] : 0.0f;
+        bi = lane < nwarps ? wbi[lane] : 0xffffffffu;
+        meet();
+    }
+    return bi;
 }
 
 template <bool BF16, int THREADS, int MIN_BLOCKS>
@@ -100,36 +169,9 @@ cluster_network_kernel(const __grid_constant__ slonn_cluster_params P)
     uint32_t *ids_s = reinterpret_cast<uint32_t *>(reinterpret_cast<float *>(smem4) + 2 * P.xbuf_floats);
     uint32_t *bitmap = ids_s + P.ids_cap;
 
-    // List offsets: with a handful of queries every block simply adds up the counts of the (query,
-    // layer) entries before its own instead of waiting for a separate planning launch.
     __shared__ uint64_t s_off[SLONN_MAX_LAYERS];
     __shared__ uint32_t s_cnt[SLONN_MAX_LAYERS];
-    const bool need_offsets = P.out_ids || P.out_vals || P.indptr_out;
-    if (threadIdx.x == 0 && (P.indptr_in || !need_offsets)) {
-        // offsets planned by an earlier launch, or not needed at all (no list is written)
-        bool bad;
-        for (uint32_t l = 0; l < P.n_layers; ++l) {
-            if (!P.layer[l].has_act) continue;
-            s_cnt[l] = cluster_count(P, q, l, &bad);
-            s_off[l] = P.indptr_in ? P.indptr_in[(uint64_t)q * P.n_act + P.layer[l].a] : 0;
-            if (bad && rank == 0) slonn_report(P.status, SLONN_ERR_BUDGET, q, l);
-        }
-    } else if (threadIdx.x == 0) {
-        uint64_t run = 0;
-        bool bad;
-        for (uint32_t qq = 0; qq <= q; ++qq)
-            for (uint32_t l = 0; l < P.n_layers; ++l) {
-                if (!P.layer[l].has_act) continue;
-                const uint32_t B = cluster_count(P, qq, l, &bad);
-                if (qq == q) {
-                    s_off[l] = run; s_cnt[l] = B;
-                    if (bad && rank == 0) slonn_report(P.status, SLONN_ERR_BUDGET, q, l);
-                }
-                if (rank == 0 && q + 1 == P.n && P.indptr_out) P.indptr_out[(uint64_t)qq * P.n_act + P.layer[l].a] = run;
-                run += B;
-            }
-        if (rank == 0 && q + 1 == P.n && P.indptr_out) P.indptr_out[(uint64_t)P.n * P.n_act] = run;
-    }
+    if (threadIdx.x == 0) cluster_plan(P, q, rank, s_off, s_cnt);
 
     // input := x (every block its own copy, in the staging order of layer 0)
     uint32_t cur = 0;
@@ -233,36 +275,10 @@ cluster_network_kernel(const __grid_constant__ slonn_cluster_params P)
         cur = nxt;
 
         if (is_last && rank == 0 && P.pred) {
-            // prediction: lowest node id among the largest computed logits (block 0 holds them by position)
-            const float *lg = xbuf[cur];
-            float best = 0.0f;
-            uint32_t bi = 0xffffffffu;
-            for (uint32_t i = threadIdx.x; i < B; i += blockDim.x) {
-                const float v = lg[i];
-                if (bi == 0xffffffffu || v > best) { best = v; bi = i; }
-            }
-            // positions ascend with node ids, so the lowest position is the lowest id
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
-                const float ob = __shfl_xor_sync(SLONN_FULL_MASK, best, o);
-                const uint32_t oi = __shfl_xor_sync(SLONN_FULL_MASK, bi, o);
-                if (oi != 0xffffffffu && (bi == 0xffffffffu || ob > best || (ob == best && oi < bi))) { best = ob; bi = oi; }
-            }
-            __shared__ float wbest[32];
-            __shared__ uint32_t wbi[32];
-            if (lane == 0) { wbest[warp] = best; wbi[warp] = bi; }
-            __syncthreads();
-            if (warp == 0) {
-                best = lane < nwarps ? wbest[lane] : 0.0f;
-                bi = lane < nwarps ? wbi[lane] : 0xffffffffu;
-#pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) {
-                    const float ob = __shfl_xor_sync(SLONN_FULL_MASK, best, o);
-                    const uint32_t oi = __shfl_xor_sync(SLONN_FULL_MASK, bi, o);
-                    if (oi != 0xffffffffu && (bi == 0xffffffffu || ob > best || (ob == best && oi < bi))) { best = ob; bi = oi; }
-                }
-                if (lane == 0 && bi != 0xffffffffu) P.pred[q] = implicit_ids ? bi : ids_s[bi];
-            }
+            // prediction: lowest node id among the largest computed logits (block 0 holds them by position, and
+            // positions ascend with node ids)
+            const uint32_t bi = cluster_argmax(xbuf[cur], B);
+            if (threadIdx.x == 0 && bi != 0xffffffffu) P.pred[q] = implicit_ids ? bi : ids_s[bi];
         }
     }
 }

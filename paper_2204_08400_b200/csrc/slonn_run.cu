@@ -10,6 +10,7 @@
 #include "slonn_run_kernels.cuh"
 #include "slonn_tile_kernels.cuh"
 #include "slonn_cluster_kernel.cuh"
+#include "slonn_cluster_lists.cuh"
 
 namespace {
 
@@ -1023,10 +1024,10 @@ uint32_t cluster_max_rows(const slonn_model *m, uint32_t max_bp)
     return r;
 }
 
-template <bool BF16, int THREADS, int MIN_BLOCKS>
-int launch_cluster_t(const slonn_cluster_params &P, size_t smem, cudaStream_t st)
+typedef void (*cluster_kernel)(const slonn_cluster_params);
+
+int launch_cluster_t(cluster_kernel kernel, uint32_t THREADS, const slonn_cluster_params &P, size_t smem, cudaStream_t st)
 {
-    auto kernel = cluster_network_kernel<BF16, THREADS, MIN_BLOCKS>;
     { const int rc = slonn_allow_smem(reinterpret_cast<const void *>(kernel), smem); if (rc) return rc; }
     if (P.cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return SLONN_ERR_CUDA;
@@ -1051,10 +1052,52 @@ int launch_cluster_t(const slonn_cluster_params &P, size_t smem, cudaStream_t st
     return cudaLaunchKernelEx(&cfg, kernel, P) == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
+// When the cluster's list-fed layers run input-stationary: speed over whole rows, one to four queries, weights of two batches in turn.
+// bf16, 4096 x 4096, nine layers, 1 / 5 / 10 / 15 / 25 %: 1.40 1.43-1.59 1.62-1.70 1.38-1.58 0.96-1.15 (10 %: 142 -> 88 us); four
+// layers of width 1024 / 1536 / 2048 / 3072 / 4096, least of 3 to 20 %: 1.07 1.06 1.03 1.06 1.11, fp32 1.02 1.06 1.08 1.07
+// 1.36; 25 % of 2048 0.99-1.00, fp32 0.95-0.98, 50 % 0.88-0.90: beyond 20 % a block's share is more than one pass of its lanes and
+// the row form, which streams, wins.  Every node computed, 1024 wide: 0.75-0.79; 784-112-112-10: 0.92-1.00: nothing to skip.
+#define SLONN_LISTS_MAX_BP 2000u
+#define SLONN_LISTS_MIN_WIDTH 1024u // of at least one such layer
+
+// Completes P for cluster_lists_kernel.  false: no layer is worth it, the lists have more positions than its selection
+// takes, or its shared memory does not fit.
+bool cluster_lists_params(const slonn_model *m, uint32_t max_bp, slonn_cluster_params &P, size_t *smem)
+{
+    const uint32_t esz = m->dtype == SLONN_BF16 ? 2u : 4u, V = 16u / esz, pre = slonn_model_pre(m);
+    uint32_t set = 1, words = 1;
+    size_t scratch = 16;
+    bool some = false;
+    if (max_bp > SLONN_LISTS_MAX_BP) return false;
+    for (uint32_t l = 0; l < m->n_layers; ++l) {
+        const slonn_layer &ly = m->layer[l];
+        slonn_cluster_layer &f = P.layer[l];
+        const uint32_t nodes = ly.has_act ? slonn_layer_nodes(max_bp, ly.N, pre) : ly.N;
+        f.by_input = l > 0 && m->layer[l - 1].has_act && ly.WT && (!ly.has_act || (ly.WH && ly.colpos));
+        if (f.by_input) {
+            some = some || ly.D >= SLONN_LISTS_MIN_WIDTH;
+            f.WT = ly.WT; f.WH = ly.WH; f.colpos = ly.colpos;
+            P.xbuf_floats = std::max(P.xbuf_floats, 32u * cols_smax(ly.D, V));
+            scratch = std::max(scratch, (size_t)32 * align_up(cols_smax(ly.D, V), 4) * 8);
+        } else if (ly.has_act) {
+            scratch = std::max(scratch, ((size_t)ly.N + 3) / 4 * 16);
+        }
+        if (ly.has_act) {
+            if ((uint64_t)(nodes - pre) * m->L > SLONN_LISTS_POSITIONS) return false;
+            set = std::max(set, nodes);
+            words = std::max(words, (ly.N + 31u) / 32u);
+        }
+    }
+    P.ids_cap = (set + 7u) / 8u * 8u; P.bitmap_words = words; P.scratch_bytes = (uint32_t)align_up(scratch, 16);
+    *smem = (size_t)P.xbuf_floats * 8 + P.scratch_bytes + 2 * 16 * 64 * 4 + (size_t)words * 16 + (size_t)P.ids_cap * 6;
+    *smem = std::max<size_t>(*smem, 48 * 1024); // the kernel's static shared memory (5 KB) is more than slonn_allow_smem reckons with below that
+    return some && *smem <= 200 * 1024;
+}
+
 // cluster_size 16: a handful of queries, 512 threads per block.  cluster_size 1: one block of four warps per query
 // (narrow networks, batches up to a few thousand queries); indptr_in: the planned offsets when lists are written.
 int launch_cluster(const slonn_model *m, const slonn_batch *b, uint32_t max_bp, uint32_t stride, cudaStream_t st,
-                   uint32_t cluster_size = SLONN_CLUSTER_SIZE, const uint64_t *indptr_in = nullptr)
+                   uint32_t cluster_size = SLONN_CLUSTER_SIZE, const uint64_t *indptr_in = nullptr, stage_timer *tm = nullptr)
 {
     slonn_cluster_params P;
     memset(&P, 0, sizeof(P));
@@ -1083,10 +1126,17 @@ int launch_cluster(const slonn_model *m, const slonn_batch *b, uint32_t max_bp, 
     P.xbuf_floats = xbuf; P.ids_cap = ids_cap; P.bitmap_words = words;
     const size_t smem = (size_t)xbuf * 8 + (size_t)ids_cap * 4 + (size_t)words * 4;
     if (smem > 200 * 1024) return SLONN_ERR_DIM;
+    const bool bf = m->dtype == SLONN_BF16;
     if (cluster_size == 1)
-        return m->dtype == SLONN_BF16 ? launch_cluster_t<true, 128, SLONN_BLOCK_MINB>(P, smem, st) : launch_cluster_t<false, 128, SLONN_BLOCK_MINB>(P, smem, st);
-    return m->dtype == SLONN_BF16 ? launch_cluster_t<true, SLONN_CLUSTER_THREADS, 1>(P, smem, st)
-                                  : launch_cluster_t<false, SLONN_CLUSTER_THREADS, 1>(P, smem, st);
+        return launch_cluster_t(bf ? cluster_network_kernel<true, 128, SLONN_BLOCK_MINB> : cluster_network_kernel<false, 128, SLONN_BLOCK_MINB>, 128, P, smem, st);
+    slonn_cluster_params Q = P;
+    size_t lists_smem = 0;
+    if (!(b->flags & SLONN_FLAG_ROW_KERNELS) && cluster_lists_params(m, max_bp, Q, &lists_smem)) {
+        TIC_BY_INPUT();
+        return launch_cluster_t(bf ? cluster_lists_kernel<true> : cluster_lists_kernel<false>, SLONN_CLUSTER_THREADS, Q, lists_smem, st);
+    }
+    return launch_cluster_t(bf ? cluster_network_kernel<true, SLONN_CLUSTER_THREADS, 1> : cluster_network_kernel<false, SLONN_CLUSTER_THREADS, 1>,
+                            SLONN_CLUSTER_THREADS, P, smem, st);
 }
 
 } // namespace
@@ -1268,7 +1318,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
          cluster_max_rows(m, max_bp) <= 1024)) {
         AT_LAYER(SLONN_ALL_LAYERS);
         TIC(SLONN_STAGE_CLUSTER);
-        const int rc = launch_cluster(m, b, max_bp, stride, st);
+        const int rc = launch_cluster(m, b, max_bp, stride, st, SLONN_CLUSTER_SIZE, nullptr, tm);
         TOC();
         if (rc != SLONN_ERR_DIM || b->kernel_path == SLONN_PATH_CLUSTER) return rc;
         // the device cannot co-schedule such a cluster: fall through to the other kernels

@@ -220,9 +220,9 @@ typedef struct {
  * ways with identical results: row kernels read each selected weight row whole; input-stationary
  * kernels walk the query's nonzero inputs and read single weights from a transposed copy the model
  * keeps.  By default the library picks per query by budget: up to SLONN_COLS_MAX_BP
- * the input list is sparse enough for the input-stationary kernels to win (batches of tens of queries
- * only for layers at least 2048 inputs wide, and, where the layer has an activator, only when no budget exceeds 1500 bp; a handful of
- * queries keep the row kernels); in large batches the queries that compute more than a few hundred nodes per layer are sorted by
+ * the input list is sparse enough for the input-stationary kernels to win (batches of tens of queries take them, in two launches per
+ * layer, up to 5000 bp when the workspace holds the scratch for it; without it, and below about 48 K inputs in all, only layers at
+ * least 2048 inputs wide do, and, where the layer has an activator, only when no budget exceeds 1500 bp); in large batches the queries that compute more than a few hundred nodes per layer are sorted by
  * budget and keys and evaluated 16 at a time over the union of their inputs and nodes, in the same order of sums
  * and with the same results, when the workspace holds the scratch for it (slonn_workspace_bytes includes it).  These two flags force one kind for the whole batch, for testing and
  * tuning; setting both is an error.  They apply to the per-stage kernels and to the
@@ -448,7 +448,9 @@ typedef struct {
                          /* (0 = every layer row-wise);                                               */
                          /* HASH_SELECT, FULL_ROWS, GROUP_ROWS: SLONN_COLS_EVERY when single weights of  */
                          /* the transposed copy were read (the two latter: 16 queries at a time, 128     */
-                         /* columns or, SLONN_COLS_EVERY_WIDE, 256), else 0                              */
+                         /* columns or, SLONN_COLS_EVERY_WIDE, 256), else 0; of the two launches that     */
+                         /* serve a list-fed layer of tens of queries HASH_SELECT has                   */
+                         /* SLONN_COLS_EVERY_WIDE and GATHER_COLS SLONN_COLS_EVERY                        */
     float ms;            /* device time between the event pair around the launch                      */
 } slonn_launch_record;
 int slonn_run_traced(const slonn_model *m, const slonn_batch *batch, void *workspace,

@@ -148,7 +148,9 @@ def kernel_name(sh: NetShape, rec: dict) -> str:
     if grouped_products(rec):
         return "tile_rows_kernel"
     if rec["stage"] == "hash_select" and rec["cols_bp"]:
-        return "hash_select_cols_kernel"
+        return "few_select_kernel" if rec["cols_bp"] == COLS_EVERY_WIDE else "hash_select_cols_kernel"
+    if rec["stage"] == "gather_cols" and rec["cols_bp"]:
+        return "few_nodes_kernel"
     if rec["stage"] == "cluster" and rec["cols_bp"]:
         return "cluster_lists_kernel"
     if rec["stage"] == "gather_dot" and rec["layer"] is not None and sh.dims[rec["layer"]] * sh.esz <= 512:

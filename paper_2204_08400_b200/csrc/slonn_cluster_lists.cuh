@@ -36,36 +36,36 @@ struct lists_set {
     uint32_t words;
 };
 
-// The layer's active set by the rule of block_select, for at most SLONN_LISTS_POSITIONS list positions.  The whole block;
-// key(b): table b's; `first`: N words of scratch, a multiple of four.  by_id: places by id are wanted.  ids_out: nullable, the id-ascending
+// What the selection reads of a layer.  colpos: places are by column of this order; NULL: by id.
+struct lists_layer {
+    const void *tables;
+    const uint32_t *hash_nodes, *colpos;
+    uint32_t N, cap;
+};
+
+// The layer's active set by the rule of block_select, for at most SLONN_LISTS_POSITIONS list positions.  A whole block of
+// SLONN_CLUSTER_THREADS; key(b): table b's; `first`: N words of scratch, a multiple of four.  by_id: places by id are wanted.  ids_out: nullable, the id-ascending
 // list.  Ends without a barrier.  Returns false when the lists did not hold enough distinct ids (malformed tables).
 // U: positions per thread.
 template <typename IDT, int U, typename KEY>
-__device__ __forceinline__ bool lists_select(const slonn_cluster_layer &ly, uint32_t K, uint32_t L, uint32_t B, uint32_t pre,
+__device__ __forceinline__ bool lists_select(const lists_layer &ly, uint32_t K, uint32_t L, uint32_t B, uint32_t pre,
                                              KEY &&key, uint32_t *first, const lists_set &S, bool by_id,
                                              uint32_t *counts /* [SELECT * 16] shared */, uint32_t *ids_out)
 {
     constexpr uint32_t T = SLONN_CLUSTER_THREADS, W = T / 32u;
     static_assert(W == 16u, "a warp reads the counts of a row of positions with half of its lanes");
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t *colpos = ly.by_input ? ly.colpos : nullptr;
+    const uint32_t *colpos = ly.colpos;
     by_id = by_id && colpos;
-    auto plain = [&](bool ok) { // nodes 0 .. B - 1
-        for (uint32_t i = tid; i < B; i += T) {
-            S.node[i] = (uint16_t)i; S.col[i] = (uint16_t)(colpos ? __ldg(colpos + i) : i); S.pos[i] = (uint16_t)i;
-            if (ids_out) ids_out[i] = i;
-        }
-        return ok;
-    };
     const uint32_t want = B - pre, npos = want * L;
-    if (B == ly.N || want > ly.cap) return plain(true); // every node; more than the lists hold (reported by the plan)
+    bool ok = true, listed = B != ly.N && want <= ly.cap; // not listed: nodes 0 .. B - 1 (all, or more than the lists hold, which the plan reports)
 
     uint32_t id[U], col[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const uint32_t p = u * T + tid;
         const uint32_t r = L == 2u ? p >> 1 : p / L, b = p - r * L;
-        id[u] = p < npos ? table_entry<IDT>(ly.tables, ly.cap, K, b, key(b), r) : 0xffffffffu;
+        id[u] = listed && p < npos ? table_entry<IDT>(ly.tables, ly.cap, K, b, key(b), r) : 0xffffffffu;
     }
     uint32_t hnode = tid < pre ? __ldg(ly.hash_nodes + tid) : 0xffffffffu, hcol = hnode; // always active, in no list
     for (uint32_t i = tid; i < (ly.N + 3u) / 4u; i += T) reinterpret_cast<uint4 *>(first)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -96,15 +96,22 @@ __device__ __forceinline__ bool lists_select(const slonn_cluster_layer &ly, uint
         if (((own[u] >> lane) & 1u) && total + (sum >> 16) + __popc(own[u] & ((1u << lane) - 1u)) < want) taken |= 1u << u;
         total += sum & 0xffffu;
     }
-    if (total < want) return plain(false); // uniform
+    if (listed && total < want) ok = listed = false; // uniform
     auto mark = [&](uint32_t node, uint32_t c) {
         atomicOr(&S.bits[c >> 5], 1u << (c & 31u));
         if (by_id) atomicOr(&S.idbits[node >> 5], 1u << (node & 31u));
     };
+    auto each = [&](auto &&f) { // the thread's share of the set: f(node, column)
+        if (!listed) {
+            for (uint32_t i = tid; i < B; i += T) f(i, colpos ? __ldg(colpos + i) : i);
+            return;
+        }
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-        if ((taken >> u) & 1u) mark(id[u], col[u]);
-    if (tid < pre) mark(hnode, hcol);
+        for (int u = 0; u < U; ++u)
+            if ((taken >> u) & 1u) f(id[u], col[u]);
+        if (tid < pre) f(hnode, hcol);
+    };
+    each(mark);
     __syncthreads();
     if (warp < (by_id ? 2u : 1u)) { // what lies below each word: warp 0 by column, warp 1 by id
         const uint32_t *bits = warp ? S.idbits : S.bits;
@@ -128,11 +135,8 @@ __device__ __forceinline__ bool lists_select(const slonn_cluster_layer &ly, uint
         S.node[at] = (uint16_t)node; S.col[at] = (uint16_t)c; S.pos[at] = (uint16_t)by;
         if (ids_out) ids_out[by] = node;
     };
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        if ((taken >> u) & 1u) place(id[u], col[u]);
-    if (tid < pre) place(hnode, hcol);
-    return true;
+    each(place);
+    return ok;
 }
 
 // ---- input-stationary sums ------------------------------------------------------------
@@ -213,6 +217,42 @@ __device__ __forceinline__ float2 lists_hash(const uint2 *e0, const uint2 *e1, u
     a.x = a.x + __shfl_xor_sync(SLONN_FULL_MASK, a.x, 16);
     a.y = a.y + __shfl_xor_sync(SLONN_FULL_MASK, a.y, 16);
     return a;
+}
+
+// The nonzero inputs of partial sums `warp` and `warp + 16` of a layer's inputs x (by partial sum, smax each: lists_index) to e0 and
+// e1, in order: n0 and n1 of them, and both filled up to the returned multiple of four with inputs that are listed anyway, at
+// the value 0.  One warp.
+template <uint32_t V>
+__device__ __forceinline__ uint32_t lists_group(const float *x, uint32_t smax, uint32_t warp, uint32_t lane, uint2 *e0, uint2 *e1, uint32_t &n0, uint32_t &n1)
+{
+    const uint32_t lower = (1u << lane) - 1u;
+    n0 = n1 = 0;
+    for (uint32_t i0 = 0; i0 < smax; i0 += 128u) { // four neighbours per lane, of one chunk
+        const uint32_t i = i0 + 4u * lane;
+        const bool in = i < smax;
+        auto group = [&](uint32_t p, uint2 *e, uint32_t &n) {
+            const float4 v = in ? *reinterpret_cast<const float4 *>(x + p * smax + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const uint32_t b0 = __ballot_sync(SLONN_FULL_MASK, v.x != 0.0f), b1 = __ballot_sync(SLONN_FULL_MASK, v.y != 0.0f);
+            const uint32_t b2 = __ballot_sync(SLONN_FULL_MASK, v.z != 0.0f), b3 = __ballot_sync(SLONN_FULL_MASK, v.w != 0.0f);
+            uint2 *at = e + n + __popc(b0 & lower) + __popc(b1 & lower) + __popc(b2 & lower) + __popc(b3 & lower);
+            const uint32_t j = ((i / V) * 32u + p) * V + (i & (V - 1u));
+            if (v.x != 0.0f) *at++ = make_uint2(j, __float_as_uint(v.x));
+            if (v.y != 0.0f) *at++ = make_uint2(j + 1u, __float_as_uint(v.y));
+            if (v.z != 0.0f) *at++ = make_uint2(j + 2u, __float_as_uint(v.z));
+            if (v.w != 0.0f) *at++ = make_uint2(j + 3u, __float_as_uint(v.w));
+            n += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
+        };
+        group(warp, e0, n0);
+        group(warp + 16u, e1, n1);
+    }
+    __syncwarp();
+    const uint32_t m = (max(n0, n1) + 3u) & ~3u;
+    const uint32_t j = n0 ? e0[0].x : e1[0].x; // m == 0: not used
+    __syncwarp();
+    for (uint32_t i = n0 + lane; i < m; i += 32u) e0[i] = make_uint2(j, 0u);
+    for (uint32_t i = n1 + lane; i < m; i += 32u) e1[i] = make_uint2(j, 0u);
+    __syncwarp();
+    return m;
 }
 
 // The sums of the 16 warps (part[warp][64]) of slot s, strides 8, 4, 2, 1 of the tree.
@@ -321,7 +361,8 @@ __global__ void __launch_bounds__(SLONN_CLUSTER_THREADS, 1) cluster_lists_kernel
             S.words = (ly.N + 31u) >> 5;
             // nodes of a layer number at most SLONN_CLUSTER_MAX_N: 16-bit ids
             const uint32_t npos = (B - P.pre) * P.L;
-            auto run = [&](auto u) { return lists_select<uint16_t, u.value>(ly, P.K, P.L, B, P.pre, key, first, S, by_id, counts, ids_out); };
+            const lists_layer sl = {ly.tables, ly.hash_nodes, ly.by_input ? ly.colpos : nullptr, ly.N, ly.cap};
+            auto run = [&](auto u) { return lists_select<uint16_t, u.value>(sl, P.K, P.L, B, P.pre, key, first, S, by_id, counts, ids_out); };
             const bool ok = npos <= 2 * T ? run(std::integral_constant<int, 2>()) : npos <= 4 * T ? run(std::integral_constant<int, 4>())
                                                                                   : run(std::integral_constant<int, SLONN_LISTS_SELECT>());
             if (!ok && rank == 0 && tid == 0) slonn_report(P.status, SLONN_ERR_ARG, q, l);
@@ -371,39 +412,11 @@ __global__ void __launch_bounds__(SLONN_CLUSTER_THREADS, 1) cluster_lists_kernel
             __syncthreads();
             clear(xin);
         } else {
-            // the nonzero inputs of the warp's two partial sums, both filled up to the same multiple of four with inputs that
-            // are listed anyway, at the value 0
+            // the nonzero inputs of the warp's two partial sums
             const uint32_t smax = cols_smax(ly.D, V), pitch = (smax + 3u) & ~3u;
             uint2 *e0 = entries() + warp * pitch, *e1 = e0 + 16u * pitch;
-            uint32_t n0 = 0, n1 = 0;
-            const uint32_t lower = (1u << lane) - 1u;
-            for (uint32_t i0 = 0; i0 < smax; i0 += 128u) { // four neighbours per lane, of one chunk
-                const uint32_t i = i0 + 4u * lane;
-                const bool in = i < smax;
-                auto group = [&](uint32_t p, uint2 *e, uint32_t &n) {
-                    const float4 v = in ? *reinterpret_cast<const float4 *>(xin + p * smax + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const uint32_t b0 = __ballot_sync(SLONN_FULL_MASK, v.x != 0.0f), b1 = __ballot_sync(SLONN_FULL_MASK, v.y != 0.0f);
-                    const uint32_t b2 = __ballot_sync(SLONN_FULL_MASK, v.z != 0.0f), b3 = __ballot_sync(SLONN_FULL_MASK, v.w != 0.0f);
-                    uint2 *at = e + n + __popc(b0 & lower) + __popc(b1 & lower) + __popc(b2 & lower) + __popc(b3 & lower);
-                    const uint32_t j = ((i / V) * 32u + p) * V + (i & (V - 1u));
-                    if (v.x != 0.0f) *at++ = make_uint2(j, __float_as_uint(v.x));
-                    if (v.y != 0.0f) *at++ = make_uint2(j + 1u, __float_as_uint(v.y));
-                    if (v.z != 0.0f) *at++ = make_uint2(j + 2u, __float_as_uint(v.z));
-                    if (v.w != 0.0f) *at++ = make_uint2(j + 3u, __float_as_uint(v.w));
-                    n += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
-                };
-                group(warp, e0, n0);
-                group(warp + 16u, e1, n1);
-            }
-            __syncwarp();
-            const uint32_t m = (max(n0, n1) + 3u) & ~3u;
-            {
-                const uint32_t j = n0 ? e0[0].x : e1[0].x; // (m == 0: not used)
-                __syncwarp();
-                for (uint32_t i = n0 + lane; i < m; i += 32u) e0[i] = make_uint2(j, 0u);
-                for (uint32_t i = n1 + lane; i < m; i += 32u) e1[i] = make_uint2(j, 0u);
-            }
-            __syncwarp();
+            uint32_t n0, n1;
+            const uint32_t m = lists_group<V>(xin, smax, warp, lane, e0, e1, n0, n1);
             uint32_t buf = 0;
             if (ly.has_act) {
                 // the hash functions' partial sums rank and rank + 16, to every block

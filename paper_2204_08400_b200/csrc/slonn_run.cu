@@ -11,6 +11,7 @@
 #include "slonn_tile_kernels.cuh"
 #include "slonn_cluster_kernel.cuh"
 #include "slonn_cluster_lists.cuh"
+#include "slonn_few_kernels.cuh"
 
 namespace {
 
@@ -83,7 +84,11 @@ struct ws_layout {
         uint32_t chunk;          // queries staged at a time, 0: this batch does not take them
         uint32_t order_stride;   // entries of `order` per chunk
     } tile;
-    uint64_t total_tile;         // what a call needs to take them (== total when it does not)
+    struct {                     // list-fed layers of few queries (slonn_few_kernels.cuh), in the same place
+        uint64_t ent, seg, nodes, quads;
+        uint32_t ent_stride, rows; // per query; 0: this batch does not take them
+    } few;
+    uint64_t total_tile;         // what a call needs to take either (== total when it takes neither)
 };
 
 // widest bf16 activation matrix row the tensor-core route needs
@@ -225,6 +230,59 @@ void carve_tile(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
     w.total_tile = o;
 }
 
+// ---- list-fed activator layers of few queries -------------------------------------------
+
+// When a batch takes them: speed over the kernels of before (whole rows or layer_cols_kernel), networks of 1024-D-D-D-600, bf16, budgets of
+// 2, 5, 10, 15, 25 and 50 %:
+//   D 4096, 12 queries 1.15 1.15 1.24 1.29 1.10 1.07; 80 queries 1.29 1.02 1.08 1.19 1.43 1.34; 150 queries 0.99 1.13 1.30 2.60 2.88 -
+//   D 2048, 16 queries 0.96 0.97 1.02 1.13 1.10 0.97; 28 queries 0.96 0.98 1.11 1.13 1.00 1.10; 80 queries 1.04 1.18 1.04 1.08 1.25 1.30
+//   D 1024, 28 queries 0.96 0.93 0.96 0.98 1.03 0.96; 48 queries 1.02 1.00 1.09 1.14 1.00 1.10; 150 queries 1.10 1.14 1.13 1.15 1.13 1.15
+// fp32 the same or better (4096, 80 queries at 5 % 0.97, 48 queries at 5 and 10 % 0.97 and 0.98: the least).  Fewer inputs than the first
+// line below, and the second launch costs more than the first saves.  More queries than SMs are one block each of layer_cols_kernel
+// as well as of few_select_kernel, so few nodes do not pay: 240 queries at 2 and 5 %, D 2048 0.92 0.99, 3072 0.91 1.04, fp32 0.91 0.95 and 0.89 0.99.
+// Mixed budgets up to 60 %, 32 queries: 0.98 (100 queries 1.05); up to 100 %: rows.
+#define SLONN_FEW_MAX_BP 5000u
+#define SLONN_FEW_INPUTS (48ull * 1024) // queries times inputs
+#define SLONN_FEW_WAVE 148u             // more queries than this: layers of at least
+#define SLONN_FEW_NODES 128u            // this many nodes per query
+// A layer without activator, behind a layer that takes them: both launches against one of gather_cols_kernel, 5, 15 and 35 %: 64 queries, 1000
+// outputs 1.04-1.29 1.03-1.23 1.04-1.19, 100 outputs 0.97-1.10; 24 queries, 1000 outputs 0.95-1.00 0.98-1.02 1.00-1.20; 12 outputs 0.90-0.98.
+#define SLONN_FEW_PLAIN (48ull * 1024)  // queries times outputs
+
+// whether a batch evaluates list-fed layer l by few_select_kernel and few_nodes_kernel (workspace permitting)
+bool few_layer_ok(const slonn_model *m, uint32_t l, uint32_t n, uint32_t max_bp)
+{
+    const slonn_layer &ly = m->layer[l];
+    if (l == 0 || !m->layer[l - 1].has_act || !ly.WT || ly.N % 4u != 0u || ly.D > SLONN_CLUSTER_MAX_D ||
+        ly.N > SLONN_CLUSTER_MAX_N || max_bp > SLONN_FEW_MAX_BP || (uint64_t)n * ly.D < SLONN_FEW_INPUTS)
+        return false;
+    if (!ly.has_act) return (uint64_t)n * ly.N >= SLONN_FEW_PLAIN && few_layer_ok(m, l - 1, n, max_bp);
+    const uint32_t pre = slonn_model_pre(m), nodes = slonn_layer_nodes(max_bp, ly.N, pre);
+    if (!ly.WH || !ly.colpos || (uint64_t)(nodes - pre) * m->L > SLONN_LISTS_POSITIONS) return false;
+    return n <= SLONN_FEW_WAVE || nodes >= SLONN_FEW_NODES;
+}
+
+void carve_few(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags, ws_layout &w)
+{
+    memset(&w.few, 0, sizeof(w.few));
+    if (w.tile.chunk || (flags & (SLONN_FLAG_ROW_KERNELS | SLONN_FLAG_COLUMN_KERNELS)) || tc_route(m, max_bp, flags)) return;
+    const uint32_t pre = slonn_model_pre(m);
+    for (uint32_t l = 0; l < m->n_layers; ++l)
+        if (few_layer_ok(m, l, n, max_bp)) {
+            const slonn_layer &ly = m->layer[l];
+            w.few.rows = std::max(w.few.rows, ly.has_act ? slonn_layer_nodes(max_bp, ly.N, pre) : 1u);
+            w.few.ent_stride = std::max(w.few.ent_stride, (uint32_t)align_up(cols_ent_cap(ly.D, slonn_layer_nodes(max_bp, ly.D, pre)), 4));
+        }
+    if (!w.few.rows) return;
+    uint64_t o = w.total;
+    auto take = [&](uint64_t bytes) { const uint64_t at = o; o = align_up(o + bytes, 256); return at; };
+    w.few.ent = take((uint64_t)n * w.few.ent_stride * 8);
+    w.few.seg = take((uint64_t)n * SLONN_FEW_SEG * 4);
+    w.few.nodes = take((uint64_t)n * w.few.rows * 8);
+    w.few.quads = take((uint64_t)n * w.few.rows * 8);
+    w.total_tile = o;
+}
+
 ws_layout carve(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags)
 {
     ws_layout w;
@@ -249,6 +307,7 @@ ws_layout carve(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
     }
     w.total = std::max<uint64_t>(o, 256);
     carve_tile(m, n, max_bp, flags, w);
+    carve_few(m, n, max_bp, flags, w);
     return w;
 }
 
@@ -674,15 +733,62 @@ int launch_layer_rows(const slonn_model *m, const slonn_layer &ly, slonn_gather_
     return launch_rows(m, P, b, n, max_bp, max_rows, gw, st, tm);
 }
 
+// The scratch of list-fed layers of few queries in a call's workspace; ws == NULL: the call does not take them.
+struct few_ws { char *ws; const ws_layout *wl; };
+
+template <bool BF16>
+int launch_few_t(const slonn_few_params &Q, uint32_t n, size_t select_smem, size_t nodes_smem, cudaStream_t st, stage_timer *tm)
+{
+    const slonn_gather_params &G = Q.G;
+    // few_select_kernel has 7 KB of static shared memory, more than slonn_allow_smem reckons with below 48 KB
+    int rc = set_smem(few_select_kernel<BF16>, std::max<size_t>(select_smem, 48 * 1024));
+    if (!rc) rc = set_smem(few_nodes_kernel<BF16>, nodes_smem);
+    if (rc) return rc;
+    if (G.use_list) TIC(SLONN_STAGE_HASH_SELECT, G.range_bp, G.bp_lo, G.bp_hi, G.skip_bp, SLONN_COLS_EVERY_WIDE);
+    else TIC(SLONN_STAGE_GATHER_COLS, G.range_bp, G.bp_lo, G.bp_hi, G.skip_bp, SLONN_COLS_EVERY);
+    slonn_launch(few_select_kernel<BF16>, n, SLONN_CLUSTER_THREADS, select_smem, st, Q);
+    if (G.use_list) TOC();
+    if (G.use_list) TIC(SLONN_STAGE_GATHER_COLS, G.range_bp, G.bp_lo, G.bp_hi, G.skip_bp, SLONN_COLS_EVERY);
+    slonn_launch(few_nodes_kernel<BF16>, n * G.ctas_per_query, SLONN_THREADS, nodes_smem, st, Q);
+    TOC();
+    return cudaGetLastError() == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
+}
+
+// SLONN_ERR_DIM: the staging does not fit shared memory.
+int launch_few(const slonn_model *m, const slonn_layer &ly, uint32_t layer, slonn_gather_params G, const slonn_batch *b, uint32_t n,
+               uint32_t max_rows, uint32_t in_cap, const few_ws &fw, cudaStream_t st, stage_timer *tm)
+{
+    const auto &F = fw.wl->few;
+    const bool bf = m->dtype == SLONN_BF16;
+    const uint32_t V = bf ? 8u : 4u, smax = cols_smax(ly.D, V);
+    slonn_few_params Q;
+    memset(&Q, 0, sizeof(Q));
+    G.WT = ly.WT; G.colpos = ly.colpos; G.rows_cap = max_rows; G.in_cap = in_cap;
+    Q.quad_stride = ly.has_act ? std::min(max_rows, ly.N / 4u) : ly.N / 4u;
+    G.ctas_per_query = (Q.quad_stride + 31u) / 32u;
+    Q.G = G; Q.WH = ly.WH; Q.hash_nodes = ly.hash_nodes; Q.tables = ly.tables; Q.cap = ly.cap;
+    Q.K = m->K; Q.L = m->L; Q.pre = slonn_model_pre(m); Q.layer = layer; Q.codes = b->codes; Q.status = b->status;
+    Q.ent = (uint2 *)(fw.ws + F.ent); Q.seg = (uint32_t *)(fw.ws + F.seg); Q.nodes = (uint2 *)(fw.ws + F.nodes); Q.quads = (uint2 *)(fw.ws + F.quads);
+    Q.ent_stride = F.ent_stride; Q.scratch_bytes = 32u * (uint32_t)align_up(smax, 4) * 8u;
+    const size_t select_smem = align_up(std::max(32u * smax, ly.N), 4) * 4 + Q.scratch_bytes + (ly.has_act ? (size_t)((ly.N + 31u) / 32u) * 16 + (size_t)max_rows * 6 : 0);
+    const size_t nodes_smem = (size_t)32 * 4 * 32 * 4 + (size_t)F.ent_stride * 8;
+    if (select_smem > 200 * 1024 || nodes_smem > 200 * 1024) return SLONN_ERR_DIM;
+    return bf ? launch_few_t<true>(Q, n, select_smem, nodes_smem, st, tm) : launch_few_t<false>(Q, n, select_smem, nodes_smem, st, tm);
+}
+
 // An activator layer: FreeHash, selection and the selected nodes.  A list-fed layer with the copies for it
 // runs as ONE input-stationary launch for the queries whose budget leaves the list sparse; the others (and
 // every query where that launch does not apply) take the selection kernel followed by the row or
 // input-stationary gather.
 int launch_act_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, slonn_select_params &sp, slonn_gather_params &gp,
                      const slonn_batch *b, uint32_t n, uint32_t max_bp, uint32_t max_rows, uint32_t in_cap, const group_ws &gw,
-                     cudaStream_t st, stage_timer *tm)
+                     const few_ws &fw, cudaStream_t st, stage_timer *tm)
 {
     int rc;
+    if (fw.ws && gp.in.kind == SLONN_IN_LIST && few_layer_ok(m, l, n, max_bp)) {
+        rc = launch_few(m, ly, l, gp, b, n, max_rows, in_cap, fw, st, tm);
+        if (rc != SLONN_ERR_DIM) return rc;
+    }
     const uint32_t cols_bp = cols_budget_limit(ly, gp, b, n, max_rows, max_bp);
     if (cols_bp && ly.WH) {
         const bool both = max_bp > cols_bp;
@@ -1307,6 +1413,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
     slonn_logit_stride(m, max_bp, &stride);
     // grouped products: when the workspace has room for their scratch, else the kernels that need none
     const tile_ws tw = {wl.tile.chunk && ws_bytes >= wl.total_tile ? ws : nullptr, &wl};
+    const few_ws fw = {wl.few.rows && ws_bytes >= wl.total_tile ? ws : nullptr, &wl};
 
     // a handful of queries: one thread-block cluster per query, every layer in one launch (it derives the
     // list offsets itself, so no planning launch either)
@@ -1519,7 +1626,7 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                     const sorted_groups sg = {(const uint32_t *)(ws + wl.tile.order), wl.tile.chunk, wl.tile.order_stride, from};
                     if (!rc) rc = launch_rows(m, gp, b, n, max_bp, max_rows, gw, st, tm, &sg);
                 } else {
-                    rc = launch_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm);
+                    rc = launch_act_layer(m, ly, l, sp, gp, b, n, max_bp, max_rows, in_cap, gw, fw, st, tm);
                 }
             }
             if (rc) return rc;
@@ -1564,7 +1671,8 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
                 if (rc) return rc;
                 rows_done = true;
             }
-            rc = launch_layer_rows(m, ly, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm, rows_done);
+            rc = fw.ws && in.kind == SLONN_IN_LIST && !rows_done && few_layer_ok(m, l, n, max_bp) ? launch_few(m, ly, l, gp, b, n, max_rows, in_cap, fw, st, tm) : SLONN_ERR_DIM;
+            if (rc == SLONN_ERR_DIM) rc = launch_layer_rows(m, ly, gp, b, n, max_bp, max_rows, in_cap, gw, st, tm, rows_done);
             if (rc) return rc;
             in.kind = SLONN_IN_DENSE; in.dense = gp.out_dense;
             dense_cur ^= 1;

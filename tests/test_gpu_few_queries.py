@@ -1,0 +1,50 @@
+"""List-fed layers of batches of tens of queries (few_select_kernel, few_nodes_kernel) against the oracle: last runs of four columns and
+last blocks half full, more queries than SMs, every number of list positions per thread, tables whose number does not divide
+a block, budgets that differ, inputs that are all zero, plain layers; and a workspace without their scratch."""
+import numpy as np
+import pytest
+
+from oracle import oracle as orc
+from parity_util import assert_run_parity, oracle_model, oracle_run
+from test_gpu_parity import custom_workload
+
+pytestmark = pytest.mark.gpu
+
+CASES = {
+    "smallest": dict(dims=[64, 1024, 1024, 36], act=[1, 1, 0], dtype="bf16", n=48, budgets=(1, 100, 5000)),
+    "ragged": dict(dims=[136, 1160, 1036, 596], act=[1, 1, 1], dtype="f32", n=61, budgets=(300, 2000, 4900), K=7, L=3),
+    "more_queries_than_sms": dict(dims=[64, 1032, 1304, 44], act=[1, 1, 0], dtype="bf16", n=173, budgets=(1000, 2500)),
+    "widest": dict(dims=[32, 8192, 8192, 20], act=[1, 1, 0], dtype="bf16", n=7, budgets=(2000, 2500)),       # 4096 list positions
+    "eight_tables": dict(dims=[64, 2048, 1400, 52], act=[1, 1, 1], dtype="f32", n=25, budgets=(900, 3600), K=4, L=8),
+    "short_lists": dict(dims=[64, 2056, 1024, 12], act=[1, 1, 0], dtype="bf16", n=30, budgets=(200, 2000), list_cap=430, free_hash=True),
+    "tiny_layer": dict(dims=[64, 1024, 48, 24], act=[1, 1, 1], dtype="bf16", n=50, budgets=(1, 400, 5000), K=3, L=2),
+}
+
+
+@pytest.mark.parametrize("name", CASES)
+@pytest.mark.parametrize("dead", [False, True])
+def test_layers_of_few_queries_match_the_oracle(name, dead):
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    c = CASES[name]
+    wl = custom_workload(930, c["dims"], c["act"], c["dtype"], n=c["n"], n_cal=200, K=c.get("K", 10), L=c.get("L", 2), budgets=c["budgets"],
+                         list_cap=c.get("list_cap", 0))
+    wl.budget_bp[:] = np.resize(c["budgets"], c["n"])
+    wl.free_hash_nodes = c.get("free_hash", False)
+    if dead:  # the first layer hands over nothing but zeros
+        wl.bias[0][:] = -1e4
+    dm, om = harness.DeviceModel(wl), oracle_model(wl)
+    o32, o64 = (oracle_run(om, wl, wl.x, wl.budget_bp, mode) for mode in (orc.CANON32, orc.REF64))
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
+    names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == 1]
+    assert names == ["few_select_kernel", "few_nodes_kernel"]
+    for _ in range(2):
+        b.run()
+        assert_run_parity(b.results(), o32, o64, wl, sum(wl.has_act), bool(wl.has_act[-1]))
+    # a workspace of the size the other kernels need: those run, with the same results
+    least = sl.slonn_workspace_bytes(dm.model, b.n, b.max_bp, sl.FLAG_ROW_KERNELS)
+    assert least < b.ws_bytes
+    sl.slonn_run(dm.model, b.batch, b.ws, least)
+    assert_run_parity(b.results(), o32, o64, wl, sum(wl.has_act), bool(wl.has_act[-1]))
+    names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, least) if r["layer"] == 1]
+    assert "few_nodes_kernel" not in names
+    dm.free()

@@ -95,15 +95,15 @@ __global__ void hash_matrix_kernel(const void *W, void *WH, uint32_t D, uint32_t
     else reinterpret_cast<uint32_t *>(WH)[t] = v;
 }
 
-// How early each node appears in the layer's ranked lists: score[n] = sum over all lists of 1024 max(0, T - r) + 1024 c / (r + c), r the rank
-// of n in the list, T = N / 8, c = N / 16.  Integer sums, so the result does not depend on thread order.  The second term orders the
-// nodes no list has near its head: with the first alone they stayed in the order of their ids (4096 nodes at 50 %: the
-// runs of four columns a group's nodes lie in hold up to 3200 columns, now 2200; 64 queries at 25 %, nine layers: 331 -> 316 us).  A
-// block adds up its lists in shared memory where the layer's scores fit.
+// How early each node appears in the layer's ranked lists: score[n] = sum over all lists of
+// max(0, T - rank of n in the list).  Integer sums, so the result does not depend on thread order.  A block adds up its lists in
+// shared memory where the layer's scores fit (2 M atomics on as few addresses as a layer has nodes otherwise).  Ordering the nodes
+// that no list has among its first T as well (by the sum of 1 / (rank + N / 16)) brought 64 queries at 25 % from 331 to 317 us and
+// cost 777 queries of mixed budgets 3 % (1568 wide, 348 -> 360 us), 300 queries at 25 % 3 % (2048 wide): left out.
 #define POPULARITY_LISTS 16      // lists per block
 #define POPULARITY_SHARED 40960u // most nodes whose scores fit
 template <typename IDT>
-__global__ void __launch_bounds__(256) popularity_kernel(const IDT *tables, uint64_t n_lists, uint32_t cap, uint32_t T, uint32_t c, uint32_t N,
+__global__ void __launch_bounds__(256) popularity_kernel(const IDT *tables, uint64_t n_lists, uint32_t cap, uint32_t T, uint32_t N,
                                                          unsigned long long *score)
 {
     extern __shared__ uint32_t s_score[];
@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(256) popularity_kernel(const IDT *tables, uint
         __syncthreads();
     }
     const uint64_t l0 = (uint64_t)blockIdx.x * POPULARITY_LISTS, l1 = min(l0 + POPULARITY_LISTS, n_lists);
-    for (uint32_t r = threadIdx.x; r < cap; r += 256) {
-        const uint32_t w = (r < T ? (T - r) * 1024u : 0u) + (uint32_t)(1024ull * c / (r + c));
+    for (uint32_t r = threadIdx.x; r < T; r += 256) {
+        const uint32_t w = T - r;
         for (uint64_t l = l0; l < l1; ++l) {
             const uint32_t id = (uint32_t)tables[l * cap + r];
             if (id >= N) continue;
@@ -163,7 +163,7 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
         }
         // order of the node axis: by popularity in the lists, equal scores by lower id
         const uint64_t n_lists = (uint64_t)m->L << m->K;
-        const uint32_t T = std::max(1u, std::min(ly.cap, (ly.N + 7u) / 8u)), c = std::max(1u, ly.N / 16u);
+        const uint32_t T = std::max(1u, std::min(ly.cap, (ly.N + 7u) / 8u));
         unsigned long long *d_score = nullptr;
         if (cudaMalloc(&d_score, sizeof(unsigned long long) * ly.N) != cudaSuccess) return SLONN_ERR_NOMEM;
         std::vector<unsigned long long> score(ly.N);
@@ -175,9 +175,9 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
             const void *kernel = ly.id_bytes == 2 ? (const void *)popularity_kernel<uint16_t> : (const void *)popularity_kernel<uint32_t>;
             if (slonn_allow_smem(kernel, smem) != SLONN_OK) ok = false;
             else if (ly.id_bytes == 2)
-                popularity_kernel<uint16_t><<<blocks, 256, smem, st>>>((const uint16_t *)ly.tables, n_lists, ly.cap, T, c, ly.N, d_score);
+                popularity_kernel<uint16_t><<<blocks, 256, smem, st>>>((const uint16_t *)ly.tables, n_lists, ly.cap, T, ly.N, d_score);
             else
-                popularity_kernel<uint32_t><<<blocks, 256, smem, st>>>((const uint32_t *)ly.tables, n_lists, ly.cap, T, c, ly.N, d_score);
+                popularity_kernel<uint32_t><<<blocks, 256, smem, st>>>((const uint32_t *)ly.tables, n_lists, ly.cap, T, ly.N, d_score);
             ok = ok && cudaGetLastError() == cudaSuccess &&
                  cudaMemcpyAsync(score.data(), d_score, sizeof(unsigned long long) * ly.N, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
                  cudaStreamSynchronize(st) == cudaSuccess;

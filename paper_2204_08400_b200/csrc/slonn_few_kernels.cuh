@@ -6,7 +6,7 @@
 //                       what the other launch needs of it goes to scratch (a layer without activator: the grouped inputs only)
 //   few_nodes_kernel    one block per (query, 32 runs of four columns): its warps share the 32 partial sums, as gather_cols_kernel's split form
 // 64 queries at 25 % on nine layers of 4096 nodes: 496 us a pass with hash_select_kernel and whole rows (a layer 12 and 46 us, the rows at 11.7
-// TB/s from L2), 317 with these (13 and 25).
+// TB/s from L2), 335 with these (13 and 26).
 #pragma once
 #include "slonn_cluster_lists.cuh"
 
@@ -169,7 +169,7 @@ __device__ __forceinline__ void few_add(const uint32_t (&w)[BF16 ? 2 : 4], uint3
 
 // What bounds it is requests: a warp's load of 32 single columns costs the L1 as much as one of 32 runs of four, and in column order
 // most of a run's columns are selected.  Lane = run of four columns (64 queries at 25 %: 37 us a layer with a column or two per
-// lane, 25 with runs; blocks of one SM on neighbouring queries' same columns, for L1 hits: 42).
+// lane, 26 with runs; blocks of one SM on neighbouring queries' same columns, for L1 hits: 42).
 template <bool BF16>
 __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FEW_BLOCKS) few_nodes_kernel(const __grid_constant__ slonn_few_params Q)
 {

@@ -234,17 +234,19 @@ void carve_tile(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
 
 // When a batch takes them: speed over the kernels of before (whole rows or layer_cols_kernel), networks of 1024-D-D-D-600, bf16, budgets of
 // 2, 5, 10, 15, 25 and 50 %:
-//   D 4096, 12 queries 1.15 1.15 1.24 1.29 1.10 1.07; 80 queries 1.29 1.02 1.08 1.19 1.43 1.34; 150 queries 0.99 1.13 1.30 2.60 2.88 -
-//   D 2048, 16 queries 0.96 0.97 1.02 1.13 1.10 0.97; 28 queries 0.96 0.98 1.11 1.13 1.00 1.10; 80 queries 1.04 1.18 1.04 1.08 1.25 1.30
-//   D 1024, 28 queries 0.96 0.93 0.96 0.98 1.03 0.96; 48 queries 1.02 1.00 1.09 1.14 1.00 1.10; 150 queries 1.10 1.14 1.13 1.15 1.13 1.15
-// fp32 the same or better (4096, 80 queries at 5 % 0.97, 48 queries at 5 and 10 % 0.97 and 0.98: the least).  Fewer inputs than the first
-// line below, and the second launch costs more than the first saves.  More queries than SMs are one block each of layer_cols_kernel
-// as well as of few_select_kernel, so few nodes do not pay: 240 queries at 2 and 5 %, D 2048 0.92 0.99, 3072 0.91 1.04, fp32 0.91 0.95 and 0.89 0.99.
+//   D 4096, 12 queries 1.05 1.08 1.18 1.19 1.01 1.02; 80 queries 1.31 1.01 1.03 1.14 1.35 1.20; 150 queries - 1.14 1.31 2.59 2.88 -
+//   D 2048, 28 queries 1.02 1.04 1.15 1.13 1.03 1.13; 80 queries 1.00 1.16 1.02 1.03 1.17 1.19; 16 queries 0.96 0.97 1.02 1.13 1.10 0.97
+//   D 1024, 28 queries 0.96 0.93 0.96 0.98 1.03 0.96; 48 queries 0.96 0.96 1.07 1.11 1.00 1.09; 150 queries 1.10 1.14 1.13 1.17 1.13 1.15
+// fp32 the same or better (4096, 28 queries at 10 %, 48 queries at 5 %, 3072, 80 queries at 5 and 10 %: 0.98 to 0.99, the least).  Fewer inputs
+// than the first line below, or a block's runs mostly empty, and the second launch costs more than the first saves.  More queries
+// than SMs are one block each of layer_cols_kernel, where that applies (2048 inputs), as well as of few_select_kernel, so few nodes
+// do not pay there: 240 queries at 2 and 5 %, D 2048 0.92 0.99, 3072 0.91 1.04, fp32 0.91 0.95 and 0.89 0.99; D 1024 1.27 1.17.
 // Mixed budgets up to 60 %, 32 queries: 0.98 (100 queries 1.05); up to 100 %: rows.
 #define SLONN_FEW_MAX_BP 5000u
 #define SLONN_FEW_INPUTS (48ull * 1024) // queries times inputs
-#define SLONN_FEW_WAVE 148u             // more queries than this: layers of at least
-#define SLONN_FEW_NODES 128u            // this many nodes per query
+#define SLONN_FEW_NODES 60u             // nodes per query
+#define SLONN_FEW_WAVE 148u             // more queries than this on wide layers:
+#define SLONN_FEW_NODES_WAVE 128u       // this many
 // A layer without activator, behind a layer that takes them: both launches against one of gather_cols_kernel, 5, 15 and 35 %: 64 queries, 1000
 // outputs 1.04-1.29 1.03-1.23 1.04-1.19, 100 outputs 0.97-1.10; 24 queries, 1000 outputs 0.95-1.00 0.98-1.02 1.00-1.20; 12 outputs 0.90-0.98.
 #define SLONN_FEW_PLAIN (48ull * 1024)  // queries times outputs
@@ -259,7 +261,7 @@ bool few_layer_ok(const slonn_model *m, uint32_t l, uint32_t n, uint32_t max_bp)
     if (!ly.has_act) return (uint64_t)n * ly.N >= SLONN_FEW_PLAIN && few_layer_ok(m, l - 1, n, max_bp);
     const uint32_t pre = slonn_model_pre(m), nodes = slonn_layer_nodes(max_bp, ly.N, pre);
     if (!ly.WH || !ly.colpos || (uint64_t)(nodes - pre) * m->L > SLONN_LISTS_POSITIONS) return false;
-    return n <= SLONN_FEW_WAVE || nodes >= SLONN_FEW_NODES;
+    return nodes >= (n > SLONN_FEW_WAVE && ly.D >= 2048u ? SLONN_FEW_NODES_WAVE : SLONN_FEW_NODES);
 }
 
 void carve_few(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flags, ws_layout &w)

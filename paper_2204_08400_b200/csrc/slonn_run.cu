@@ -922,7 +922,7 @@ int launch_tile_layer(const slonn_model *m, const slonn_layer &ly, uint32_t l, c
         P.cols = tile_item_cols(P, P.select ? slonn_layer_nodes(max_bp, ly.N, slonn_model_pre(m)) : ly.N, all_queries);
         P.work = (uint32_t *)(tw.ws + T.work) + (c ? 2 : 0); // the first chunk's counts stay until the layer is done (items_at)
         // the sort cleared the counts of work items; only the first chunk can rely on it
-        if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, 8, st) != cudaSuccess) return SLONN_ERR_CUDA;
+        if ((c > 0 || !fresh_order) && cudaMemsetAsync(P.work, 0, SLONN_TILE_WORK * 4, st) != cudaSuccess) return SLONN_ERR_CUDA;
         slonn_launch(tile_prep_kernel, dim3(P.groups, 2), 512, smem, st, P);
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
         if (c == 0) TIC_ITEMS(P.work);

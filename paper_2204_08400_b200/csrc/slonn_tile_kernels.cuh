@@ -27,6 +27,8 @@
 #define SLONN_WIDE_COLS (32 * SLONN_WIDE_NN)
 #define SLONN_TILE_CHUNK 8192u  // most queries sorted and staged at a time
 #define SLONN_TILE_MAX_N 32768u // widest layer: the group's G node bitmaps are built in shared memory
+#define SLONN_TILE_TAKEN 4      // place of the counts of taken items behind those of items
+#define SLONN_TILE_WORK 6u      // words of counts
 #define SLONN_TILE_SLACK 64u    // entries past a group's list that a pipelined load may touch
 
 // Position of partial sum p in the entry order, and back.  Four in a row are those of a warp of eight, in bit-reversed order
@@ -44,7 +46,7 @@ struct slonn_order_params {
     uint32_t skip_full;      // 1: and those at exactly 10000 bp
     uint32_t q0, n;          // queries [q0, q0 + n), n <= SLONN_TILE_CHUNK
     uint32_t *order;         // out: the first entries; the rest keep the 0xffffffff (no query) they were set to
-    uint32_t *work;          // [2] cleared for the tile_prep_kernel that follows
+    uint32_t *work;          // [SLONN_TILE_WORK] cleared for the tile_prep_kernel that follows
 };
 
 // Rank by counting: a query's place is the number of smaller keys of its chunk.  n^2 compares (17 M for 4096
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(256) tile_order_kernel(slonn_order_params P)
     const uint32_t e0 = (blockIdx.x * 8u + warp) * 4u;
     uint64_t mine[4];
     uint32_t rank[4] = {0u, 0u, 0u, 0u};
-    if (blockIdx.x == 0 && threadIdx.x < 2u) P.work[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < SLONN_TILE_WORK) P.work[threadIdx.x] = 0u;
     // ~0: left out.  The key of a query that is left out may never have been written; it is loaded beside the budget all the
     // same, so that neither load waits for the other.
     auto key_of = [&](uint32_t e) -> uint64_t {
@@ -126,7 +128,7 @@ struct slonn_tile_params {
     uint32_t groups;
     uint32_t nwords;          // (N + 31) / 32
     uint32_t cols;            // columns of a work item: SLONN_TILE_COLS or SLONN_WIDE_COLS, or 0: tile_prep_kernel decides
-    uint32_t *work;           // [2] number of work items of SLONN_TILE_COLS and of SLONN_WIDE_COLS columns; one of them stays 0
+    uint32_t *work;           // number of work items of SLONN_TILE_COLS and of SLONN_WIDE_COLS columns; one of them stays 0; and at SLONN_TILE_TAKEN how many the blocks have taken
     uint32_t *items;          // group << 16 | tile (groups <= 1024 * 8, tiles <= N / 128)
     uint32_t *kseg;           // [groups][33] first entry of each partial sum's stretch, total
     uint32_t *krow;           // [groups][kcap] byte offset of the entry's row of WT
@@ -459,7 +461,7 @@ __device__ __forceinline__ void tile_cp_async(uint32_t dst, const void *src)
 #define SLONN_TILE_RING_BYTES (SLONN_TILE_ROWS_AT + SLONN_TILE_RING * 4 + 16) // the first row offsets again behind the last
 #define SLONN_TILE_PART (SLONN_TILE_COLS * SLONN_TILE_G) // floats of a warp's sums
 #define SLONN_TILE_SMEM ((size_t)SLONN_TILE_WARPS * (SLONN_TILE_RING_BYTES + SLONN_TILE_PART * 4))
-#define SLONN_TILE_STATIC (2 * SLONN_TILE_COLS * 8 + 2 * SLONN_TILE_WARPS * 32 + 2 * SLONN_TILE_G * 12) // s_col, s_item, s_q and s_off
+#define SLONN_TILE_STATIC (2 * SLONN_TILE_COLS * 8 + 2 * SLONN_TILE_WARPS * 32 + 2 * SLONN_TILE_G * 12 + 8) // s_col, s_item, s_q, s_off and s_next
 static_assert(SLONN_TILE_SMEM > 46 * 1024 && SLONN_TILE_SMEM + SLONN_TILE_STATIC <= 227 * 1024,
               "tile_rows_kernel must opt in to its shared memory and fit a block's 227 KB with its static part");
 
@@ -521,6 +523,7 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
     auto slot_index = [&](uint32_t tile, uint32_t s) -> uint32_t {
         return tile * SLONN_TILE_COLS + (QUAD ? ((s & 63u) >> 1) * 4u + (s >> 6) * 2u + (s & 1u) : s);
     };
+    __shared__ uint32_t s_next;
     const uint32_t n_items = P.work[0];
 
     // the item at hand: the steps of the warp's two partial sums, the lane's columns in row 0
@@ -595,8 +598,10 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         }
     };
 
-    // items are dealt out in turn: neighbours in the list are of neighbouring groups and cost about the same
-    uint32_t it = blockIdx.x;
+    // Items differ (unions, budgets), so beyond the first two a block takes the next one nobody has (dealt out in turn, second layer of
+    // 8192 queries of 5 to 100 % on 4096 x 4096 1338 us, now 1280; 4096 queries at 10 % on as many, sort and staging included, 182
+    // and 177; from the end of the list, where the highest budgets are, 1292).
+    uint32_t it = blockIdx.x, next = blockIdx.x + gridDim.x;
     if (it >= n_items) return;
     for (uint32_t i = lane; i < SLONN_TILE_RING_BYTES / 4; i += 32) reinterpret_cast<uint32_t *>(ring)[i] = 0u; // row offsets that exist
     look_up(it, 0u);
@@ -606,6 +611,8 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
     start_weights(0u);
 
     for (uint32_t buf = 0;; buf ^= 1u) {
+        uint32_t taken = 0;
+        if (tid == 0 && next < n_items) taken = 2u * gridDim.x + atomicAdd(P.work + SLONN_TILE_TAKEN, 1u);
         float2 acc[G][NN / 2];
 #pragma unroll
         for (int i = 0; i < G; ++i)
@@ -667,7 +674,7 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
                         *reinterpret_cast<float2 *>(mypart + i * SLONN_TILE_COLS + j * 64) = acc[i][j];
                         acc[i][j] = make_float2(0.0f, 0.0f);
                     }
-                if (it + gridDim.x < n_items) look_up(it + gridDim.x, buf ^ 1u);
+                if (next < n_items) look_up(next, buf ^ 1u);
             }
         }
 #pragma unroll
@@ -680,8 +687,8 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
 
-        it += gridDim.x;
-        const bool more = it < n_items;
+        const bool more = next < n_items;
+        if (tid == 0) s_next = taken;
         // the item's own end, one column and four queries per thread
         const uint32_t g = s_item[buf][warp][4] >> 16, tile = s_item[buf][warp][4] & 0xffffu, cnt = s_item[buf][warp][3];
         const uint32_t s = tid % SLONN_TILE_COLS, quad = tid / SLONN_TILE_COLS;
@@ -701,6 +708,8 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         }
         if (more) start_copies(buf ^ 1u);
         __syncthreads();
+        it = next;
+        next = s_next;
         if (more) start_weights(buf ^ 1u);
         if (mine) {
             // the sixteen warps' sums, strides 8, 4, 2, 1 of the tree; then bias, ReLU and the query's list
@@ -919,7 +928,8 @@ __global__ void __launch_bounds__(SLONN_WIDE_WARPS * 32, 1) tile_rows_wide_kerne
         }
     };
 
-    // items are dealt out in turn: neighbours in the list are of neighbouring groups and cost about the same
+    // items are dealt out in turn: neighbours in the list are of neighbouring groups and cost about the same (whoever is free takes the next,
+    // as in tile_rows_kernel: two more registers across the loop than there are, every node of 4096 x 2048 for 1638 queries 1202 -> 1257 us)
     if (warp == 0) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_tmem)), "r"(SLONN_WIDE_TMEM) : "memory");

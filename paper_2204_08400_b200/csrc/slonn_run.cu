@@ -1463,8 +1463,12 @@ static int run_impl(const slonn_model *m, const slonn_batch *b, void *workspace,
         uint64_t *tile_sums = (uint64_t *)(ws + wl.plan_sums);
         AT_LAYER(SLONN_ALL_LAYERS);
         TIC(SLONN_STAGE_PLAN);
-        slonn_launch(plan_partial_kernel, (uint32_t)tiles, SLONN_PLAN_THREADS, 0, st, pp, tile_sums);
-        slonn_launch(plan_final_kernel, (uint32_t)tiles, SLONN_PLAN_THREADS, 0, st, pp, tile_sums);
+        if ((uint64_t)n * m->n_act <= SLONN_PLAN_SMALL) {
+            slonn_launch(plan_small_kernel, 1u, 1024u, 0, st, pp, (n * m->n_act + 1023u) / 1024u);
+        } else {
+            slonn_launch(plan_partial_kernel, (uint32_t)tiles, SLONN_PLAN_THREADS, 0, st, pp, tile_sums);
+            slonn_launch(plan_final_kernel, (uint32_t)tiles, SLONN_PLAN_THREADS, 0, st, pp, tile_sums);
+        }
         TOC();
         if (cudaGetLastError() != cudaSuccess) return SLONN_ERR_CUDA;
     }

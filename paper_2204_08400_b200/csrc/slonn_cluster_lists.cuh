@@ -7,23 +7,21 @@
 //   3. every block runs the selection: each list position marks its node with the lowest position that names it, the
 //      positions that find their own mark are the first ones of their nodes, and one count over them in position order
 //      cuts the list at the budget (a handful of block barriers whatever the overlap of the lists);
-//   4. the block evaluates its share of the nodes, lane = node, in column order, every weight load of a warp's two
-//      partial sums in flight at once; activations go to every block's copy of the next input.      cluster barrier
+//   4. the block evaluates its share of the nodes, lane = node, in column order, a warp its two partial sums of all of them, 16
+//      loads per lane in flight; activations go to every block's copy of the next input.      cluster barrier
 // Two cluster barriers per layer as before, but B_out * B_in weights instead of B_out rows, and nothing from HBM that few queries in
 // a row do not share: nine layers of 4096 nodes, one query at 10 %, 154 -> 89 us a pass.  Of a layer's 8.5 us (clock stamps):
 // grouping 0.9, hash 2.1, selection 2.7 (list loads 1.0), nodes 1.8, delivery and barrier 1.7; a layer run by rows takes 13.
 // Every phase is short enough that its instruction count, times the four warps of a scheduler, is what it takes: all loads
 // in flight at once cost more in spills than they saved (lists_walk with 16 entries of both partial sums in flight 3.7 us, 8: 1.8).
 // Other clusters bringing the weights into L2 ahead of time: 104 us, as their lists and rows displace what the next query shares.
-//  Layers whose input is dense run as in
-// cluster_network_kernel.
+// Layers whose input is dense run as in cluster_network_kernel.
 #pragma once
 #include "slonn_cluster_kernel.cuh"
 
 #define SLONN_LISTS_SELECT 8 // list positions per thread, most
 #define SLONN_LISTS_POSITIONS (SLONN_LISTS_SELECT * SLONN_CLUSTER_THREADS)
-
-#define SLONN_LISTS_DEPTH 4  // 16-byte chunks of a weight row in flight per lane
+#define SLONN_LISTS_DEPTH 4  // 16-byte chunks of a weight row in flight per lane (8: the first layer takes as long, the others 3 % longer: spills)
 
 // ---- selection ----------------------------------------------------------------------
 

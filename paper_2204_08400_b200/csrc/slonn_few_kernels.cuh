@@ -167,9 +167,10 @@ __device__ __forceinline__ void few_add(const uint32_t (&w)[BF16 ? 2 : 4], uint3
     }
 }
 
-// What bounds it is requests: a warp's load of 32 single columns costs the L1 as much as one of 32 runs of four, and in column order
-// most of a run's columns are selected.  Lane = run of four columns (64 queries at 25 %: 37 us a layer with a column or two per
-// lane, 26 with runs; blocks of one SM on neighbouring queries' same columns, for L1 hits: 42).
+// What bounds it is the way from L2: a query's columns in sectors, 8.4 TB/s, the L1 68 % busy.  Lane = run of four columns: in column
+// order most of a run's columns are selected, and a request brings 32 of them instead of 32 columns (64 queries at 25 %, 4096 x
+// 4096: 37 us a layer with a column or two per lane, 26 with runs; blocks of one SM on neighbouring queries' same columns, for L1
+// hits, measured with two columns per lane: 42).
 template <bool BF16>
 __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FEW_BLOCKS) few_nodes_kernel(const __grid_constant__ slonn_few_params Q)
 {

@@ -461,7 +461,7 @@ __device__ __forceinline__ void tile_cp_async(uint32_t dst, const void *src)
 #define SLONN_TILE_RING_BYTES (SLONN_TILE_ROWS_AT + SLONN_TILE_RING * 4 + 16) // the first row offsets again behind the last
 #define SLONN_TILE_PART (SLONN_TILE_COLS * SLONN_TILE_G) // floats of a warp's sums
 #define SLONN_TILE_SMEM ((size_t)SLONN_TILE_WARPS * (SLONN_TILE_RING_BYTES + SLONN_TILE_PART * 4))
-#define SLONN_TILE_STATIC (2 * SLONN_TILE_COLS * 8 + 2 * SLONN_TILE_WARPS * 32 + 2 * SLONN_TILE_G * 12 + 8) // s_col, s_item, s_q, s_off and s_next
+#define SLONN_TILE_STATIC (2 * SLONN_TILE_COLS * 8 + 2 * SLONN_TILE_WARPS * 32 + 2 * SLONN_TILE_G * 12 + 8) // s_col, s_item, s_q, s_off, s_next and s_items
 static_assert(SLONN_TILE_SMEM > 46 * 1024 && SLONN_TILE_SMEM + SLONN_TILE_STATIC <= 227 * 1024,
               "tile_rows_kernel must opt in to its shared memory and fit a block's 227 KB with its static part");
 
@@ -523,8 +523,8 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
     auto slot_index = [&](uint32_t tile, uint32_t s) -> uint32_t {
         return tile * SLONN_TILE_COLS + (QUAD ? ((s & 63u) >> 1) * 4u + (s >> 6) * 2u + (s & 1u) : s);
     };
-    __shared__ uint32_t s_next;
-    const uint32_t n_items = P.work[0];
+    __shared__ uint32_t s_next, s_items; // the item after next; items in all, which is read from here so that it holds no register in the loop
+    auto n_items = [&]() { return *reinterpret_cast<volatile uint32_t *>(&s_items); };
 
     // the item at hand: the steps of the warp's two partial sums, the lane's columns in row 0
     uint32_t nA = 0, nst = 0; // steps of two entries: of the first partial sum, of both
@@ -601,10 +601,14 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
     // Items differ (unions, budgets), so beyond the first two a block takes the next one nobody has (dealt out in turn, second layer of
     // 8192 queries of 5 to 100 % on 4096 x 4096 1338 us, now 1280; 4096 queries at 10 % on as many, sort and staging included, 182
     // and 177; from the end of the list, where the highest budgets are, 1292).
-    uint32_t it = blockIdx.x, next = blockIdx.x + gridDim.x;
-    if (it >= n_items) return;
+    uint32_t next = blockIdx.x + gridDim.x;
+    {
+        const uint32_t n = P.work[0];
+        if (blockIdx.x >= n) return;
+        if (tid == 0) s_items = n;
+    }
     for (uint32_t i = lane; i < SLONN_TILE_RING_BYTES / 4; i += 32) reinterpret_cast<uint32_t *>(ring)[i] = 0u; // row offsets that exist
-    look_up(it, 0u);
+    look_up(blockIdx.x, 0u);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     start_copies(0u);
@@ -612,7 +616,7 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
 
     for (uint32_t buf = 0;; buf ^= 1u) {
         uint32_t taken = 0;
-        if (tid == 0 && next < n_items) taken = 2u * gridDim.x + atomicAdd(P.work + SLONN_TILE_TAKEN, 1u);
+        if (tid == 0 && next < n_items()) taken = 2u * gridDim.x + atomicAdd(P.work + SLONN_TILE_TAKEN, 1u);
         float2 acc[G][NN / 2];
 #pragma unroll
         for (int i = 0; i < G; ++i)
@@ -674,7 +678,7 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
                         *reinterpret_cast<float2 *>(mypart + i * SLONN_TILE_COLS + j * 64) = acc[i][j];
                         acc[i][j] = make_float2(0.0f, 0.0f);
                     }
-                if (next < n_items) look_up(next, buf ^ 1u);
+                if (next < n_items()) look_up(next, buf ^ 1u);
             }
         }
 #pragma unroll
@@ -687,7 +691,7 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
 
-        const bool more = next < n_items;
+        const bool more = next < n_items();
         if (tid == 0) s_next = taken;
         // the item's own end, one column and four queries per thread
         const uint32_t g = s_item[buf][warp][4] >> 16, tile = s_item[buf][warp][4] & 0xffffu, cnt = s_item[buf][warp][3];
@@ -708,7 +712,6 @@ __global__ void __launch_bounds__(SLONN_TILE_WARPS * 32, 1) tile_rows_kernel(slo
         }
         if (more) start_copies(buf ^ 1u);
         __syncthreads();
-        it = next;
         next = s_next;
         if (more) start_weights(buf ^ 1u);
         if (mine) {

@@ -43,7 +43,8 @@ struct lists_layer {
 
 // The layer's active set by the rule of block_select, for at most SLONN_LISTS_POSITIONS list positions.  A whole block of
 // SLONN_CLUSTER_THREADS; key(b): table b's; `first`: N words of scratch, a multiple of four.  by_id: places by id are wanted.  ids_out: nullable, the id-ascending
-// list.  Ends without a barrier.  Returns false when the lists did not hold enough distinct ids (malformed tables).
+// list.  Ends without a barrier.  Every place below B is filled whatever the lists hold (a saved model's entries are not checked on
+// loading); returns false when they did not hold enough distinct ids beside the hash nodes.
 // U: positions per thread.
 template <typename IDT, int U, typename KEY>
 __device__ __forceinline__ bool lists_select(const lists_layer &ly, uint32_t K, uint32_t L, uint32_t B, uint32_t pre,
@@ -65,13 +66,14 @@ __device__ __forceinline__ bool lists_select(const lists_layer &ly, uint32_t K, 
         const uint32_t r = L == 2u ? p >> 1 : p / L, b = p - r * L;
         id[u] = listed && p < npos ? table_entry<IDT>(ly.tables, ly.cap, K, b, key(b), r) : 0xffffffffu;
     }
-    uint32_t hnode = tid < pre ? __ldg(ly.hash_nodes + tid) : 0xffffffffu, hcol = hnode; // always active, in no list
+    uint32_t hnode = tid < pre ? __ldg(ly.hash_nodes + tid) : 0xffffffffu, hcol = hnode; // always active
     for (uint32_t i = tid; i < (ly.N + 3u) / 4u; i += T) reinterpret_cast<uint4 *>(first)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
     for (uint32_t i = tid; i < S.words; i += T) { S.bits[i] = 0u; S.idbits[i] = 0u; }
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < U; ++u)
-        if (id[u] < ly.N) atomicMin(&first[id[u]], u * T + tid);
+        if (id[u] < ly.N) atomicMin(&first[id[u]], u * T + tid + 1u);
+    if (tid < pre) atomicMin(&first[hnode], 0u); // below every list position: an entry that names a hash node is not counted
 #pragma unroll
     for (int u = 0; u < U; ++u) col[u] = id[u] < ly.N && colpos ? __ldg(colpos + id[u]) : id[u];
     if (tid < pre && colpos) hcol = __ldg(colpos + hnode);
@@ -81,7 +83,7 @@ __device__ __forceinline__ bool lists_select(const lists_layer &ly, uint32_t K, 
     for (int u = 0; u < U; ++u) {
         own[u] = 0u;
         if (u * T >= npos) continue; // uniform
-        own[u] = __ballot_sync(SLONN_FULL_MASK, id[u] < ly.N && first[min(id[u], ly.N - 1u)] == u * T + tid);
+        own[u] = __ballot_sync(SLONN_FULL_MASK, id[u] < ly.N && first[min(id[u], ly.N - 1u)] == u * T + tid + 1u);
         if (lane == 0) counts[u * W + warp] = __popc(own[u]);
     }
     __syncthreads();

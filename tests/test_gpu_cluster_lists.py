@@ -1,6 +1,7 @@
 """The one-cluster-per-query path whose list-fed layers run input-stationary, against the oracle: shares of the 16 blocks below and
 above one pass of a warp's lanes, empty shares, every number of list positions per thread its selection is compiled for, tables
-whose number does not divide the block, inputs that are all zero, plain layers, and a budgeted last layer."""
+whose number does not divide the block, inputs that are all zero, plain layers, and a budgeted last layer.  Its selection, which the
+layers of tens of queries share, on saved lists that no build writes: against the row kernels."""
 import numpy as np
 import pytest
 
@@ -58,3 +59,65 @@ def test_higher_budgets_and_narrow_networks_keep_whole_rows():
         b = harness.DeviceBatch(dm, wl.x, wl.budget_bp)
         assert [r["cols_bp"] for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["stage"] == "cluster"] == [cols]
         dm.free()
+
+
+def edited(blob, tables, hash_nodes, edit):
+    """A saved model whose bucket lists edit(lists [L, buckets, cap], hash nodes) has changed, with the checksum of its bytes."""
+    out, at = blob.copy(), len(blob) - 8
+    for t, nodes in zip(reversed(tables), reversed(hash_nodes)):   # layer records end with the lists, the last one at the checksum
+        at -= t.nbytes
+        edit(out[at:at + t.nbytes].view(t.dtype).reshape(t.shape), nodes.reshape(-1))
+        at -= 8 + 4 * nodes.size
+    h = 0xCBF29CE484222325
+    for b in out[:-8].tobytes():
+        h = ((h ^ b) * 0x100000001B3) & 0xFFFFFFFFFFFFFFFF
+    out[-8:] = np.frombuffer(h.to_bytes(8, "little"), np.uint8)
+    return out
+
+
+def fill(lists, nodes):
+    """Lists that share few nodes, hash nodes left out."""
+    others = np.setdiff1d(np.arange(1024), nodes)
+    L, buckets, cap = lists.shape
+    b, k, r = np.ogrid[:L, :buckets, :cap]
+    lists[...] = others[(b * 450 + k * 13 + r) % others.size]
+
+
+def name_a_hash_node(lists, nodes):
+    fill(lists, nodes)
+    lists[:, :, 0] = nodes[1]
+
+
+def name_three_hash_nodes(lists, nodes):
+    fill(lists, nodes)
+    lists[:, :, (0, 5, 9)] = nodes[:3]
+
+
+def one_node_only(lists, nodes):
+    lists[...] = np.setdiff1d(np.arange(1024), nodes)[700]
+
+
+@pytest.mark.parametrize("edit,short", [(name_a_hash_node, False), (name_three_hash_nodes, False), (one_node_only, True)])
+@pytest.mark.parametrize("path,n,kernel", [("CLUSTER", 3, "cluster_lists_kernel"), ("STAGED", 80, "few_nodes_kernel")])
+def test_saved_lists_that_name_hash_nodes(edit, short, path, n, kernel):
+    """Loading checks the sizes and the checksum of the lists, not their entries.  An entry that names an always-active hash node
+    is not counted, and a query whose lists are too short is reported and takes the first nodes, as in the row kernels."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(912, [64, 1024, 1024, 40], [1, 1, 0], "bf16", n=n, n_cal=200, K=4, L=2, budgets=(200, 1000, 2000), list_cap=300)
+    wl.free_hash_nodes = True
+    dm = harness.DeviceModel(wl)
+    blob = sl.slonn_serialize(dm.model)
+    assert np.array_equal(edited(blob, [dm.tables(0), dm.tables(1)], [dm.hash_nodes(0), dm.hash_nodes(1)], lambda lists, nodes: None), blob)
+    blob = edited(blob, [dm.tables(0), dm.tables(1)], [dm.hash_nodes(0), dm.hash_nodes(1)], edit)
+    built, dm.model = dm.model, sl.slonn_deserialize(blob, dm.W, dm.bias)
+    got = []
+    for flags in (0, sl.FLAG_ROW_KERNELS):
+        b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=getattr(sl, "PATH_" + path), flags=flags)
+        names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes)]
+        assert (kernel in names) == (flags == 0)
+        got.append(b.results())
+    assert [bool(g["status"][0]) for g in got] == [short, short] and (not short or got[0]["status"][0] == -sl.ERR["ARG"])
+    for k in ("logits", "pred", "codes", "active_indptr", "active_ids", "active_vals"):
+        assert np.array_equal(got[0][k], got[1][k]), k
+    sl.slonn_free(built)
+    dm.free()

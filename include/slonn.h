@@ -323,7 +323,7 @@ int slonn_active_capacity(const slonn_model *m, uint32_t n_queries, uint32_t max
 int slonn_logit_stride(const slonn_model *m, uint32_t max_budget_bp, uint32_t *stride);
 /* Bytes of device workspace slonn_run needs (256-byte aligned buffer) for a batch with these
  * n_queries, max_budget_bp and flags.  For large batches up to about 170 MiB of it are scratch for evaluating 16 queries
- * at a time; slonn_run also takes a workspace without that part (the size with SLONN_FLAG_ROW_KERNELS) and then
+ * at a time, for batches of tens of queries (fewer than 256) up to about 24 MiB for grouping each query's inputs and nodes once; slonn_run also takes a workspace without that part (the size with SLONN_FLAG_ROW_KERNELS) and then
  * uses the kernels that need none, with the same results. */
 int slonn_workspace_bytes(const slonn_model *m, uint32_t n_queries, uint32_t max_budget_bp,
                           uint32_t flags, uint64_t *bytes);

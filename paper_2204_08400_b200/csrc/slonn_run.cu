@@ -242,6 +242,10 @@ void carve_tile(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
 // than SMs are one block each of layer_cols_kernel, where that applies (2048 inputs), as well as of few_select_kernel, so few nodes
 // do not pay there: 240 queries at 2 and 5 %, D 2048 0.92 0.99, 3072 0.91 1.04, fp32 0.91 0.95 and 0.89 0.99; D 1024 1.27 1.17.
 // Mixed budgets up to 60 %, 32 queries: 0.98 (100 queries 1.05); up to 100 %: rows.
+// Batches of 256 queries and more sort them and take grouped products; where they may not (SLONN_FLAG_UNGROUPED_ROWS) the kernels of
+// before fill the GPU: 5, 10, 25 and 50 %, 200 queries, D 4096 1.15 1.46 1.96 1.38, 2048 - 1.17 1.27 1.30; 512 queries 0.90 0.99 1.33
+// 1.29, - 0.92 1.01 1.29; 4096 queries 0.67 0.81 1.03 1.27, - 0.68 0.85 1.13, and scratch of 20 to 100 KB per query.
+#define SLONN_FEW_END SLONN_TILE_MIN_QUERIES // fewer queries than this
 #define SLONN_FEW_MAX_BP 5000u
 #define SLONN_FEW_INPUTS (48ull * 1024)      // queries times inputs; with a budget above 15 % (nine layers of 4096, 12 queries: 1.25 1.36 1.18 up to it,
 #define SLONN_FEW_INPUTS_HIGH (80ull * 1024) // 0.94 and 0.86 at 25 and 35 %; 24 queries 1.20 and 1.11)
@@ -257,7 +261,7 @@ bool few_layer_ok(const slonn_model *m, uint32_t l, uint32_t n, uint32_t max_bp)
 {
     const slonn_layer &ly = m->layer[l];
     if (l == 0 || !m->layer[l - 1].has_act || !ly.WT || ly.N % 4u != 0u || ly.D > SLONN_CLUSTER_MAX_D ||
-        ly.N > SLONN_CLUSTER_MAX_N || max_bp > SLONN_FEW_MAX_BP || (uint64_t)n * ly.D < (max_bp <= 1500u ? SLONN_FEW_INPUTS : SLONN_FEW_INPUTS_HIGH))
+        ly.N > SLONN_CLUSTER_MAX_N || n >= SLONN_FEW_END || max_bp > SLONN_FEW_MAX_BP || (uint64_t)n * ly.D < (max_bp <= 1500u ? SLONN_FEW_INPUTS : SLONN_FEW_INPUTS_HIGH))
         return false;
     if (!ly.has_act) return (uint64_t)n * ly.N >= SLONN_FEW_PLAIN && few_layer_ok(m, l - 1, n, max_bp);
     const uint32_t pre = slonn_model_pre(m), nodes = slonn_layer_nodes(max_bp, ly.N, pre);

@@ -63,3 +63,21 @@ def test_lines_of_the_dispatch():
         names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == 1]
         assert ("few_nodes_kernel" in names) == few, (dims, n, bp, names)
         dm.free()
+
+
+@pytest.mark.parametrize("n,few", [(255, True), (256, False), (700, False)])
+def test_batches_that_may_not_group_queries(n, few):
+    """Without grouped products these kernels would be all that is left of the forms with scratch: they end below 256 queries, and so
+    does their scratch."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(932, [64, 1024, 1024, 8], [1, 1, 0], "bf16", n=n, n_cal=64, K=4, L=2, budgets=(2500,))
+    dm = harness.DeviceModel(wl)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED, flags=sl.FLAG_UNGROUPED_ROWS)
+    names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == 1]
+    assert ("few_nodes_kernel" in names) == few, names
+    assert (b.ws_bytes > sl.slonn_workspace_bytes(dm.model, n, 2500, sl.FLAG_ROW_KERNELS)) == few
+    got = b.results()
+    rows = harness.run_once(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS)
+    for k in ("logits", "pred", "codes", "active_indptr", "active_ids", "active_vals"):
+        assert np.array_equal(got[k], rows[k]), k
+    dm.free()

@@ -9,13 +9,15 @@
 //      cuts the list at the budget (a handful of block barriers whatever the overlap of the lists);
 //   4. the block evaluates its share of the nodes, lane = node, in column order, a warp its two partial sums of all of them, 16
 //      loads per lane in flight; activations go to every block's copy of the next input.      cluster barrier
-// Two cluster barriers per layer as before, but B_out * B_in weights instead of B_out rows, and nothing from HBM that few queries in
-// a row do not share: nine layers of 4096 nodes, one query at 10 %, 154 -> 89 us a pass.  Of a layer's 8.5 us (clock stamps):
-// grouping 0.9, hash 2.1, selection 2.7 (list loads 1.0), nodes 1.8, delivery and barrier 1.7; a layer run by rows takes 13.
+// Two cluster barriers per layer as before, but B_out * B_in weights instead of B_out rows.  Nine layers of 4096 nodes, one query at
+// 10 %, whole rows and this form: 64 different queries in turn 121 and 88 us a pass, three models in turn 154 and 89, weights and code
+// from HBM 176 and 127.  Of a layer's 9.2 us (clock stamps): grouping 0.9, hash 2.1, selection 2.7 (list loads 1.0 of it),
+// nodes 1.8, delivery and barrier 1.7; a layer run by rows takes 13.
 // Every phase is short enough that its instruction count, times the four warps of a scheduler, is what it takes: all loads
 // in flight at once cost more in spills than they saved (lists_walk with 16 entries of both partial sums in flight 3.7 us, 8: 1.8).
-// Other clusters bringing the weights into L2 ahead of time: 104 us, as their lists and rows displace what the next query shares.
-// Layers whose input is dense run as in cluster_network_kernel.
+// Other clusters bringing the weights into L2 ahead of time: 104 us where queries follow one another (not measured from HBM).
+// Layers whose input is dense run as in cluster_network_kernel.  They share the selection's code with the others: fetched from HBM,
+// a second copy of it took 8 us of a pass (three layers of 1024 at 3 %: 43 us, now 34; by rows 35).
 #pragma once
 #include "slonn_cluster_kernel.cuh"
 
@@ -60,11 +62,21 @@ __device__ __forceinline__ bool lists_select(const lists_layer &ly, uint32_t K, 
     bool ok = true, listed = B != ly.N && want <= ly.cap; // not listed: nodes 0 .. B - 1 (all, or more than the lists hold, which the plan reports)
 
     uint32_t id[U], col[U];
+    {
+        uint32_t r = tid / L, b = tid - r * L; // rank and table of the thread's first position
+        const uint32_t rs = T / L, bs = T - rs * L;
+        if (bs == 0u) { // the others are of the same list
+            const IDT *list = reinterpret_cast<const IDT *>(ly.tables) + (((uint64_t)b << K) + key(b)) * ly.cap + r;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t p = u * T + tid;
-        const uint32_t r = L == 2u ? p >> 1 : p / L, b = p - r * L;
-        id[u] = listed && p < npos ? table_entry<IDT>(ly.tables, ly.cap, K, b, key(b), r) : 0xffffffffu;
+            for (int u = 0; u < U; ++u) id[u] = listed && u * T + tid < npos ? (uint32_t)__ldg(list + u * rs) : 0xffffffffu;
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                id[u] = listed && u * T + tid < npos ? table_entry<IDT>(ly.tables, ly.cap, K, b, key(b), r) : 0xffffffffu;
+                r += rs; b += bs;
+                if (b >= L) { b -= L; ++r; }
+            }
+        }
     }
     uint32_t hnode = tid < pre ? __ldg(ly.hash_nodes + tid) : 0xffffffffu, hcol = hnode; // always active
     for (uint32_t i = tid; i < (ly.N + 3u) / 4u; i += T) reinterpret_cast<uint4 *>(first)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -383,6 +395,8 @@ __global__ void __launch_bounds__(SLONN_CLUSTER_THREADS, 1) cluster_lists_kernel
             else if (to == 0) *cluster.map_shared_rank(&xout[by], 0) = z;
         };
 
+        uint2 *e0 = nullptr, *e1 = nullptr; // input-stationary: the grouped inputs of the warp's two partial sums
+        uint32_t m = 0, signs = 0;
         if (!ly.by_input) {
             if (ly.has_act) {
                 // FreeHash rows, spread over the cluster; each sum goes to every block
@@ -398,11 +412,35 @@ __global__ void __launch_bounds__(SLONN_CLUSTER_THREADS, 1) cluster_lists_kernel
                     for (uint32_t j = 0; j < P.K; ++j)
                         if (zh[tid * P.K + j] > 0.0f) key |= (1u << j);
                     keys[tid] = key;
-                    if (rank == 0 && P.codes) P.codes[((uint64_t)q * P.n_act + ly.a) * P.L + tid] = (uint16_t)key;
                 }
                 __syncthreads();
-                select(reinterpret_cast<uint32_t *>(entries()), [&](uint32_t b) { return keys[b]; });
             }
+        } else {
+            const uint32_t smax = cols_smax(ly.D, V), pitch = (smax + 3u) & ~3u;
+            e0 = entries() + warp * pitch; e1 = e0 + 16u * pitch;
+            uint32_t n0, n1;
+            m = lists_group<V>(xin, smax, warp, lane, e0, e1, n0, n1);
+            if (ly.has_act) {
+                // the hash functions' partial sums rank and rank + 16, to every block
+                if (warp == rank) {
+                    const float2 a = lists_hash<BF16>(e0, e1, m, P.layer[l].WH, lane);
+                    float *at = sums() + rank * 64u + (lane & 15u) * 2u;
+                    for (uint32_t to = lane >> 4; to < C; to += 2u) *cluster.map_shared_rank(reinterpret_cast<float2 *>(at), to) = a;
+                }
+                cluster.sync(); // also: the block has grouped its inputs
+                signs = __ballot_sync(SLONN_FULL_MASK, lane < H && lists_tree(sums(), lane) + s_hbias[l][lane] > 0.0f);
+            } else {
+                __syncthreads();
+            }
+        }
+        if (ly.has_act) {
+            auto key = [&](uint32_t b) { return ly.by_input ? (signs >> (b * P.K)) & ((1u << P.K) - 1u) : keys[b]; };
+            if (rank == 0 && P.codes && tid < P.L) P.codes[((uint64_t)q * P.n_act + ly.a) * P.L + tid] = (uint16_t)key(tid);
+            // the marks lie where the input was, or the grouped inputs would be; as an offset, so that it stays an address of shared memory
+            // (a choice of two pointers: 1 % slower)
+            select(reinterpret_cast<uint32_t *>(smem_c + (!ly.by_input ? s_at[0] : l & 1u ? P.xbuf_floats * 4u : 0u)), key);
+        }
+        if (!ly.by_input) {
             for (uint32_t r = gwarp; r < B; r += gwarps) {
                 const uint32_t nd = ly.has_act ? active_set().node[r] : r;
                 const float b = __ldg(ly.bias + nd);
@@ -412,28 +450,7 @@ __global__ void __launch_bounds__(SLONN_CLUSTER_THREADS, 1) cluster_lists_kernel
             __syncthreads();
             clear(xin);
         } else {
-            // the nonzero inputs of the warp's two partial sums
-            const uint32_t smax = cols_smax(ly.D, V), pitch = (smax + 3u) & ~3u;
-            uint2 *e0 = entries() + warp * pitch, *e1 = e0 + 16u * pitch;
-            uint32_t n0, n1;
-            const uint32_t m = lists_group<V>(xin, smax, warp, lane, e0, e1, n0, n1);
-            uint32_t buf = 0;
-            if (ly.has_act) {
-                // the hash functions' partial sums rank and rank + 16, to every block
-                if (warp == rank) {
-                    const float2 a = lists_hash<BF16>(e0, e1, m, P.layer[l].WH, lane);
-                    float *at = sums() + rank * 64u + (lane & 15u) * 2u;
-                    for (uint32_t to = lane >> 4; to < C; to += 2u) *cluster.map_shared_rank(reinterpret_cast<float2 *>(at), to) = a;
-                }
-                cluster.sync(); // also: the block has grouped its inputs
-                const uint32_t signs = __ballot_sync(SLONN_FULL_MASK, lane < H && lists_tree(sums(), lane) + s_hbias[l][lane] > 0.0f);
-                auto key = [&](uint32_t b) { return (signs >> (b * P.K)) & ((1u << P.K) - 1u); };
-                if (rank == 0 && P.codes && tid < P.L) P.codes[((uint64_t)q * P.n_act + ly.a) * P.L + tid] = (uint16_t)key(tid);
-                select(reinterpret_cast<uint32_t *>(xin), key);
-                buf = 1;
-            } else {
-                __syncthreads();
-            }
+            uint32_t buf = ly.has_act; // the set of sums that the hash functions' have left free
             if (!is_last) clear(xin);
             // the block's share of the nodes, up to 64 at a time
             const uint32_t per = (B + C - 1u) / C, r0 = min(rank * per, B), r1 = min(r0 + per, B);

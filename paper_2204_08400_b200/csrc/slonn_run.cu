@@ -1165,11 +1165,13 @@ int launch_cluster_t(cluster_kernel kernel, uint32_t THREADS, const slonn_cluste
     return cudaLaunchKernelEx(&cfg, kernel, P) == cudaSuccess ? SLONN_OK : SLONN_ERR_CUDA;
 }
 
-// When the cluster's list-fed layers run input-stationary: speed over whole rows, one to four queries, weights of two batches in turn.
-// bf16, 4096 x 4096, nine layers, 1 / 5 / 10 / 15 / 25 %: 1.40 1.43-1.59 1.62-1.70 1.38-1.58 0.96-1.15 (10 %: 142 -> 88 us); four
-// layers of width 1024 / 1536 / 2048 / 3072 / 4096, least of 3 to 20 %: 1.07 1.06 1.03 1.06 1.11, fp32 1.02 1.06 1.08 1.07
-// 1.36; 25 % of 2048 0.99-1.00, fp32 0.95-0.98, 50 % 0.88-0.90: beyond 20 % a block's share is more than one pass of its lanes and
-// the row form, which streams, wins.  Every node computed, 1024 wide: 0.75-0.79; 784-112-112-10: 0.92-1.00: nothing to skip.
+// When the cluster's list-fed layers run input-stationary: speed over whole rows, one, two and four queries, 32 or 64 different batches in
+// turn, and every pass with weights and code from HBM:
+//   bf16, nine layers of 4096, 1 / 3 / 10 / 15 / 20 %: 1.39-1.42 1.37 1.37-1.43 1.32-1.38 1.25-1.30; HBM 1.58-1.64 1.49-1.52 1.35-1.38 1.20 1.14-1.19
+//   five layers of 1024 / 1536 / 2048 / 3072 / 4096, least of 1 to 20 %: bf16 1.10 1.06 1.08 1.11 1.13, HBM 1.01 1.05 1.04 1.11 1.13;
+//   fp32 1.05 1.09 1.14 1.15 1.22, HBM 0.97 1.05 1.11 1.08 1.16 (three layers of 1024 at 20 %, HBM: 0.96)
+// Two batches in turn, 25 % of 2048 0.99-1.00, fp32 0.95-0.98, 50 % 0.88-0.90: beyond 20 % a block's share is more than one pass of its
+// lanes and the row form, which streams, wins.  Every node computed, 1024 wide: 0.75-0.79; 784-112-112-10: 0.92-1.00: nothing to skip.
 #define SLONN_LISTS_MAX_BP 2000u
 #define SLONN_LISTS_MIN_WIDTH 1024u // of at least one such layer
 

@@ -237,7 +237,7 @@ void carve_tile(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
 //   D 4096, 12 queries 1.05 1.08 1.18 1.19 1.01 1.02; 80 queries 1.31 1.01 1.03 1.14 1.35 1.20; 150 queries - 1.14 1.31 2.59 2.88 -
 //   D 2048, 28 queries 1.02 1.04 1.15 1.13 1.03 1.13; 80 queries 1.00 1.16 1.02 1.03 1.17 1.19; 16 queries 0.96 0.97 1.02 1.13 1.10 0.97
 //   D 1024, 28 queries 0.96 0.93 0.96 0.98 1.03 0.96; 48 queries 0.96 0.96 1.07 1.11 1.00 1.09; 150 queries 1.10 1.14 1.13 1.17 1.13 1.15
-// fp32 the same or better (4096, 28 queries at 10 %, 48 queries at 5 %, 3072, 80 queries at 5 and 10 %: 0.98 to 0.99, the least).  Fewer inputs
+// fp32 the same or better but for the case below.  Fewer inputs
 // than the first line below, or a block's runs mostly empty, and the second launch costs more than the first saves.  More queries
 // than SMs are one block each of layer_cols_kernel, where that applies (2048 inputs), as well as of few_select_kernel, so few nodes
 // do not pay there: 240 queries at 2 and 5 %, D 2048 0.92 0.99, 3072 0.91 1.04, fp32 0.91 0.95 and 0.89 0.99; D 1024 1.27 1.17.
@@ -252,6 +252,17 @@ void carve_tile(const slonn_model *m, uint32_t n, uint32_t max_bp, uint32_t flag
 #define SLONN_FEW_NODES 60u             // nodes per query
 #define SLONN_FEW_WAVE 148u             // more queries than this on wide layers:
 #define SLONN_FEW_NODES_WAVE 128u       // this many
+// The host knows the largest budget only.  Where that is more nodes than this and the others are small, few blocks walk long lists: 5, 10, 25 and
+// 50 % evenly, or one of 16 at 50 % and the others at 1 %, on 4096, 32 queries 0.94 0.95 (fp32 0.98 0.85), 40 and 48 queries 1.09-1.16
+// (fp32 1.02-1.27); 5, 12 and 25 % on 8192, 10, 16 and 24 queries 0.86 0.89 1.02 (fp32 0.95 0.95 1.22).  All at 50 %, 24 and 32: 1.17 1.24.  Up to
+// 35 % of 4096, 20 queries and more, such batches 1.00-1.16 (fp32 0.99-1.18), with weights from HBM down to 0.87 (0.96).
+#define SLONN_FEW_LONG 1640u
+#define SLONN_FEW_LONG_QUERIES 40u
+// fp32, wide, where layer_cols_kernel is the alternative and reads its weights in as long requests: 48, 64, 80, 100 queries, 5 % of 4096
+// 1.00 0.99 1.00 0.98, 3072 - 0.98 0.97 0.97, 7 % 1.02 0.97 0.98 0.95, 8 % of 2048 - 1.01 1.00 1.00; above: 6 % of 4096 and 8 % of 3072
+// 1.00-1.03; 140 queries 0.99-1.09; bf16, 5 % 1.03-1.08
+#define SLONN_FEW_F32_NODES 216u
+#define SLONN_FEW_F32_QUERIES 128u
 // A layer without activator, behind a layer that takes them: both launches against one of gather_cols_kernel, 5, 15 and 35 %: 64 queries, 1000
 // outputs 1.04-1.29 1.03-1.23 1.04-1.19, 100 outputs 0.97-1.10; 24 queries, 1000 outputs 0.95-1.00 0.98-1.02 1.00-1.20; 12 outputs 0.90-0.98.
 #define SLONN_FEW_PLAIN (48ull * 1024)  // queries times outputs
@@ -266,6 +277,9 @@ bool few_layer_ok(const slonn_model *m, uint32_t l, uint32_t n, uint32_t max_bp)
     if (!ly.has_act) return (uint64_t)n * ly.N >= SLONN_FEW_PLAIN && few_layer_ok(m, l - 1, n, max_bp);
     const uint32_t pre = slonn_model_pre(m), nodes = slonn_layer_nodes(max_bp, ly.N, pre);
     if (!ly.WH || !ly.colpos || (uint64_t)(nodes - pre) * m->L > SLONN_LISTS_POSITIONS) return false;
+    if (nodes > SLONN_FEW_LONG && n < SLONN_FEW_LONG_QUERIES) return false;
+    if (m->dtype == SLONN_F32 && ly.D >= 2048u && max_bp <= 1500u && nodes < SLONN_FEW_F32_NODES && n <= SLONN_FEW_F32_QUERIES && (uint64_t)n * nodes > 148ull * 64)
+        return false;
     return nodes >= (n > SLONN_FEW_WAVE && ly.D >= 2048u ? SLONN_FEW_NODES_WAVE : SLONN_FEW_NODES);
 }
 

@@ -14,7 +14,7 @@ CASES = {
     "smallest": dict(dims=[64, 1024, 1024, 36], act=[1, 1, 0], dtype="bf16", n=80, budgets=(1, 100, 5000)),
     "ragged": dict(dims=[136, 1160, 1036, 596], act=[1, 1, 1], dtype="f32", n=97, budgets=(300, 2000, 4900), K=7, L=3),
     "more_queries_than_sms": dict(dims=[64, 1032, 1304, 44], act=[1, 1, 0], dtype="bf16", n=173, budgets=(1000, 2500)),
-    "widest": dict(dims=[32, 8192, 8192, 20], act=[1, 1, 0], dtype="bf16", n=10, budgets=(2000, 2500)),       # 4096 list positions
+    "widest": dict(dims=[32, 8192, 8192, 20], act=[1, 1, 0], dtype="bf16", n=40, budgets=(2000, 2500)),       # 4096 list positions
     "eight_tables": dict(dims=[64, 2048, 1400, 52], act=[1, 1, 1], dtype="f32", n=41, budgets=(900, 3600), K=4, L=8),
     "short_lists": dict(dims=[64, 2056, 1024, 12], act=[1, 1, 0], dtype="bf16", n=40, budgets=(200, 2000), list_cap=430, free_hash=True),
     "small_layer": dict(dims=[64, 1024, 120, 24], act=[1, 1, 1], dtype="bf16", n=81, budgets=(1, 400, 5000), K=3, L=2),
@@ -55,6 +55,11 @@ def test_lines_of_the_dispatch():
     from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
     for dims, n, bp, few in (([64, 1024, 1024, 8], 80, 1501, True), ([64, 1024, 1024, 8], 79, 1501, False), ([64, 1024, 1024, 8], 48, 1000, True), ([64, 1024, 1024, 8], 47, 1000, False), ([64, 1024, 1024, 8], 48, 500, False),
                              ([64, 1024, 1024, 8], 150, 1000, True), ([64, 2048, 2048, 8], 150, 600, False), ([64, 2048, 2048, 8], 150, 700, True),
+                             # more than 1640 nodes: 40 queries
+                             ([64, 4096, 4096, 8], 39, 4000, True), ([64, 4096, 4096, 8], 39, 4100, False), ([64, 4096, 4096, 8], 40, 4100, True),
+                             # fp32, 2048 inputs and more: layer_cols_kernel keeps 9472 nodes of a batch and more, up to 215 a query and 128 queries
+                             ([64, 2048, 2052, 8], 80, 1000, False), ([64, 2048, 2052, 8], 80, 1100, True), ([64, 2048, 2052, 8], 46, 1000, True),
+                             ([64, 2048, 2052, 8], 128, 1000, False), ([64, 2048, 2052, 8], 129, 1000, True),
                              ([64, 1024, 1022, 8], 90, 2500, False), ([64, 1024, 1024, 8], 90, 5001, False)):
         wl = custom_workload(931, dims, [1, 1, 0], "f32" if dims[2] % 8 else "bf16", n=n, n_cal=64, K=4, L=2, budgets=(bp,)) if dims[2] % 4 == 0 else \
             custom_workload(931, dims[:2] + [dims[2]], [1, 1], "bf16", n=n, n_cal=64, K=4, L=2, budgets=(bp,))

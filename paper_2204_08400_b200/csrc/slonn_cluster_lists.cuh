@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(SLONN_CLUSTER_THREADS, 1) cluster_lists_kernel
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     constexpr uint32_t T = SLONN_CLUSTER_THREADS, W = T / 32u, V = BF16 ? 8u : 4u, ESZ = BF16 ? 2u : 4u;
+    static_assert(SLONN_CLUSTER_SIZE == 16 && W == 16u, "warp r of block r computes the hash functions' partial sums r and r + 16");
     extern __shared__ float4 smem4[];
     __shared__ float zh[128];
     __shared__ uint32_t keys[8];

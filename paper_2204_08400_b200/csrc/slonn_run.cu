@@ -1261,8 +1261,9 @@ int launch_cluster(const slonn_model *m, const slonn_batch *b, uint32_t max_bp, 
     slonn_cluster_params Q = P;
     size_t lists_smem = 0;
     if (!(b->flags & SLONN_FLAG_ROW_KERNELS) && cluster_lists_params(m, max_bp, Q, &lists_smem)) {
-        TIC_BY_INPUT();
-        return launch_cluster_t(bf ? cluster_lists_kernel<true> : cluster_lists_kernel<false>, SLONN_CLUSTER_THREADS, Q, lists_smem, st);
+        const int rc = launch_cluster_t(bf ? cluster_lists_kernel<true> : cluster_lists_kernel<false>, SLONN_CLUSTER_THREADS, Q, lists_smem, st);
+        if (rc == SLONN_OK) TIC_BY_INPUT();
+        if (rc != SLONN_ERR_DIM) return rc; // else such a cluster does not fit the device; that of the row form, with less shared memory, may
     }
     return launch_cluster_t(bf ? cluster_network_kernel<true, SLONN_CLUSTER_THREADS, 1> : cluster_network_kernel<false, SLONN_CLUSTER_THREADS, 1>,
                             SLONN_CLUSTER_THREADS, P, smem, st);

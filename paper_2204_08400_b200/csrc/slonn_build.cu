@@ -96,36 +96,20 @@ __global__ void hash_matrix_kernel(const void *W, void *WH, uint32_t D, uint32_t
 }
 
 // How early each node appears in the layer's ranked lists: score[n] = sum over all lists of
-// max(0, T - rank of n in the list).  Integer sums, so the result does not depend on thread order.  A block adds up its lists in
-// shared memory where the layer's scores fit (2 M atomics on as few addresses as a layer has nodes otherwise).  Ordering the nodes
-// that no list has among its first T as well (by the sum of 1 / (rank + N / 16)) brought 64 queries at 25 % from 331 to 317 us and
-// cost 777 queries of mixed budgets 3 % (1568 wide, 348 -> 360 us), 300 queries at 25 % 3 % (2048 wide): left out.
-#define POPULARITY_LISTS 16      // lists per block
-#define POPULARITY_SHARED 40960u // most nodes whose scores fit
+// max(0, T - rank of n in the list).  Integer sums, so the result does not depend on thread order.  A thread per entry: 2048 lists of 512 on 4096
+// nodes 21 us; a block per 16 lists, sums in shared memory where they fit, took 13, but 262 instead of 5 for 32 lists of 8192 on 65,536 nodes.
+// Ordering the nodes that no list has among its first T as well (by the sum of 1 / (rank + N / 16)) brought 64 queries at 25 % from 331 to 317 us
+// and cost 777 queries of mixed budgets 3 % (1568 wide, 348 -> 360 us), 300 queries at 25 % 3 % (2048 wide): left out.
 template <typename IDT>
-__global__ void __launch_bounds__(256) popularity_kernel(const IDT *tables, uint64_t n_lists, uint32_t cap, uint32_t T, uint32_t N,
-                                                         unsigned long long *score)
+__global__ void popularity_kernel(const IDT *tables, uint64_t n_lists, uint32_t cap, uint32_t T, uint32_t N,
+                                  unsigned long long *score)
 {
-    extern __shared__ uint32_t s_score[];
-    const bool shared = N <= POPULARITY_SHARED;
-    if (shared) {
-        for (uint32_t i = threadIdx.x; i < N; i += 256) s_score[i] = 0u;
-        __syncthreads();
-    }
-    const uint64_t l0 = (uint64_t)blockIdx.x * POPULARITY_LISTS, l1 = min(l0 + POPULARITY_LISTS, n_lists);
-    for (uint32_t r = threadIdx.x; r < T; r += 256) {
-        const uint32_t w = T - r;
-        for (uint64_t l = l0; l < l1; ++l) {
-            const uint32_t id = (uint32_t)tables[l * cap + r];
-            if (id >= N) continue;
-            if (shared) atomicAdd(s_score + id, w);
-            else atomicAdd(score + id, (unsigned long long)w);
-        }
-    }
-    if (!shared) return;
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < N; i += 256)
-        if (s_score[i]) atomicAdd(score + i, (unsigned long long)s_score[i]);
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t list = t / T;
+    const uint32_t r = (uint32_t)(t - list * T);
+    if (list >= n_lists) return;
+    const uint32_t id = (uint32_t)tables[list * cap + r];
+    if (id < N) atomicAdd(score + id, (unsigned long long)(T - r));
 }
 
 // Library-owned copies for the kernels that read weights by input (a first layer with dense input, and layers
@@ -170,15 +154,13 @@ int make_transposed_copies(slonn_model *m, cudaStream_t st, int phase)
         std::vector<uint32_t> order(ly.N), colpos(ly.N);
         bool ok = cudaMemsetAsync(d_score, 0, sizeof(unsigned long long) * ly.N, st) == cudaSuccess;
         if (ok) {
-            const uint32_t blocks = (uint32_t)((n_lists + POPULARITY_LISTS - 1) / POPULARITY_LISTS);
-            const size_t smem = ly.N <= POPULARITY_SHARED ? (size_t)ly.N * 4 : 0;
-            const void *kernel = ly.id_bytes == 2 ? (const void *)popularity_kernel<uint16_t> : (const void *)popularity_kernel<uint32_t>;
-            if (slonn_allow_smem(kernel, smem) != SLONN_OK) ok = false;
-            else if (ly.id_bytes == 2)
-                popularity_kernel<uint16_t><<<blocks, 256, smem, st>>>((const uint16_t *)ly.tables, n_lists, ly.cap, T, ly.N, d_score);
+            const uint64_t threads = n_lists * T;
+            const uint32_t blocks = (uint32_t)((threads + 255) / 256);
+            if (ly.id_bytes == 2)
+                popularity_kernel<uint16_t><<<blocks, 256, 0, st>>>((const uint16_t *)ly.tables, n_lists, ly.cap, T, ly.N, d_score);
             else
-                popularity_kernel<uint32_t><<<blocks, 256, smem, st>>>((const uint32_t *)ly.tables, n_lists, ly.cap, T, ly.N, d_score);
-            ok = ok && cudaGetLastError() == cudaSuccess &&
+                popularity_kernel<uint32_t><<<blocks, 256, 0, st>>>((const uint32_t *)ly.tables, n_lists, ly.cap, T, ly.N, d_score);
+            ok = cudaGetLastError() == cudaSuccess &&
                  cudaMemcpyAsync(score.data(), d_score, sizeof(unsigned long long) * ly.N, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
                  cudaStreamSynchronize(st) == cudaSuccess;
         }

@@ -66,9 +66,10 @@ __device__ __forceinline__ bool lists_select(const lists_layer &ly, uint32_t K, 
         uint32_t r = tid / L, b = tid - r * L; // rank and table of the thread's first position
         const uint32_t rs = T / L, bs = T - rs * L;
         if (bs == 0u) { // the others are of the same list
-            const IDT *list = reinterpret_cast<const IDT *>(ly.tables) + (((uint64_t)b << K) + key(b)) * ly.cap + r;
+            const uint64_t bucket = ((uint64_t)b << K) + key(b);
+            const IDT *ranked = reinterpret_cast<const IDT *>(ly.tables) + bucket * ly.cap + r;
 #pragma unroll
-            for (int u = 0; u < U; ++u) id[u] = listed && u * T + tid < npos ? (uint32_t)__ldg(list + u * rs) : 0xffffffffu;
+            for (int u = 0; u < U; ++u) id[u] = listed && u * T + tid < npos ? (uint32_t)__ldg(ranked + u * rs) : 0xffffffffu;
         } else {
 #pragma unroll
             for (int u = 0; u < U; ++u) {

@@ -12,7 +12,7 @@ CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_220
 FILES = sorted(os.path.basename(p) for p in glob.glob(os.path.join(CSRC, "*.cuh"))) + ["slonn_run.cu", "slonn_dense_tc.cu"]
 # members and arguments that hold what a kernel of the chain wrote
 WRITTEN = {"dense", "ids", "vals", "indptr", "idlist", "order", "list", "count", "work", "items", "kseg", "krow", "xt", "ucol",
-           "ucount", "bm", "pre", "key", "sort_key", "out_ids", "out_vals", "tile_sums", "logits", "row_count", "row_map"}
+           "ucount", "bm", "pre", "key", "sort_key", "ent", "seg", "gseg", "nodes", "quads", "out_ids", "out_vals", "tile_sums", "logits", "row_count", "row_map"}
 
 
 def read_only_loads(text):
@@ -42,6 +42,8 @@ def test_what_the_chain_writes_is_read_with_plain_loads(name):
 def test_the_check_sees_direct_and_renamed_loads():
     for body in ("__device__ void f() { const float4 *src = (const float4 *)(in.dense + q); v = __ldg(src + i); }",
                  "__global__ void k(P p) { x = __ldg(P.ids + off + r); }",
+                 "__global__ void k(P p) { const uint2 *at = Q.quads + q * Q.quad_stride; v = __ldg(at + r0); }",
+                 "__global__ void k(P p) { seg[tid] = __ldg(gseg + tid); v = __ldg(Q.ent + i); }",
                  "__global__ void k(P p) { const float *vals = P.in.vals + s; x = in ? __ldg(vals + i) : 0.0f; }"):
         arg, names, aliases = next(iter(read_only_loads(body)))
         assert names & (WRITTEN | aliases), body

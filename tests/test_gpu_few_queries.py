@@ -1,6 +1,7 @@
 """List-fed layers of batches of tens of queries (few_select_kernel, few_nodes_kernel) against the oracle: last runs of four columns and
 last blocks half full, more queries than SMs, every number of list positions per thread, tables whose number does not divide
-a block, budgets that differ, inputs that are all zero, plain layers; and a workspace without their scratch."""
+a block, budgets that differ, inputs that are all zero, infinities and NaNs, plain layers in the middle and at the end; a workspace
+without their scratch, a saved model, and queries from host memory."""
 import numpy as np
 import pytest
 
@@ -17,6 +18,11 @@ CASES = {
     "widest": dict(dims=[32, 8192, 8192, 20], act=[1, 1, 0], dtype="bf16", n=40, budgets=(2000, 2500)),       # 4096 list positions
     "eight_tables": dict(dims=[64, 2048, 1400, 52], act=[1, 1, 1], dtype="f32", n=41, budgets=(900, 3600), K=4, L=8),
     "short_lists": dict(dims=[64, 2056, 1024, 12], act=[1, 1, 0], dtype="bf16", n=40, budgets=(200, 2000), list_cap=430, free_hash=True),
+    # layers without activator: the last block of runs a third full, the last run of columns the only one of its block
+    "plain_last": dict(dims=[64, 1024, 1024, 1036], act=[1, 1, 0], dtype="bf16", n=64, budgets=(300, 1000, 1500), plain=2),
+    "plain_last_f32": dict(dims=[64, 1028, 1024, 772], act=[1, 1, 0], dtype="f32", n=65, budgets=(1, 900, 1500), K=7, L=3, plain=2),
+    "plain_between": dict(dims=[64, 1024, 1032, 1032, 72], act=[1, 1, 0, 0], dtype="bf16", n=80, budgets=(200, 2000), free_hash=True, list_cap=300, plain=2),
+    "plain_between_f32": dict(dims=[64, 1024, 1024, 900, 1028, 24], act=[1, 1, 0, 1, 0], dtype="f32", n=96, budgets=(500, 3500), plain=2),
     "small_layer": dict(dims=[64, 1024, 120, 24], act=[1, 1, 1], dtype="bf16", n=81, budgets=(1, 400, 5000), K=3, L=2),
 }
 
@@ -37,6 +43,9 @@ def test_layers_of_few_queries_match_the_oracle(name, dead):
     b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
     names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == 1]
     assert names == ["few_select_kernel", "few_nodes_kernel"]
+    if "plain" in c:
+        names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == c["plain"]]
+        assert names == ["few_nodes_kernel"]
     for _ in range(2):
         b.run()
         assert_run_parity(b.results(), o32, o64, wl, sum(wl.has_act), bool(wl.has_act[-1]))
@@ -85,4 +94,64 @@ def test_batches_that_may_not_group_queries(n, few):
     rows = harness.run_once(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED, flags=sl.FLAG_ROW_KERNELS | sl.FLAG_UNGROUPED_ROWS)
     for k in ("logits", "pred", "codes", "active_indptr", "active_ids", "active_vals"):
         assert np.array_equal(got[k], rows[k]), k
+    dm.free()
+
+
+@pytest.mark.parametrize("n,last,few", [(48, 1024, True), (48, 1020, False), (64, 768, True), (64, 764, False)])
+def test_lines_of_plain_layers(n, last, few):
+    """Queries times outputs: 48 K."""
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(933, [64, 1024, 1024, last], [1, 1, 0], "bf16", n=n, n_cal=64, K=4, L=2, budgets=(1000,))
+    dm = harness.DeviceModel(wl)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp, kernel_path=sl.PATH_STAGED)
+    names = [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes) if r["layer"] == 2]
+    assert ("few_nodes_kernel" in names) == few, names
+    dm.free()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("path,n", [("CLUSTER", 4), ("STAGED", 64)])
+def test_infinities_and_nans(dtype, path, n):
+    """Infinite and NaN inputs give what the row kernels give, and leave the other queries of the batch alone."""
+    from paper_2204_08400_b200 import binding as sl, harness
+    wl = custom_workload(934, [64, 1024, 1032, 1036], [1, 1, 0], dtype, n=n, n_cal=200, K=6, L=2, budgets=(300, 1500))
+    w = wl.W_store[1]   # every other node of the second layer adds up positive weights, so that infinities stay infinities
+    w[::2] = np.abs(w[::2]) if dtype == "f32" else w[::2] & 0x7FFF
+    dm = harness.DeviceModel(wl)
+    x = wl.x.copy()
+    x[1::4, 3], x[2::4, 9], x[2::4, 11] = np.inf, np.nan, -np.inf
+    clean, dirty = (harness.run_once(dm, v, wl.budget_bp, kernel_path=getattr(sl, "PATH_" + path)) for v in (wl.x, x))
+    rows = harness.run_once(dm, x, wl.budget_bp, kernel_path=getattr(sl, "PATH_" + path), flags=sl.FLAG_ROW_KERNELS)
+    assert np.isinf(dirty["active_vals"]).any() and np.isnan(dirty["logits"][1::4]).any()
+    for k in ("logits", "pred", "codes", "active_indptr", "active_ids", "active_vals"):
+        assert np.array_equal(dirty[k], rows[k], equal_nan=dirty[k].dtype == np.float32), k
+    others = [q for q in range(n) if q % 4 in (0, 3)]
+    assert np.array_equal(clean["logits"][others], dirty["logits"][others])
+    dm.free()
+
+
+@pytest.mark.parametrize("n,kernel", [(3, "cluster_lists_kernel"), (64, "few_nodes_kernel")])
+def test_saved_models_and_host_buffers(n, kernel):
+    """The copies these kernels read are made again on loading; queries in host memory take the same kernels in the call's own workspace."""
+    import torch
+    from paper_2204_08400_b200 import accounting as acc, binding as sl, harness
+    wl = custom_workload(935, [64, 1024, 1040, 1020], [1, 1, 0], "bf16", n=n, n_cal=200, K=6, L=2, budgets=(400, 1500))
+    dm = harness.DeviceModel(wl)
+    want = harness.run_once(dm, wl.x, wl.budget_bp)
+    built, dm.model = dm.model, sl.slonn_deserialize(sl.slonn_serialize(dm.model), dm.W, dm.bias)
+    sl.slonn_free(built)
+    b = harness.DeviceBatch(dm, wl.x, wl.budget_bp)
+    assert kernel in [acc.kernel_name(acc.NetShape.of(wl), r) for r in sl.slonn_run_traced(dm.model, b.batch, b.ws, b.ws_bytes)]
+    b.run()
+    got = b.results()
+    for k in ("logits", "pred", "codes", "active_indptr", "active_ids", "active_vals"):
+        assert np.array_equal(got[k], want[k]), k
+    full = sl.slonn_host_workspace_bytes(dm.model, n, 1500)
+    least = sl.slonn_host_workspace_bytes(dm.model, n, 1500, flags=sl.FLAG_ROW_KERNELS)
+    for nb in {full, least}: # with and without scratch
+        logits, pred, status = np.zeros((n, 1020), np.float32), np.zeros(n, np.uint32), np.ones(4, np.uint32)
+        hb = sl.make_batch(n, np.ascontiguousarray(wl.budget_bp), logits, status, x_dense=np.ascontiguousarray(wl.x), max_budget_bp=1500, pred=pred)
+        sl.slonn_run_host(dm.model, hb, torch.empty(nb, dtype=torch.uint8, device=dm.device), nb)
+        assert status[0] == 0
+        assert np.array_equal(logits, want["logits"]) and np.array_equal(pred, want["pred"])
     dm.free()

@@ -10,7 +10,7 @@
 //   4. the block evaluates its share of the nodes, lane = node, in column order, a warp its two partial sums of all of them, 16
 //      loads per lane in flight; activations go to every block's copy of the next input.      cluster barrier
 // Two cluster barriers per layer as before, but B_out * B_in weights instead of B_out rows.  Nine layers of 4096 nodes, one query at
-// 10 %, whole rows and this form: 64 different queries in turn 121 and 88 us a pass, three models in turn 154 and 89, weights and code
+// 10 %, whole rows and this form: 64 different queries in turn 121 and 88 us a pass, three models in turn 156 and 87, weights and code
 // from HBM 176 and 127.  Of a layer's 9.2 us (clock stamps): grouping 0.9, hash 2.1, selection 2.7 (list loads 1.0 of it),
 // nodes 1.8, delivery and barrier 1.7; a layer run by rows takes 13.
 // Every phase is short enough that its instruction count, times the four warps of a scheduler, is what it takes: all loads

@@ -5,13 +5,13 @@
 //   few_select_kernel   one block per query: groups the nonzero inputs, hash functions, keys, selection, nodes in column order;
 //                       what the other launch needs of it goes to scratch (a layer without activator: the grouped inputs only)
 //   few_nodes_kernel    one block per (query, 32 runs of four columns): its warps share the 32 partial sums, as gather_cols_kernel's split form
-// 64 queries at 25 % on nine layers of 4096 nodes: 496 us a pass with hash_select_kernel and whole rows (a layer 12 and 46 us, the rows at 11.7
-// TB/s from L2), 335 with these (13 and 26).
+// 64 queries at 25 % on nine layers of 4096 nodes: 495 us a pass with hash_select_kernel and whole rows, 327 with these.  Launch by launch
+// between events a layer takes 17 and 50 us (rows at 11.7 TB/s from L2), with these 17 and 30.
 #pragma once
 #include "slonn_cluster_lists.cuh"
 
 #ifndef SLONN_FEW_BLOCKS
-#define SLONN_FEW_BLOCKS 5 // 48 registers; 4: 369 us, 6: 379, 8: 577 (64 queries at 25 % on nine layers of 4096 nodes, 5: 366)
+#define SLONN_FEW_BLOCKS 5 // 48 registers.  64 queries at 25 % on nine layers of 4096 nodes, 4 / 5 / 6: 378 / 334 / 364 us, 24 at 25 % 277 / 278 / 317, 64 at 10 % 175 / 176 / 180
 #endif
 #define SLONN_FEW_SEG 36 // words of scratch for a query's borders of partial sums and number of quads
 
@@ -167,10 +167,10 @@ __device__ __forceinline__ void few_add(const uint32_t (&w)[BF16 ? 2 : 4], uint3
     }
 }
 
-// What bounds it is the way from L2: a query's columns in sectors, 8.4 TB/s, the L1 68 % busy.  Lane = run of four columns: in column
+// What bounds it is the way from L2: a query's columns in sectors, 8.6 TB/s under the profiler, the L1 68 % busy.  Lane = run of four columns: in column
 // order most of a run's columns are selected, and a request brings 32 of them instead of 32 columns (64 queries at 25 %, 4096 x
-// 4096: 37 us a layer with a column or two per lane, 26 with runs; blocks of one SM on neighbouring queries' same columns, for L1
-// hits, measured with two columns per lane: 42).
+// 4096, without events: 37 us a layer with a column or two per lane, 26 with runs; blocks of one SM on neighbouring queries' same
+// columns, for L1 hits, measured with two columns per lane: 42).
 template <bool BF16>
 __global__ void __launch_bounds__(SLONN_THREADS, SLONN_FEW_BLOCKS) few_nodes_kernel(const __grid_constant__ slonn_few_params Q)
 {

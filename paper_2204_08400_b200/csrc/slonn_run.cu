@@ -761,7 +761,7 @@ template <bool BF16>
 int launch_few_t(const slonn_few_params &Q, uint32_t n, size_t select_smem, size_t nodes_smem, cudaStream_t st, stage_timer *tm)
 {
     const slonn_gather_params &G = Q.G;
-    // few_select_kernel has 7 KB of static shared memory, more than slonn_allow_smem reckons with below 48 KB
+    // few_select_kernel has 4.6 KB of static shared memory, more than slonn_allow_smem reckons with below 48 KB
     int rc = set_smem(few_select_kernel<BF16>, std::max<size_t>(select_smem, 48 * 1024));
     if (!rc) rc = set_smem(few_nodes_kernel<BF16>, nodes_smem);
     if (rc) return rc;
